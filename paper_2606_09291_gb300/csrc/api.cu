@@ -703,7 +703,7 @@ static mlsgd_status step_core(mlsgd_ctx* ctx, const mlsgd_level_stats* stats, in
   const double denom = std::max(floor_y, ey);
   if (!std::isfinite(denom) || !std::isfinite(cstar)) return fail(ctx, MLSGD_ENONFINITE, "mlsgd_step: non-finite shift");
   const long long nc = cells_of(ctx->Nc());
-  const int nblk = (int)((nc + 255) / 256);
+  const int nblk = combine_blocks(nc);
   const int rows = n_levels + 5;
   const size_t part_bytes = al((size_t)(rows + 1) * nblk * 8 + 64 * 8);
   mlsgd_status s = ensure_ws(ctx, part_bytes + al(16 * 8) + (adaptive ? al((size_t)nc * 8) : 0), st);

@@ -788,33 +788,75 @@ void launch_stats_reset(double* field, double* scalars, long long ncells, cudaSt
 }
 
 // Chan merge of two statistics records: src into dst, both rescaled to the larger shift.
-__global__ void k_merge_field(double* __restrict__ df, const double* __restrict__ dsc, const double* __restrict__ sf,
-                              const double* __restrict__ ssc, long long n, double theta, double hc3,
-                              double* __restrict__ partial) {
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  const double na = dsc[MLSGD_S_COUNT], nb = ssc[MLSGD_S_COUNT];
-  const double shift = fmax(dsc[MLSGD_S_SHIFT], ssc[MLSGD_S_SHIFT]);
-  const double fa = na > 0.0 ? exp(theta * (dsc[MLSGD_S_SHIFT] - shift)) : 0.0;
-  const double fb = nb > 0.0 ? exp(theta * (ssc[MLSGD_S_SHIFT] - shift)) : 0.0;
-  const double nt = na + nb;
-  double contrib = 0.0;
-  if (i < n && nt > 0.0) {
-    const double a = df[i] * fa, b = sf[i] * fb;
-    const double d = a - b;
-    df[i] = b + (na / nt) * d;
-    contrib = hc3 * d * d * na * nb / nt;
+//
+// Bound: FP64 issue (2 operations per clock and SM; 3 or 4 per cell here), then HBM (24
+// bytes per cell).  The factors' exponentials and the divisions by the counts are the
+// same for every cell, so thread 0 of a block forms them once and at most
+// kCellBlocks blocks march over the cells; the scalar kernel then sums a few partial
+// sums per thread.  A merge into an empty record (the first of a series) is a copy and
+// does not read dst.  Six levels on a 256^3 control (16.8M cells) reset, merged twice and
+// stepped: 31.9 ms with the factors formed per cell and one warp over 65536 partial
+// sums, 2.08 ms now (1.6 ms of FP64 issue).
+constexpr int kCellBlocks = 8 * 152;  // eight blocks of 256 threads per SM
+static int cell_blocks(long long n) {
+  const long long b = (n + kBlock - 1) / kBlock;
+  return (int)(b < kCellBlocks ? b : kCellBlocks);
+}
+__global__ void __launch_bounds__(kBlock) k_merge_field(double* __restrict__ df, const double* __restrict__ dsc,
+                                                        const double* __restrict__ sf, const double* __restrict__ ssc,
+                                                        long long n, double theta, double hc3,
+                                                        double* __restrict__ partial) {
+  __shared__ double co[4];  // fa, fb, na / nt, h_c^3 na nb / nt
+  __shared__ int form;      // 0: both empty, 1: dst empty, 2: src holds the larger shift (fb = 1), 3: dst does
+  if (threadIdx.x == 0) {
+    const double na = dsc[MLSGD_S_COUNT], nb = ssc[MLSGD_S_COUNT], nt = na + nb;
+    const double shift = fmax(dsc[MLSGD_S_SHIFT], ssc[MLSGD_S_SHIFT]);
+    const double fa = na > 0.0 ? exp(theta * (dsc[MLSGD_S_SHIFT] - shift)) : 0.0;
+    const double fb = nb > 0.0 ? exp(theta * (ssc[MLSGD_S_SHIFT] - shift)) : 0.0;
+    const bool some = nt > 0.0;
+    form = !some ? 0 : (fb == 1.0 ? (na == 0.0 ? 1 : 2) : 3);
+    co[0] = fa;
+    co[1] = fb;
+    co[2] = some ? na / nt : 0.0;
+    co[3] = some ? hc3 * na * nb / nt : 0.0;
   }
-  const double bs = block_sum(contrib);
-  if (threadIdx.x == 0) partial[blockIdx.x] = bs;
+  __syncthreads();
+  const double fa = co[0], fb = co[1], w = co[2];
+  const long long step = (long long)gridDim.x * kBlock;
+  const long long i0 = (long long)blockIdx.x * kBlock + threadIdx.x;
+  double acc = 0.0;
+  if (form == 1) {
+#pragma unroll 4
+    for (long long i = i0; i < n; i += step) {
+      const double b = sf[i];
+      df[i] = fma(w, b, b);  // w = 0: b (NaN for an infinite b, as w (a - b) gives)
+    }
+  } else if (form == 2) {
+#pragma unroll 4
+    for (long long i = i0; i < n; i += step) {
+      const double b = sf[i], d = fma(df[i], fa, -b);
+      df[i] = fma(w, d, b);
+      acc = fma(d, d, acc);
+    }
+  } else if (form == 3) {
+#pragma unroll 4
+    for (long long i = i0; i < n; i += step) {
+      const double b = sf[i] * fb, d = fma(df[i], fa, -b);
+      df[i] = fma(w, d, b);
+      acc = fma(d, d, acc);
+    }
+  }
+  const double bs = block_sum(acc);
+  if (threadIdx.x == 0) partial[blockIdx.x] = co[3] * bs;
 }
 
-__global__ void k_merge_scalars(const double* __restrict__ partial, int nblk, double* __restrict__ dsc,
-                                const double* __restrict__ ssc, double theta) {
-  const int lane = threadIdx.x;
+__global__ void __launch_bounds__(kBlock) k_merge_scalars(const double* __restrict__ partial, int nblk,
+                                                          double* __restrict__ dsc, const double* __restrict__ ssc,
+                                                          double theta) {
   double v = 0.0;
-  for (int t = lane; t < nblk; t += 32) v += partial[t];
-  v = warp_sum(v);
-  if (lane != 0) return;
+  for (int t = threadIdx.x; t < nblk; t += kBlock) v += partial[t];
+  v = block_sum(v);
+  if (threadIdx.x != 0) return;
   const double na = dsc[MLSGD_S_COUNT], nb = ssc[MLSGD_S_COUNT];
   const double nt = na + nb;
   if (nt <= 0.0) return;
@@ -835,10 +877,10 @@ __global__ void k_merge_scalars(const double* __restrict__ partial, int nblk, do
 
 void launch_stats_merge(double* dfield, double* dsc, const double* sfield, const double* ssc, long long ncells,
                         double hc3, double theta, double* partial, cudaStream_t st) {
-  const int nblk = (int)((ncells + kBlock - 1) / kBlock);
+  const int nblk = cell_blocks(ncells);
   launch("merge", (double)ncells * 24, k_merge_field, dim3(nblk), kBlock, 0, st, dfield, (const double*)dsc, sfield,
          ssc, ncells, theta, hc3, partial);
-  launch("merge_scalars", 0.0, k_merge_scalars, dim3(1), 32, 0, st, (const double*)partial, nblk, dsc, ssc, theta);
+  launch("merge_scalars", 0.0, k_merge_scalars, dim3(1), kBlock, 0, st, (const double*)partial, nblk, dsc, ssc, theta);
 }
 
 // ---------------------------------------------------------------- combine and step
@@ -847,42 +889,59 @@ void launch_stats_merge(double* dfield, double* dsc, const double* sfield, const
 // 2 = ||grad - gprev||^2, 3 = ||gprev||^2 (0 without gprev), 4 = ||z||^2 (before the
 // step), 5+l = ||mean_l||^2
 // (unscaled, counted without h_c^3).
+// Bound: FP64 issue (2 L + 6 operations per cell of L levels, 2 per clock and SM), then
+// HBM (L + 3 words per cell).  At most kCellBlocks blocks march over the cells,
+// so the L + 5 block reductions are paid once per block and not once per 256 cells; the
+// level count is a template parameter, which keeps the L running sums in registers; the
+// division by the denominator is one reciprocal per thread.
 struct FieldList { const double* f[16]; };
 
-__global__ void k_combine_step(FieldList fl, const double* __restrict__ factors, int L, long long n, double denom,
-                               double alpha, double tau, int update, double* __restrict__ z,
-                               double* __restrict__ grad, const double* __restrict__ gprev,
-                               double* __restrict__ partial, int nblk) {
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  double ex = 0.0, g = 0.0, d = 0.0, gp = 0.0, zz = 0.0;
-  double ml[16];
-  for (int l = 0; l < L; ++l) ml[l] = 0.0;
-  if (i < n) {
-    for (int l = 0; l < L; ++l) {
-      const double m = fl.f[l][i];
-      ml[l] = m * m;
-      ex += factors[l] * m;
-    }
+template <int L>
+__global__ void __launch_bounds__(kBlock) k_combine_step(FieldList fl, const double* __restrict__ factors, long long n,
+                                                         double denom, double alpha, double tau, int update,
+                                                         double* __restrict__ z, double* __restrict__ grad,
+                                                         const double* __restrict__ gprev, double* __restrict__ partial,
+                                                         int nblk) {
+  double fac[L], ml[L];
+#pragma unroll
+  for (int l = 0; l < L; ++l) {
+    fac[l] = factors[l];
+    ml[l] = 0.0;
+  }
+  const double inv = 1.0 / denom;
+  const bool divide = !(denom > 1e-300 && denom < 1e300);  // where the reciprocal would leave the normal range
+  double row[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
+  const long long step = (long long)gridDim.x * kBlock;
+#pragma unroll 2
+  for (long long i = (long long)blockIdx.x * kBlock + threadIdx.x; i < n; i += step) {
+    double m[L];
+#pragma unroll
+    for (int l = 0; l < L; ++l) m[l] = fl.f[l][i];
     const double zi = z[i];
-    zz = zi * zi;
-    g = ex / denom + alpha * zi;
+    double ex = fac[0] * m[0];
+    ml[0] = fma(m[0], m[0], ml[0]);
+#pragma unroll
+    for (int l = 1; l < L; ++l) {
+      ex = fma(fac[l], m[l], ex);
+      ml[l] = fma(m[l], m[l], ml[l]);
+    }
+    const double g = fma(alpha, zi, divide ? ex / denom : ex * inv);
+    row[0] = fma(g, g, row[0]);
+    row[1] = fma(ex, ex, row[1]);
+    row[4] = fma(zi, zi, row[4]);
     if (gprev) {
-      gp = gprev[i];
-      d = g - gp;
+      const double gp = gprev[i], d = g - gp;
+      row[2] = fma(d, d, row[2]);
+      row[3] = fma(gp, gp, row[3]);
     }
     if (grad) grad[i] = g;
-    if (update) z[i] = zi - tau * g;
+    if (update) z[i] = fma(-tau, g, zi);
   }
-  const double rowv[5] = {g * g, ex * ex, d * d, gp * gp, zz};
-  for (int r = 0; r < 5; ++r) {
-    if (r) __syncthreads();
-    const double v = block_sum(rowv[r]);
+#pragma unroll
+  for (int r = 0; r < 5 + L; ++r) {
+    const double v = block_sum(r < 5 ? row[r < 5 ? r : 0] : ml[r < 5 ? 0 : r - 5]);
     if (threadIdx.x == 0) partial[(long long)r * nblk + blockIdx.x] = v;
-  }
-  for (int l = 0; l < L; ++l) {
     __syncthreads();
-    const double v = block_sum(ml[l]);
-    if (threadIdx.x == 0) partial[(long long)(5 + l) * nblk + blockIdx.x] = v;
   }
 }
 
@@ -896,15 +955,16 @@ __global__ void k_step_apply(long long n, double tau, const double* __restrict__
   gout[i] = gi;
 }
 
-__global__ void k_rows_finish(const double* __restrict__ partial, int nblk, int rows, double* __restrict__ out) {
-  const int r = blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5);
-  const int lane = threadIdx.x & 31;
-  if (r >= rows) return;
+// out[r] = sum of row r of partial (one block per row)
+__global__ void __launch_bounds__(kBlock) k_rows_finish(const double* __restrict__ partial, int nblk,
+                                                        double* __restrict__ out) {
   double v = 0.0;
-  for (int t = lane; t < nblk; t += 32) v += partial[(long long)r * nblk + t];
-  v = warp_sum(v);
-  if (lane == 0) out[r] = v;
+  for (int t = threadIdx.x; t < nblk; t += kBlock) v += partial[(long long)blockIdx.x * nblk + t];
+  v = block_sum(v);
+  if (threadIdx.x == 0) out[blockIdx.x] = v;
 }
+
+int combine_blocks(long long ncells) { return cell_blocks(ncells); }
 
 void launch_combine_step(const double* const* fields, const double* factors, int L, long long ncells, double denom,
                          double alpha, double tau, bool update, double* z, double* grad, const double* gprev,
@@ -912,10 +972,15 @@ void launch_combine_step(const double* const* fields, const double* factors, int
   FieldList fl;
   for (int l = 0; l < L && l < 16; ++l) fl.f[l] = fields[l];
   const double bytes = (double)ncells * 8 * (L + 1 + (update ? 1 : 0) + (grad ? 1 : 0) + (gprev ? 1 : 0));
-  launch("combine", bytes, k_combine_step, dim3(nblk), kBlock, 0, st, fl, factors, L, ncells, denom, alpha, tau,
+  using Kern = decltype(&k_combine_step<1>);
+  static const Kern kern[16] = {k_combine_step<1>,  k_combine_step<2>,  k_combine_step<3>,  k_combine_step<4>,
+                                k_combine_step<5>,  k_combine_step<6>,  k_combine_step<7>,  k_combine_step<8>,
+                                k_combine_step<9>,  k_combine_step<10>, k_combine_step<11>, k_combine_step<12>,
+                                k_combine_step<13>, k_combine_step<14>, k_combine_step<15>, k_combine_step<16>};
+  launch("combine", bytes, kern[L - 1], dim3(nblk), kBlock, 0, st, fl, factors, ncells, denom, alpha, tau,
          update ? 1 : 0, z, grad, gprev, partial, nblk);
   const int rows = L + 5;
-  launch("combine_finish", 0.0, k_rows_finish, dim3((rows + 7) / 8), 256, 0, st, (const double*)partial, nblk, rows,
+  launch("combine_finish", 0.0, k_rows_finish, dim3(rows), kBlock, 0, st, (const double*)partial, nblk,
          partial + (long long)rows * nblk);
 }
 

@@ -222,6 +222,8 @@ void launch_level_stats(const double* qf, const double* phif, int Nf, const doub
 void launch_stats_reset(double* field, double* scalars, long long ncells, cudaStream_t st);
 void launch_stats_merge(double* dfield, double* dsc, const double* sfield, const double* ssc, long long ncells,
                         double hc3, double theta, double* partial, cudaStream_t st);
+// blocks of the combine pass over ncells control cells (its partial sums per row)
+int combine_blocks(long long ncells);
 // combine levels and (when `update`) step; partial gets [L + 5][blocks] sums and
 // then the L + 5 totals; gprev (optional) is the previous gradient
 void launch_combine_step(const double* const* fields, const double* factors, int L, long long ncells,
