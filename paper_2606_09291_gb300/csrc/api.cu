@@ -200,14 +200,23 @@ mlsgd_status solve_grid(mlsgd_ctx* ctx, int N, int S, const GridFields& f, const
   PcgParams prm{ctx->cfg.rtol, ctx->cfg.max_iter, ctx->cfg.omega > 0 ? ctx->cfg.omega : 0.6, 4};
   const int inner = ctx->cfg.inner_iters > 0 ? ctx->cfg.inner_iters : 6;
   const int inner2 = ctx->cfg.inner_iters_next > 0 ? ctx->cfg.inner_iters_next : inner;
-  if (ctx->mixed()) build_hierarchy_mixed(B, f.abf, prm.omega, st);
-  else build_hierarchy_fp64(B, f.a64, prm.omega, st);
+  const bool small = ctx->mixed() && small_supported(N);  // 8^3, 16^3: a solve is one launch
+  if (ctx->mixed()) {
+    if (!small) build_hierarchy_mixed(B, f.abf, prm.omega, st);
+  } else {
+    build_hierarchy_fp64(B, f.a64, prm.omega, st);
+  }
   launch_rhs_state(z, ctx->Nc(), N, b, st);
   const int fixed = ctx->cfg.ir_steps > 0 ? ctx->cfg.ir_steps : 0;
   const bool pairs = want_pairs && ctx->mixed() && N >= kTiledMinN && B.J >= 1;
   if (pairs_out) *pairs_out = pairs;
-  cudaError_t e = ctx->mixed() ? ir_mixed(B, f.a32, f.abf, b, 0, ytmp, r64, prm, inner, st, fixed, nullptr, pairs, inner2)
-                               : pcg_fp64(B, f.a64, b, 0, ytmp, prm, st);
+  auto solve = [&](const double* rhs, const float2* rhs_pair, long long stride, double* x) {
+    if (!ctx->mixed()) return pcg_fp64(B, f.a64, rhs, stride, x, prm, st);
+    if (small)
+      return small_mixed(B, f.a32, f.abf, rhs, stride, x, r64, prm, inner, inner2, fixed, rhs_pair, pairs, st);
+    return ir_mixed(B, f.a32, f.abf, rhs, stride, x, r64, prm, inner, st, fixed, rhs_pair, pairs, inner2);
+  };
+  cudaError_t e = solve(b, nullptr, 0, ytmp);
   CK(e);
   launch("record", 0.0, k_record, dim3((S + 127) / 128), 128, 0, st, (const SolveScalars*)B.sc, S, (int)ctx->mixed(),
          iters, status, 0);
@@ -217,12 +226,10 @@ mlsgd_status solve_grid(mlsgd_ctx* ctx, int N, int S, const GridFields& f, const
   if (pairs) {
     launch_phi_adjrhs_df((const float2*)ytmp, N, S, (float2*)badj, phi, B.partial, ctx->d_gtab2[lev],
                          ctx->d_mgtab2[lev], st);
-    e = ir_mixed(B, f.a32, f.abf, nullptr, (long long)nodes, q, r64, prm, inner, st, fixed, (const float2*)badj, true,
-                 inner2);
+    e = solve(nullptr, (const float2*)badj, (long long)nodes, q);
   } else {
     launch_phi_adjrhs(ytmp, N, S, badj, phi, B.partial, ctx->d_gtab[lev], ctx->d_mgtab[lev], st, ctx->freq());
-    e = ctx->mixed() ? ir_mixed(B, f.a32, f.abf, badj, (long long)nodes, q, r64, prm, inner, st, fixed, nullptr, false, inner2)
-                     : pcg_fp64(B, f.a64, badj, (long long)nodes, q, prm, st);
+    e = solve(badj, nullptr, (long long)nodes, q);
   }
   CK(e);
   launch("record", 0.0, k_record, dim3((S + 127) / 128), 128, 0, st, (const SolveScalars*)B.sc, S, (int)ctx->mixed(),

@@ -24,17 +24,13 @@
 #include "internal.cuh"
 #include "kernels.h"
 #include "launch.h"
+#include "levels.cuh"
 
 namespace mlsgd {
 
 namespace {
 
 constexpr int kCT = 768;  // threads per block (24 warps: two blocks per SM hide the shared-memory latency)
-
-template <int N>
-struct Lv {
-  static constexpr int n1 = N + 1, nodes = n1 * n1 * n1, cells = N * N * N;
-};
 
 // shared-memory layout (elements of T)
 template <typename T>
@@ -51,149 +47,6 @@ struct CoarseSmem {
   static constexpr int total = a2 + L2::cells;
   static constexpr size_t bytes = sizeof(T) * (size_t)total;
 };
-
-// the eight cells around interior node (i, j, k) of an N^3 level held in shared memory
-template <typename T>
-__device__ __forceinline__ void cells8(Cells8<T, T>& C, const T* a, int i, int j, int k, int N) {
-  C.sum = T(0);
-#pragma unroll
-  for (int r = 0; r < 2; ++r)
-#pragma unroll
-    for (int q = 0; q < 2; ++q)
-#pragma unroll
-      for (int p = 0; p < 2; ++p) {
-        const T v = a[(i - 1 + p) + N * ((j - 1 + q) + N * (k - 1 + r))];
-        C.c[p][q][r] = v;
-        C.sum += v;
-      }
-}
-
-__device__ __forceinline__ double rcp(double x) { return 1.0 / x; }
-__device__ __forceinline__ float rcp(float x) { return __fdividef(1.0f, x); }
-
-// D^-1 of the 16^3 level at every node (0 on the boundary)
-template <typename T>
-__device__ void dinv_level(const T* a, T* d) {
-  constexpr int N = 16, n1 = N + 1;
-  const T h3 = T(1.0 / (3.0 * N));
-  for (int n = threadIdx.x; n < Lv<N>::nodes; n += kCT) {
-    int i, j, k;
-    node_ijk(n, n1, i, j, k);
-    T v = T(0);
-    if (interior(i, j, k, N)) {
-      auto sum4 = [&](int c) {
-        const T* p = a + (i - 1) + N * (j - 1) + N * N * c;
-        return (p[0] + p[1]) + (p[N] + p[N + 1]);
-      };
-      v = rcp(h3 * (sum4(k - 1) + sum4(k)));
-    }
-    d[n] = v;
-  }
-}
-
-// pre-smoothing from 0 and the residual: x = omega D^-1 r (from d, or dividing by D),
-// t = r - A x
-template <int N, bool DTAB, typename T>
-__device__ void pre_level(const T* r, const T* a, const T* d, T* x, T* t, T omega) {
-  constexpr int n1 = N + 1;
-  const T h3 = T(1.0 / (3.0 * N)), sc = T(1.0 / (12.0 * N));
-  for (int n = threadIdx.x; n < Lv<N>::nodes; n += kCT) {
-    int i, j, k;
-    node_ijk(n, n1, i, j, k);
-    T v = T(0);
-    if (interior(i, j, k, N)) {
-      if (DTAB) {
-        v = omega * r[n] * d[n];
-      } else {
-        Cells8<T, T> C;
-        cells8(C, a, i, j, k, N);
-        v = omega * r[n] / (h3 * C.sum);
-      }
-    }
-    x[n] = v;
-  }
-  __syncthreads();
-  for (int n = threadIdx.x; n < Lv<N>::nodes; n += kCT) {
-    int i, j, k;
-    node_ijk(n, n1, i, j, k);
-    T v = T(0);
-    if (interior(i, j, k, N)) {
-      Cells8<T, T> C;
-      cells8(C, a, i, j, k, N);
-      v = r[n] - sc * q1_row(C, x, i, j, k, n1);
-    }
-    t[n] = v;
-  }
-}
-
-// rc = P^T tf (coarse level Nc, weights 1 and 1/2 per axis around the even fine node)
-template <int NC, typename T>
-__device__ void restrict_level(const T* tf, T* rc) {
-  constexpr int n1c = NC + 1, n1f = 2 * NC + 1;
-  for (int n = threadIdx.x; n < Lv<NC>::nodes; n += kCT) {
-    int I, J, K;
-    node_ijk(n, n1c, I, J, K);
-    T v = T(0);
-    if (interior(I, J, K, NC)) {
-      const T* f = tf + 2 * I + n1f * (2 * J) + n1f * n1f * (2 * K);
-#pragma unroll
-      for (int w = -1; w <= 1; ++w)
-#pragma unroll
-        for (int u = -1; u <= 1; ++u)
-#pragma unroll
-          for (int q = -1; q <= 1; ++q) {
-            const T wt = T((q == 0 ? 1.0 : 0.5) * (u == 0 ? 1.0 : 0.5) * (w == 0 ? 1.0 : 0.5));
-            v += wt * f[q + n1f * u + n1f * n1f * w];
-          }
-    }
-    rc[n] = v;
-  }
-}
-
-// xf += P ec (trilinear; ec holds 0 on its boundary)
-template <int NF, typename T>
-__device__ void prolong_level(T* xf, const T* ec) {
-  constexpr int n1f = NF + 1, n1c = NF / 2 + 1;
-  for (int n = threadIdx.x; n < Lv<NF>::nodes; n += kCT) {
-    int i, j, k;
-    node_ijk(n, n1f, i, j, k);
-    if (!interior(i, j, k, NF)) continue;
-    const int i0 = i >> 1, j0 = j >> 1, k0 = k >> 1;
-    const int i1 = i0 + (i & 1), j1 = j0 + (j & 1), k1 = k0 + (k & 1);
-    const T wi = (i & 1) ? T(0.5) : T(1), wj = (j & 1) ? T(0.5) : T(1), wk = (k & 1) ? T(0.5) : T(1);
-    auto at = [&](int a, int b, int c) { return ec[a + n1c * b + n1c * n1c * c]; };
-    T v;
-    if ((i & 1) == 0 && (j & 1) == 0 && (k & 1) == 0) {
-      v = at(i0, j0, k0);
-    } else {
-      v = wi * wj * wk *
-          (at(i0, j0, k0) + ((i & 1) ? at(i1, j0, k0) : T(0)) + ((j & 1) ? at(i0, j1, k0) : T(0)) +
-           ((k & 1) ? at(i0, j0, k1) : T(0)) + (((i & 1) && (j & 1)) ? at(i1, j1, k0) : T(0)) +
-           (((i & 1) && (k & 1)) ? at(i1, j0, k1) : T(0)) + (((j & 1) && (k & 1)) ? at(i0, j1, k1) : T(0)) +
-           (((i & 1) && (j & 1) && (k & 1)) ? at(i1, j1, k1) : T(0)));
-    }
-    xf[n] += v;
-  }
-}
-
-// post-smoothing z = x + omega D^-1 (r - A x), written to z (shared or global)
-template <int N, bool DTAB, typename T>
-__device__ void post_level(const T* r, const T* a, const T* d, const T* x, T* z, T omega) {
-  constexpr int n1 = N + 1;
-  const T h3 = T(1.0 / (3.0 * N)), sc = T(1.0 / (12.0 * N));
-  for (int n = threadIdx.x; n < Lv<N>::nodes; n += kCT) {
-    int i, j, k;
-    node_ijk(n, n1, i, j, k);
-    T v = T(0);
-    if (interior(i, j, k, N)) {
-      Cells8<T, T> C;
-      cells8(C, a, i, j, k, N);
-      const T res = r[n] - sc * q1_row(C, x, i, j, k, n1);
-      v = DTAB ? x[n] + omega * res * d[n] : x[n] + omega * res / (h3 * C.sum);
-    }
-    z[n] = v;
-  }
-}
 
 // asynchronous element copy into shared memory (4 or 8 bytes; the thread waits for its
 // own copies, a block barrier then publishes them)
@@ -234,20 +87,20 @@ __global__ void __launch_bounds__(kCT, sizeof(T) == 4 ? 2 : 1) k_coarse_vcycle(C
   asm volatile("cp.async.commit_group;\n" ::: "memory");
   asm volatile("cp.async.wait_all;\n" ::: "memory");
   __syncthreads();
-  dinv_level<T>(sm + M::a16, sm + M::d16);
+  dinv_level<kCT, T>(sm + M::a16, sm + M::d16);
   __syncthreads();
   // down: 16^3, 8^3, 4^3
-  pre_level<16, true, T>(sm + M::r16, sm + M::a16, sm + M::d16, sm + M::x16, sm + M::t16, omega);
+  pre_level<kCT, 16, true, T>(sm + M::r16, sm + M::a16, sm + M::d16, sm + M::x16, sm + M::t16, omega);
   __syncthreads();
-  restrict_level<8, T>(sm + M::t16, sm + M::r8);
+  restrict_level<kCT, 8, T>(sm + M::t16, sm + M::r8);
   __syncthreads();
-  pre_level<8, false, T>(sm + M::r8, sm + M::a8, nullptr, sm + M::x8, sm + M::t8, omega);
+  pre_level<kCT, 8, false, T>(sm + M::r8, sm + M::a8, nullptr, sm + M::x8, sm + M::t8, omega);
   __syncthreads();
-  restrict_level<4, T>(sm + M::t8, sm + M::r4);
+  restrict_level<kCT, 4, T>(sm + M::t8, sm + M::r4);
   __syncthreads();
-  pre_level<4, false, T>(sm + M::r4, sm + M::a4, nullptr, sm + M::x4, sm + M::t4, omega);
+  pre_level<kCT, 4, false, T>(sm + M::r4, sm + M::a4, nullptr, sm + M::x4, sm + M::t4, omega);
   __syncthreads();
-  restrict_level<2, T>(sm + M::t4, sm + M::r2);
+  restrict_level<kCT, 2, T>(sm + M::t4, sm + M::r2);
   __syncthreads();
   // 2^3: the single interior unknown (node 13), x = r / D
   for (int n = threadIdx.x; n < Lv<2>::nodes; n += kCT) {
@@ -261,17 +114,17 @@ __global__ void __launch_bounds__(kCT, sizeof(T) == 4 ? 2 : 1) k_coarse_vcycle(C
   }
   __syncthreads();
   // up: 4^3, 8^3 (the smoothed corrections overwrite the dead residuals t), then 16^3
-  prolong_level<4, T>(sm + M::x4, sm + M::x2);
+  prolong_level<kCT, 4, T>(sm + M::x4, sm + M::x2);
   __syncthreads();
-  post_level<4, false, T>(sm + M::r4, sm + M::a4, nullptr, sm + M::x4, sm + M::t4, omega);
+  post_level<kCT, 4, false, T>(sm + M::r4, sm + M::a4, nullptr, sm + M::x4, sm + M::t4, omega);
   __syncthreads();
-  prolong_level<8, T>(sm + M::x8, sm + M::t4);
+  prolong_level<kCT, 8, T>(sm + M::x8, sm + M::t4);
   __syncthreads();
-  post_level<8, false, T>(sm + M::r8, sm + M::a8, nullptr, sm + M::x8, sm + M::t8, omega);
+  post_level<kCT, 8, false, T>(sm + M::r8, sm + M::a8, nullptr, sm + M::x8, sm + M::t8, omega);
   __syncthreads();
-  prolong_level<16, T>(sm + M::x16, sm + M::t8);
+  prolong_level<kCT, 16, T>(sm + M::x16, sm + M::t8);
   __syncthreads();
-  post_level<16, true, T>(sm + M::r16, sm + M::a16, sm + M::d16, sm + M::x16,
+  post_level<kCT, 16, true, T>(sm + M::r16, sm + M::a16, sm + M::d16, sm + M::x16,
                           (T*)A.z + (long long)s * Lv<16>::nodes, omega);
 }
 

@@ -193,6 +193,13 @@ template <typename T>
 void coarse_vcycle(const T* r16, const T* const a[4], T* z16, const SolveScalars* sc, const Batch& bt, double omega,
                    cudaStream_t st);
 
+// a whole mixed-precision solve per sample in one launch on 8^3 and 16^3 grids (small.cu);
+// builds the coefficient hierarchy itself; arguments as ir_mixed
+bool small_supported(int N);
+cudaError_t small_mixed(SolverBufs& B, const float* a32, const __nv_bfloat16* abf, const double* b, long long bstride,
+                        double* x_out, double* r64, const PcgParams& prm, int inner_iters, int inner_next,
+                        int fixed_steps, const float2* b_pair, bool pair_out, cudaStream_t st);
+
 // tensor-core KL synthesis (kl_gemm.cu)
 size_t kl_gemm_b_bytes(int N, int K);
 size_t kl_gemm_a_bytes(int S, int K);

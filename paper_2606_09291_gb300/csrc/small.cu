@@ -1,0 +1,780 @@
+// small.cu - a whole mixed-precision solve on an 8^3 or 16^3 grid in one launch, one
+// block per sample (rows a4, a6).
+//
+// On these grids a pass over a sample is a few thousand nodes: run pass by pass, a solve
+// is some 200 dependent launches (22 per inner PCG iteration with the V-cycle level by
+// level), each a few microseconds of launch latency, partial sums in global memory and
+// tail, whatever the batch.  Everything a sample needs fits the shared memory of one
+// block (8^3: 27 KB; 16^3: 108 KB), so here a block keeps its sample's coefficient
+// levels, operand and residuals on the SM and runs the refinement loop to the end:
+// coarse coefficients, FP32 inner PCG with its V(1,1)-cycle, FP64-accurate residual,
+// stop test.  What bounds it is the latency between block barriers (about 14 per inner
+// iteration) and, on 16^3, the shared-memory loads of three 21-point stencils.
+// Measured (three refinement steps of six iterations, state or adjoint): 1024 samples of
+// 8^3 400 us a solve against 2.2 ms in passes, 256 of 16^3 320 us against 3.1 ms, 64 of
+// 16^3 200 us against 1.6 ms.
+//
+// Arithmetic: that of the pass-by-pass solver on the same grid, operation by operation
+// and sum by sum (solver.cu for 8^3: FP64 refinement residual and solution, partial sums
+// per 256 consecutive nodes; tiled.cu for 16^3: solution and b as FP32 pairs, partial
+// sums per thread over 8 planes and the rows of a thread), so a sample's iterates, its
+// iteration count and its result are the ones those passes give.
+#include "internal.cuh"
+#include "kernels.h"
+#include "launch.h"
+#include "levels.cuh"
+#include "refine.cuh"
+
+namespace mlsgd {
+
+namespace {
+
+struct SmallArgs {
+  const float* a32;           // operator coefficient [S][N^3]
+  const __nv_bfloat16* abf;   // V-cycle coefficient [S][N^3]
+  const double* b;            // right-hand side (FP64), or null with bp
+  const float2* bp;           // right-hand side as FP32 (hi, lo) pairs (16^3 only)
+  long long bstride;          // nodes between samples of b / bp (0: one vector for all)
+  double* x64;                // solution in FP64 [S][nodes], or null with xp
+  float2* xp;                 // 16^3: solution as FP32 pairs [S][nodes] (always written)
+  SolveScalars* sc;
+  double tol2;
+  float omega;
+  int fixed;                  // > 0: that many refinement steps
+  int cap;                    // refinement steps after which a solve gives up
+  int inner, inner_next;      // inner iterations of the first and the later steps
+};
+
+// The refinement loop's per-sample state, held by lane 0 of warp 0.
+struct Outer {
+  double bb, rr, rz;
+  int iters, status, pad;
+};
+
+// x = 8^3 level and below: the V(1,1)-cycle with the level's residual r8 in shared memory,
+// correction left in z8 (block of CT threads, thread n < 729 owns node n of the level).
+// The levels 4^3 and 2^3 (27 and 1 interior nodes) are one warp's work.
+struct CoarseLevels {
+  float *r8, *x8, *t8;              // [729]; t8 also receives the correction
+  const float* a8;                  // [512]
+  float *x4, *t4;                   // [125]
+  const float *a4, *a2;             // [64], [8]
+};
+constexpr int kCoarse8Floats = 3 * 729 + 512 + 2 * 125 + 64 + 8;
+constexpr int kCoarse8Own = 2 * 729 + 2 * 125 + 64 + 8;  // without r8 and a8
+
+template <int N>
+__device__ __forceinline__ float diag_of(const float* a, int i, int j, int k) {  // D = (h/3) sum_8 a
+  Cells8<float, float> C;
+  cells8(C, a, i, j, k, N);
+  return float(1.0 / (3.0 * N)) * C.sum;
+}
+
+// levels 4^3 and 2^3 by one warp: restricts t8, leaves the 4^3 correction in L.t4
+__device__ __forceinline__ void coarse4(const CoarseLevels& L, float omega) {
+  const int lane = threadIdx.x & 31;
+  const int I = 1 + lane % 3, J = 1 + (lane / 3) % 3, K = 1 + lane / 9;  // lane < 27
+  const int n = I + 5 * (J + 5 * K);
+  const bool own = lane < 27;
+  float r = 0.f, D = 1.f;
+  if (own) {
+    const float* f = L.t8 + 2 * I + 9 * (2 * J) + 81 * (2 * K);
+    float v = 0.f;
+#pragma unroll
+    for (int w = -1; w <= 1; ++w)
+#pragma unroll
+      for (int u = -1; u <= 1; ++u)
+#pragma unroll
+        for (int q = -1; q <= 1; ++q) {
+          const float wt = float((q == 0 ? 1.0 : 0.5) * (u == 0 ? 1.0 : 0.5) * (w == 0 ? 1.0 : 0.5));
+          v += wt * f[q + 9 * u + 81 * w];
+        }
+    r = v;
+    D = diag_of<4>(L.a4, I, J, K);
+    L.x4[n] = omega * r / D;
+  }
+  __syncwarp();
+  Cells8<float, float> C;
+  if (own) {
+    cells8(C, L.a4, I, J, K, 4);
+    L.t4[n] = r - float(1.0 / 48.0) * q1_row(C, (const float*)L.x4, I, J, K, 5);
+  }
+  __syncwarp();
+  // restriction to the single unknown of 2^3 and its exact solution (every lane the same)
+  float e2;
+  {
+    const float* f = L.t4 + 62;
+    float v = 0.f;
+#pragma unroll
+    for (int w = -1; w <= 1; ++w)
+#pragma unroll
+      for (int u = -1; u <= 1; ++u)
+#pragma unroll
+        for (int q = -1; q <= 1; ++q) {
+          const float wt = float((q == 0 ? 1.0 : 0.5) * (u == 0 ? 1.0 : 0.5) * (w == 0 ? 1.0 : 0.5));
+          v += wt * f[q + 5 * u + 25 * w];
+        }
+    Cells8<float, float> C2;
+    cells8(C2, L.a2, 1, 1, 1, 2);
+    e2 = v / (float(1.0 / 6.0) * C2.sum);
+  }
+  if (own) {  // trilinear: the one coarse node, weight 1/2 per odd index (I, J, K in 1..3)
+    const float w = ((I & 1) ? 0.5f : 1.f) * ((J & 1) ? 0.5f : 1.f) * ((K & 1) ? 0.5f : 1.f);
+    L.x4[n] += w * e2;
+  }
+  __syncwarp();
+  if (own) {
+    const float res = r - float(1.0 / 48.0) * q1_row(C, (const float*)L.x4, I, J, K, 5);
+    L.t4[n] = L.x4[n] + omega * res / D;
+  }
+}
+
+// V-cycle from the 8^3 level; r8 is complete (barrier passed), z in L.t8 after the return
+// of all threads and one more barrier.  own: this thread's node of the level; D its
+// diagonal.  Returns the correction at the own node.
+template <int CT>
+__device__ __forceinline__ float vcycle8(const CoarseLevels& L, int n, int i, int j, int k, bool in, float D,
+                                         float omega) {
+  constexpr float sc = float(1.0 / 96.0);
+  const float r = n < 729 ? L.r8[n] : 0.f;
+  if (in) L.x8[n] = omega * r / D;
+  __syncthreads();
+  if (in) {
+    Cells8<float, float> C;
+    cells8(C, L.a8, i, j, k, 8);
+    L.t8[n] = r - sc * q1_row(C, (const float*)L.x8, i, j, k, 9);
+  }
+  __syncthreads();
+  if (threadIdx.x < 32) coarse4(L, omega);
+  __syncthreads();
+  if (in) {
+    const int i0 = i >> 1, j0 = j >> 1, k0 = k >> 1;
+    const int i1 = i0 + (i & 1), j1 = j0 + (j & 1), k1 = k0 + (k & 1);
+    const float wi = (i & 1) ? 0.5f : 1.f, wj = (j & 1) ? 0.5f : 1.f, wk = (k & 1) ? 0.5f : 1.f;
+    const float* ec = L.t4;
+    auto at = [&](int a, int b, int c) { return ec[a + 5 * b + 25 * c]; };
+    float v;
+    if ((i & 1) == 0 && (j & 1) == 0 && (k & 1) == 0) {
+      v = at(i0, j0, k0);
+    } else {
+      v = wi * wj * wk *
+          (at(i0, j0, k0) + ((i & 1) ? at(i1, j0, k0) : 0.f) + ((j & 1) ? at(i0, j1, k0) : 0.f) +
+           ((k & 1) ? at(i0, j0, k1) : 0.f) + (((i & 1) && (j & 1)) ? at(i1, j1, k0) : 0.f) +
+           (((i & 1) && (k & 1)) ? at(i1, j0, k1) : 0.f) + (((j & 1) && (k & 1)) ? at(i0, j1, k1) : 0.f) +
+           (((i & 1) && (j & 1) && (k & 1)) ? at(i1, j1, k1) : 0.f));
+    }
+    L.x8[n] += v;
+  }
+  __syncthreads();
+  float z = 0.f;
+  if (in) {
+    Cells8<float, float> C;
+    cells8(C, L.a8, i, j, k, 8);
+    const float res = r - sc * q1_row(C, (const float*)L.x8, i, j, k, 9);
+    z = L.x8[n] + omega * res / D;
+    L.t8[n] = z;
+  }
+  return z;
+}
+
+// mean of the eight children (the coarse coefficient), FP32 sums in the order of k_coarsen_coef
+__device__ __forceinline__ float coarsen_cell(const float* af, int c, int Nc) {
+  const int I = c % Nc, J = (c / Nc) % Nc, K = c / (Nc * Nc), Nf = 2 * Nc;
+  const float* f = af + 2 * I + Nf * (2 * J + Nf * 2 * K);
+  float acc = 0.f;
+#pragma unroll
+  for (int r = 0; r < 2; ++r)
+#pragma unroll
+    for (int q = 0; q < 2; ++q)
+#pragma unroll
+      for (int p = 0; p < 2; ++p) acc += f[p + Nf * (q + Nf * r)];
+  return 0.125f * acc;
+}
+
+// scalar updates of the PCG (see SM_ALPHA, SM_BETA in solver.cu)
+__device__ __forceinline__ float pcg_alpha(const Outer& o, double v) {
+  return (float)((v > 0.0 && o.rz != 0.0) ? o.rz / v : 0.0);
+}
+__device__ __forceinline__ float pcg_beta(Outer& o, double v) {
+  const double b = o.rz != 0.0 ? v / o.rz : 0.0;
+  o.rz = v;
+  return (float)b;
+}
+// the refinement's stop test (SM_OUTER_CONV): true while the sample goes on
+__device__ __forceinline__ bool outer_go(Outer& o, double v, double tol2, int cap) {
+  o.rr = v;
+  if (v <= tol2 * o.bb) return false;
+  if (!(v < INFINITY)) { o.status = 2; return false; }
+  if (o.iters >= cap) { o.status = 1; return false; }
+  return true;
+}
+__device__ __forceinline__ void store_scalars(SolveScalars* sc, const Outer& o) {
+  SolveScalars c;
+  c.bb = o.bb; c.rz = o.rz; c.alpha = 0.0; c.beta = 0.0; c.rr = o.rr;
+  c.active = 0; c.iters = o.iters; c.status = o.status; c.pad = o.pad;
+  *sc = c;
+}
+
+// ---------------------------------------------------------------- 8^3
+// thread n < 729 owns node n; partial sums per 256 consecutive nodes (warps 0-7, 8-15,
+// 16-23), then over the three of them, as block_sum and k_scalar form them
+constexpr int kT8 = 768;
+
+template <typename T>
+__device__ __forceinline__ double sum_groups(T v) {  // lane l holds warp l's sum (l < 24, else 0)
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  double p = (double)v;  // lanes 8g: the block sum of group g
+  const double p0 = __shfl_sync(0xffffffffu, p, 0), p1 = __shfl_sync(0xffffffffu, p, 8),
+               p2 = __shfl_sync(0xffffffffu, p, 16);
+  return (p0 + p2) + p1;
+}
+
+struct Smem8 {
+  double xd[729];       // solution for the refinement residual
+  double redd[24];
+  float a32[512], abf[512];
+  float op[729];        // operand of A p
+  float r8[729];        // residual of the V-cycle
+  float lv[kCoarse8Own];
+  float redf[2][24];
+  float bc;             // alpha or beta
+  int go;
+};
+
+__global__ void __launch_bounds__(kT8, 2) k_small8(SmallArgs A) {
+  __shared__ Smem8 M;
+  const int s = blockIdx.x, n = threadIdx.x, lane = n & 31, warp = n >> 5;
+  const float omega = A.omega;
+  for (int c = n; c < 512; c += kT8) {
+    M.a32[c] = A.a32[(long long)s * 512 + c];
+    M.abf[c] = __bfloat162float(A.abf[(long long)s * 512 + c]);
+  }
+  if (n < 729) M.op[n] = M.r8[n] = 0.f;
+  for (int e = n; e < kCoarse8Own; e += kT8) M.lv[e] = 0.f;
+  CoarseLevels L;
+  L.r8 = M.r8; L.a8 = M.abf;
+  L.x8 = M.lv; L.t8 = L.x8 + 729;
+  L.x4 = L.t8 + 729; L.t4 = L.x4 + 125;
+  float* a4 = L.t4 + 125;
+  float* a2 = a4 + 64;
+  L.a4 = a4; L.a2 = a2;
+  int i = 0, j = 0, k = 0;
+  if (n < 729) node_ijk(n, 9, i, j, k);
+  const bool in = n < 729 && interior(i, j, k, 8);
+  const double bv = n < 729 ? A.b[s * A.bstride + n] : 0.0;
+  __syncthreads();
+  if (n < 64) a4[n] = coarsen_cell(M.abf, n, 4);
+  const float D = in ? diag_of<8>(M.abf, i, j, k) : 1.f;
+  __syncthreads();
+  if (n < 8) a2[n] = coarsen_cell(a4, n, 2);
+  Outer o{0.0, 0.0, 0.0, 0, 0, 0};
+  // block sum of a double, result in warp 0
+  auto sum64 = [&](double v) {
+    v = warp_sum(v);
+    if (lane == 0) M.redd[warp] = v;
+    __syncthreads();
+    return warp == 0 ? sum_groups<double>(lane < 24 ? M.redd[lane] : 0.0) : 0.0;
+  };
+  int par = 0;
+  auto sum32 = [&](float v) {
+    v = warp_sum(v);
+    if (lane == 0) M.redf[par][warp] = v;
+    __syncthreads();
+    const double d = warp == 0 ? sum_groups<float>(lane < 24 ? M.redf[par][lane] : 0.f) : 0.0;
+    par ^= 1;
+    return d;
+  };
+  {
+    const double v = sum64(bv * bv);
+    if (n == 0) {
+      o.bb = o.rr = v;
+      bool go = v > 0.0;
+      if (!(v < INFINITY)) { go = false; o.status = 2; }
+      M.go = go;
+    }
+  }
+  __syncthreads();
+  double x = 0.0;
+  bool go = M.go != 0;
+  for (int step = 0; go; ++step) {
+    double r64 = bv;
+    if (step > 0) {  // r = b - A x in FP64
+      if (n < 729) M.xd[n] = x;
+      __syncthreads();
+      r64 = 0.0;
+      if (in) {
+        Cells8<double, float> C;
+        C.sum = 0.0;
+#pragma unroll
+        for (int r = 0; r < 2; ++r)
+#pragma unroll
+          for (int q = 0; q < 2; ++q)
+#pragma unroll
+            for (int p = 0; p < 2; ++p) {
+              const double v = (double)M.a32[(i - 1 + p) + 8 * ((j - 1 + q) + 8 * (k - 1 + r))];
+              C.c[p][q][r] = v;
+              C.sum += v;
+            }
+        r64 = bv - (1.0 / (12.0 * 8)) * q1_row(C, (const double*)M.xd, i, j, k, 9);
+      }
+      const double v = sum64(r64 * r64);
+      if (n == 0) M.go = outer_go(o, v, A.tol2, A.cap);
+      __syncthreads();
+      go = M.go != 0;
+      if (!go) break;
+    }
+    if (A.fixed > 0 && step == A.fixed) break;
+    const int inner = step == 0 ? A.inner : A.inner_next;
+    float r = (float)r64, d = 0.f, p = 0.f;
+    for (int it = 0;; ++it) {
+      if (n < 729) M.r8[n] = r;
+      __syncthreads();
+      const float z = vcycle8<kT8>(L, n, i, j, k, in, D, omega);
+      {
+        const double v = sum32(r * z);
+        if (n == 0) {
+          if (it == 0) o.rz = v;
+          else M.bc = pcg_beta(o, v);
+        }
+      }
+      if (it > 0) {
+        __syncthreads();
+        p = z + M.bc * p;
+      } else {
+        p = z;
+      }
+      if (n < 729) M.op[n] = p;
+      __syncthreads();
+      float q = 0.f;
+      if (in) {
+        Cells8<float, float> C;
+        cells8(C, M.a32, i, j, k, 8);
+        q = float(1.0 / (12.0 * 8)) * q1_row(C, (const float*)M.op, i, j, k, 9);
+      }
+      const double v = sum32(p * q);
+      if (n == 0) M.bc = pcg_alpha(o, v);
+      __syncthreads();
+      const float al = M.bc;
+      d += al * p;
+      if (it == inner - 1) break;
+      r = r - al * q;
+    }
+    x += (double)d;
+    if (n == 0) { o.iters += 1; o.pad += inner; }
+  }
+  if (n < 729) A.x64[(long long)s * 729 + n] = x;
+  if (n == 0) store_scalars(A.sc + s, o);
+}
+
+// ---------------------------------------------------------------- 16^3
+// 1024 threads: thread (xq, yq, g) owns the nodes x = xq + 1, y = yq + 1 of the planes
+// 4g + 1 .. 4g + 4 (xq, yq < 15; plane 16 is the boundary), whose r, p, z, q, correction
+// and omega D^-1 stay in its registers.  Shared memory holds what neighbours read: the
+// operand, the residual to restrict, and the vectors whose dot product the threads of the
+// tile passes would sum.
+constexpr int kT16 = 1024;
+constexpr int kN16 = 17 * 17 * 17;
+
+struct Smem16 {
+  float b0[kN16];  // operand of a stencil; with b1: the solution pairs of a refinement residual
+  float b1[kN16];  // t, then r (dot)
+  float b2[kN16];  // z, q or the refinement residual (dot)
+  float a32[4096], abf[4096];
+  float lv[kCoarse8Floats];
+  double redd[24];
+  float redf[8];
+  float bc;
+  int go;
+};
+static_assert(sizeof(Smem16) <= 227 * 1024, "shared memory");
+
+// operator row over h/12 of tiled.cu's passes: three partial sums, operand window and
+// cells read from shared memory
+__device__ __forceinline__ float q1_tile(const float* x, const float* a, int n, int c) {
+  float C[2][2][2];  // [r][p][q]
+#pragma unroll
+  for (int r = 0; r < 2; ++r)
+#pragma unroll
+    for (int p = 0; p < 2; ++p)
+#pragma unroll
+      for (int q = 0; q < 2; ++q) C[r][p][q] = a[c + p + 16 * q + 256 * r];
+  auto X = [&](int pl, int u, int v) { return x[n + (u - 1) + 17 * (v - 1) + 289 * (pl - 1)]; };
+  float pxy[2][2], pxz[2][2], pyz[2][2];
+#pragma unroll
+  for (int u = 0; u < 2; ++u)
+#pragma unroll
+    for (int v = 0; v < 2; ++v) {
+      pxy[v][u] = C[0][u][v] + C[1][u][v];
+      pxz[v][u] = C[v][u][0] + C[v][u][1];
+      pyz[v][u] = C[v][0][u] + C[v][1][u];
+    }
+  const float sum8 = (pxy[0][0] + pxy[0][1]) + (pxy[1][0] + pxy[1][1]);
+  float accp[3];
+  accp[1] = 4.f * sum8 * X(1, 1, 1);
+#pragma unroll
+  for (int v = 0; v < 2; ++v)
+#pragma unroll
+    for (int u = 0; u < 2; ++u) accp[1] -= pxy[v][u] * X(1, 2 * u, 2 * v);
+#pragma unroll
+  for (int r = 0; r < 2; ++r) {
+    const int pl = 2 * r;
+    float a2 = 0.f;
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      a2 -= pxz[r][u] * X(pl, 2 * u, 1);
+      a2 -= pyz[r][u] * X(pl, 1, 2 * u);
+    }
+#pragma unroll
+    for (int q = 0; q < 2; ++q)
+#pragma unroll
+      for (int p = 0; p < 2; ++p) a2 -= C[r][p][q] * X(pl, 2 * p, 2 * q);
+    accp[pl] = a2;
+  }
+  return accp[1] + (accp[0] + accp[2]);
+}
+
+__global__ void __launch_bounds__(kT16, 1) k_small16(SmallArgs A) {
+  extern __shared__ __align__(16) unsigned char smraw[];
+  Smem16& M = *reinterpret_cast<Smem16*>(smraw);
+  const int s = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int xq = tid & 15, yq = (tid >> 4) & 15, g = tid >> 8;
+  const float omega = A.omega, scale = float(1.0 / (12.0 * 16));
+  const bool col = xq < 15 && yq < 15;
+  const int nu = col ? (g == 3 ? 3 : 4) : 0;               // own nodes
+  const int n0 = (xq + 1) + 17 * (yq + 1) + 289 * (4 * g + 1);  // first own node
+  const int c0 = xq + 16 * yq + 256 * (4 * g);                  // its lowest cell
+  for (int c = tid; c < 4096; c += kT16) {
+    M.a32[c] = A.a32[(long long)s * 4096 + c];
+    M.abf[c] = __bfloat162float(A.abf[(long long)s * 4096 + c]);
+  }
+  for (int e = tid; e < kN16; e += kT16) M.b0[e] = M.b1[e] = 0.f;
+  for (int e = tid; e < kCoarse8Floats; e += kT16) M.lv[e] = 0.f;
+  CoarseLevels L;
+  L.r8 = M.lv; L.x8 = L.r8 + 729; L.t8 = L.x8 + 729;
+  float* a8 = L.t8 + 729;
+  L.x4 = a8 + 512; L.t4 = L.x4 + 125;
+  float* a4 = L.t4 + 125;
+  float* a2 = a4 + 64;
+  L.a8 = a8; L.a4 = a4; L.a2 = a2;
+  // the right-hand side's pair at node n of this sample
+  auto b_pair = [&](int n) {
+    return A.bp ? A.bp[s * A.bstride + n] : df_split(A.b[s * A.bstride + n]);
+  };
+  // boundary nodes of the outputs
+  for (int e = tid; e < kN16; e += kT16) {
+    int i, j, k;
+    node_ijk(e, 17, i, j, k);
+    const bool in = interior(i, j, k, 16);
+    M.b2[e] = 0.f;
+    if (!in) {
+      A.xp[(long long)s * kN16 + e] = make_float2(0.f, 0.f);
+      if (A.x64) A.x64[(long long)s * kN16 + e] = 0.0;
+    }
+  }
+  __syncthreads();
+  float r[4], p[4], z[4], d[4], dv[4], q[4];
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    r[u] = p[u] = z[u] = d[u] = dv[u] = q[u] = 0.f;
+    if (u < nu) {
+      r[u] = b_pair(n0 + 289 * u).x;
+      M.b2[n0 + 289 * u] = r[u];
+      auto sum4 = [&](int c) { return (M.abf[c] + M.abf[c + 1]) + (M.abf[c + 16] + M.abf[c + 17]); };
+      const float below = sum4(c0 + 256 * u), above = sum4(c0 + 256 * (u + 1));
+      dv[u] = omega * __fdividef(1.0f, float(1.0 / 48.0) * (below + above));
+    }
+  }
+  for (int c = tid; c < 512; c += kT16) a8[c] = coarsen_cell(M.abf, c, 8);
+  __syncthreads();
+  if (tid < 64) a4[tid] = coarsen_cell(a8, tid, 4);
+  // node of the 8^3 level
+  int i8 = 0, j8 = 0, k8 = 0;
+  if (tid < 729) node_ijk(tid, 9, i8, j8, k8);
+  const bool in8 = tid < 729 && interior(i8, j8, k8, 8);
+  const float D8 = in8 ? diag_of<8>(a8, i8, j8, k8) : 1.f;
+  __syncthreads();
+  if (tid < 8) a2[tid] = coarsen_cell(a4, tid, 2);
+  Outer o{0.0, 0.0, 0.0, 0, 0, 0};
+  // ||b||^2 as the solver's init pass sums it: three blocks of 256 threads, eight nodes a
+  // thread at stride 256 (FP32 over the pair heads; FP64 for an FP64 right-hand side of its own)
+  {
+    const bool own64 = !A.bp && A.bstride != 0;
+    double v = 0.0;
+    if (tid < 768) {
+      const int m0 = (tid >> 8) * 2048 + (tid & 255);
+      float f = 0.f;
+#pragma unroll
+      for (int t = 0; t < 8; ++t) {
+        const int n = m0 + 256 * t;
+        if (n >= kN16) continue;
+        if (own64) {
+          int ii, jj, kk;
+          node_ijk(n, 17, ii, jj, kk);
+          if (interior(ii, jj, kk, 16)) {
+            const double bv = A.b[s * A.bstride + n];
+            v = fma(bv, bv, v);
+          }
+        } else {
+          f = __fmaf_rn(M.b2[n], M.b2[n], f);
+        }
+      }
+      if (!own64) v = (double)f;
+      v = warp_sum(v);
+      if (lane == 0) M.redd[warp] = v;
+    }
+    __syncthreads();
+    if (warp == 0) {
+      v = sum_groups<double>(lane < 24 ? M.redd[lane] : 0.0);
+      if (lane == 0) {
+        o.bb = o.rr = v;
+        bool go = v > 0.0;
+        if (!(v < INFINITY)) { go = false; o.status = 2; }
+        M.go = go;
+      }
+    }
+  }
+  __syncthreads();
+  // dot product of two shared vectors in the order of the tile passes: thread (tx, ty) of
+  // segment sg sums rows 4 ty + 1 .. 4 ty + 4 over the segment's eight planes, then the
+  // block sum of the segment, then the two segments (result in warp 0)
+  auto dot = [&](const float* u, const float* v) {
+    if (warp < 8) {
+      const int sg = warp >> 2, ty = warp & 3;
+      float red = 0.f;
+      if (lane < 15) {
+        const int base = lane + 1 + 17 * (4 * ty + 1) + 289 * (8 * sg + 1);
+#pragma unroll
+        for (int k = 0; k < 8; ++k)
+#pragma unroll
+          for (int t = 0; t < 4; ++t)
+            if (8 * sg + k < 15 && 4 * ty + t < 15) {
+              const int n = base + 17 * t + 289 * k;
+              red = __fmaf_rn(u[n], v[n], red);
+            }
+      }
+      red = warp_sum(red);
+      if (lane == 0) M.redf[warp] = red;
+    }
+    __syncthreads();
+    if (warp != 0) return 0.0;
+    float w = lane < 8 ? M.redf[lane] : 0.f;
+    w += __shfl_xor_sync(0xffffffffu, w, 2);
+    w += __shfl_xor_sync(0xffffffffu, w, 1);
+    const double p0 = (double)__shfl_sync(0xffffffffu, w, 0), p1 = (double)__shfl_sync(0xffffffffu, w, 4);
+    return p0 + p1;
+  };
+  bool go = M.go != 0;
+  const float2 zero2 = make_float2(0.f, 0.f);
+  if (!go) {  // no step is taken: x = 0
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (u < nu) A.xp[(long long)s * kN16 + n0 + 289 * u] = zero2;
+  }
+  for (int step = 0; go; ++step) {
+    if (step > 0) {  // r = b - A x from the pairs, error-free products and sums in FP32
+      float2* xs = reinterpret_cast<float2*>(M.b0);  // b0 and b1
+      __syncthreads();                               // the last step's reads of b0, b1
+      for (int e = tid; e < kN16; e += kT16) xs[e] = A.xp[(long long)s * kN16 + e];
+      __syncthreads();
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (u < nu) {
+          const int n = n0 + 289 * u, c = c0 + 256 * u;
+          auto X = [&](int pl, int a, int b) { return xs[n + (a - 1) + 17 * (b - 1) + 289 * (pl - 1)]; };
+          auto C = [&](int rr, int pp, int qq) { return M.a32[c + pp + 16 * qq + 256 * rr]; };
+          r[u] = refine_residual(C, X, b_pair(n), 16);
+          M.b2[n] = r[u];
+        }
+      __syncthreads();
+      double v = 0.0;
+      if (warp < 16) {  // rows 2 ty + 1, 2 ty + 2 of segment sg
+        const int sg = warp >> 3, ty = warp & 7;
+        float red = 0.f;
+        if (lane < 15) {
+          const int base = lane + 1 + 17 * (2 * ty + 1) + 289 * (8 * sg + 1);
+#pragma unroll
+          for (int k = 0; k < 8; ++k)
+#pragma unroll
+            for (int t = 0; t < 2; ++t)
+              if (8 * sg + k < 15 && 2 * ty + t < 15) {
+                const float rv = M.b2[base + 17 * t + 289 * k];
+                red = __fmaf_rn(rv, rv, red);
+              }
+        }
+        v = warp_sum((double)red);
+        if (lane == 0) M.redd[warp] = v;
+      }
+      __syncthreads();
+      if (warp == 0) {
+        v = lane < 16 ? M.redd[lane] : 0.0;
+#pragma unroll
+        for (int w = 4; w > 0; w >>= 1) v += __shfl_xor_sync(0xffffffffu, v, w);
+        v = __shfl_sync(0xffffffffu, v, 0) + __shfl_sync(0xffffffffu, v, 8);
+        if (lane == 0) M.go = outer_go(o, v, A.tol2, A.cap);
+      }
+      for (int e = tid; e < 2 * kN16; e += kT16) M.b0[e] = 0.f;  // boundary nodes of b0 and b1
+      __syncthreads();
+      go = M.go != 0;
+      if (!go) break;
+    }
+    if (A.fixed > 0 && step == A.fixed) break;
+    const int inner = step == 0 ? A.inner : A.inner_next;
+    float al = 0.f;
+    for (int it = 0;; ++it) {
+      // V-cycle on r: pre-smoothing, residual, 8^3 and below, prolongation, post-smoothing
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (u < nu) M.b0[n0 + 289 * u] = r[u] * dv[u];
+      __syncthreads();
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (u < nu) M.b1[n0 + 289 * u] = __fmaf_rn(-scale, q1_tile(M.b0, M.abf, n0 + 289 * u, c0 + 256 * u), r[u]);
+      __syncthreads();
+      if (in8) {
+        const float* f = M.b1 + 2 * i8 + 17 * (2 * j8) + 289 * (2 * k8);
+        float v = 0.f;
+#pragma unroll
+        for (int w = -1; w <= 1; ++w)
+#pragma unroll
+          for (int b = -1; b <= 1; ++b)
+#pragma unroll
+            for (int a = -1; a <= 1; ++a) {
+              const float wt = float((a == 0 ? 1.0 : 0.5) * (b == 0 ? 1.0 : 0.5) * (w == 0 ? 1.0 : 0.5));
+              v += wt * f[a + 17 * b + 289 * w];
+            }
+        L.r8[tid] = v;
+      }
+      __syncthreads();
+      (void)vcycle8<kT16>(L, tid, i8, j8, k8, in8, D8, omega);
+      __syncthreads();
+      const int px = (xq + 1) & 1, py = (yq + 1) & 1;
+      const float* e8 = L.t8 + ((xq + 1) >> 1) + 9 * ((yq + 1) >> 1);
+      auto plane = [&](int c) {  // coarse plane c interpolated in x and y
+        const float* e = e8 + 81 * c;
+        const float e00 = e[0];
+        if (!px && !py) return e00;
+        if (!py) return (e00 + e[1]) * 0.5f;
+        if (!px) return (e00 + e[9]) * 0.5f;
+        return ((e00 + e[1]) * 0.5f + (e[9] + e[10]) * 0.5f) * 0.5f;
+      };
+      float x2[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (u < nu) {
+          const int k = 4 * g + 1 + u;
+          const float y = (k & 1) ? (plane(k >> 1) + plane((k >> 1) + 1)) * 0.5f : plane(k >> 1);
+          x2[u] = __fadd_rn(__fmul_rn(r[u], dv[u]), y);  // rounded product first, as the tile pass
+          M.b0[n0 + 289 * u] = x2[u];
+        }
+      __syncthreads();
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (u < nu) {
+          const float res = __fmaf_rn(-scale, q1_tile(M.b0, M.abf, n0 + 289 * u, c0 + 256 * u), r[u]);
+          z[u] = __fmaf_rn(res, dv[u], x2[u]);
+          M.b1[n0 + 289 * u] = r[u];
+          M.b2[n0 + 289 * u] = z[u];
+        }
+      __syncthreads();
+      {
+        const double v = dot(M.b1, M.b2);
+        if (tid == 0) {
+          if (it == 0) {
+            o.rz = v;
+            M.bc = 0.f;
+          } else {
+            M.bc = pcg_beta(o, v);
+          }
+        }
+      }
+      __syncthreads();
+      // p = z + beta p, q = A p
+      const float be = M.bc;
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (u < nu) {
+          p[u] = it == 0 ? z[u] : __fmaf_rn(be, p[u], z[u]);
+          M.b0[n0 + 289 * u] = p[u];
+        }
+      __syncthreads();
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (u < nu) {
+          q[u] = scale * q1_tile(M.b0, M.a32, n0 + 289 * u, c0 + 256 * u);
+          M.b2[n0 + 289 * u] = q[u];
+        }
+      __syncthreads();
+      {
+        const double v = dot(M.b0, M.b2);
+        if (tid == 0) M.bc = pcg_alpha(o, v);
+      }
+      __syncthreads();
+      al = M.bc;
+      if (it == inner - 1) break;
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        d[u] = it == 0 ? al * p[u] : __fmaf_rn(al, p[u], d[u]);
+        r[u] = __fmaf_rn(-al, q[u], r[u]);
+      }
+    }
+    // x (+)= d + alpha p in pair arithmetic
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (u < nu) {
+        const float inc = inner > 1 ? __fmaf_rn(al, p[u], d[u]) : al * p[u];
+        float2* xo = A.xp + (long long)s * kN16 + n0 + 289 * u;
+        *xo = step == 0 ? make_float2(inc, 0.f) : pair_add(*xo, inc);
+      }
+    if (tid == 0) { o.iters += 1; o.pad += inner; }
+  }
+  if (A.x64) {
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (u < nu) {
+        const long long e = (long long)s * kN16 + n0 + 289 * u;
+        const float2 v = A.xp[e];
+        A.x64[e] = (double)v.x + (double)v.y;
+      }
+  }
+  if (tid == 0) store_scalars(A.sc + s, o);
+}
+
+}  // namespace
+
+bool small_supported(int N) { return N == 8 || N == 16; }
+
+cudaError_t small_mixed(SolverBufs& B, const float* a32, const __nv_bfloat16* abf, const double* b, long long bstride,
+                        double* x_out, double* r64, const PcgParams& prm, int inner_iters, int inner_next,
+                        int fixed_steps, const float2* b_pair, bool pair_out, cudaStream_t st) {
+  const int N = B.N, S = B.S;
+  if (N == 8 && (b_pair || pair_out)) return cudaErrorInvalidValue;
+  SmallArgs A{};
+  A.a32 = a32; A.abf = abf; A.b = b; A.bp = b_pair; A.bstride = bstride;
+  A.x64 = pair_out ? nullptr : x_out;
+  A.xp = pair_out ? (float2*)x_out : (float2*)r64;
+  A.sc = B.sc;
+  A.tol2 = prm.rtol * prm.rtol;
+  A.omega = (float)prm.omega;
+  A.fixed = fixed_steps > 0 ? fixed_steps : 0;
+  A.cap = fixed_steps > 0 ? fixed_steps : prm.max_iter;
+  A.inner = inner_iters;
+  A.inner_next = inner_next > 0 ? inner_next : inner_iters;
+  const double nodes = (double)nodes_of(N), cells = (double)cells_of(N);
+  const double bytes = (bstride ? S : 1) * nodes * 8 + S * (nodes * 8 + cells * 6);
+  if (N == 8) {
+    launch("small_f32", bytes, k_small8, dim3((unsigned)S), dim3(kT8), 0, st, A);
+  } else {
+    static bool smem_set = false;  // once (capture-friendly)
+    if (!smem_set) {
+      const cudaError_t e =
+          cudaFuncSetAttribute(k_small16, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Smem16));
+      if (e != cudaSuccess) return e;
+      smem_set = true;
+    }
+    launch("small_f32", bytes, k_small16, dim3((unsigned)S), dim3(kT16), sizeof(Smem16), st, A);
+  }
+  return cudaGetLastError();
+}
+
+}  // namespace mlsgd

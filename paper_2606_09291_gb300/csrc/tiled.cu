@@ -33,6 +33,7 @@
 #include "internal.cuh"
 #include "kernels.h"
 #include "launch.h"
+#include "refine.cuh"
 
 namespace mlsgd {
 
@@ -125,27 +126,6 @@ struct TiledSmem {
   static constexpr size_t total = cells + sizeof(TA) * RING * G::CPL;
 };
 
-
-// ---- error-free FP32 arithmetic for the refinement residual (TM_RES64)
-// two_sum: s + e == a + b exactly (Knuth); products use the FMA to split
-// c * x into p + pe exactly.  A coefficient is an unevaluated pair (h, l).
-struct F2 { float h, l; };
-__device__ __forceinline__ F2 two_sum(float a, float b) {  // intrinsics: never contracted
-  const float s = __fadd_rn(a, b);
-  const float bb = __fsub_rn(s, a);
-  return F2{s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb))};
-}
-// (S, comp) += sgn * (c.h + c.l) * (x.x + x.y), sgn = +1 or -1
-template <bool NEG>
-__device__ __forceinline__ void df_term(float& S, float& comp, F2 c, float2 x) {
-  const float p = __fmul_rn(c.h, x.x);
-  const float pe = __fmaf_rn(c.h, x.x, -p);
-  const float low = __fmaf_rn(c.h, x.y, __fmaf_rn(c.l, x.x, pe));
-  const float q = NEG ? -p : p;
-  const F2 t = two_sum(S, q);
-  S = t.h;
-  comp = __fadd_rn(comp, __fadd_rn(t.l, NEG ? -low : low));
-}
 
 template <typename T, typename TA, int MODE>
 __global__ void __launch_bounds__(NT) k_tiled(TiledArgs A) {
