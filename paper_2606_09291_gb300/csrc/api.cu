@@ -200,18 +200,16 @@ mlsgd_status solve_grid(mlsgd_ctx* ctx, int N, int S, const GridFields& f, const
   PcgParams prm{ctx->cfg.rtol, ctx->cfg.max_iter, ctx->cfg.omega > 0 ? ctx->cfg.omega : 0.6, 4};
   const int inner = ctx->cfg.inner_iters > 0 ? ctx->cfg.inner_iters : 6;
   const int inner2 = ctx->cfg.inner_iters_next > 0 ? ctx->cfg.inner_iters_next : inner;
-  const bool small = ctx->mixed() && small_supported(N);  // 8^3, 16^3: a solve is one launch
-  if (ctx->mixed()) {
-    if (!small) build_hierarchy_mixed(B, f.abf, prm.omega, st);
-  } else {
-    build_hierarchy_fp64(B, f.a64, prm.omega, st);
-  }
+  const bool small = small_supported(N);  // 8^3, 16^3: a solve is one launch
+  if (!small && ctx->mixed()) build_hierarchy_mixed(B, f.abf, prm.omega, st);
+  if (!small && !ctx->mixed()) build_hierarchy_fp64(B, f.a64, prm.omega, st);
   launch_rhs_state(z, ctx->Nc(), N, b, st);
   const int fixed = ctx->cfg.ir_steps > 0 ? ctx->cfg.ir_steps : 0;
   const bool pairs = want_pairs && ctx->mixed() && N >= kTiledMinN && B.J >= 1;
   if (pairs_out) *pairs_out = pairs;
   auto solve = [&](const double* rhs, const float2* rhs_pair, long long stride, double* x) {
-    if (!ctx->mixed()) return pcg_fp64(B, f.a64, rhs, stride, x, prm, st);
+    if (!ctx->mixed())
+      return small ? small_fp64(B, f.a64, rhs, stride, x, prm, st) : pcg_fp64(B, f.a64, rhs, stride, x, prm, st);
     if (small)
       return small_mixed(B, f.a32, f.abf, rhs, stride, x, r64, prm, inner, inner2, fixed, rhs_pair, pairs, st);
     return ir_mixed(B, f.a32, f.abf, rhs, stride, x, r64, prm, inner, st, fixed, rhs_pair, pairs, inner2);

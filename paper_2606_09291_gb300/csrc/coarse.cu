@@ -67,7 +67,7 @@ struct CoarseArgs {
 };
 
 template <typename T>
-__global__ void __launch_bounds__(kCT, sizeof(T) == 4 ? 2 : 1) k_coarse_vcycle(CoarseArgs A) {
+__global__ void __launch_bounds__(kCT, 2) k_coarse_vcycle(CoarseArgs A) {
   using M = CoarseSmem<T>;
   const int s = A.act != nullptr ? A.act[blockIdx.x] : (int)blockIdx.x;
   if (A.sc != nullptr && !A.sc[s].active) return;
@@ -132,13 +132,12 @@ __global__ void __launch_bounds__(kCT, sizeof(T) == 4 ? 2 : 1) k_coarse_vcycle(C
 
 bool coarse_vcycle_applies(int N, int j) { return j >= 1 && (N >> j) == 16; }
 
-template <typename T>
-void coarse_vcycle(const T* r16, const T* const a[4], T* z16, const SolveScalars* sc, const Batch& bt, double omega,
-                   cudaStream_t st) {
-  using M = CoarseSmem<T>;
-  static bool smem_set = false;  // once per instantiation (capture-friendly)
+void coarse_vcycle(const float* r16, const float* const a[4], float* z16, const SolveScalars* sc, const Batch& bt,
+                   double omega, cudaStream_t st) {
+  using M = CoarseSmem<float>;
+  static bool smem_set = false;  // once (capture-friendly)
   if (!smem_set) {
-    cudaFuncSetAttribute(k_coarse_vcycle<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)M::bytes);
+    cudaFuncSetAttribute(k_coarse_vcycle<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)M::bytes);
     smem_set = true;
   }
   CoarseArgs A{};
@@ -149,15 +148,9 @@ void coarse_vcycle(const T* r16, const T* const a[4], T* z16, const SolveScalars
   A.act = bt.act;
   A.omega = omega;
   // per sample: r and z on 17^3 nodes, the four coefficient levels
-  const double bytes = (double)bt.n * sizeof(T) *
+  const double bytes = (double)bt.n * sizeof(float) *
                        (2.0 * Lv<16>::nodes + Lv<16>::cells + Lv<8>::cells + Lv<4>::cells + Lv<2>::cells);
-  launch(sizeof(T) == 4 ? "coarse_f32" : "coarse_f64", bytes, k_coarse_vcycle<T>, dim3((unsigned)bt.n), dim3(kCT),
-         M::bytes, st, A);
+  launch("coarse_f32", bytes, k_coarse_vcycle<float>, dim3((unsigned)bt.n), dim3(kCT), M::bytes, st, A);
 }
-
-template void coarse_vcycle<float>(const float*, const float* const[4], float*, const SolveScalars*, const Batch&,
-                                   double, cudaStream_t);
-template void coarse_vcycle<double>(const double*, const double* const[4], double*, const SolveScalars*,
-                                    const Batch&, double, cudaStream_t);
 
 }  // namespace mlsgd

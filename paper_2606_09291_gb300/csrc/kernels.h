@@ -189,9 +189,16 @@ void slab_res(const float* d, const float* p, bool d_zero, const SolveScalars* s
 // launch, one block per launched sample (coarse.cu): r16 the restricted residual, a the
 // coefficients of the levels 16^3 .. 2^3, z16 the correction
 bool coarse_vcycle_applies(int N, int j);
-template <typename T>
-void coarse_vcycle(const T* r16, const T* const a[4], T* z16, const SolveScalars* sc, const Batch& bt, double omega,
-                   cudaStream_t st);
+void coarse_vcycle(const float* r16, const float* const a[4], float* z16, const SolveScalars* sc, const Batch& bt,
+                   double omega, cudaStream_t st);
+// the same in FP64 with a cluster of eight blocks per sample (small64.cu); wd: omega D^-1 of
+// the levels 16^3, 8^3 and 4^3
+cudaError_t coarse_vcycle64(const double* r16, const double* const a[4], const double* const wd[3], double* z16,
+                            const SolveScalars* sc, const Batch& bt, double omega, cudaStream_t st);
+// a whole FP64 PCG solve per sample in one launch on 8^3 and 16^3 grids (small64.cu);
+// builds the coefficient hierarchy itself; arguments as pcg_fp64
+cudaError_t small_fp64(SolverBufs& B, const double* a64, const double* b, long long bstride, double* x_out,
+                       const PcgParams& prm, cudaStream_t st);
 
 // a whole mixed-precision solve per sample in one launch on 8^3 and 16^3 grids (small.cu);
 // builds the coefficient hierarchy itself; arguments as ir_mixed

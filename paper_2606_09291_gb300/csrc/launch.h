@@ -28,4 +28,26 @@ inline void launch_flops(const char* cls, double bytes, double flops, void (*ker
   prof_end(cls, st, bytes, flops);
 }
 
+// a kernel whose blocks form clusters of `cluster` consecutive blocks
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_cluster(const char* cls, double bytes, void (*kern)(KArgs...), dim3 grid, dim3 block,
+                                  unsigned cluster, size_t smem, cudaStream_t st, Args&&... args) {
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = cluster;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  prof_begin(cls, st);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, std::forward<Args>(args)...);
+  prof_end(cls, st, bytes, 0.0);
+  return e;
+}
+
 }  // namespace mlsgd

@@ -653,17 +653,24 @@ __global__ void k_dinv(const TA* __restrict__ a, T* __restrict__ dinv, int N, T 
 
 template <typename T, typename TA0>
 static void build_dinv(SolverBufs& B, const TA0* a0, double omega, cudaStream_t st) {
-  for (int j = 0; j <= B.J; ++j) {
-    if (!B.dinv[j]) continue;
+  auto level = [&](int j, T* out) {
     const int Nj = B.N >> j;
     const dim3 g((unsigned)(((Nj + 1) * (Nj + 1) + kBlock - 1) / kBlock), (unsigned)B.S,
                  (unsigned)((Nj - 1 + kDinvPlanes - 1) / kDinvPlanes));
     if (j == 0)
-      launch("dinv", nbytes<T, TA0>(Nj, B.S, 1, 1), k_dinv<T, TA0>, g, kBlock, 0, st, a0, (T*)B.dinv[0], Nj,
-             (T)omega);
+      launch("dinv", nbytes<T, TA0>(Nj, B.S, 1, 1), k_dinv<T, TA0>, g, kBlock, 0, st, a0, out, Nj, (T)omega);
     else
-      launch("dinv", nbytes<T, T>(Nj, B.S, 1, 1), k_dinv<T, T>, g, kBlock, 0, st, (const T*)B.acoef[j],
-             (T*)B.dinv[j], Nj, (T)omega);
+      launch("dinv", nbytes<T, T>(Nj, B.S, 1, 1), k_dinv<T, T>, g, kBlock, 0, st, (const T*)B.acoef[j], out, Nj,
+             (T)omega);
+  };
+  for (int j = 0; j <= B.J; ++j)
+    if (B.dinv[j]) level(j, (T*)B.dinv[j]);
+  if constexpr (std::is_same<T, double>::value) {
+    // the FP64 cluster V-cycle below a 32^3 level multiplies by omega D^-1 on 8^3 and 4^3
+    // as well; those levels' iterates (vx) are not used otherwise
+    for (int j = 1; j + 2 <= B.J; ++j)
+      if (coarse_vcycle_applies(B.N, j))
+        for (int t = 1; t <= 2; ++t) level(j + t, (T*)B.vx[j + t]);
   }
 }
 
@@ -756,7 +763,12 @@ static int vcycle(SolverBufs& B, const T* r0, const TA0* a0, const SolveScalars*
   if (jc < J) {
     const T* const al[4] = {(const T*)B.acoef[jc], (const T*)B.acoef[jc + 1], (const T*)B.acoef[jc + 2],
                             (const T*)B.acoef[jc + 3]};
-    coarse_vcycle<T>(rin(jc), al, (T*)B.vt[jc], sc, bt, (double)omega, st);
+    if constexpr (std::is_same<T, double>::value) {
+      const double* const wd[3] = {(const double*)B.dinv[jc], (const double*)B.vx[jc + 1], (const double*)B.vx[jc + 2]};
+      (void)coarse_vcycle64(rin(jc), al, wd, (double*)B.vt[jc], sc, bt, (double)omega, st);  // checked by the caller
+    } else {
+      coarse_vcycle(rin(jc), al, (T*)B.vt[jc], sc, bt, (double)omega, st);
+    }
   } else if (J == 0) {
     launch("coarsest", 0.0, k_coarsest<T, TA0>, dim3((n + 127) / 128), 128, 0, st, rin(0), a0, (T*)B.vt[0], sc, n,
            act);

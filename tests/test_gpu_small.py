@@ -56,6 +56,15 @@ def test_mixed_against_oracle(lib, grid, S, knobs):
     _check(grid, la, y, q, phi, z, 1e-6, range(S))
 
 
+@pytest.mark.parametrize("grid", [0, 1, 2, 3])
+@pytest.mark.parametrize("S", [1, 47])
+def test_fp64_against_oracle(lib, grid, S):
+    z = inputs.z_test(32) + inputs.z_random(32, 3)
+    code, la, y, q, phi, it, st = _solve(lib, grid, S, z, precision="fp64", rtol=1e-13)
+    assert code == 0 and not st.any() and (it > 0).all()
+    _check(grid, la, y, q, phi, z, 1e-10, sorted({0, S // 2, S - 1}))
+
+
 @pytest.mark.parametrize("grid,S", [(1, 700), (2, 310)])
 def test_mixed_more_than_one_wave(lib, grid, S):
     z = inputs.z_test(32)
