@@ -200,10 +200,11 @@ mlsgd_status solve_grid(mlsgd_ctx* ctx, int N, int S, const GridFields& f, const
   PcgParams prm{ctx->cfg.rtol, ctx->cfg.max_iter, ctx->cfg.omega > 0 ? ctx->cfg.omega : 0.6, 4};
   const int inner = ctx->cfg.inner_iters > 0 ? ctx->cfg.inner_iters : 6;
   const int inner2 = ctx->cfg.inner_iters_next > 0 ? ctx->cfg.inner_iters_next : inner;
+  // B z first: the solver's vectors, not yet in use, are its scratch
+  launch_rhs_state(z, ctx->Nc(), N, b, scratch, (size_t)(p - scratch), st);
   const bool small = small_supported(N);  // 8^3, 16^3: a solve is one launch
   if (!small && ctx->mixed()) build_hierarchy_mixed(B, f.abf, prm.omega, st);
   if (!small && !ctx->mixed()) build_hierarchy_fp64(B, f.a64, prm.omega, st);
-  launch_rhs_state(z, ctx->Nc(), N, b, st);
   const int fixed = ctx->cfg.ir_steps > 0 ? ctx->cfg.ir_steps : 0;
   const bool pairs = want_pairs && ctx->mixed() && N >= kTiledMinN && B.J >= 1;
   if (pairs_out) *pairs_out = pairs;
@@ -220,13 +221,14 @@ mlsgd_status solve_grid(mlsgd_ctx* ctx, int N, int S, const GridFields& f, const
          iters, status, 0);
   int lev = 0;
   while ((ctx->cfg.n0 << lev) < N) ++lev;
-  if (!pairs) CK(cudaMemsetAsync(badj, 0, S * nodes * sizeof(double), st));  // boundary rows stay 0
+  // the tiled Phi pass writes interior rows only: the boundary rows stay 0
+  if (!pairs && N >= kTiledMinN) CK(cudaMemsetAsync(badj, 0, S * nodes * sizeof(double), st));
   if (pairs) {
     launch_phi_adjrhs_df((const float2*)ytmp, N, S, (float2*)badj, phi, B.partial, ctx->d_gtab2[lev],
                          ctx->d_mgtab2[lev], st);
     e = solve(nullptr, (const float2*)badj, (long long)nodes, q);
   } else {
-    launch_phi_adjrhs(ytmp, N, S, badj, phi, B.partial, ctx->d_gtab[lev], ctx->d_mgtab[lev], st, ctx->freq());
+    launch_phi_adjrhs(ytmp, N, S, badj, phi, B.partial, ctx->d_gtab[lev], ctx->d_mgtab[lev], st);
     e = solve(badj, nullptr, (long long)nodes, q);
   }
   CK(e);

@@ -12,6 +12,15 @@
 
 namespace mlsgd {
 
+// Passes over the control cells march over them with at most kCellBlocks blocks, so that
+// what is the same for every cell, and the FP64 block reductions (five additions per
+// warp, as much as the cell's own work), are paid once per block.
+constexpr int kCellBlocks = 8 * 152;  // eight blocks of 256 threads per SM
+static int cell_blocks(long long n) {
+  const long long b = (n + kBlock - 1) / kBlock;
+  return (int)(b < kCellBlocks ? b : kCellBlocks);
+}
+
 // (B z)_n = int z phi_n (<B u, v> = int u v, Sec. 5) for a cellwise-constant control
 // z on the control grid Nc.
 //
@@ -40,10 +49,116 @@ __global__ void k_rhs_state(const double* __restrict__ z, int Nc, int N, double*
 // Control grid at least as fine as the grid (Nc = r N): the midpoint rule on each
 // control cell c is exact for the multilinear phi_n, so (B z)_n = h_c^3 sum_c z_c
 // phi_n(x_c) over the (2r)^3 control cells of the support.  phi_n(x_c) is a product of
-// one hat weight per axis, w(m) = 1 - |(m + 1/2) / r - 1| for the m-th of the 2r control
-// cells along that axis.  One block per node row (j, k): threads along cx contract
-// the (2r)^2 control rows (cy, cz) of the row's support with w(y) w(z) into a column
-// sum per cx, then each node i of the row contracts its 2r columns with w(x).
+// one hat weight per axis: t = (m + 1/2) / r for the right and 1 - t for the left node of
+// the level cell that holds the m-th control cell along the axis.
+//
+// Bound: FP64 issue, then one read of z.  Contracted axis by axis every control cell
+// costs two FMAs (to the two nodes of its level cell along y), where contracting the
+// (2r)^2 rows of each node row's support costs 4 (and reads z four times).
+// k_rhs_xy: one block per (level cell row ey, control plane cz) contracts y, then x, into
+// u[cz][ey][side][i]; k_rhs_z contracts z.  A 256^3 control onto 8^3: 615 us by node
+// rows, 116 us now.
+__global__ void __launch_bounds__(kBlock) k_rhs_xy(const double* __restrict__ z, int Nc, int N,
+                                                   double* __restrict__ u) {
+  extern __shared__ double sm[];  // t[r], left and right sums [2][Nc]
+  const int r = Nc / N, n1 = N + 1;
+  double* t = sm;
+  double* col = sm + r;
+  const int ey = blockIdx.x, cz = blockIdx.y;
+  const double inv_r = 1.0 / r;
+  for (int m = threadIdx.x; m < r; m += blockDim.x) t[m] = (m + 0.5) * inv_r;
+  __syncthreads();
+  const double* zp = z + (long long)Nc * ((long long)r * ey + (long long)Nc * cz);
+  for (int cx = threadIdx.x; cx < Nc; cx += blockDim.x) {
+    double all = 0.0, right = 0.0;
+#pragma unroll 4
+    for (int m = 0; m < r; ++m) {
+      const double v = zp[(long long)Nc * m + cx];
+      all += v;
+      right = fma(t[m], v, right);
+    }
+    col[cx] = all - right;
+    col[Nc + cx] = right;
+  }
+  __syncthreads();
+  double* ub = u + ((long long)cz * N + ey) * 2 * n1;
+  for (int e = threadIdx.x; e < 2 * n1; e += blockDim.x) {
+    const int side = e / n1, i = e - side * n1;
+    double v = 0.0;
+    if (i > 0 && i < N) {
+      const double* cp = col + side * Nc + r * (i - 1);
+      for (int m = 0; m < r; ++m) v = fma(t[m], cp[m], fma(1.0 - t[m], cp[m + r], v));
+    }
+    ub[e] = v;
+  }
+}
+// node (i, j, k): the right side of cell row j - 1 and the left side of row j, over 2r planes
+__global__ void __launch_bounds__(kBlock) k_rhs_z(const double* __restrict__ u, int Nc, int N,
+                                                  double* __restrict__ b) {
+  const int n1 = N + 1, r = Nc / N;
+  const int n = blockIdx.x * blockDim.x + threadIdx.x;
+  if (n >= n1 * n1 * n1) return;
+  int i, j, k;
+  node_ijk(n, n1, i, j, k);
+  double v = 0.0;
+  if (interior(i, j, k, N)) {
+    const long long plane = (long long)N * 2 * n1;
+    const double* up = u + (long long)r * (k - 1) * plane + (long long)(2 * (j - 1) + 1) * n1 + i;
+    const double inv_r = 1.0 / r;
+    for (int m = 0; m < 2 * r; ++m, up += plane) {
+      const double w = m < r ? (m + 0.5) * inv_r : 2.0 - (m + 0.5) * inv_r;
+      v = fma(w, up[0] + up[n1], v);
+    }
+    const double hc = 1.0 / Nc;
+    v *= hc * hc * hc;
+  }
+  b[n] = v;
+}
+// Control and level grid equal: (B z)_n = h^3 / 8 sum of the eight cells, summed along y,
+// z and x in that order (the order of k_rhs_rows, whose weights are all 1/2 here).  One
+// thread per node column marches over kRhsPlanes planes; a plane's sums serve two nodes.
+constexpr int kRhsPlanes = 16;
+__global__ void __launch_bounds__(kBlock) k_rhs_equal(const double* __restrict__ z, int N, double* __restrict__ b) {
+  const int n1 = N + 1;
+  const int col = blockIdx.x * blockDim.x + threadIdx.x;
+  if (col >= n1 * n1) return;
+  const int j = col / n1, i = col - j * n1;
+  const int k0 = kRhsPlanes * (int)blockIdx.y, k1 = min(N, k0 + kRhsPlanes - 1);
+  const long long pn = (long long)n1 * n1, pc = (long long)N * N;
+  double* o = b + pn * k0 + col;
+  const bool in = i > 0 && j > 0 && i < N && j < N;
+  const double* c = z + (in ? (i - 1) + (long long)N * (j - 1) : 0);
+  const double h = 1.0 / N, w = 0.125 * (h * h * h);
+  double lo0 = 0.0, lo1 = 0.0;  // y sums of the cell columns i - 1 and i in the plane below
+  if (in && k0 > 0) {
+    const double* p = c + pc * (k0 - 1);
+    lo0 = p[0] + p[N];
+    lo1 = p[1] + p[N + 1];
+  }
+  c += pc * k0;
+  for (int k = k0; k <= k1; ++k, o += pn, c += pc) {
+    double v = 0.0;
+    if (in && k < N) {
+      const double up0 = c[0] + c[N], up1 = c[1] + c[N + 1];
+      if (k > 0) v = w * ((lo0 + up0) + (lo1 + up1));
+      lo0 = up0;
+      lo1 = up1;
+    }
+    *o = v;
+  }
+}
+
+// The by-axis form from r = Nc / N = 4 on.  At r = 2 it takes about as many operations as
+// the node rows (145 against 156 us of FP64 issue for a 256^3 control on 128^3), which
+// need no scratch.
+constexpr int kRhsAxisR = 4;
+size_t rhs_scratch_bytes(int Nc, int N) {  // u of k_rhs_xy
+  return Nc >= kRhsAxisR * N ? (size_t)Nc * N * 2 * (N + 1) * sizeof(double) : 0;
+}
+
+// The form of r = 2, and without scratch of any r: one block per node row (j, k); threads along cx contract the
+// (2r)^2 control rows (cy, cz) of the row's support with w(y) w(z) into a column sum per
+// cx, then each node i of the row contracts its 2r columns with w(x).
 __global__ void __launch_bounds__(kBlock) k_rhs_rows(const double* __restrict__ z, int Nc, int N,
                                                      double* __restrict__ b) {
   extern __shared__ double sm[];  // w[2r], col[Nc]
@@ -84,10 +199,23 @@ __global__ void __launch_bounds__(kBlock) k_rhs_rows(const double* __restrict__ 
   }
 }
 
-void launch_rhs_state(const double* z, int Nc, int N, double* b, cudaStream_t st) {
+// scratch: memory the launch may overwrite (the by-axis form needs rhs_scratch_bytes)
+void launch_rhs_state(const double* z, int Nc, int N, double* b, void* scratch, size_t scratch_bytes,
+                      cudaStream_t st) {
   const double bytes = (double)cells_of(Nc) * 8 + (double)nodes_of(N) * 8;
   if (N > Nc) {
     launch("rhs", bytes, k_rhs_state, dim3(node_blocks(N)), kBlock, 0, st, z, Nc, N, b);
+  } else if (N == Nc) {
+    launch("rhs", bytes, k_rhs_equal,
+           dim3((unsigned)(((N + 1) * (N + 1) + kBlock - 1) / kBlock), (unsigned)((N + kRhsPlanes) / kRhsPlanes)), kBlock,
+           0, st, z, N, b);
+  } else if (Nc >= kRhsAxisR * N && rhs_scratch_bytes(Nc, N) <= scratch_bytes) {
+    double* u = (double*)scratch;
+    const double ub = (double)rhs_scratch_bytes(Nc, N);
+    launch("rhs", (double)cells_of(Nc) * 8 + ub, k_rhs_xy, dim3((unsigned)N, (unsigned)Nc), kBlock,
+           (size_t)(Nc / N + 2 * Nc) * sizeof(double), st, z, Nc, N, u);
+    launch("rhs", ub + (double)nodes_of(N) * 8, k_rhs_z, dim3(node_blocks(N)), kBlock, 0, st, (const double*)u, Nc, N,
+           b);
   } else {
     const size_t smem = (size_t)(2 * (Nc / N) + Nc) * sizeof(double);
     launch("rhs", bytes, k_rhs_rows, dim3((unsigned)(N + 1), (unsigned)(N + 1)), kBlock, smem, st, z, Nc, N, b);
@@ -98,51 +226,43 @@ void launch_rhs_state(const double* z, int Nc, int N, double* b, cudaStream_t st
 // (M e)_n with the consistent Q1 mass M = (h/6)^3 [1 4 1]^(x3); badj = M e on
 // interior rows (adjoint right-hand side <y - g, v>_H, Sec. 2.2) and
 // Phi = 1/2 e^T M e (eq:cost), reduced per sample in FP64.
-__global__ void k_phi_adjrhs(const double* __restrict__ y, int N, double* __restrict__ badj,
-                             double* __restrict__ partial, int freq) {
-  const int s = blockIdx.y;
-  const int n1 = N + 1;
-  const long long nodes = (long long)n1 * n1 * n1;
-  const int n = blockIdx.x * blockDim.x + threadIdx.x;
-  const double* ys = y + s * nodes;
+// One block per sample (grids below the tiled ones, at most 9^3 nodes): y in shared memory,
+// the mass [1 4 1] axis by axis, g and M g from the 1D tables (both separable), Phi summed
+// in the block.  1024 samples of 8^3: 314 us with nine sines and 27 weighted products per
+// node, 29 us now.
+__global__ void __launch_bounds__(kBlock) k_phi_small(const double* __restrict__ y, int N, double* __restrict__ badj,
+                                                      double* __restrict__ phi, const double* __restrict__ gtab,
+                                                      const double* __restrict__ mgtab) {
+  __shared__ double u[729], v[729];
+  const int s = blockIdx.x, n1 = N + 1, nodes = n1 * n1 * n1;
+  const double* ys = y + (long long)s * nodes;
+  for (int n = threadIdx.x; n < nodes; n += kBlock) u[n] = ys[n];  // 0 on the boundary
+  __syncthreads();
+  for (int n = threadIdx.x; n < nodes; n += kBlock) {
+    const int i = n % n1;
+    v[n] = (i > 0 && i < N) ? fma(4.0, u[n], u[n - 1] + u[n + 1]) : 0.0;
+  }
+  __syncthreads();
+  for (int n = threadIdx.x; n < nodes; n += kBlock) {
+    const int j = (n / n1) % n1;
+    u[n] = (j > 0 && j < N) ? fma(4.0, v[n], v[n - n1] + v[n + n1]) : 0.0;
+  }
+  __syncthreads();
+  const double h6 = 1.0 / (6.0 * N), h63 = h6 * h6 * h6;
   double contrib = 0.0;
-  if (n < nodes) {
+  for (int n = threadIdx.x; n < nodes; n += kBlock) {
     int i, j, k;
     node_ijk(n, n1, i, j, k);
     double me = 0.0;
     if (interior(i, j, k, N)) {
-      const double invN = (double)freq / N;  // g = prod sin(freq pi x)
-      double gx[3], gy[3], gz[3];
-      for (int d = -1; d <= 1; ++d) {
-        gx[d + 1] = sinpi((i + d) * invN);
-        gy[d + 1] = sinpi((j + d) * invN);
-        gz[d + 1] = sinpi((k + d) * invN);
-      }
-      for (int w = -1; w <= 1; ++w) {
-        const int kk = k + w;
-        const double mz = (w == 0) ? 4.0 : 1.0;
-        const double gzv = (kk == 0 || kk == N) ? 0.0 : gz[w + 1];
-        for (int v = -1; v <= 1; ++v) {
-          const int jj = j + v;
-          const double my = (v == 0) ? 4.0 : 1.0;
-          const double gyv = (jj == 0 || jj == N) ? 0.0 : gy[v + 1];
-          for (int u = -1; u <= 1; ++u) {
-            const int ii = i + u;
-            const double mx = (u == 0) ? 4.0 : 1.0;
-            const double gxv = (ii == 0 || ii == N) ? 0.0 : gx[u + 1];
-            const double e = ys[ii + (long long)n1 * (jj + (long long)n1 * kk)] - gxv * gyv * gzv;
-            me += mx * my * mz * e;
-          }
-        }
-      }
-      const double h6 = 1.0 / (6.0 * N);
-      me *= h6 * h6 * h6;
-      contrib = (ys[n] - gx[1] * gy[1] * gz[1]) * me;
+      const double my = fma(4.0, u[n], u[n - n1 * n1] + u[n + n1 * n1]);
+      me = h63 * my - mgtab[i] * mgtab[j] * mgtab[k];
+      contrib = fma(ys[n] - gtab[i] * gtab[j] * gtab[k], me, contrib);
     }
-    badj[s * nodes + n] = me;
+    badj[(long long)s * nodes + n] = me;
   }
-  const double bs = block_sum(contrib);
-  if (threadIdx.x == 0) partial[(long long)s * gridDim.x + blockIdx.x] = bs;
+  contrib = block_sum(contrib);
+  if (threadIdx.x == 0) phi[s] = 0.5 * contrib;
 }
 
 __global__ void k_phi_finish(const double* __restrict__ partial, int nblk, int S, double* __restrict__ phi) {
@@ -164,22 +284,20 @@ void launch_phi_adjrhs_df(const float2* y, int N, int S, float2* badj, double* p
 }
 
 void launch_phi_adjrhs(const double* y, int N, int S, double* badj, double* phi, double* partial, const double* gtab,
-                       const double* mgtab, cudaStream_t st, int freq) {
+                       const double* mgtab, cudaStream_t st) {
   if (S == 0) return;
-  if (N >= kTiledMinN && gtab != nullptr) {
-    const int nb = tiled_phi(y, N, S, gtab, mgtab, badj, partial, st);
-    launch("phi_finish", 0.0, k_phi_finish, dim3((S + 7) / 8), 256, 0, st, (const double*)partial, nb, S, phi);
+  if (N < kTiledMinN) {
+    launch("phi_adjrhs", (double)S * nodes_of(N) * 16, k_phi_small, dim3((unsigned)S), kBlock, 0, st, y, N, badj, phi,
+           gtab, mgtab);
     return;
   }
-  const int nb = node_blocks(N);
-  launch("phi_adjrhs", (double)S * nodes_of(N) * 16, k_phi_adjrhs, dim3(nb, S), kBlock, 0, st, y, N, badj, partial,
-         freq);
+  const int nb = tiled_phi(y, N, S, gtab, mgtab, badj, partial, st);
   launch("phi_finish", 0.0, k_phi_finish, dim3((S + 7) / 8), 256, 0, st, (const double*)partial, nb, S, phi);
 }
 
 // ---------------------------------------------------------------- level statistics
 // work layout: [0] shift_new, [1] scale_old = exp(theta (shift_old - shift_new)),
-// [2] n_old, [3] n_batch, [4..4+S) w_fine, [4+S..4+2S) w_coarse, then the same
+// [2] n_old, [3] n_old / (n_old + S), [4..4+S) w_fine, [4+S..4+2S) w_coarse, then the same
 // weights as FP32 (hi, lo) pairs (8 bytes each): [4+2S..4+3S) fine, [4+3S..4+4S) coarse.
 //
 // Single block: shift, per-sample weights Y~ = exp(theta (Phi - shift)), and
@@ -206,7 +324,7 @@ __global__ void k_level_scalars(const double* __restrict__ phif, const double* _
     work[0] = shift;
     work[1] = (n_old > 0.0) ? exp(theta * (shift_old - shift)) : 0.0;
     work[2] = n_old;
-    work[3] = (double)S;
+    work[3] = n_old / (n_old + S);
   }
   __syncthreads();
   const double shift = work[0];
@@ -305,6 +423,19 @@ __device__ __forceinline__ double eval_at_ctrl(const double* __restrict__ q, int
   return (c00 * (1 - ty) + c10 * ty) * (1 - tz) + (c01 * (1 - ty) + c11 * ty) * tz;
 }
 
+// FP32 -> FP64 by moving the fields (IEEE 754 binary32 and binary64 layouts), in
+// integer instructions instead of the FP64 conversion: exponent rebiased by
+// 1023 - 127, mantissa shifted into the top of the 52-bit field; 0 and subnormals
+// give a signed 0, Inf and NaN keep their class (a NaN stays a NaN).
+__device__ __forceinline__ double f2d(float f) {
+  const uint32_t u = __float_as_uint(f);
+  const uint32_t e = (u >> 23) & 0xffu, m = u & 0x7fffffu;
+  const uint32_t e11 = e == 0u ? 0u : (e == 0xffu ? 0x7ffu : e + 896u);
+  const uint32_t mh = e == 0u ? 0u : ((m >> 3) | ((e == 0xffu && m != 0u) ? 0x80000u : 0u));
+  const uint32_t hi = (u & 0x80000000u) | (e11 << 20) | mh;
+  const uint32_t lo = e == 0u ? 0u : (m << 29);
+  return __hiloint2double((int)hi, (int)lo);
+}
 // The eight trilinear weights of a control-cell centre inside a level cell
 // (level no finer than the control grid), set up once per control cell.
 struct CellInterp {
@@ -312,17 +443,20 @@ struct CellInterp {
   long long sy, sz;
   double w[8];     // weight of node (ex + a, ey + b, ez + c) at index a + 2b + 4c
   float w32[8];    // the same weights (exact in FP32: r is a power of two)
+  // the weights are dyadic and exact in FP32, so they are formed there (an FP64 division
+  // is some 20 operations of the pipe that bounds the kernel)
   __device__ void setup(int N, int Nc, int cx, int cy, int cz) {
     const int n1 = N + 1, r = Nc / N;
-    const double tx = ((cx % r) + 0.5) / r, ty = ((cy % r) + 0.5) / r, tz = ((cz % r) + 0.5) / r;
+    const float ir = 1.0f / (float)r;
+    const float tx = ((cx % r) + 0.5f) * ir, ty = ((cy % r) + 0.5f) * ir, tz = ((cz % r) + 0.5f) * ir;
     base = (cx / r) + (long long)n1 * ((cy / r) + (long long)n1 * (cz / r));
     sy = n1;
     sz = (long long)n1 * n1;
 #pragma unroll
-    for (int e = 0; e < 8; ++e)
-      w[e] = ((e & 1) ? tx : 1.0 - tx) * ((e & 2) ? ty : 1.0 - ty) * ((e & 4) ? tz : 1.0 - tz);
-#pragma unroll
-    for (int e = 0; e < 8; ++e) w32[e] = (float)w[e];
+    for (int e = 0; e < 8; ++e) {
+      w32[e] = ((e & 1) ? tx : 1.0f - tx) * ((e & 2) ? ty : 1.0f - ty) * ((e & 4) ? tz : 1.0f - tz);
+      w[e] = f2d(w32[e]);
+    }
   }
   // the same average of an FP32 pair field, in pair arithmetic
   __device__ __forceinline__ DF eval(const float2* __restrict__ q) const {
@@ -353,37 +487,52 @@ struct CellInterp {
   }
 };
 
-// The same trilinear average for FP32 pair fields with the weights kept as three
-// per-axis pairs (exact dyadic values, so each product equals CellInterp's w32) and a
-// 32-bit node index: fewer registers per thread, so more threads in flight.
+// The same trilinear average for FP32 pair fields on a grid R times coarser than the
+// control grid, R known at compile time: three per-axis weight pairs (exact dyadic values,
+// so each product equals CellInterp's w32), a 32-bit node index, and for R = 1 no product
+// at all (every weight is 1/8: the sum is scaled, which is exact).
+template <int R>
 struct PairInterp {
   int base, sy, sz;
-  float wx[2], wy[2], wz[2];
-  __device__ void setup(int N, int Nc, int cx, int cy, int cz) {
-    const int n1 = N + 1, r = Nc / N;
-    const float ir = 1.0f / (float)r;  // r a power of two: exact
-    const float tx = ((cx % r) + 0.5f) * ir, ty = ((cy % r) + 0.5f) * ir, tz = ((cz % r) + 0.5f) * ir;
-    wx[0] = 1.0f - tx; wx[1] = tx;
-    wy[0] = 1.0f - ty; wy[1] = ty;
-    wz[0] = 1.0f - tz; wz[1] = tz;
-    base = (cx / r) + n1 * ((cy / r) + n1 * (cz / r));
+  float tx, ty, tz;
+  __device__ __forceinline__ void setup(int N, int cx, int cy, int cz) {
+    const int n1 = N + 1;
+    constexpr float ir = 1.0f / R;
+    tx = ((cx % R) + 0.5f) * ir;
+    ty = ((cy % R) + 0.5f) * ir;
+    tz = ((cz % R) + 0.5f) * ir;
+    base = (cx / R) + n1 * ((cy / R) + n1 * (cz / R));
     sy = n1;
     sz = n1 * n1;
   }
   __device__ __forceinline__ DF eval(const float2* __restrict__ q) const {
     const float2* b = q + base;
+    float2 v[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) v[e] = b[(e & 1) + ((e >> 1) & 1) * sy + (e >> 2) * sz];
     float s = 0.f, c = 0.f;
 #pragma unroll
     for (int e = 0; e < 8; ++e) {
-      const float w = (wx[e & 1] * wy[(e >> 1) & 1]) * wz[e >> 2];  // exact
-      const float2 v = b[(e & 1) + ((e >> 1) & 1) * sy + (e >> 2) * sz];
-      const float p = __fmul_rn(w, v.x);
-      const float pe = __fmaf_rn(w, v.y, __fmaf_rn(w, v.x, -p));
+      float p, pe;
+      if constexpr (R == 1) {
+        p = v[e].x;
+        pe = v[e].y;
+      } else {
+        const float w = (((e & 1) ? tx : 1.0f - tx) * ((e & 2) ? ty : 1.0f - ty)) * ((e & 4) ? tz : 1.0f - tz);  // exact
+        p = __fmul_rn(w, v[e].x);
+        pe = __fmaf_rn(w, v[e].y, __fmaf_rn(w, v[e].x, -p));
+      }
+      if (e == 0) {
+        s = p;
+        c = pe;
+        continue;
+      }
       const float t = __fadd_rn(s, p);  // two-sum (intrinsics: never contracted)
       const float bb = __fsub_rn(t, s);
       c = __fadd_rn(c, __fadd_rn(__fadd_rn(__fsub_rn(s, __fsub_rn(t, bb)), __fsub_rn(p, bb)), pe));
       s = t;
     }
+    if constexpr (R == 1) return df_norm(0.125f * s, 0.125f * c);
     return df_norm(s, c);
   }
 };
@@ -428,19 +577,6 @@ __device__ __forceinline__ double ctrl_avg(const CellInterp& I, bool fast, const
                                            int cy, int cz) {
   return fast ? I.eval(q) : eval_at_ctrl(q, N, Nc, cx, cy, cz);
 }
-// FP32 -> FP64 by moving the fields (IEEE 754 binary32 and binary64 layouts), in
-// integer instructions instead of the FP64 conversion: exponent rebiased by
-// 1023 - 127, mantissa shifted into the top of the 52-bit field; 0 and subnormals
-// give a signed 0, Inf and NaN keep their class (a NaN stays a NaN).
-__device__ __forceinline__ double f2d(float f) {
-  const uint32_t u = __float_as_uint(f);
-  const uint32_t e = (u >> 23) & 0xffu, m = u & 0x7fffffu;
-  const uint32_t e11 = e == 0u ? 0u : (e == 0xffu ? 0x7ffu : e + 896u);
-  const uint32_t mh = e == 0u ? 0u : ((m >> 3) | ((e == 0xffu && m != 0u) ? 0x80000u : 0u));
-  const uint32_t hi = (u & 0x80000000u) | (e11 << 20) | mh;
-  const uint32_t lo = e == 0u ? 0u : (m << 29);
-  return __hiloint2double((int)hi, (int)lo);
-}
 __device__ __forceinline__ DF ctrl_avg_df(const CellInterp& I, bool fast, const float2* q, int N, int Nc, int cx,
                                           int cy, int cz) {
   return fast ? I.eval(q) : eval_at_ctrl(q, N, Nc, cx, cy, cz);
@@ -449,46 +585,31 @@ __device__ __forceinline__ double ctrl_avg(const CellInterp& I, bool fast, const
                                            int cy, int cz) {
   return df_to_double(ctrl_avg_df(I, fast, q, N, Nc, cx, cy, cz));
 }
-template <bool PF, bool PC, bool FAST = false>
-__global__ void k_level_field(const void* __restrict__ qf_, int Nf, const void* __restrict__ qc_, int Ncs, int S,
-                              int Nc, const double* __restrict__ work, double* __restrict__ field,
-                              double* __restrict__ partial) {
+template <bool PF, bool PC>
+__global__ void __launch_bounds__(kBlock) k_level_field(const void* __restrict__ qf_, int Nf,
+                                                        const void* __restrict__ qc_, int Ncs, int S, int Nc,
+                                                        double inv_s, const double* __restrict__ work,
+                                                        double* __restrict__ field, double* __restrict__ partial) {
   using QF = typename std::conditional<PF, float2, double>::type;
   using QC = typename std::conditional<PC, float2, double>::type;
   const QF* qf = (const QF*)qf_;
   const QC* qc = (const QC*)qc_;
-  const long long ncell = (long long)Nc * Nc * Nc;
-  const long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  const unsigned ncell = (unsigned)Nc * Nc * Nc;  // at most 1024^3
+  const unsigned step = gridDim.x * kBlock;
+  const long long nf = nodes_of(Nf), ncn = qc ? nodes_of(Ncs) : 0;
+  const double* wf = work + 4;
+  const double* wc = work + 4 + S;
+  const float2* wfp = (const float2*)(work + 4 + 2 * S);
+  const float2* wcp = wfp + S;
+  // level grids no finer than the control grid: weights hoisted out of the sample loop
+  const bool fast_f = Nf <= Nc, fast_c = !qc || Ncs <= Nc;
+  const double n_old = work[2], scale = work[1], a = work[3];
+  const double as = a * S;  // n_old S / (n_old + S)
   double contrib = 0.0;
-  if (c < ncell) {
-    const int cx = (int)(c % Nc), cy = (int)((c / Nc) % Nc), cz = (int)(c / ((long long)Nc * Nc));
-    const long long nf = nodes_of(Nf), ncn = qc ? nodes_of(Ncs) : 0;
-    const double* wf = work + 4;
-    const double* wc = work + 4 + S;
-    const float2* wfp = (const float2*)(work + 4 + 2 * S);
-    const float2* wcp = wfp + S;
-    // level grids no finer than the control grid: weights hoisted out of the sample loop
-    const bool fast_f = Nf <= Nc, fast_c = !qc || Ncs <= Nc;
+  for (unsigned c = blockIdx.x * kBlock + threadIdx.x; c < ncell; c += step) {
+    const unsigned row = c / (unsigned)Nc;
+    const int cx = (int)(c - row * Nc), cz = (int)(row / (unsigned)Nc), cy = (int)(row - (unsigned)cz * Nc);
     double ref = 0.0, sd = 0.0, sd2 = 0.0;
-    if constexpr (PF && PC && FAST) {  // both grids no finer than the control grid
-      PairInterp Pf{}, Pc{};
-      Pf.setup(Nf, Nc, cx, cy, cz);
-      Pc.setup(Ncs, Nc, cx, cy, cz);
-      // sample pointers advanced by addition: a 64-bit multiply per sample would issue
-      // on the FP64 pipe of this part, the kernel's bottleneck
-      const QF* qfs = qf;
-      const QC* qcs = qc;
-      for (int s = 0; s < S; ++s, qfs += nf, qcs += ncn) {
-        const DF vf = df_mul(df_make(wfp[s]), Pf.eval(qfs));
-        const DF vc = df_mul(df_make(wcp[s]), Pc.eval(qcs));
-        const DF vd = df_add(vf, df_neg(vc));
-        const double v = f2d(vd.h) + f2d(vd.l);
-        if (s == 0) ref = v;
-        const double d = v - ref;
-        sd += d;
-        sd2 = fma(d, d, sd2);
-      }
-    } else {
     CellInterp If{}, Ic{};
     if (fast_f) If.setup(Nf, Nc, cx, cy, cz);
     if (qc && fast_c) Ic.setup(Ncs, Nc, cx, cy, cz);
@@ -508,19 +629,92 @@ __global__ void k_level_field(const void* __restrict__ qf_, int Nf, const void* 
       sd += d;
       sd2 = fma(d, d, sd2);
     }
-    }
-    const double mean = ref + sd / S;
-    const double m2 = fmax(sd2 - sd * (sd / S), 0.0);
-    const double n_old = work[2], scale = work[1];
-    const double n = n_old + S;
+    const double mean = fma(sd, inv_s, ref);
+    const double m2 = fmax(fma(-sd * inv_s, sd, sd2), 0.0);
     const double mo = (n_old > 0.0) ? field[c] * scale : 0.0;
     const double delta = mo - mean;
-    field[c] = mean + (n_old / n) * delta;
-    const double hc = 1.0 / Nc;
-    contrib = hc * hc * hc * (m2 + delta * delta * n_old * S / n);
+    field[c] = fma(a, delta, mean);
+    contrib += fma(as * delta, delta, m2);
   }
   const double bs = block_sum(contrib);
-  if (threadIdx.x == 0) partial[blockIdx.x] = bs;
+  const double hc = 1.0 / Nc;
+  if (threadIdx.x == 0) partial[blockIdx.x] = hc * hc * hc * bs;
+}
+
+// k_level_field for pairs on both grids, the fine one RF (1 or 2) times coarser than the
+// control grid: the bulk of a difference level's statistics.  The FP32 pair arithmetic and
+// the FP64 sums (four operations per cell and sample) take about the same time, and the
+// 16 scattered loads need threads in flight: 64 registers, four blocks per SM.  G = 4
+// splits the samples of a cell over four threads (their sums joined in a fixed order), for
+// batches on control grids too small to fill the SMs with one thread per cell: 512 samples
+// of 64^3 on a 64^3 control: 1.6 ms; 4
+// samples of 128^3 on 256^3: 2.8 ms with the divisions and a block sum per 256 cells, 0.94 ms now.
+constexpr int kPairBlocks = 4 * 152;
+template <int RF, int G>
+__global__ void __launch_bounds__(kBlock, 4) k_level_pairs(const float2* __restrict__ qf, int Nf,
+                                                           const float2* __restrict__ qc, int S, int Nc, double inv_s,
+                                                           const double* __restrict__ work, double* __restrict__ field,
+                                                           double* __restrict__ partial) {
+  constexpr int CB = kBlock / G;  // cells per block
+  __shared__ double sums[G > 1 ? 2 : 1][G][CB];
+  const unsigned ncell = (unsigned)Nc * Nc * Nc;
+  const int tc = threadIdx.x % CB, g = threadIdx.x / CB;
+  const int Ncs = Nf / 2;
+  const long long nf = nodes_of(Nf), nc = nodes_of(Ncs);
+  const float2* wfp = (const float2*)(work + 4 + 2 * S);
+  const float2* wcp = wfp + S;
+  double contrib = 0.0;
+  for (unsigned c0 = blockIdx.x * CB; c0 < ncell; c0 += gridDim.x * CB) {  // ncell is a multiple of 8
+    const unsigned c = c0 + tc < ncell ? c0 + tc : ncell - 1;
+    const unsigned row = c / (unsigned)Nc;
+    const int cx = (int)(c - row * Nc), cz = (int)(row / (unsigned)Nc), cy = (int)(row - (unsigned)cz * Nc);
+    PairInterp<RF> Pf;
+    PairInterp<2 * RF> Pc;
+    Pf.setup(Nf, cx, cy, cz);
+    Pc.setup(Ncs, cx, cy, cz);
+    auto value = [&](int s, const float2* f, const float2* k) {
+      const DF vf = df_mul(df_make(wfp[s]), Pf.eval(f));
+      const DF vc = df_mul(df_make(wcp[s]), Pc.eval(k));
+      const DF vd = df_add(vf, df_neg(vc));
+      return f2d(vd.h) + f2d(vd.l);
+    };
+    // sample pointers advanced by addition: a 64-bit multiply per sample would issue on
+    // the FP64 pipe
+    const double ref = value(0, qf, qc);
+    double sd = 0.0, sd2 = 0.0;
+    const int s0 = g == 0 ? G : g;  // sample 0 is the reference: its deviation is 0
+    const float2 *f = qf + (long long)s0 * nf, *k = qc + (long long)s0 * nc;
+    for (int s = s0; s < S; s += G, f += G * nf, k += G * nc) {
+      const double d = value(s, f, k) - ref;
+      sd += d;
+      sd2 = fma(d, d, sd2);
+    }
+    if constexpr (G > 1) {
+      sums[0][g][tc] = sd;
+      sums[1][g][tc] = sd2;
+      __syncthreads();
+      if (g == 0) {
+#pragma unroll
+        for (int q = 1; q < G; ++q) {
+          sd += sums[0][q][tc];
+          sd2 += sums[1][q][tc];
+        }
+      }
+      __syncthreads();
+    }
+    if (g == 0 && c0 + tc < ncell) {
+      const double a = work[3];  // n_old / (n_old + S)
+      const double mean = fma(sd, inv_s, ref);
+      const double m2 = fmax(fma(-sd * inv_s, sd, sd2), 0.0);
+      const double mo = (work[2] > 0.0) ? field[c] * work[1] : 0.0;
+      const double delta = mo - mean;
+      field[c] = fma(a, delta, mean);
+      contrib += fma(a * S * delta, delta, m2);
+    }
+  }
+  const double bs = block_sum(contrib);
+  const double hc = 1.0 / Nc;
+  if (threadIdx.x == 0) partial[blockIdx.x] = hc * hc * hc * bs;
 }
 
 // ---- statistics of a level whose grids are coarser than the control grid (Nc = r Nf,
@@ -528,163 +722,201 @@ __global__ void k_level_field(const void* __restrict__ qf_, int Nf, const void* 
 // x_s = w_f[s] q_f[s] - w_c[s] P q_c[s] on the level's fine grid (P q_c: the coarse
 // trilinear function at the fine nodes, which interpolation to the control cells
 // reproduces exactly) the batch mean field is the interpolation of the nodal mean,
-// and ||I x||_U^2 = sum over level cells e of x_e^T G x_e with the fixed 8 x 8 Gram
-// matrix G = h_f^3 (g x g x g), g = (1/r) sum_m w(t_m) w(t_m)^T, w(t) = (1 - t, t),
-// t_m = (m + 1/2)/r (the midpoint rule over the r^3 control cells of a level cell is
-// exact for the integrand of these trilinear weights).  M2 of the batch is then
-// sum_s ||d_s||_G^2 - S ||mean d||_G^2 with d_s = x_s - x_0 (deviations from the
-// first sample, as in k_level_field).  Work per sample: the level's nodes and cells,
-// not the control cells.
+// and ||I x||_U^2 = h_f^3 x^T (g x g x g) x with the 1D Gram matrix g assembled from
+// (1/r) sum_m w(t_m) w(t_m)^T, w(t) = (1 - t, t), t_m = (m + 1/2)/r (the midpoint rule over
+// the r^3 control cells of a level cell is exact for the integrand of these trilinear
+// weights): rows [B, 2A, B], x is 0 on the boundary.  M2 of the batch is the sum over
+// samples of that form of x_s - mean.  Work per sample: the level's nodes, not the
+// control cells.
+//
+// Bound: FP64 issue.  The form is applied axis by axis (three operations per node and
+// axis) to the deviations from the mean, where the 8 x 8 matrix per level cell took 64 per
+// cell.  Values given as FP32 pairs enter FP64 by integer instructions (f2d) and one addition.
 __device__ __forceinline__ double ldq(const double* p, long long i) { return p[i]; }
 __device__ __forceinline__ double ldq(const float2* p, long long i) {
   const float2 v = p[i];
-  return (double)v.x + (double)v.y;
-}
-template <typename QF, typename QC>
-__device__ __forceinline__ double lvl_x(const QF* qfs, const QC* qcs, int Nf, int i, int j, int k, double wf,
-                                        double wc) {
-  const int n1 = Nf + 1;
-  double v = wf * ldq(qfs, i + (long long)n1 * (j + (long long)n1 * k));
-  if (qcs) {
-    const int c1 = Nf / 2 + 1;
-    const int di = i & 1, dj = j & 1, dk = k & 1;
-    const long long b = (i >> 1) + (long long)c1 * ((j >> 1) + (long long)c1 * (k >> 1));
-    double acc = 0.0;
-    for (int c = 0; c <= dk; ++c)
-      for (int bb = 0; bb <= dj; ++bb)
-        for (int a = 0; a <= di; ++a) acc += ldq(qcs, b + a + (long long)c1 * (bb + (long long)c1 * c));
-    v -= wc * acc * (1.0 / (double)(1 << (di + dj + dk)));
-  }
-  return v;
+  return f2d(v.x) + f2d(v.y);
 }
 // x_s at every node of the level grid, written over q_f (same 8-byte slots; q_f is
 // not needed after the statistics)
 template <typename QF, typename QC>
-__global__ void k_lvl_x(QF* __restrict__ qf, int Nf, const QC* __restrict__ qc, int S,
-                        const double* __restrict__ work) {
+__global__ void __launch_bounds__(kBlock) k_lvl_x(QF* __restrict__ qf, int Nf, const QC* __restrict__ qc, int S,
+                                                  const double* __restrict__ work) {
   const int s = blockIdx.y;
-  const int n1 = Nf + 1;
-  const long long nodes = (long long)n1 * n1 * n1;
-  const long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  const int n1 = Nf + 1, nodes = n1 * n1 * n1;  // at most 257^3 (the control grid is 4x finer)
+  const int n = blockIdx.x * blockDim.x + threadIdx.x;
   if (n >= nodes) return;
-  const int i = (int)(n % n1), j = (int)((n / n1) % n1), k = (int)(n / ((long long)n1 * n1));
-  const long long ncn = qc ? nodes_of(Nf / 2) : 0;
-  const double x = lvl_x(qf + s * nodes, qc ? qc + s * ncn : (const QC*)nullptr, Nf, i, j, k, work[4 + s],
-                         work[4 + S + s]);
-  reinterpret_cast<double*>(qf)[s * nodes + n] = x;
-}
-// nodal x_0 and sum_s (x_s - x_0)
-__global__ void k_lvl_nodes(const double* __restrict__ x, long long nodes, int S, double* __restrict__ x0,
-                            double* __restrict__ dsum) {
-  const long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (n >= nodes) return;
-  const double xr = x[n];
-  double ds = 0.0;
-  for (int s = 1; s < S; ++s) ds += x[s * nodes + n] - xr;
-  x0[n] = xr;
-  dsum[n] = ds;
-}
-// d^T G d for the 8 nodal values of a level cell (index a + 2b + 4c)
-__device__ __forceinline__ double gram8(const double* d, double A, double B) {
-  double t[8], u[8];
-#pragma unroll
-  for (int e = 0; e < 8; e += 2) { t[e] = A * d[e] + B * d[e + 1]; t[e + 1] = B * d[e] + A * d[e + 1]; }
-#pragma unroll
-  for (int e = 0; e < 8; ++e) {
-    if (e & 2) continue;
-    u[e] = A * t[e] + B * t[e + 2];
-    u[e + 2] = B * t[e] + A * t[e + 2];
-  }
-  double q = 0.0;
-#pragma unroll
-  for (int e = 0; e < 4; ++e) q += d[e] * (A * u[e] + B * u[e + 4]) + d[e + 4] * (B * u[e] + A * u[e + 4]);
-  return q;
-}
-// per level cell: sum_s ||d_s||^2 - S ||mean d||^2 over the cell, block partials;
-// blockIdx.y takes samples y, y + gridDim.y, ... (the mean term goes with y = 0)
-__global__ void k_lvl_cells(const double* __restrict__ x, int Nf, int S, const double* __restrict__ x0,
-                            const double* __restrict__ dsum, double A, double B, double hf3,
-                            double* __restrict__ partial) {
-  const long long cells = (long long)Nf * Nf * Nf;
-  const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  double contrib = 0.0;
-  if (e < cells) {
-    const int ci = (int)(e % Nf), cj = (int)((e / Nf) % Nf), ck = (int)(e / ((long long)Nf * Nf));
-    const int n1 = Nf + 1;
-    const long long nodes = (long long)n1 * n1 * n1;
-    long long nv[8];
-    double xr[8];
-#pragma unroll
-    for (int v = 0; v < 8; ++v) {
-      nv[v] = (ci + (v & 1)) + (long long)n1 * ((cj + ((v >> 1) & 1)) + (long long)n1 * (ck + (v >> 2)));
-      xr[v] = x0[nv[v]];
-    }
+  int i, j, k;
+  node_ijk(n, n1, i, j, k);
+  QF* qs = qf + (long long)s * nodes;
+  double x = work[4 + s] * ldq(qs, n);
+  if (qc) {
+    const int c1 = Nf / 2 + 1;
+    const QC* q = qc + (long long)s * (c1 * c1 * c1) + (i >> 1) + c1 * ((j >> 1) + c1 * (k >> 1));
+    const int di = i & 1, dj = j & 1, dk = k & 1;
     double acc = 0.0;
-    for (int s = blockIdx.y; s < S; s += gridDim.y) {
-      const double* xs = x + s * nodes;
-      double d[8];
-#pragma unroll
-      for (int v = 0; v < 8; ++v) d[v] = xs[nv[v]] - xr[v];
-      acc += gram8(d, A, B);
-    }
-    if (blockIdx.y == 0) {
-      double db[8];
-#pragma unroll
-      for (int v = 0; v < 8; ++v) db[v] = dsum[nv[v]] / S;
-      acc -= S * gram8(db, A, B);
-    }
-    contrib = hf3 * acc;
+    for (int c = 0; c <= dk; ++c)
+      for (int b = 0; b <= dj; ++b)
+        for (int a = 0; a <= di; ++a) acc += ldq(q, a + c1 * (b + c1 * c));
+    x = fma(-work[4 + S + s] * (di ? 0.5 : 1.0), (dj ? 0.5 : 1.0) * (dk ? 0.5 : 1.0) * acc, x);
   }
-  const double bs = block_sum(contrib);
-  if (threadIdx.x == 0) partial[blockIdx.x + (long long)gridDim.x * blockIdx.y] = bs;
+  reinterpret_cast<double*>(qs)[n] = x;
+}
+// nodal mean over the samples, by deviations from the first one: a block takes 32 nodes
+// and splits the samples over its eight warps (summed in a fixed order)
+__global__ void __launch_bounds__(kBlock) k_lvl_mean(const double* __restrict__ x, int nodes, int S, double inv_s,
+                                                     double* __restrict__ mean) {
+  __shared__ double part[8][32];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int n = blockIdx.x * 32 + lane;
+  double d = 0.0, xr = 0.0;
+  if (n < nodes) {
+    xr = x[n];
+#pragma unroll 4
+    for (int s = w; s < S; s += 8) d += x[(long long)s * nodes + n] - xr;
+  }
+  part[w][lane] = d;
+  __syncthreads();
+  if (w == 0 && n < nodes) {
+#pragma unroll
+    for (int v = 1; v < 8; ++v) d += part[v][lane];
+    mean[n] = fma(d, inv_s, xr);
+  }
+}
+// sum over samples of d^T (g x g x g) d, d = x_s - mean, grids of at most 16^3: a sample in
+// shared memory, one axis after the other; blockIdx.x takes samples x, x + gridDim.x, ..
+__global__ void __launch_bounds__(kBlock) k_lvl_s2_small(const double* __restrict__ x, int N, int S,
+                                                         const double* __restrict__ mean, double A2, double B,
+                                                         double hf3, double* __restrict__ partial) {
+  extern __shared__ double sm[];
+  const int n1 = N + 1, nodes = n1 * n1 * n1, m1 = N - 1, inner = m1 * m1 * m1;
+  double *d = sm, *u = sm + nodes, *v = sm + 2 * nodes;
+  double acc = 0.0;
+  auto node = [&](int e) {  // interior node e of (N - 1)^3
+    const int t = e / m1, i = e - t * m1, k = t / m1, j = t - k * m1;
+    return (i + 1) + n1 * ((j + 1) + n1 * (k + 1));
+  };
+  for (int e = threadIdx.x; e < 3 * nodes; e += kBlock) sm[e] = 0.0;
+  for (int s = blockIdx.x; s < S; s += gridDim.x) {
+    __syncthreads();
+    for (int e = threadIdx.x; e < inner; e += kBlock) {
+      const int n = node(e);
+      d[n] = x[(long long)s * nodes + n] - mean[n];
+    }
+    __syncthreads();
+    for (int e = threadIdx.x; e < inner; e += kBlock) {
+      const int n = node(e);
+      u[n] = fma(A2, d[n], B * (d[n - 1] + d[n + 1]));
+    }
+    __syncthreads();
+    for (int e = threadIdx.x; e < inner; e += kBlock) {
+      const int n = node(e);
+      v[n] = fma(A2, u[n], B * (u[n - n1] + u[n + n1]));
+    }
+    __syncthreads();
+    for (int e = threadIdx.x; e < inner; e += kBlock) {
+      const int n = node(e);
+      acc = fma(d[n], fma(A2, v[n], B * (v[n - n1 * n1] + v[n + n1 * n1])), acc);
+    }
+  }
+  const double bs = block_sum(acc);
+  if (threadIdx.x == 0) partial[blockIdx.x] = hf3 * bs;
+}
+// the same on larger grids: 32 x 32 tiles (four rows per thread) marching over kLvlPlanes
+// planes of one sample; blockIdx.z: (sample group, z chunk), samples g, g + groups, ..
+constexpr int kLvlPlanes = 16, kLvlTY = 32;
+__global__ void __launch_bounds__(kBlock) k_lvl_s2(const double* __restrict__ x, int N, int S, int groups,
+                                                   const double* __restrict__ mean, double A2, double B, double hf3,
+                                                   double* __restrict__ partial) {
+  __shared__ double d[kLvlTY + 2][34], u[kLvlTY + 2][32];
+  const int n1 = N + 1, tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  const long long nodes = (long long)n1 * n1 * n1, pn = (long long)n1 * n1;
+  const int x0 = 1 + 32 * blockIdx.x, y0 = 1 + kLvlTY * blockIdx.y;
+  const int chunk = blockIdx.z / groups, group = blockIdx.z % groups;
+  const int k0 = 1 + kLvlPlanes * chunk, k1 = min(N - 1, k0 + kLvlPlanes - 1);
+  double acc = 0.0;
+  for (int s = group; s < S; s += groups) {
+    const double* xs = x + s * nodes;
+    double below[4], here[4], dc[4], dn[4];  // v of planes k - 1 and k, d of the own nodes of planes k and k + 1
+#pragma unroll
+    for (int t = 0; t < 4; ++t) below[t] = here[t] = dc[t] = 0.0;
+    for (int m = k0 - 1; m <= k1 + 1; ++m) {
+      const bool mok = m > 0 && m < N;
+      __syncthreads();
+      for (int e = threadIdx.x; e < (kLvlTY + 2) * 34; e += kBlock) {
+        const int ly = e / 34, lx = e - 34 * ly, i = x0 - 1 + lx, j = y0 - 1 + ly;
+        const bool ok = mok && i > 0 && j > 0 && i < N && j < N;
+        const long long n = i + (long long)n1 * j + pn * m;
+        d[ly][lx] = ok ? xs[n] - mean[n] : 0.0;
+      }
+      __syncthreads();
+      for (int e = ty; e < kLvlTY + 2; e += 8) u[e][tx] = fma(A2, d[e][tx + 1], B * (d[e][tx] + d[e][tx + 2]));
+      __syncthreads();
+#pragma unroll
+      for (int t = 0; t < 4; ++t) {
+        const int ly = 4 * ty + t;
+        const double v = fma(A2, u[ly + 1][tx], B * (u[ly][tx] + u[ly + 2][tx]));
+        dn[t] = d[ly + 1][tx + 1];  // 0 outside the interior
+        if (m > k0) acc = fma(dc[t], fma(A2, here[t], B * (below[t] + v)), acc);
+        below[t] = here[t];
+        here[t] = v;
+        dc[t] = dn[t];
+      }
+    }
+  }
+  const double bs = block_sum(acc);
+  const int bid = (blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
+  if (threadIdx.x == 0) partial[bid] = hf3 * bs;
 }
 // per control cell: batch mean = interpolated nodal mean; Chan merge with the old
 // field; block partials of h_c^3 delta^2 n_old S / n.  A block takes kLvlRows rows
 // (cy, cz) of control cells, 256 cells of a row per block in x; per row the
-// level-node columns are first interpolated in (y, z) into shared memory, then each
-// cell interpolates linearly in x between the two columns of its level cell.
+// level-node columns are first interpolated in (y, z) into shared memory with their
+// differences, then each cell interpolates linearly in x between the two columns of its
+// level cell.  An empty record (n_old = 0) is not read.
 constexpr int kLvlRows = 16;
-__global__ void __launch_bounds__(kBlock) k_lvl_field(const double* __restrict__ x0, const double* __restrict__ dsum,
-                                                      int Nf, int Nc, int S, const double* __restrict__ work,
-                                                      double* __restrict__ field, double* __restrict__ partial) {
-  extern __shared__ double col[];  // [2][Nf + 1]: x0 and dsum interpolated in (y, z)
+__global__ void __launch_bounds__(kBlock) k_lvl_field(const double* __restrict__ xm, int Nf, int Nc, int S,
+                                                      const double* __restrict__ work, double* __restrict__ field,
+                                                      double* __restrict__ partial) {
+  extern __shared__ double col[];  // [2][Nf + 1]: the mean interpolated in (y, z), and its x differences
   const int n1 = Nf + 1, r = Nc / Nf;
   const long long sz = (long long)n1 * n1;
-  const double inv_r = 1.0 / r;
-  const double n_old = work[2], scale = work[1];
-  const double n = n_old + S;
-  const double inv_s = 1.0 / S, a = n_old / n;
+  const float inv_r = 1.0f / (float)r;  // r a power of two: the weights are exact in FP32
+  const double n_old = work[2], scale = work[1], a = work[3];
   const int cx = blockIdx.x * blockDim.x + threadIdx.x;
   const int ex = cx / r;
-  const double tx = (cx - ex * r + 0.5) * inv_r;
+  const double tx = f2d(((float)(cx - ex * r) + 0.5f) * inv_r);
   const long long rows = (long long)Nc * Nc;
   double contrib = 0.0;
   for (long long row = (long long)blockIdx.y * kLvlRows; row < rows && row < (long long)(blockIdx.y + 1) * kLvlRows;
        ++row) {
-    const int cy = (int)(row % Nc), cz = (int)(row / Nc);
+    const int cz = (int)((unsigned)row / (unsigned)Nc), cy = (int)row - cz * Nc;
     const int ey = cy / r, ez = cz / r;
-    const double ty = (cy - ey * r + 0.5) * inv_r, tz = (cz - ez * r + 0.5) * inv_r;
+    const float ty = ((float)(cy - ey * r) + 0.5f) * inv_r, tz = ((float)(cz - ez * r) + 0.5f) * inv_r;
+    const double w00 = f2d((1.f - ty) * (1.f - tz)), w10 = f2d(ty * (1.f - tz)), w01 = f2d((1.f - ty) * tz),
+                 w11 = f2d(ty * tz);
     __syncthreads();  // the previous row's columns are no longer read
     for (int c = threadIdx.x; c < n1; c += blockDim.x) {
-      const long long b = c + (long long)n1 * ey + sz * ez;
-      const double w00 = (1.0 - ty) * (1.0 - tz), w10 = ty * (1.0 - tz), w01 = (1.0 - ty) * tz, w11 = ty * tz;
-      col[c] = w00 * x0[b] + w10 * x0[b + n1] + w01 * x0[b + sz] + w11 * x0[b + sz + n1];
-      col[n1 + c] = w00 * dsum[b] + w10 * dsum[b + n1] + w01 * dsum[b + sz] + w11 * dsum[b + sz + n1];
+      const double* b = xm + c + (long long)n1 * ey + sz * ez;
+      col[c] = fma(w11, b[sz + n1], fma(w01, b[sz], fma(w10, b[n1], w00 * b[0])));
     }
     __syncthreads();
+    for (int c = threadIdx.x; c < Nf; c += blockDim.x) col[n1 + c] = col[c + 1] - col[c];
+    __syncthreads();
     if (cx < Nc) {
-      const double xv = fma(tx, col[ex + 1] - col[ex], col[ex]);
-      const double dv = fma(tx, col[n1 + ex + 1] - col[n1 + ex], col[n1 + ex]);
-      const double mean = fma(dv, inv_s, xv);
+      const double mean = fma(tx, col[n1 + ex], col[ex]);
       const long long c = cx + row * Nc;
-      const double mo = (n_old > 0.0) ? field[c] * scale : 0.0;
-      const double delta = mo - mean;
-      field[c] = fma(a, delta, mean);
-      contrib = fma(delta, delta, contrib);
+      if (n_old > 0.0) {
+        const double delta = fma(field[c], scale, -mean);
+        field[c] = fma(a, delta, mean);
+        contrib = fma(delta, delta, contrib);
+      } else {
+        field[c] = mean;
+      }
     }
   }
   const double hc = 1.0 / Nc;
-  contrib *= hc * hc * hc * n_old * S / n;
+  contrib *= hc * hc * hc * a * S;
   const double bs = block_sum(contrib);
   if (threadIdx.x == 0) partial[blockIdx.x + (long long)gridDim.x * blockIdx.y] = bs;
 }
@@ -693,9 +925,7 @@ __global__ void __launch_bounds__(kBlock) k_lvl_field(const double* __restrict__
 template <typename QF, typename QC>
 static int launch_lvl(const void* qf, int Nf, const void* qc, int S, int Nc, const double* work, double* field,
                       double* partial, double* nodebuf, cudaStream_t st) {
-  const long long nodes = nodes_of(Nf), cells = cells_of(Nf), ncell = cells_of(Nc);
-  double* x0 = nodebuf;
-  double* dsum = nodebuf + nodes;
+  const long long nodes = nodes_of(Nf), ncell = cells_of(Nc);
   const int r = Nc / Nf;
   double A = 0.0, B = 0.0;
   for (int m = 0; m < r; ++m) {
@@ -703,37 +933,50 @@ static int launch_lvl(const void* qf, int Nf, const void* qc, int S, int Nc, con
     A += (1.0 - t) * (1.0 - t) / r;
     B += t * (1.0 - t) / r;
   }
-  const double hf = 1.0 / Nf;
+  const double hf = 1.0 / Nf, hf3 = hf * hf * hf;
   const double qb = (double)S * sizeof(QF) * (nodes + (qc ? nodes_of(Nf / 2) : 0));
   const unsigned nbn = (unsigned)((nodes + kBlock - 1) / kBlock);
   launch("level_x", qb + (double)S * nodes * 8, k_lvl_x<QF, QC>, dim3(nbn, (unsigned)S), kBlock, 0, st,
          (QF*)const_cast<void*>(qf), Nf, (const QC*)qc, S, work);
   const double* x = (const double*)qf;
-  launch("level_nodes", (double)S * nodes * 8 + (double)nodes * 16, k_lvl_nodes, dim3(nbn), kBlock, 0, st, x, nodes,
-         S, x0, dsum);
+  double* mean = nodebuf;
+  launch("level_nodes", (double)S * nodes * 8 + (double)nodes * 8, k_lvl_mean, dim3((unsigned)((nodes + 31) / 32)), kBlock,
+         0, st, x, (int)nodes, S, 1.0 / S, mean);
   const unsigned fx = (unsigned)((Nc + kBlock - 1) / kBlock);
   const unsigned fy = (unsigned)(((long long)Nc * Nc + kLvlRows - 1) / kLvlRows);
   const long long nf = (long long)fx * fy;
-  launch("level_field", (double)nodes * 16 + (double)ncell * 16, k_lvl_field, dim3(fx, fy), kBlock,
-         (size_t)2 * (Nf + 1) * sizeof(double), st, (const double*)x0, (const double*)dsum, Nf, Nc, S, work, field,
-         partial);
-  // samples spread over blockIdx.y: about 4 blocks per SM, within the partial buffer
-  const long long cb = (cells + kBlock - 1) / kBlock;
-  long long g = std::min<long long>((level_partial_cap(Nc, Nf) - nf) / cb, (4LL * 152 + cb - 1) / cb);
-  g = std::max<long long>(1, std::min<long long>(g, S));
-  launch("level_cells", (double)S * nodes * 8 + (double)nodes * 16, k_lvl_cells, dim3((unsigned)cb, (unsigned)g),
-         kBlock, 0, st, x, Nf, S, (const double*)x0, (const double*)dsum, A, B, hf * hf * hf, partial + nf);
-  return (int)(nf + cb * g);
+  launch("level_field", (double)nodes * 8 + (double)ncell * 16, k_lvl_field, dim3(fx, fy), kBlock,
+         (size_t)2 * (Nf + 1) * sizeof(double), st, (const double*)mean, Nf, Nc, S, work, field, partial);
+  // samples spread over blocks within the partial buffer
+  const long long room = level_partial_cap(Nc, Nf) - nf;
+  const double sb = (double)S * nodes * 8 + (double)nodes * 8;
+  if (Nf <= 16) {
+    const int g = (int)std::min<long long>(S, room);
+    const size_t smem = 3 * (size_t)nodes * sizeof(double);
+    static bool smem_set = false;  // once (capture-friendly)
+    if (smem > 48 * 1024 && !smem_set) {
+      cudaFuncSetAttribute(k_lvl_s2_small, cudaFuncAttributeMaxDynamicSharedMemorySize, 3 * 17 * 17 * 17 * 8);
+      smem_set = true;
+    }
+    launch("level_cells", sb, k_lvl_s2_small, dim3((unsigned)g), kBlock, smem, st, x, Nf, S, (const double*)mean, 2.0 * A, B,
+           hf3, partial + nf);
+    return (int)(nf + g);
+  }
+  const int bx = (Nf - 1 + 31) / 32, by = (Nf - 1 + kLvlTY - 1) / kLvlTY, bz = (Nf - 1 + kLvlPlanes - 1) / kLvlPlanes;
+  const long long tiles = (long long)bx * by * bz;
+  const int g = (int)std::max<long long>(1, std::min<long long>(S, std::min<long long>(room / tiles, (8LL * 152 + tiles - 1) / tiles)));
+  launch("level_cells", sb, k_lvl_s2, dim3((unsigned)bx, (unsigned)by, (unsigned)(bz * g)), kBlock, 0, st, x, Nf, S, g,
+         (const double*)mean, 2.0 * A, B, hf3, partial + nf);
+  return (int)(nf + tiles * g);
 }
 
-// s2_dx = old * scale^2 + sum of partials (fixed order, one warp)
-__global__ void k_level_finish(const double* __restrict__ partial, int nblk, const double* __restrict__ work,
-                               double* __restrict__ sc) {
-  const int lane = threadIdx.x;
+// s2_dx = old * scale^2 + sum of partials (fixed order, one block)
+__global__ void __launch_bounds__(kBlock) k_level_finish(const double* __restrict__ partial, int nblk,
+                                                         const double* __restrict__ work, double* __restrict__ sc) {
   double v = 0.0;
-  for (int t = lane; t < nblk; t += 32) v += partial[t];
-  v = warp_sum(v);
-  if (lane == 0) {
+  for (int t = threadIdx.x; t < nblk; t += kBlock) v += partial[t];
+  v = block_sum(v);
+  if (threadIdx.x == 0) {
     const double scale = work[1];
     sc[MLSGD_S_S2_DX] = (work[2] > 0.0 ? sc[MLSGD_S_S2_DX] * scale * scale : 0.0) + v;
   }
@@ -753,38 +996,48 @@ void launch_level_stats(const double* qf, const double* phif, int Nf, const doub
     const int nb = (qf_pairs && qc_pairs) ? launch_lvl<float2, float2>(qf, Nf, qc, S, Nc, work, field, partial, nodebuf, st)
                    : qf_pairs             ? launch_lvl<float2, double>(qf, Nf, qc, S, Nc, work, field, partial, nodebuf, st)
                                           : launch_lvl<double, double>(qf, Nf, qc, S, Nc, work, field, partial, nodebuf, st);
-    launch("level_finish", 0.0, k_level_finish, dim3(1), 32, 0, st, (const double*)partial, nb, (const double*)work,
+    launch("level_finish", 0.0, k_level_finish, dim3(1), kBlock, 0, st, (const double*)partial, nb, (const double*)work,
            scalars);
     return;
   }
   const long long ncell = (long long)Nc * Nc * Nc;
-  const int nblk = (int)((ncell + kBlock - 1) / kBlock);
+  const int nblk = cell_blocks(ncell);
   const double qbytes = (double)S * 8 * (nodes_of(Nf) + (qc ? nodes_of(Ncoarse) : 0));
+  // both grids in pairs, the fine one the control grid or one level below it
+  if (qf_pairs && qc_pairs && (Nf == Nc || 2 * Nf == Nc)) {
+    const bool split = S >= 16 && ncell < (long long)kPairBlocks * kBlock * 4;
+    const int cb = split ? kBlock / 4 : kBlock;
+    const int nb = (int)std::min<long long>((ncell + cb - 1) / cb, split ? kPairBlocks : cell_blocks(ncell));
+    auto kp = Nf == Nc ? (split ? k_level_pairs<1, 4> : k_level_pairs<1, 1>)
+                       : (split ? k_level_pairs<2, 4> : k_level_pairs<2, 1>);
+    launch_flops("level_field", qbytes + (double)ncell * 16, (double)S * ncell * 4.0, kp, dim3(nb), kBlock, 0, st,
+                 (const float2*)qf, Nf, (const float2*)qc, S, Nc, 1.0 / S, (const double*)work, field, partial);
+    launch("level_finish", 0.0, k_level_finish, dim3(1), kBlock, 0, st, (const double*)partial, nb, (const double*)work,
+           scalars);
+    return;
+  }
   // pairs on the coarse grid only come with pairs on the fine grid (it is at least as large)
-  const bool fast = Nf <= Nc && (!qc || Ncoarse <= Nc);
-  auto lf = qf_pairs ? (qc_pairs ? (fast ? k_level_field<true, true, true> : k_level_field<true, true>)
-                                 : k_level_field<true, false>)
-                     : k_level_field<false, false>;
+  auto lf = qf_pairs ? (qc_pairs ? k_level_field<true, true> : k_level_field<true, false>) : k_level_field<false, false>;
   // FP64 operations per control cell and sample: both grids in pairs, the pair value
   // to FP64 (2 conversions, 1 add), its deviation and the two sums; otherwise also the
   // FP64 weighting and, for FP64 fields, the 8-node averages
-  const double f64ops = qf_pairs && qc_pairs ? (fast ? 4.0 : 6.0) : (qf_pairs ? 16.0 : 21.0);
+  const double f64ops = qf_pairs && qc_pairs ? 6.0 : (qf_pairs ? 16.0 : 21.0);
   launch_flops("level_field", qbytes + (double)ncell * 16, (double)S * ncell * f64ops, lf, dim3(nblk), kBlock, 0, st,
-               (const void*)qf, Nf, (const void*)qc, Ncoarse, S, Nc, (const double*)work, field, partial);
-  launch("level_finish", 0.0, k_level_finish, dim3(1), 32, 0, st, (const double*)partial, nblk, (const double*)work,
+               (const void*)qf, Nf, (const void*)qc, Ncoarse, S, Nc, 1.0 / S, (const double*)work, field, partial);
+  launch("level_finish", 0.0, k_level_finish, dim3(1), kBlock, 0, st, (const double*)partial, nblk, (const double*)work,
          scalars);
 }
 
-__global__ void k_stats_reset(double* __restrict__ field, double* __restrict__ sc, long long n) {
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) field[i] = 0.0;
-  if (i < MLSGD_NSCALARS) sc[i] = (i == MLSGD_S_SHIFT || i == MLSGD_S_PHI_MAX) ? -INFINITY : 0.0;
+__global__ void __launch_bounds__(kBlock) k_stats_reset(double* __restrict__ field, double* __restrict__ sc, long long n) {
+  const long long i0 = (long long)blockIdx.x * kBlock + threadIdx.x, step = (long long)gridDim.x * kBlock;
+  if (i0 < MLSGD_NSCALARS) sc[i0] = (i0 == MLSGD_S_SHIFT || i0 == MLSGD_S_PHI_MAX) ? -INFINITY : 0.0;
+#pragma unroll 4
+  for (long long i = i0; i < n; i += step) field[i] = 0.0;
 }
 
 void launch_stats_reset(double* field, double* scalars, long long ncells, cudaStream_t st) {
-  const long long n = ncells > MLSGD_NSCALARS ? ncells : MLSGD_NSCALARS;
-  launch("stats_reset", (double)ncells * 8, k_stats_reset, dim3((unsigned)((n + kBlock - 1) / kBlock)), kBlock, 0, st,
-         field, scalars, ncells);
+  launch("stats_reset", (double)ncells * 8, k_stats_reset, dim3((unsigned)cell_blocks(ncells)), kBlock, 0, st, field,
+         scalars, ncells);
 }
 
 // Chan merge of two statistics records: src into dst, both rescaled to the larger shift.
@@ -797,11 +1050,6 @@ void launch_stats_reset(double* field, double* scalars, long long ncells, cudaSt
 // does not read dst.  Six levels on a 256^3 control (16.8M cells) reset, merged twice and
 // stepped: 31.9 ms with the factors formed per cell and one warp over 65536 partial
 // sums, 2.08 ms now (1.6 ms of FP64 issue).
-constexpr int kCellBlocks = 8 * 152;  // eight blocks of 256 threads per SM
-static int cell_blocks(long long n) {
-  const long long b = (n + kBlock - 1) / kBlock;
-  return (int)(b < kCellBlocks ? b : kCellBlocks);
-}
 __global__ void __launch_bounds__(kBlock) k_merge_field(double* __restrict__ df, const double* __restrict__ dsc,
                                                         const double* __restrict__ sf, const double* __restrict__ ssc,
                                                         long long n, double theta, double hc3,

@@ -99,7 +99,7 @@ __global__ void k_field(const double* __restrict__ xi, int K, const ModeTable mt
 }
 
 // FP32-coefficient synthesis (the mixed path needs only a = exp(log a) rounded to
-// FP32 and BF16).  One block per (chunk of kFieldPlanes z planes, sample): the 1D
+// FP32 and BF16).  One block per (chunk of `planes` z planes, sample): the 1D
 // tables and c_k are split into FP32 pairs once per block (the only FP64 work),
 // then per plane c_k phi_{iz_k}(z) is a pair product and stage 1 (T2) runs in FP32
 // pair arithmetic;
@@ -110,11 +110,13 @@ __global__ void k_field(const double* __restrict__ xi, int K, const ModeTable mt
 // Dynamic shared memory: c_k phi(z) pairs and c_k pairs [K rounded up to even each],
 // then T2 hi/lo [n1x][N] and phi hi/lo [n1d][N] (floats; 16-byte aligned for the
 // float4 reads since N % 4 == 0 is required).
+// planes: at most kFieldPlanes, halved while the blocks would not fill the SMs twice (one
+// 256^3 sample: 16 blocks and 1.45 ms with 16 planes each, 0.15 ms with one).
 constexpr int kFieldPlanes = 16;
 constexpr float kLn2Hi = 0.693145751953125f;        // ln 2 truncated to 16 bits
 constexpr float kLn2Lo = 1.4286068202862268e-06f;   // ln 2 - kLn2Hi
 __global__ void k_field_df(const double* __restrict__ xi, int K, const ModeTable mt, const double* __restrict__ phi,
-                           int N, float* __restrict__ a32, __nv_bfloat16* __restrict__ abf) {
+                           int N, int planes, float* __restrict__ a32, __nv_bfloat16* __restrict__ abf) {
   extern __shared__ __align__(16) unsigned char smf[];
   float2* cz = reinterpret_cast<float2*>(smf);  // c_k phi_{iz_k}(z) as pairs
   float2* ck = cz + ((K + 1) & ~1);             // c_k as pairs
@@ -130,7 +132,7 @@ __global__ void k_field_df(const double* __restrict__ xi, int K, const ModeTable
     Ph[e] = h;
     Pl[e] = (float)(v - (double)h);
   }
-  const int z0 = kFieldPlanes * blockIdx.x, z1 = min(N, z0 + kFieldPlanes);
+  const int z0 = planes * blockIdx.x, z1 = min(N, z0 + planes);
   for (int z = z0; z < z1; ++z) {
     __syncthreads();  // the tables (first plane); the previous plane's T2 reads done
     for (int k = threadIdx.x; k < K; k += blockDim.x) {
@@ -205,10 +207,12 @@ cudaError_t launch_field(const double* xi, int K, const ModeTable& mt, const dou
       smem_df = smem;
     }
     const double cells = (double)S * N * N * N;
+    int planes = kFieldPlanes;
+    while (planes > 1 && (long long)S * ((N + planes - 1) / planes) < 2 * 152) planes /= 2;
     launch_flops("field", (double)S * K * 8 + cells * ((out.a32 ? 4 : 0) + (out.abf ? 2 : 0)),
                  2.0 * cells * mt.n1x + 2.0 * (double)S * K * N * N, k_field_df,
-                 dim3((unsigned)((N + kFieldPlanes - 1) / kFieldPlanes), S), kBlock, smem, st, xi, K,
-                 mt, phi, N, out.a32, out.abf);
+                 dim3((unsigned)((N + planes - 1) / planes), S), kBlock, smem, st, xi, K, mt, phi, N, planes, out.a32,
+                 out.abf);
     return cudaGetLastError();
   }
   const size_t smem = field_smem_bytes(mt, K, N);

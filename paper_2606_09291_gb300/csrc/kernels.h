@@ -216,16 +216,19 @@ cudaError_t kl_gemm(const double* xi, const double* scale, int S, int K, const _
                     __nv_bfloat16* A_scratch, __nv_bfloat16* abf, float* loga, int* err, cudaStream_t st);
 
 // ---------------------------------------------------------------- estimator
-void launch_rhs_state(const double* z, int Nc, int N, double* b, cudaStream_t st);
+// scratch: scratch_bytes of device memory the launch may overwrite (rhs_scratch_bytes for
+// the by-axis form of a finer control grid; less falls back to a slower form)
+size_t rhs_scratch_bytes(int Nc, int N);
+void launch_rhs_state(const double* z, int Nc, int N, double* b, void* scratch, size_t scratch_bytes, cudaStream_t st);
 // Phi = 1/2 e^T M e, badj = M e (interior rows), e = y - g_h
 void launch_phi_adjrhs(const double* y, int N, int S, double* badj, double* phi, double* partial,
-                       const double* gtab, const double* mgtab, cudaStream_t st, int freq = 1);
+                       const double* gtab, const double* mgtab, cudaStream_t st);
 // the same for a state stored as FP32 pairs on a tiled grid (tables and M e as pairs)
 void launch_phi_adjrhs_df(const float2* y, int N, int S, float2* badj, double* phi, double* partial,
                           const float2* gtab, const float2* mgtab, cudaStream_t st);
 // batch statistics of one level merged into stats (see mlsgd_level_stats)
 // qf_pairs / qc_pairs: the adjoint solutions are stored as FP32 (hi, lo) pairs;
-// work holds 4 + 4 S doubles; nodebuf (2 (Nf+1)^3 doubles, optional): when the
+// work holds 4 + 4 S doubles; nodebuf ((Nf+1)^3 doubles, optional): when the
 // level's grids are at least 4x coarser than the control grid the statistics are
 // formed on the level grid (qf is then overwritten; partial needs cells(Nc)/256 +
 // cells(Nf)/256 + 2 entries)

@@ -98,3 +98,32 @@ def test_combine_levels(lib, L, ctrl_level, adaptive):
         lh = np.sqrt(((g - prev) ** 2).sum()) / (tau * np.sqrt((prev ** 2).sum()))
         assert abs(rep["l_hat"] - lh) <= TOL * lh
     ctx.close()
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+@pytest.mark.parametrize("n0,level,ctrl_level", [(4, 0, 0), (4, 0, 2), (4, 1, 3), (4, 2, 4), (4, 3, 5), (4, 3, 2), (8, 2, 2), (8, 2, 1),
+                                                 (2, 1, 6)])
+def test_level_record_against_oracle(lib, precision, n0, level, ctrl_level):
+    """Level grids coarser than, equal to and finer than the control grid (every right-hand
+    side and statistics kernel), two calls merged, against the oracle at the parity bars."""
+    from oracle import mlmc
+    from paper_2606_09291_gb300 import inputs
+    L = max(level, ctrl_level) + 1
+    c = dict(n_levels=L, n0=n0, n_modes=16, corr_len=0.3, sigma=1.0, theta=5.0, alpha=1e-4, seed=6, ctrl_level=ctrl_level)
+    rtol, tol = (1e-13, 1e-10) if precision == "fp64" else (1e-8, 1e-6)
+    Nc = n0 << ctrl_level
+    z = inputs.z_test(Nc) + inputs.z_random(Nc, 2)
+    ctx = lib.Context(**dict(c, rtol=rtol, max_iter=400, precision=precision))
+    zt = torch.tensor(z, dtype=torch.float64, device="cuda")
+    st = ctx.new_stats(level)
+    ctx.mlsgd_level_gradient(3, level, 0, 2, zt, st)
+    ctx.mlsgd_level_gradient(3, level, 2, 3, zt, st)
+    W = mlmc.Workload(**c)
+    ref = mlmc.level_batch(W, 3, level, range(5), z)
+    h = st.host()
+    fac = np.exp(5.0 * (h["shift"] - ref["shift"]))
+    f, o = st.field.cpu().numpy() * fac, ref["stats"].mean_x
+    assert h["count"] == 5
+    assert np.abs(f - o).max() <= tol * np.abs(o).max()
+    assert abs(h["s2_dx"] * fac ** 2 - ref["stats"].s2_x) <= tol * ref["stats"].s2_x
+    ctx.close()
