@@ -30,6 +30,9 @@ struct mlsgd_ctx {
   double* d_scale = nullptr;
   int* d_order = nullptr;
   int* d_offs = nullptr;
+  int* d_order4 = nullptr;
+  int* d_iy4 = nullptr;
+  int* d_offs4 = nullptr;
   std::vector<double*> d_phi;  // per level: [n1d][N] at cell centres
   std::vector<double*> d_gtab;   // per level: [N+1] sin(pi i / N), 0 at i = 0, N (nodal interpolant of g)
   std::vector<double*> d_mgtab;  // per level: [N+1] (h/6)(g[i-1] + 4 g[i] + g[i+1]) (1D mass times g)
@@ -44,6 +47,8 @@ struct mlsgd_ctx {
   ModeTable mt() const {
     ModeTable m;
     m.iy = d_iy; m.iz = d_iz; m.scale = d_scale; m.order = d_order; m.offs = d_offs;
+    m.order4 = d_order4; m.iy4 = d_iy4; m.offs4 = d_offs4;
+    m.even = cfg.field_model == 1 ? 1 : 0;  // cos((n + 1) pi x); else even n are the cosines about the centre
     m.n1x = n1x; m.n1d = kl.n1d;
     return m;
   }
@@ -337,6 +342,20 @@ mlsgd_status mlsgd_create(const mlsgd_config* cfg, mlsgd_ctx** out) {
   std::vector<int> fill(offs.begin(), offs.end() - 1);
   for (int k = 0; k < K; ++k) order[fill[ctx->kl.ix[k]]++] = k;
   ctx->n1x = n1x;
+  // the x-index groups split by the parity of the y and z modes
+  const int even = c.field_model == 1 ? 1 : 0;
+  std::vector<int> offs4(4 * n1x + 1, 0), order4(K), iy4(K);
+  auto cls4 = [&](int k) {
+    return 4 * ctx->kl.ix[k] + ((iy[k] & 1) != even ? 1 : 0) + ((iz[k] & 1) != even ? 2 : 0);
+  };
+  for (int k = 0; k < K; ++k) offs4[cls4(k) + 1]++;
+  for (int i = 0; i < 4 * n1x; ++i) offs4[i + 1] += offs4[i];
+  std::vector<int> fill4(offs4.begin(), offs4.end() - 1);
+  for (int k = 0; k < K; ++k) {
+    const int t = fill4[cls4(k)]++;
+    order4[t] = k;
+    iy4[t] = iy[k];
+  }
   auto up = [&](void** d, const void* h, size_t n) -> bool {
     return cudaMalloc(d, n) == cudaSuccess && cudaMemcpy(*d, h, n, cudaMemcpyHostToDevice) == cudaSuccess;
   };
@@ -346,7 +365,10 @@ mlsgd_status mlsgd_create(const mlsgd_config* cfg, mlsgd_ctx** out) {
             up((void**)&ctx->d_iy, iy.data(), K * sizeof(int)) && up((void**)&ctx->d_iz, iz.data(), K * sizeof(int)) &&
             up((void**)&ctx->d_scale, scale.data(), K * sizeof(double)) &&
             up((void**)&ctx->d_order, order.data(), K * sizeof(int)) &&
-            up((void**)&ctx->d_offs, offs.data(), (n1x + 1) * sizeof(int));
+            up((void**)&ctx->d_offs, offs.data(), (n1x + 1) * sizeof(int)) &&
+            up((void**)&ctx->d_order4, order4.data(), K * sizeof(int)) &&
+            up((void**)&ctx->d_iy4, iy4.data(), K * sizeof(int)) &&
+            up((void**)&ctx->d_offs4, offs4.data(), offs4.size() * sizeof(int));
   ctx->d_phiT.assign(c.n_levels, nullptr);
   for (int l = 0; ok && l < c.n_levels; ++l) {
     std::vector<double> phi = kl_cell_table(ctx->kl, ctx->N(l));
@@ -386,6 +408,7 @@ void mlsgd_destroy(mlsgd_ctx* ctx) {
   cudaFree(ctx->d_ix); cudaFree(ctx->d_err);
   for (__nv_bfloat16* b : ctx->d_phiT) cudaFree(b);
   cudaFree(ctx->d_iy); cudaFree(ctx->d_iz); cudaFree(ctx->d_scale); cudaFree(ctx->d_order); cudaFree(ctx->d_offs);
+  cudaFree(ctx->d_order4); cudaFree(ctx->d_iy4); cudaFree(ctx->d_offs4);
   for (double* d : ctx->d_phi) cudaFree(d);
   for (double* d : ctx->d_gtab) cudaFree(d);
   for (double* d : ctx->d_mgtab) cudaFree(d);

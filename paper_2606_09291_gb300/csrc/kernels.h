@@ -14,6 +14,12 @@ struct ModeTable {
   const double* scale;  // [K] sigma * sqrt(lambda_k)
   const int* order;     // [K] modes sorted by x-index
   const int* offs;      // [n1x+1] start of each x-index group in `order`
+  // the same order split by parity class: modes of x-index i, class (iy odd) + 2 (iz odd) at
+  // offs4[4 i + class] .. in order4; iy4: their y-indices in that order
+  const int* order4;    // [K]
+  const int* iy4;       // [K]
+  const int* offs4;     // [4 n1x + 1]
+  int even;             // index parity of the 1D modes that are even about x = 1/2 (the others are odd)
   int n1x;              // number of x-indices (max + 1)
   int n1d;              // number of 1D modes in the phi tables
 };
@@ -31,7 +37,6 @@ void launch_draw_xi(uint64_t seed, int iter, int level, long long first, int S, 
                     double half_width = 0.0);
 cudaError_t launch_field(const double* xi, int K, const ModeTable& mt, const double* phi, int N, int S,
                          const FieldOut& out, cudaStream_t st);
-size_t field_smem_bytes(const ModeTable& mt, int K, int N);
 void launch_exp_field(const double* la, const FieldOut& out, long long n, cudaStream_t st);
 
 // ---------------------------------------------------------------- solver
