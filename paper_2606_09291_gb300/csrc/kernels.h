@@ -190,6 +190,17 @@ void slab_res(const float* d, const float* p, bool d_zero, const SolveScalars* s
               long long rr_stride, float2* rr_out, float2* x, bool assign, const float* a, float* r32,
               double* partial, const SolveScalars* sco, int N, const Batch& bt, cudaStream_t st);
 
+// the FP32 passes on the other tiled grids (tile32.cu): APPLY (x null) or APPLYX; PRE (q null)
+// or PREU, t stored; POST
+void tile32_apply(const float* z, const float* pold, float* pnew, const float* a, float* q, float* x, double* partial,
+                  const SolveScalars* sc, int N, const Batch& bt, bool first, bool x_first, cudaStream_t st);
+template <typename TA>
+void tile32_pre(const float* r, const float* q, const TA* a, const float* wdinv, float* t, float* rnew,
+                const SolveScalars* sc, int N, const Batch& bt, cudaStream_t st);
+template <typename TA>
+void tile32_post(const float* r, const TA* a, const float* wdinv, const float* ec, float* z, double* partial,
+                 const SolveScalars* sc, int N, const Batch& bt, cudaStream_t st);
+
 // the V-cycle from a coarse 16^3 level (j >= 1 of a grid with N cells) down to 2^3 in one
 // launch, one block per launched sample (coarse.cu): r16 the restricted residual, a the
 // coefficients of the levels 16^3 .. 2^3, z16 the correction

@@ -43,9 +43,6 @@ constexpr int NPY = TY + 2, NP = NPX * NPY;      // the Phi kernels' staged plan
 constexpr int NT = TX * TY;
 
 enum TiledMode { TM_APPLY = 0, TM_PRE = 1, TM_POST = 2, TM_RES64 = 3, TM_PREU = 4, TM_APPLYX = 5 };
-// TM_PREU  : PRE with the CG residual update fused in: r_new = r - alpha q (staged from
-//            both), t = r_new - A x1, x1 = omega D^{-1} r_new; writes t and r_new
-// TM_APPLYX: APPLY with the previous iteration's x += alpha_prev p_old fused in
 
 struct TiledArgs {
   const void* in0;   // APPLY: z   PRE/POST: r    RES64: x (FP64)
@@ -788,13 +785,16 @@ void tiled_apply(const T* z, const T* pold, T* pnew, const TA* a, T* q, double* 
   if constexpr (std::is_same<T, float>::value && std::is_same<TA, float>::value) {
     if (bt.stencil == 0 && slab_supported(N)) {
       slab_apply(z, pold, pnew, a, q, nullptr, partial, sc, N, bt, first != 0, false, false, st);
-      return;
+    } else {
+      tile32_apply(z, pold, pnew, a, q, nullptr, partial, sc, N, bt, first != 0, false, st);
     }
-  }
+    return;
+  } else {
   TiledArgs A{};
   A.in0 = z; A.in1 = pold; A.a = a; A.out0 = q; A.out1 = pnew; A.partial = partial; A.sc = sc; A.N = N;
   A.first = first;
-  run_tiled<T, TA, TM_APPLY>(name("apply", tag<T>()), vbytes<T, TA>(N, bt.n, first ? 3 : 4, 1), A, bt, st);
+  run_tiled<T, TA, TM_APPLY>("apply_f64", vbytes<T, TA>(N, bt.n, first ? 3 : 4, 1), A, bt, st);
+  }
 }
 // fused variants of the mixed inner solve (see TM_PREU / TM_APPLYX)
 void tiled_apply_x(const float* z, const float* pold, float* pnew, const float* a, float* q, float* x, double* partial,
@@ -803,10 +803,7 @@ void tiled_apply_x(const float* z, const float* pold, float* pnew, const float* 
     slab_apply(z, pold, pnew, a, q, x, partial, sc, N, bt, false, true, x_first, st);
     return;
   }
-  TiledArgs A{};
-  A.in0 = z; A.in1 = pold; A.a = a; A.out0 = q; A.out1 = pnew; A.x = x; A.partial = partial; A.sc = sc; A.N = N;
-  A.xfirst = x_first ? 1 : 0;
-  run_tiled<float, float, TM_APPLYX>("apply_f32", vbytes<float, float>(N, bt.n, x_first ? 5 : 6, 1), A, bt, st);
+  tile32_apply(z, pold, pnew, a, q, x, partial, sc, N, bt, false, x_first, st);
 }
 bool tiled_pre_update(const float* r, const float* q, const __nv_bfloat16* a, const float* dinv, float* t,
                       float* rnew, float* rc, const SolveScalars* sc, int N, const Batch& bt, cudaStream_t st) {
@@ -814,9 +811,7 @@ bool tiled_pre_update(const float* r, const float* q, const __nv_bfloat16* a, co
     slab_pre<__nv_bfloat16>(r, q, a, dinv, rnew, rc, sc, N, bt, st);
     return true;
   }
-  TiledArgs A{};
-  A.in0 = r; A.q = q; A.a = a; A.dinv = dinv; A.out0 = t; A.out1 = rnew; A.sc = sc; A.N = N;
-  run_tiled<float, __nv_bfloat16, TM_PREU>("pre_f32", vbytes<float, __nv_bfloat16>(N, bt.n, 5, 1), A, bt, st);
+  tile32_pre<__nv_bfloat16>(r, q, a, dinv, t, rnew, sc, N, bt, st);
   return false;
 }
 
@@ -828,10 +823,12 @@ bool tiled_pre(const T* r, const TA* a, const T* dinv, T* t, T* rc, const SolveS
       slab_pre<TA>(r, nullptr, a, dinv, nullptr, rc, sc, N, bt, st);
       return true;
     }
-  }
+    tile32_pre<TA>(r, nullptr, a, dinv, t, nullptr, sc, N, bt, st);
+  } else {
   TiledArgs A{};
   A.in0 = r; A.a = a; A.dinv = dinv; A.out0 = t; A.sc = sc; A.N = N;
-  run_tiled<T, TA, TM_PRE>(name("pre", tag<T>()), vbytes<T, TA>(N, bt.n, 3, 1), A, bt, st);
+  run_tiled<T, TA, TM_PRE>("pre_f64", vbytes<T, TA>(N, bt.n, 3, 1), A, bt, st);
+  }
   return false;
 }
 template <typename T, typename TA>
@@ -840,13 +837,14 @@ void tiled_post(const T* r, const TA* a, const T* dinv, const T* ec, T* z, doubl
   if constexpr (std::is_same<T, float>::value) {
     if (bt.stencil == 0 && slab_supported(N)) {
       slab_post<TA>(r, a, dinv, ec, z, partial, sc, N, bt, st);
-      return;
+    } else {
+      tile32_post<TA>(r, a, dinv, ec, z, partial, sc, N, bt, st);
     }
-  }
+  } else {
   TiledArgs A{};
   A.in0 = r; A.a = a; A.dinv = dinv; A.ec = ec; A.out0 = z; A.partial = partial; A.sc = sc; A.N = N;
-  run_tiled<T, TA, TM_POST>(name("post", tag<T>()), vbytes<T, TA>(N, bt.n, 3, 1) + vbytes<T, T>(N / 2, bt.n, 1, 0), A,
-                            bt, st);
+  run_tiled<T, TA, TM_POST>("post_f64", vbytes<T, TA>(N, bt.n, 3, 1) + vbytes<T, T>(N / 2, bt.n, 1, 0), A, bt, st);
+  }
 }
 void tiled_res64(const float2* b, long long bstride, const float2* x, const float* a, float* r32, double* partial,
                  const SolveScalars* sc, int N, const Batch& bt, cudaStream_t st) {
