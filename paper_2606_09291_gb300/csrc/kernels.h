@@ -216,6 +216,14 @@ cudaError_t coarse_vcycle64(const double* r16, const double* const a[4], const d
 cudaError_t small_fp64(SolverBufs& B, const double* a64, const double* b, long long bstride, double* x_out,
                        const PcgParams& prm, cudaStream_t st);
 
+// FP32 work on 32^3 levels with a cluster of four blocks per sample (cluster32.cu): the
+// V-cycle from a coarse 32^3 level down (below: cells of 16^3 .. 2^3), and the whole solve
+// on a 32^3 grid after the init pass (B.r, B.sc; b as pairs in rr_in), x as FP32 pairs
+cudaError_t vcycle32(const float* r, const float* a, const float* dinv, const float* const below[4], float* z,
+                     const SolveScalars* sc, const Batch& bt, double omega, cudaStream_t st);
+cudaError_t solve32(SolverBufs& B, const float* a32, const __nv_bfloat16* abf, const float2* rr_in, long long rr_stride,
+                    float2* x, const PcgParams& prm, int inner, int inner_next, int fixed_steps, cudaStream_t st);
+
 // a whole mixed-precision solve per sample in one launch on 8^3 and 16^3 grids (small.cu);
 // builds the coefficient hierarchy itself; arguments as ir_mixed
 bool small_supported(int N);

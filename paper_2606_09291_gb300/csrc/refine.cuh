@@ -25,6 +25,26 @@ __device__ __forceinline__ void df_term(float& S, float& comp, F2 c, float2 x) {
   comp = __fadd_rn(comp, __fadd_rn(t.l, NEG ? -low : low));
 }
 
+// (S, comp) += sgn (c.h + c.l) x for an FP32 operand x: the product c.h x is split
+// exactly by the FMA, c.l x enters the compensation
+template <bool NEG>
+__device__ __forceinline__ void res_term(float& S, float& comp, F2 c, float x) {
+  const float p = __fmul_rn(c.h, x);
+  const float low = __fmaf_rn(c.l, x, __fmaf_rn(c.h, x, -p));
+  const F2 t = two_sum(S, NEG ? -p : p);
+  S = t.h;
+  comp = __fadd_rn(comp, __fadd_rn(t.l, NEG ? -low : low));
+}
+// the same for a single FP32 coefficient c (a cell of the body diagonals)
+template <bool NEG>
+__device__ __forceinline__ void res_term1(float& S, float& comp, float c, float x) {
+  const float p = __fmul_rn(c, x);
+  const float low = __fmaf_rn(c, x, -p);
+  const F2 t = two_sum(S, NEG ? -p : p);
+  S = t.h;
+  comp = __fadd_rn(comp, __fadd_rn(t.l, NEG ? -low : low));
+}
+
 // (b - A x) at one interior node of an N^3 grid, rounded to FP32: exact pair sums of the
 // cells C(r, p, q) (plane, x, y offset), exact products with the operand pairs
 // X(plane, x, y), compensated sums, the scale h/12 and the subtraction from b in the same

@@ -63,6 +63,7 @@
 #include "internal.cuh"
 #include "kernels.h"
 #include "launch.h"
+#include "refine.cuh"
 
 namespace mlsgd {
 
@@ -107,33 +108,7 @@ struct SlabArgs {
   float* rc;                // PRE/PREU: the restricted residual on grid N/2, [S][(N/2+1)^3]
 };
 
-// ---- error-free FP32 arithmetic of the refinement step (RES)
-// two_sum: s + e == a + b exactly (Knuth); a coefficient is an unevaluated pair (h, l)
-struct P2 { float h, l; };
-__device__ __forceinline__ P2 two_sum(float a, float b) {  // intrinsics: never contracted
-  const float s = __fadd_rn(a, b);
-  const float bb = __fsub_rn(s, a);
-  return P2{s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb))};
-}
-// (S, comp) += sgn (c.h + c.l) x for an FP32 operand x: the product c.h x is split
-// exactly by the FMA, c.l x enters the compensation
-template <bool NEG>
-__device__ __forceinline__ void res_term(float& S, float& comp, P2 c, float x) {
-  const float p = __fmul_rn(c.h, x);
-  const float low = __fmaf_rn(c.l, x, __fmaf_rn(c.h, x, -p));
-  const P2 t = two_sum(S, NEG ? -p : p);
-  S = t.h;
-  comp = __fadd_rn(comp, __fadd_rn(t.l, NEG ? -low : low));
-}
-// the same for a single FP32 coefficient c (a cell of the body diagonals)
-template <bool NEG>
-__device__ __forceinline__ void res_term1(float& S, float& comp, float c, float x) {
-  const float p = __fmul_rn(c, x);
-  const float low = __fmaf_rn(c, x, -p);
-  const P2 t = two_sum(S, NEG ? -p : p);
-  S = t.h;
-  comp = __fadd_rn(comp, __fadd_rn(t.l, NEG ? -low : low));
-}
+using P2 = F2;  // an unevaluated pair (refine.cuh)
 
 template <int N>
 struct SlabGeo {

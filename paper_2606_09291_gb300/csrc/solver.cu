@@ -697,6 +697,12 @@ void build_hierarchy_mixed(SolverBufs& B, const __nv_bfloat16* abf, double omega
   build_dinv<float, __nv_bfloat16>(B, abf, omega, st);
 }
 
+// Up to this many samples the 32^3 level's work runs in clusters (cluster32.cu), which take
+// four SMs per sample: one wave.  The whole 32^3 solve (three steps of six iterations):
+// 0.55 ms up to 32 samples, 1.1 ms at 38 (a second wave), against 0.95 to 1.0 ms in
+// passes; the V-cycle from 32^3 down 18 us against 38 us in three passes, 38 us at 38.
+constexpr int kCluster32Max = 32;
+
 // One V(1,1)-cycle on r0 (level-0 coefficient a0); the result is left in vt[0].
 // Grids with N >= kTiledMinN run the fine level with the tiled passes (PRE
 // fuses the pre-smoothing into the residual, POST fuses prolongation,
@@ -720,6 +726,13 @@ static int vcycle(SolverBufs& B, const T* r0, const TA0* a0, const SolveScalars*
   if (tiled)
     for (int j = 1; j < J; ++j)
       if (coarse_vcycle_applies(B.N, j) && J - j == 3) jc = j;
+  // small batches: from the coarse 32^3 level on the V-cycle is one launch of clusters
+  bool from32 = false;
+  if constexpr (std::is_same<T, float>::value)
+    if (tiled && jc < J && jc >= 2 && B.stencil == 0 && n <= kCluster32Max) {
+      from32 = true;
+      --jc;
+    }
   for (int j = 0; j < jc; ++j) {
     const int Nj = B.N >> j;
     const bool fine = j == 0;
@@ -763,9 +776,13 @@ static int vcycle(SolverBufs& B, const T* r0, const TA0* a0, const SolveScalars*
   if (jc < J) {
     const T* const al[4] = {(const T*)B.acoef[jc], (const T*)B.acoef[jc + 1], (const T*)B.acoef[jc + 2],
                             (const T*)B.acoef[jc + 3]};
+    const T* const below[4] = {al[1], al[2], al[3], from32 ? (const T*)B.acoef[jc + 4] : nullptr};
     if constexpr (std::is_same<T, double>::value) {
+      (void)below;
       const double* const wd[3] = {(const double*)B.dinv[jc], (const double*)B.vx[jc + 1], (const double*)B.vx[jc + 2]};
       (void)coarse_vcycle64(rin(jc), al, wd, (double*)B.vt[jc], sc, bt, (double)omega, st);  // checked by the caller
+    } else if (from32) {
+      (void)vcycle32(rin(jc), al[0], (const float*)B.dinv[jc], below, (float*)B.vt[jc], sc, bt, (double)omega, st);
     } else {
       coarse_vcycle(rin(jc), al, (T*)B.vt[jc], sc, bt, (double)omega, st);
     }
@@ -1096,6 +1113,14 @@ cudaError_t ir_mixed(SolverBufs& B, const float* a32, const __nv_bfloat16* abf, 
       }
     });
     scalar(B, sco, SM_INIT, 0, 0, st, init_blocks(N));
+    if (sres && N == 32 && S <= kCluster32Max) {  // the rest of the solve is one launch of clusters
+      e = solve32(B, a32, abf, bdf, bstride, xdf, prm, inner_iters, inner_next, fixed_steps, st);
+      if (e != cudaSuccess) return e;
+      if (!pair_out)
+        launch("store_x", (double)S * nodes * 16, k_store_pair, grid_nodes(N, S), kBlock, 0, st, x_out,
+               (const float2*)xdf, nodes);
+      return cudaGetLastError();
+    }
   } else {
     launch("init_f64", bb + nbytes<double, double>(N, S, 2, 0), k_init<double>, g(), kBlock, 0, st, b, bstride, r64,
            x_out, B.partial, nodes);

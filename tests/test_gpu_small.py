@@ -25,7 +25,7 @@ def lib():
 
 
 def _solve(lib, grid, S, z, **cfg):
-    ctx = lib.Context(**dict(CFG, max_iter=400, **cfg))
+    ctx = lib.Context(**dict(dict(CFG, max_iter=400), **cfg))
     N = 4 << grid
     f64 = dict(dtype=torch.float64, device="cuda")
     la = torch.zeros(S, N ** 3, **f64)
@@ -93,3 +93,23 @@ def test_zero_nonfinite_and_capped(lib, grid, precision):
     assert ctx.mlsgd_solve_state_adjoint(grid, 2, la, torch.tensor(inputs.z_test(32), **f64), *buf) == 3
     assert (buf[4].cpu().numpy() == 1).all()
     ctx.close()
+
+
+@pytest.mark.parametrize("grid", [3, 4, 5])  # 32^3: the whole solve; 64^3 and 128^3: the V-cycle from 32^3 down
+@pytest.mark.parametrize("knobs", [dict(), dict(inner_iters=1), dict(ir_steps=2, inner_iters=4, inner_iters_next=7)])
+def test_clusters_and_passes_agree(lib, grid, knobs):
+    """Up to 32 samples the 32^3 level runs in clusters, above in passes: the same bits."""
+    z = inputs.z_test(32) + inputs.z_random(32, 3)
+    big = _solve(lib, grid, 33, z, precision="mixed", rtol=1e-8, n_levels=6, ctrl_level=3, **knobs)
+    few = _solve(lib, grid, 3, z, precision="mixed", rtol=1e-8, n_levels=6, ctrl_level=3, **knobs)
+    for a, b in zip(big[1:], few[1:]):
+        assert np.array_equal(a[:3], b)
+
+
+def test_cluster_zero_and_nonfinite(lib):
+    z = np.zeros(32 ** 3)
+    code, la, y, q, phi, it, st = _solve(lib, 3, 3, z, precision="mixed", rtol=1e-8)
+    assert code == 0 and not y.any() and not st.any()
+    z[100] = np.inf
+    code, la, y, q, phi, it, st = _solve(lib, 3, 3, z, precision="mixed", rtol=1e-8)
+    assert code == 4 and (st & 2).all()
