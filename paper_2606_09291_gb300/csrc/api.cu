@@ -12,6 +12,7 @@
 #include <string>
 #include <vector>
 
+#include "internal.cuh"
 #include "kernels.h"
 #include "launch.h"
 #include "kl_table.h"
@@ -152,6 +153,7 @@ GridFields carve_fields(const mlsgd_ctx* ctx, int N, int S, Bump& bp) {
 // sample are OR-ed.
 __global__ void k_record(const SolveScalars* __restrict__ sc, int S, int mixed, int* __restrict__ iters,
                          int* __restrict__ status, int accumulate) {
+  pdl_entry();
   const int s = blockIdx.x * blockDim.x + threadIdx.x;
   if (s >= S) return;
   const int it = mixed ? sc[s].pad : sc[s].iters;
@@ -163,6 +165,7 @@ __global__ void k_record(const SolveScalars* __restrict__ sc, int S, int mixed, 
 // OR of the S per-sample status flags into *out (one block of kAnyBlock threads)
 constexpr int kAnyBlock = 256;
 __global__ void k_status_any(const int* __restrict__ status, int S, int* __restrict__ out) {
+  pdl_entry();
   int v = 0;
   for (int s = threadIdx.x; s < S; s += blockDim.x) v |= status[s];
   for (int o = 16; o > 0; o >>= 1) v |= __shfl_xor_sync(0xffffffffu, v, o);

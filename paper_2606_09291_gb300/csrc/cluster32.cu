@@ -392,6 +392,7 @@ struct VArgs {
   float omega;
 };
 __global__ void __launch_bounds__(kNT, 1) k_vcycle32(VArgs A) {
+  pdl_entry();
   cg::cluster_group cl = cg::this_cluster();
   const int rank = (int)cl.block_rank(), tb = blockIdx.x / kC;
   const int s = A.act != nullptr ? A.act[tb] : tb;
@@ -438,6 +439,7 @@ struct SArgs {
 };
 
 __global__ void __launch_bounds__(kNT, 1) k_solve32(SArgs A) {
+  pdl_entry();
   cg::cluster_group cl = cg::this_cluster();
   const int rank = (int)cl.block_rank(), s = blockIdx.x / kC, tid = threadIdx.x;
   extern __shared__ __align__(16) unsigned char smraw[];

@@ -68,6 +68,7 @@ struct CoarseArgs {
 
 template <typename T>
 __global__ void __launch_bounds__(kCT, 2) k_coarse_vcycle(CoarseArgs A) {
+  pdl_entry();
   using M = CoarseSmem<T>;
   const int s = A.act != nullptr ? A.act[blockIdx.x] : (int)blockIdx.x;
   if (A.sc != nullptr && !A.sc[s].active) return;

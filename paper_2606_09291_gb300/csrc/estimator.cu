@@ -27,6 +27,7 @@ static int cell_blocks(long long n) {
 // Control coarser than the grid (N = r Nc): each of the 8 cells around node n lies in
 // one control cell (its parent) and int_e phi_n = h^3 / 8.
 __global__ void k_rhs_state(const double* __restrict__ z, int Nc, int N, double* __restrict__ b) {
+  pdl_entry();
   const int n1 = N + 1;
   const long long nodes = (long long)n1 * n1 * n1;
   const int n = blockIdx.x * blockDim.x + threadIdx.x;
@@ -60,6 +61,7 @@ __global__ void k_rhs_state(const double* __restrict__ z, int Nc, int N, double*
 // rows, 116 us now.
 __global__ void __launch_bounds__(kBlock) k_rhs_xy(const double* __restrict__ z, int Nc, int N,
                                                    double* __restrict__ u) {
+  pdl_entry();
   extern __shared__ double sm[];  // t[r], left and right sums [2][Nc]
   const int r = Nc / N, n1 = N + 1;
   double* t = sm;
@@ -95,6 +97,7 @@ __global__ void __launch_bounds__(kBlock) k_rhs_xy(const double* __restrict__ z,
 // node (i, j, k): the right side of cell row j - 1 and the left side of row j, over 2r planes
 __global__ void __launch_bounds__(kBlock) k_rhs_z(const double* __restrict__ u, int Nc, int N,
                                                   double* __restrict__ b) {
+  pdl_entry();
   const int n1 = N + 1, r = Nc / N;
   const int n = blockIdx.x * blockDim.x + threadIdx.x;
   if (n >= n1 * n1 * n1) return;
@@ -119,6 +122,7 @@ __global__ void __launch_bounds__(kBlock) k_rhs_z(const double* __restrict__ u, 
 // thread per node column marches over kRhsPlanes planes; a plane's sums serve two nodes.
 constexpr int kRhsPlanes = 16;
 __global__ void __launch_bounds__(kBlock) k_rhs_equal(const double* __restrict__ z, int N, double* __restrict__ b) {
+  pdl_entry();
   const int n1 = N + 1;
   const int col = blockIdx.x * blockDim.x + threadIdx.x;
   if (col >= n1 * n1) return;
@@ -161,6 +165,7 @@ size_t rhs_scratch_bytes(int Nc, int N) {  // u of k_rhs_xy
 // cx, then each node i of the row contracts its 2r columns with w(x).
 __global__ void __launch_bounds__(kBlock) k_rhs_rows(const double* __restrict__ z, int Nc, int N,
                                                      double* __restrict__ b) {
+  pdl_entry();
   extern __shared__ double sm[];  // w[2r], col[Nc]
   const int n1 = N + 1, r = Nc / N, w2 = 2 * r;
   const int j = blockIdx.x, k = blockIdx.y;
@@ -233,6 +238,7 @@ void launch_rhs_state(const double* z, int Nc, int N, double* b, void* scratch, 
 __global__ void __launch_bounds__(kBlock) k_phi_small(const double* __restrict__ y, int N, double* __restrict__ badj,
                                                       double* __restrict__ phi, const double* __restrict__ gtab,
                                                       const double* __restrict__ mgtab) {
+  pdl_entry();
   __shared__ double u[729], v[729];
   const int s = blockIdx.x, n1 = N + 1, nodes = n1 * n1 * n1;
   const double* ys = y + (long long)s * nodes;
@@ -266,6 +272,7 @@ __global__ void __launch_bounds__(kBlock) k_phi_small(const double* __restrict__
 }
 
 __global__ void k_phi_finish(const double* __restrict__ partial, int nblk, int S, double* __restrict__ phi) {
+  pdl_entry();
   const int s = blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (s >= S) return;
@@ -306,6 +313,7 @@ void launch_phi_adjrhs(const double* y, int N, int S, double* badj, double* phi,
 __global__ void k_level_scalars(const double* __restrict__ phif, const double* __restrict__ phic, int S,
                                 double theta, double* __restrict__ sc, double* __restrict__ work,
                                 const int* __restrict__ iters, const int* __restrict__ status) {
+  pdl_entry();
   __shared__ double smax[kBlock / 32];
   double m = -INFINITY;
   for (int s = threadIdx.x; s < S; s += blockDim.x) {
@@ -590,6 +598,7 @@ __global__ void __launch_bounds__(kBlock) k_level_field(const void* __restrict__
                                                         const void* __restrict__ qc_, int Ncs, int S, int Nc,
                                                         double inv_s, const double* __restrict__ work,
                                                         double* __restrict__ field, double* __restrict__ partial) {
+  pdl_entry();
   using QF = typename std::conditional<PF, float2, double>::type;
   using QC = typename std::conditional<PC, float2, double>::type;
   const QF* qf = (const QF*)qf_;
@@ -655,6 +664,7 @@ __global__ void __launch_bounds__(kBlock, 4) k_level_pairs(const float2* __restr
                                                            const float2* __restrict__ qc, int S, int Nc, double inv_s,
                                                            const double* __restrict__ work, double* __restrict__ field,
                                                            double* __restrict__ partial) {
+  pdl_entry();
   constexpr int CB = kBlock / G;  // cells per block
   __shared__ double sums[G > 1 ? 2 : 1][G][CB];
   const unsigned ncell = (unsigned)Nc * Nc * Nc;
@@ -742,6 +752,7 @@ __device__ __forceinline__ double ldq(const float2* p, long long i) {
 template <typename QF, typename QC>
 __global__ void __launch_bounds__(kBlock) k_lvl_x(QF* __restrict__ qf, int Nf, const QC* __restrict__ qc, int S,
                                                   const double* __restrict__ work) {
+  pdl_entry();
   const int s = blockIdx.y;
   const int n1 = Nf + 1, nodes = n1 * n1 * n1;  // at most 257^3 (the control grid is 4x finer)
   const int n = blockIdx.x * blockDim.x + threadIdx.x;
@@ -766,6 +777,7 @@ __global__ void __launch_bounds__(kBlock) k_lvl_x(QF* __restrict__ qf, int Nf, c
 // and splits the samples over its eight warps (summed in a fixed order)
 __global__ void __launch_bounds__(kBlock) k_lvl_mean(const double* __restrict__ x, int nodes, int S, double inv_s,
                                                      double* __restrict__ mean) {
+  pdl_entry();
   __shared__ double part[8][32];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int n = blockIdx.x * 32 + lane;
@@ -788,6 +800,7 @@ __global__ void __launch_bounds__(kBlock) k_lvl_mean(const double* __restrict__ 
 __global__ void __launch_bounds__(kBlock) k_lvl_s2_small(const double* __restrict__ x, int N, int S,
                                                          const double* __restrict__ mean, double A2, double B,
                                                          double hf3, double* __restrict__ partial) {
+  pdl_entry();
   extern __shared__ double sm[];
   const int n1 = N + 1, nodes = n1 * n1 * n1, m1 = N - 1, inner = m1 * m1 * m1;
   double *d = sm, *u = sm + nodes, *v = sm + 2 * nodes;
@@ -828,6 +841,7 @@ constexpr int kLvlPlanes = 16, kLvlTY = 32;
 __global__ void __launch_bounds__(kBlock) k_lvl_s2(const double* __restrict__ x, int N, int S, int groups,
                                                    const double* __restrict__ mean, double A2, double B, double hf3,
                                                    double* __restrict__ partial) {
+  pdl_entry();
   __shared__ double d[kLvlTY + 2][34], u[kLvlTY + 2][32];
   const int n1 = N + 1, tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
   const long long nodes = (long long)n1 * n1 * n1, pn = (long long)n1 * n1;
@@ -878,6 +892,7 @@ constexpr int kLvlRows = 16;
 __global__ void __launch_bounds__(kBlock) k_lvl_field(const double* __restrict__ xm, int Nf, int Nc, int S,
                                                       const double* __restrict__ work, double* __restrict__ field,
                                                       double* __restrict__ partial) {
+  pdl_entry();
   extern __shared__ double col[];  // [2][Nf + 1]: the mean interpolated in (y, z), and its x differences
   const int n1 = Nf + 1, r = Nc / Nf;
   const long long sz = (long long)n1 * n1;
@@ -973,6 +988,7 @@ static int launch_lvl(const void* qf, int Nf, const void* qc, int S, int Nc, con
 // s2_dx = old * scale^2 + sum of partials (fixed order, one block)
 __global__ void __launch_bounds__(kBlock) k_level_finish(const double* __restrict__ partial, int nblk,
                                                          const double* __restrict__ work, double* __restrict__ sc) {
+  pdl_entry();
   double v = 0.0;
   for (int t = threadIdx.x; t < nblk; t += kBlock) v += partial[t];
   v = block_sum(v);
@@ -1029,6 +1045,7 @@ void launch_level_stats(const double* qf, const double* phif, int Nf, const doub
 }
 
 __global__ void __launch_bounds__(kBlock) k_stats_reset(double* __restrict__ field, double* __restrict__ sc, long long n) {
+  pdl_entry();
   const long long i0 = (long long)blockIdx.x * kBlock + threadIdx.x, step = (long long)gridDim.x * kBlock;
   if (i0 < MLSGD_NSCALARS) sc[i0] = (i0 == MLSGD_S_SHIFT || i0 == MLSGD_S_PHI_MAX) ? -INFINITY : 0.0;
 #pragma unroll 4
@@ -1054,6 +1071,7 @@ __global__ void __launch_bounds__(kBlock) k_merge_field(double* __restrict__ df,
                                                         const double* __restrict__ sf, const double* __restrict__ ssc,
                                                         long long n, double theta, double hc3,
                                                         double* __restrict__ partial) {
+  pdl_entry();
   __shared__ double co[4];  // fa, fb, na / nt, h_c^3 na nb / nt
   __shared__ int form;      // 0: both empty, 1: dst empty, 2: src holds the larger shift (fb = 1), 3: dst does
   if (threadIdx.x == 0) {
@@ -1101,6 +1119,7 @@ __global__ void __launch_bounds__(kBlock) k_merge_field(double* __restrict__ df,
 __global__ void __launch_bounds__(kBlock) k_merge_scalars(const double* __restrict__ partial, int nblk,
                                                           double* __restrict__ dsc, const double* __restrict__ ssc,
                                                           double theta) {
+  pdl_entry();
   double v = 0.0;
   for (int t = threadIdx.x; t < nblk; t += kBlock) v += partial[t];
   v = block_sum(v);
@@ -1150,6 +1169,7 @@ __global__ void __launch_bounds__(kBlock) k_combine_step(FieldList fl, const dou
                                                          double* __restrict__ z, double* __restrict__ grad,
                                                          const double* __restrict__ gprev, double* __restrict__ partial,
                                                          int nblk) {
+  pdl_entry();
   double fac[L], ml[L];
 #pragma unroll
   for (int l = 0; l < L; ++l) {
@@ -1196,6 +1216,7 @@ __global__ void __launch_bounds__(kBlock) k_combine_step(FieldList fl, const dou
 // z <- z - tau g, and gout <- g (the gradient kept for the next step size)
 __global__ void k_step_apply(long long n, double tau, const double* __restrict__ g, double* __restrict__ z,
                              double* __restrict__ gout) {
+  pdl_entry();
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const double gi = g[i];
@@ -1206,6 +1227,7 @@ __global__ void k_step_apply(long long n, double tau, const double* __restrict__
 // out[r] = sum of row r of partial (one block per row)
 __global__ void __launch_bounds__(kBlock) k_rows_finish(const double* __restrict__ partial, int nblk,
                                                         double* __restrict__ out) {
+  pdl_entry();
   double v = 0.0;
   for (int t = threadIdx.x; t < nblk; t += kBlock) v += partial[(long long)blockIdx.x * nblk + t];
   v = block_sum(v);

@@ -16,6 +16,7 @@ namespace mlsgd {
 // half_width > 0: xi uniform on (-half_width, half_width] from the same uniforms
 __global__ void k_draw_xi(uint32_t key0, uint32_t key1, uint32_t iter, uint32_t level, long long first,
                           int S, int K, double half_width, double* __restrict__ xi) {
+  pdl_entry();
   const int pairs = (K + 1) / 2;
   const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= (long long)S * pairs) return;
@@ -69,6 +70,7 @@ __device__ __forceinline__ float exp_to_f32(double la) {
 template <int PL>
 __global__ void __launch_bounds__(kBlock) k_field(const double* __restrict__ xi, int K, const ModeTable mt,
                                                   const double* __restrict__ phi, int N, FieldOut out) {
+  pdl_entry();
   extern __shared__ double sm[];
   const int H = N / 2;
   double* cz = sm;
@@ -154,6 +156,7 @@ constexpr float kLn2Hi = 0.693145751953125f;        // ln 2 truncated to 16 bits
 constexpr float kLn2Lo = 1.4286068202862268e-06f;   // ln 2 - kLn2Hi
 __global__ void k_field_df(const double* __restrict__ xi, int K, const ModeTable mt, const double* __restrict__ phi,
                            int N, int planes, float* __restrict__ a32, __nv_bfloat16* __restrict__ abf) {
+  pdl_entry();
   extern __shared__ __align__(16) unsigned char smf[];
   float2* cz = reinterpret_cast<float2*>(smf);  // c_k phi_{iz_k}(z) as pairs
   float2* ck = cz + ((K + 1) & ~1);             // c_k as pairs
@@ -272,11 +275,13 @@ cudaError_t launch_field(const double* xi, int K, const ModeTable& mt, const dou
 // exp of a stored log field (used when the caller passes log a)
 template <typename TO>
 __global__ void k_exp_field(const double* __restrict__ la, TO* __restrict__ a, long long n) {
+  pdl_entry();
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) a[i] = (TO)exp(la[i]);
 }
 __global__ void k_exp_field_mixed(const double* __restrict__ la, float* __restrict__ a32,
                                   __nv_bfloat16* __restrict__ abf, long long n) {
+  pdl_entry();
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) {
     const double a = exp(la[i]);

@@ -31,6 +31,16 @@ template <typename T> __device__ __forceinline__ T smem_coef(double v) { return 
 template <typename T> __device__ __forceinline__ T smem_coef(float v) { return (T)v; }
 template <typename T> __device__ __forceinline__ T smem_coef(__nv_bfloat16 v) { return (T)__bfloat162float(v); }
 
+// ---------------------------------------------------------------- programmatic launch
+// First statement of every kernel: waits until the kernels before it in the stream have
+// completed and their writes are visible (nothing is read or written before), then lets
+// the next kernel's blocks be launched as soon as all of this kernel's have started, so
+// that their launch latency is hidden (launch.h sets the attribute).
+__device__ __forceinline__ void pdl_entry() {
+  asm volatile("griddepcontrol.wait;\n" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
+}
+
 // ---------------------------------------------------------------- Philox4x32-10
 // Salmon, Moraes, Dror, Shaw, "Parallel random numbers: as easy as 1, 2, 3"
 // (SC'11): 10 rounds; a round multiplies counter words 0 and 2 by the two

@@ -82,6 +82,7 @@ __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::
 __global__ void __launch_bounds__(128, kGemmCtasPerSm)
     k_kl_gemm(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, int S, int cells, int K,
               __nv_bfloat16* __restrict__ abf, float* __restrict__ loga, int* __restrict__ err) {
+  pdl_entry();
   extern __shared__ unsigned char gsm_raw[];
   // 1024-byte aligned base for the swizzled stages
   const uint32_t raw = su32(gsm_raw);
@@ -220,12 +221,14 @@ __global__ void __launch_bounds__(128, kGemmCtasPerSm)
 // A operand: A[s][k] = bf16(scale_k * xi[s][k])
 __global__ void k_gemm_a(const double* __restrict__ xi, const double* __restrict__ scale, int S, int K,
                          __nv_bfloat16* __restrict__ A) {
+  pdl_entry();
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < (long long)S * K) A[i] = __float2bfloat16_rn((float)(scale[i % K] * xi[i]));
 }
 // B operand (cells x K, K contiguous): phi_ix(x) phi_iy(y) phi_iz(z) at the cell centres
 __global__ void k_gemm_b(const double* __restrict__ phi, const int* __restrict__ ix, const int* __restrict__ iy,
                          const int* __restrict__ iz, int N, int K, __nv_bfloat16* __restrict__ B) {
+  pdl_entry();
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   const long long cells = (long long)N * N * N;
   if (i >= cells * K) return;

@@ -217,6 +217,7 @@ __device__ __forceinline__ void ld_cell_pair(const __nv_bfloat16* c, float& a, f
 
 template <int N, typename TA, int MODE>
 __global__ void __launch_bounds__(256, 3) k_slab(SlabArgs A) {
+  pdl_entry();
   using G = SlabGeo<N>;
   using L = SlabSmem<N, TA, MODE>;
   constexpr int RX = G::RX, RY = G::RY, TYT = G::TYT, N1 = G::N1, NR = G::NR, XS = G::XS;
@@ -1026,6 +1027,7 @@ void slab_res(const float* d, const float* p, bool d_zero, const SolveScalars* s
 template <int N>
 __global__ void __launch_bounds__(256) k_zero_seams(float* __restrict__ rc, const int* __restrict__ act,
                                                     const SolveScalars* __restrict__ sc) {
+  pdl_entry();
   using G = SlabGeo<N>;
   const int s = act != nullptr ? act[blockIdx.x] : (int)blockIdx.x;
   if (sc != nullptr && !sc[s].active) return;

@@ -88,6 +88,7 @@ struct Smem8 {
 };
 
 __global__ void __launch_bounds__(kT8, 2) k_small8(SmallArgs A) {
+  pdl_entry();
   __shared__ Smem8 M;
   const int s = blockIdx.x, n = threadIdx.x, lane = n & 31, warp = n >> 5;
   const float omega = A.omega;
@@ -280,6 +281,7 @@ __device__ __forceinline__ float q1_tile(const float* x, const float* a, int n, 
 }
 
 __global__ void __launch_bounds__(kT16, 1) k_small16(SmallArgs A) {
+  pdl_entry();
   extern __shared__ __align__(16) unsigned char smraw[];
   Smem16& M = *reinterpret_cast<Smem16*>(smraw);
   const int s = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;

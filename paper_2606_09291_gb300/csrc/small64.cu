@@ -341,6 +341,7 @@ struct CoarseArgs64 {
 using SmemV = With8<16, Smem<16>>;
 
 __global__ void __launch_bounds__(256, 2) k_vcycle64(CoarseArgs64 A) {
+  pdl_entry();
   cg::cluster_group cl = cg::this_cluster();
   const int rank = (int)cl.block_rank(), t = blockIdx.x / 8;
   const int s = A.act != nullptr ? A.act[t] : t;
@@ -409,6 +410,7 @@ __device__ __forceinline__ double omega_over_d(const double* c, int i, int j, in
 
 template <int N>
 __global__ void __launch_bounds__(Cfg<N>::NT, N == 16 ? 2 : 8) k_small64(SolveArgs64 A) {
+  pdl_entry();
   using K = Cfg<N>;
   using SM = With8<N, SmemSolve<N>>;
   constexpr int S1 = K::n1, S2 = K::PL, C = K::C, NT = K::NT;

@@ -36,6 +36,7 @@ template <typename T, typename TA>
 __global__ void k_apply_dot(const T* __restrict__ x, const TA* __restrict__ a, T* __restrict__ y,
                             double* __restrict__ partial, const SolveScalars* __restrict__ sc, int N,
                             const int* __restrict__ act) {
+  pdl_entry();
   SAMPLE_GUARD(sc);
   const int n1 = N + 1;
   const long long nodes = (long long)n1 * n1 * n1;
@@ -61,6 +62,7 @@ __global__ void k_apply_dot(const T* __restrict__ x, const TA* __restrict__ a, T
 template <typename T>
 __global__ void k_dot(const T* __restrict__ u, const T* __restrict__ v, double* __restrict__ partial,
                       const SolveScalars* __restrict__ sc, long long nodes, const int* __restrict__ act) {
+  pdl_entry();
   SAMPLE_GUARD(sc);
   const int n = blockIdx.x * blockDim.x + threadIdx.x;
   T contrib = T(0);
@@ -74,6 +76,7 @@ template <typename T, bool REDUCE>
 __global__ void k_update_xr(T* __restrict__ x, T* __restrict__ r, const T* __restrict__ p, const T* __restrict__ q,
                             double* __restrict__ partial, const SolveScalars* __restrict__ sc, long long nodes,
                             const int* __restrict__ act) {
+  pdl_entry();
   SAMPLE_GUARD(sc);
   const int n = blockIdx.x * blockDim.x + threadIdx.x;
   const T al = (T)sc[s].alpha;
@@ -94,6 +97,7 @@ __global__ void k_update_xr(T* __restrict__ x, T* __restrict__ r, const T* __res
 template <typename T>
 __global__ void k_p_update(T* __restrict__ p, const T* __restrict__ z, const SolveScalars* __restrict__ sc,
                            long long nodes, int first, const int* __restrict__ act) {
+  pdl_entry();
   SAMPLE_GUARD(sc);
   const int n = blockIdx.x * blockDim.x + threadIdx.x;
   if (n < nodes) {
@@ -106,6 +110,7 @@ __global__ void k_p_update(T* __restrict__ p, const T* __restrict__ z, const Sol
 template <typename T>
 __global__ void k_init(const double* __restrict__ b, long long bstride, T* __restrict__ r, T* __restrict__ x,
                        double* __restrict__ partial, long long nodes) {
+  pdl_entry();
   const int s = blockIdx.y;
   const int n = blockIdx.x * blockDim.x + threadIdx.x;
   double contrib = 0.0;
@@ -124,6 +129,7 @@ __global__ void k_init(const double* __restrict__ b, long long bstride, T* __res
 __global__ void k_scalar(const double* __restrict__ partial, int nblk, SolveScalars* __restrict__ sc, int n,
                          const int* __restrict__ act, int mode, double tol2, int max_iter, int inner_iters,
                          const SolveScalars* __restrict__ outer) {
+  pdl_entry();
   const int t = blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (t >= n) return;
@@ -171,6 +177,7 @@ __global__ void k_scalar(const double* __restrict__ partial, int nblk, SolveScal
 // each chunk's offsets come from warp ballots and a scan of the warp counts.
 __global__ void __launch_bounds__(kBlock) k_compact(const SolveScalars* __restrict__ sc, int S, int* __restrict__ act,
                                                     int* __restrict__ count) {
+  pdl_entry();
   __shared__ int wcount[kBlock / 32];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   int base = 0;
@@ -194,6 +201,7 @@ __global__ void __launch_bounds__(kBlock) k_compact(const SolveScalars* __restri
 template <typename T, typename TA>
 __global__ void k_jacobi0(const T* __restrict__ r, const TA* __restrict__ a, T* __restrict__ x,
                           const SolveScalars* __restrict__ sc, int N, T omega, const int* __restrict__ act) {
+  pdl_entry();
   SAMPLE_GUARD(sc);
   const int n1 = N + 1;
   const long long nodes = (long long)n1 * n1 * n1;
@@ -215,6 +223,7 @@ template <typename T, typename TA, int MODE>
 __global__ void k_resid_smooth(const T* __restrict__ r, const T* __restrict__ x, const TA* __restrict__ a,
                                T* __restrict__ t, const SolveScalars* __restrict__ sc, int N, T omega,
                                const int* __restrict__ act) {
+  pdl_entry();
   SAMPLE_GUARD(sc);
   const int n1 = N + 1;
   const long long nodes = (long long)n1 * n1 * n1;
@@ -237,6 +246,7 @@ __global__ void k_resid_smooth(const T* __restrict__ r, const T* __restrict__ x,
 template <typename T, int NCC = 0>
 __global__ void k_restrict(const T* __restrict__ tf, T* __restrict__ rc, const SolveScalars* __restrict__ sc,
                            int Nc_, const int* __restrict__ act) {
+  pdl_entry();
   SAMPLE_GUARD(sc);
   const int Nc = NCC ? NCC : Nc_;  // a compile-time grid makes the index divisions multiplications
   const int n1c = Nc + 1, Nf = 2 * Nc, n1f = Nf + 1;
@@ -269,6 +279,7 @@ constexpr int kRestrictPlanes = 8;
 template <typename T, int NCC>
 __global__ void k_restrict_zm(const T* __restrict__ tf, T* __restrict__ rc, const SolveScalars* __restrict__ sc,
                               const int* __restrict__ act) {
+  pdl_entry();
   SAMPLE_GUARD(sc);
   constexpr int Nc = NCC, n1c = Nc + 1, n1f = 2 * Nc + 1;
   constexpr long long nc = (long long)n1c * n1c * n1c, nf = (long long)n1f * n1f * n1f;
@@ -307,6 +318,7 @@ __global__ void k_restrict_zm(const T* __restrict__ tf, T* __restrict__ rc, cons
 template <typename T>
 __global__ void k_prolong_add(T* __restrict__ xf, const T* __restrict__ ec, const SolveScalars* __restrict__ sc,
                               int Nf, const int* __restrict__ act) {
+  pdl_entry();
   SAMPLE_GUARD(sc);
   const int n1f = Nf + 1, Nc = Nf / 2, n1c = Nc + 1;
   const long long nf = (long long)n1f * n1f * n1f, nc = (long long)n1c * n1c * n1c;
@@ -337,6 +349,7 @@ __global__ void k_prolong_add(T* __restrict__ xf, const T* __restrict__ ec, cons
 template <typename T, typename TA>
 __global__ void k_coarsest(const T* __restrict__ r, const TA* __restrict__ a, T* __restrict__ x,
                            const SolveScalars* __restrict__ sc, int n, const int* __restrict__ act) {
+  pdl_entry();
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= n) return;
   const int s = act != nullptr ? act[t] : t;
@@ -355,6 +368,7 @@ template <typename TI, typename TO>
 // (8-bit significands, the coefficient's range spans well under 16 binary orders), and
 // the coarse coefficients only shape the preconditioner; the FP64 path sums in FP64.
 __global__ void k_coarsen_coef(const TI* __restrict__ af, TO* __restrict__ ac, int Nc) {
+  pdl_entry();
   using Acc = typename std::conditional<std::is_same<TO, double>::value, double, float>::type;
   const int cc = Nc * Nc * Nc;
   const int c = blockIdx.x * blockDim.x + threadIdx.x;
@@ -380,6 +394,7 @@ template <typename TA>
 __global__ void k_residual64(const double* __restrict__ b, long long bstride, const double* __restrict__ x,
                              const TA* __restrict__ a, double* __restrict__ r, double* __restrict__ partial,
                              const SolveScalars* __restrict__ sc, int N, const int* __restrict__ act) {
+  pdl_entry();
   SAMPLE_GUARD(sc);
   const int n1 = N + 1;
   const long long nodes = (long long)n1 * n1 * n1;
@@ -404,6 +419,7 @@ __global__ void k_residual64(const double* __restrict__ b, long long bstride, co
 // r32 = (float) r64, d = 0
 __global__ void k_demote(const double* __restrict__ r64, float* __restrict__ r32, float* __restrict__ d,
                          const SolveScalars* __restrict__ sc, long long nodes, const int* __restrict__ act) {
+  pdl_entry();
   SAMPLE_GUARD(sc);
   const int n = blockIdx.x * blockDim.x + threadIdx.x;
   if (n < nodes) {
@@ -423,6 +439,7 @@ template <bool PAIR_B, int NN = 0>
 __global__ void k_init32(const double* __restrict__ b, const float2* __restrict__ bp, long long bstride,
                          float* __restrict__ r32, float2* __restrict__ bdf, double* __restrict__ partial,
                          long long nodes, int N_) {
+  pdl_entry();
   const int N = NN ? NN : N_;
   const int s = blockIdx.y;
   const long long n0 = (long long)blockIdx.x * blockDim.x * kInitPer + threadIdx.x;
@@ -467,6 +484,7 @@ template <int NN = 0>
 __global__ void k_finish_step(float2* __restrict__ x, const float* __restrict__ d, const float* __restrict__ p,
                               const SolveScalars* __restrict__ sci, const SolveScalars* __restrict__ sco,
                               long long nodes, int N_, int assign, int d_zero, const int* __restrict__ act) {
+  pdl_entry();
   const int N = NN ? NN : N_;
   const int s = act != nullptr ? act[blockIdx.y] : (int)blockIdx.y;
   const bool on = sco[s].active != 0;
@@ -497,6 +515,7 @@ __global__ void k_finish_step(float2* __restrict__ x, const float* __restrict__ 
 
 // x64 = hi + lo of the FP32 pair solution (every sample, after the refinement)
 __global__ void k_store_pair(double* __restrict__ x, const float2* __restrict__ xp, long long nodes) {
+  pdl_entry();
   const int s = blockIdx.y;
   const int n = blockIdx.x * blockDim.x + threadIdx.x;
   if (n >= nodes) return;
@@ -507,6 +526,7 @@ __global__ void k_store_pair(double* __restrict__ x, const float2* __restrict__ 
 // x64 += d
 __global__ void k_accumulate(double* __restrict__ x, const float* __restrict__ d, const SolveScalars* __restrict__ sc,
                              long long nodes, const int* __restrict__ act) {
+  pdl_entry();
   SAMPLE_GUARD(sc);
   const int n = blockIdx.x * blockDim.x + threadIdx.x;
   if (n < nodes) x[s * nodes + n] += (double)d[s * nodes + n];
@@ -619,6 +639,7 @@ __device__ __forceinline__ float recip(float x) { return __fdividef(1.0f, x); }
 constexpr int kDinvPlanes = 8;
 template <typename T, typename TA>
 __global__ void k_dinv(const TA* __restrict__ a, T* __restrict__ dinv, int N, T omega) {
+  pdl_entry();
   const int s = blockIdx.y;
   const int n1 = N + 1;
   const int col = blockIdx.x * blockDim.x + threadIdx.x;
@@ -995,6 +1016,7 @@ static cudaError_t pcg_inner_fused(SolverBufs& B, const float* a32, const __nv_b
 struct ZeroList { void* v[6]; };
 template <typename T>
 __global__ void k_zero_boundary(ZeroList zl, int nv, int N) {
+  pdl_entry();
   const int s = blockIdx.y;
   const int n1 = N + 1;
   const long long plane = (long long)n1 * n1;

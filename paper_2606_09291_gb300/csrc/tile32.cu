@@ -107,6 +107,7 @@ __device__ __forceinline__ float cell_f(__nv_bfloat16 c) { return __bfloat162flo
 
 template <typename TA, int MODE>
 __global__ void __launch_bounds__(256, 3) k_tile32(Args A) {
+  pdl_entry();
   using SM = Smem<TA, MODE>;
   constexpr bool kX = MODE == T_APPLYX, kApply = MODE == T_APPLY || kX, kPost = MODE == T_POST;
   constexpr bool kPre = MODE == T_PRE || MODE == T_PREU;

@@ -126,6 +126,7 @@ struct TiledSmem {
 
 template <typename T, typename TA, int MODE>
 __global__ void __launch_bounds__(NT) k_tiled(TiledArgs A) {
+  pdl_entry();
   using L = TiledSmem<T, TA, MODE>;
   constexpr int RY = L::RY;
   using G = typename L::G;
@@ -563,6 +564,7 @@ __global__ void __launch_bounds__(NT) k_tiled(TiledArgs A) {
 __global__ void __launch_bounds__(NT) k_phi_tiled(const double* __restrict__ y, int N, const double* __restrict__ gtab,
                                                   const double* __restrict__ mgtab, double* __restrict__ badj,
                                                   double* __restrict__ partial, int nzc, int zc, int nseg) {
+  pdl_entry();
   __shared__ double ys[NP];
   __shared__ double xsum[NPY][TX];
   __shared__ double mxy[3][NT];
@@ -632,6 +634,7 @@ constexpr size_t kPhiSmem = sizeof(float2) * (2 * kPhiNP + kPhiNPY * TX + 3 * kP
 __global__ void __launch_bounds__(NT) k_phi_tiled_df(const float2* __restrict__ y, int N, const float2* __restrict__ gtab,
                                                      const float2* __restrict__ mgtab, float2* __restrict__ badj,
                                                      double* __restrict__ partial, int nzc, int zc, int nseg) {
+  pdl_entry();
   extern __shared__ __align__(16) unsigned char smp[];
   float2* ysb = reinterpret_cast<float2*>(smp);  // [2][kPhiNP]: plane m in buffer m & 1
   float2(*xsum)[TX] = reinterpret_cast<float2(*)[TX]>(ysb + 2 * kPhiNP);                   // [kPhiNPY][TX]
