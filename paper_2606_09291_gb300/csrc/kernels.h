@@ -134,29 +134,37 @@ void build_hierarchy_mixed(SolverBufs& B, const __nv_bfloat16* abf, double omega
 size_t solver_bytes(int N, int S, int elem);
 void carve_solver(SolverBufs& B, int N, int S, int elem, char*& ptr);
 
-// tiled fine-grid kernels (tiled.cu); partial sums land in [S][blocks_per_sample], one
-// entry per (xy tile, segment of 8 interior planes), independent of the z chunking
+// tiled fine-grid passes: partial sums land in [S][blocks_per_sample], one entry per (xy
+// tile, segment of 8 interior planes), independent of the z chunking
 struct TiledShape { int bx, by, nzc, zc, nseg, blocks_per_sample; };
 TiledShape tiled_shape(int N, int S, int rows_per_thread, int zchunks = 0);
-// partial-sum entries per sample of the solver passes for elements of `elem` bytes
-// (slab: the whole-row slab passes' geometry)
-int tiled_blocks_per_sample(int N, int S, int elem, bool slab);
-template <typename T, typename TA>
-void tiled_apply(const T* z, const T* pold, T* pnew, const TA* a, T* q, double* partial, const SolveScalars* sc, int N,
-                 const Batch& bt, int first, cudaStream_t st);
+// partial-sum entries per sample of the FP32 passes (slab: the whole-row slab passes' geometry)
+int tiled_blocks_per_sample(int N, int S, bool slab);
+int res64_blocks_per_sample(int N, int S);  // of tiled_res64
+// The FP32 passes: slab.cu on 32^3 and 64^3 grids (unless Batch::stencil is 1), else tile32.cu
+void tiled_apply(const float* z, const float* pold, float* pnew, const float* a, float* q, double* partial,
+                 const SolveScalars* sc, int N, const Batch& bt, int first, cudaStream_t st);
 // PRE (and PREU): t = r - A x1 with x1 = omega D^-1 r (PREU: r <- r - alpha q first, stored
 // in rnew).  True when the pass also restricted t to rc on grid N/2 (the slab passes;
 // t is then not stored), false when t was stored for a separate restriction.
-template <typename T, typename TA>
-bool tiled_pre(const T* r, const TA* a, const T* wdinv, T* t, T* rc, const SolveScalars* sc, int N, const Batch& bt,
-               cudaStream_t st);
-template <typename T, typename TA>
-void tiled_post(const T* r, const TA* a, const T* wdinv, const T* ec, T* z, double* partial, const SolveScalars* sc,
-                int N, const Batch& bt, cudaStream_t st);
+template <typename TA>
+bool tiled_pre(const float* r, const TA* a, const float* wdinv, float* t, float* rc, const SolveScalars* sc, int N,
+               const Batch& bt, cudaStream_t st);
+template <typename TA>
+void tiled_post(const float* r, const TA* a, const float* wdinv, const float* ec, float* z, double* partial,
+                const SolveScalars* sc, int N, const Batch& bt, cudaStream_t st);
 void tiled_apply_x(const float* z, const float* pold, float* pnew, const float* a, float* q, float* x, double* partial,
                    const SolveScalars* sc, int N, const Batch& bt, cudaStream_t st, bool x_first);
 bool tiled_pre_update(const float* r, const float* q, const __nv_bfloat16* a, const float* wdinv, float* t,
                       float* rnew, float* rc, const SolveScalars* sc, int N, const Batch& bt, cudaStream_t st);
+// The FP64 passes on grids of 32^3 and up (tile64.cu)
+int tile64_blocks_per_sample(int N);
+void tile64_apply(const double* z, const double* pold, double* pnew, const double* a, double* q, double* partial,
+                  const SolveScalars* sc, int N, const Batch& bt, bool first, cudaStream_t st);
+void tile64_pre(const double* r, const double* a, const double* wdinv, double* t, const SolveScalars* sc, int N,
+                const Batch& bt, double omega, cudaStream_t st);
+void tile64_post(const double* r, const double* a, const double* wdinv, const double* ec, double* z, double* partial,
+                 const SolveScalars* sc, int N, const Batch& bt, double omega, cudaStream_t st);
 // r32 = (float)(b - A x) to FP64 accuracy with x, b as FP32 (hi, lo) pairs and error-free
 // FP32 products and sums; partial r.r
 void tiled_res64(const float2* b, long long bstride, const float2* x, const float* a, float* r32, double* partial,

@@ -563,6 +563,13 @@ static int mg_levels(int N) {
 // the whole-row slab passes run the FP32 fused passes of grid N
 static bool uses_slab(const SolverBufs& B, int N, int elem) { return elem == 4 && B.stencil == 0 && slab_supported(N); }
 
+// partial sums per sample of the fine level's tiled passes
+template <typename T>
+static int fine_blocks(const SolverBufs& B) {
+  if (std::is_same<T, double>::value) return tile64_blocks_per_sample(B.N);
+  return tiled_blocks_per_sample(B.N, B.S, uses_slab(B, B.N, 4));
+}
+
 // levels whose smoothing runs in the tiled passes (they read a precomputed D^{-1})
 static bool tiled_level(int N, int j) { return N >= kTiledMinN && mg_levels(N) >= 1 && (N >> j) >= kTiledMinN; }
 
@@ -734,7 +741,7 @@ constexpr int kCluster32Max = 32;
 template <typename T, typename TA0>
 static int vcycle(SolverBufs& B, const T* r0, const TA0* a0, const SolveScalars* sc, T omega, cudaStream_t st,
                   const T* fuse_q = nullptr, T* r_new = nullptr, T* z0 = nullptr) {
-  const int S = B.S, J = B.J;
+  const int J = B.J;
   const int n = B.n_act;            // samples launched (the active ones when compacted)
   const int* act = B.actp;
   const Batch bt = B.batch();
@@ -762,10 +769,13 @@ static int vcycle(SolverBufs& B, const T* r0, const TA0* a0, const SolveScalars*
     if (fine && tiled && fuse_q) {
       if constexpr (std::is_same<T, float>::value && std::is_same<TA0, __nv_bfloat16>::value)
         restricted = tiled_pre_update(r0, fuse_q, a0, (const T*)B.dinv[0], (T*)B.vt[0], r_new, rc, sc, Nj, bt, st);
-    } else if (fine && tiled) {
-      restricted = tiled_pre<T, TA0>(r0, a0, (const T*)B.dinv[0], (T*)B.vt[0], rc, sc, Nj, bt, st);
-    } else if (!fine && tiled && Nj >= kTiledMinN) {
-      restricted = tiled_pre<T, T>(rin(j), (const T*)B.acoef[j], (const T*)B.dinv[j], (T*)B.vt[j], rc, sc, Nj, bt, st);
+    } else if (tiled && Nj >= kTiledMinN) {
+      if constexpr (std::is_same<T, double>::value)
+        tile64_pre(rin(j), fine ? a0 : (const T*)B.acoef[j], (const T*)B.dinv[j], (T*)B.vt[j], sc, Nj, bt, omega, st);
+      else if (fine)
+        restricted = tiled_pre<TA0>(r0, a0, (const T*)B.dinv[0], (T*)B.vt[0], rc, sc, Nj, bt, st);
+      else
+        restricted = tiled_pre<T>(rin(j), (const T*)B.acoef[j], (const T*)B.dinv[j], (T*)B.vt[j], rc, sc, Nj, bt, st);
     } else if (fine) {
       launch(cls<T>("jacobi0", true), nbytes<T, TA0>(Nj, n, 2, 1), k_jacobi0<T, TA0>, grid_nodes(Nj, n), kBlock, 0,
              st, rin(0), a0, (T*)B.vx[0], sc, Nj, omega, act);
@@ -817,15 +827,17 @@ static int vcycle(SolverBufs& B, const T* r0, const TA0* a0, const SolveScalars*
   for (int j = jc - 1; j >= 0; --j) {
     const int Nj = B.N >> j;
     const bool fine = j == 0;
-    if (fine && tiled) {
-      tiled_post<T, TA0>(rfine, a0, (const T*)B.dinv[0], (const T*)B.vt[1], z0 ? z0 : (T*)B.vt[0], B.partial, sc, Nj,
-                         bt, st);
-      return tiled_blocks_per_sample(Nj, S, (int)sizeof(T), uses_slab(B, Nj, (int)sizeof(T)));
-    }
-    if (!fine && tiled && Nj >= kTiledMinN) {
+    if (tiled && Nj >= kTiledMinN) {
       // the r.z partial sums of a coarse level are overwritten by the fine level's POST
-      tiled_post<T, T>(rin(j), (const T*)B.acoef[j], (const T*)B.dinv[j], (const T*)B.vt[j + 1], (T*)B.vt[j],
-                       B.partial, sc, Nj, bt, st);
+      T* zj = fine && z0 ? z0 : (T*)B.vt[j];
+      const T* ec = (const T*)B.vt[j + 1];
+      if constexpr (std::is_same<T, double>::value)
+        tile64_post(rin(j), fine ? a0 : (const T*)B.acoef[j], (const T*)B.dinv[j], ec, zj, B.partial, sc, Nj, bt, omega, st);
+      else if (fine)
+        tiled_post<TA0>(rfine, a0, (const T*)B.dinv[0], ec, zj, B.partial, sc, Nj, bt, st);
+      else
+        tiled_post<T>(rin(j), (const T*)B.acoef[j], (const T*)B.dinv[j], ec, zj, B.partial, sc, Nj, bt, st);
+      if (fine) return fine_blocks<T>(B);
       continue;
     }
     launch(cls<T>("prolong", fine), nbytes<T, T>(Nj, n, 2, 0) + nbytes<T, T>(Nj / 2, n, 1, 0), k_prolong_add<T>,
@@ -878,7 +890,7 @@ static cudaError_t compact_active(SolverBufs& B, const SolveScalars* sc, cudaStr
 template <typename T, typename TAop, typename TA0>
 static cudaError_t pcg_loop(SolverBufs& B, const TAop* aop, const TA0* a0, T* x, T* r, SolveScalars* sc,
                             const PcgParams& prm, int fixed_iters, cudaStream_t st) {
-  const int S = B.S, N = B.N;
+  const int N = B.N;
   const long long nodes = nodes_of(N);
   const int nb = node_blocks(N);
   const T omega = (T)prm.omega;
@@ -904,12 +916,15 @@ static cudaError_t pcg_loop(SolverBufs& B, const TAop* aop, const TA0* a0, T* x,
            (const SolveScalars*)sc, nodes, 1, B.actp);
   const double tol2 = prm.rtol * prm.rtol;
   const int nit = fixed_iters > 0 ? fixed_iters : prm.max_iter;
-  const int napply = tiled ? tiled_blocks_per_sample(N, S, (int)sizeof(T), uses_slab(B, N, (int)sizeof(T))) : nb;
+  const int napply = tiled ? fine_blocks<T>(B) : nb;
   for (int it = 0; it < nit; ++it) {
     T* p;
     if (tiled) {
       p = pbuf[cur ^ 1];
-      tiled_apply<T, TAop>(z, pbuf[cur], p, aop, q, B.partial, sc, N, B.batch(), it == 0, st);
+      if constexpr (std::is_same<T, double>::value)
+        tile64_apply(z, pbuf[cur], p, aop, q, B.partial, sc, N, B.batch(), it == 0, st);
+      else
+        tiled_apply(z, pbuf[cur], p, aop, q, B.partial, sc, N, B.batch(), it == 0, st);
       cur ^= 1;
     } else {
       p = pbuf[0];
@@ -953,7 +968,7 @@ static cudaError_t pcg_inner_fused(SolverBufs& B, const float* a32, const __nv_b
                                    SolveScalars* sc, const PcgParams& prm, int iters, cudaStream_t st,
                                    float2* x_out, const SolveScalars* sco, bool assign_out,
                                    const float** p_last = nullptr) {
-  const int S = B.S, N = B.N, n = B.n_act;
+  const int N = B.N, n = B.n_act;
   const Batch bt = B.batch();
   const long long nodes = nodes_of(N);
   const float omega = (float)prm.omega;
@@ -971,7 +986,7 @@ static cudaError_t pcg_inner_fused(SolverBufs& B, const float* a32, const __nv_b
   };
   float* z = vb[0];
   float* pold = vb[1];  // not read by the first pass
-  const int napply = tiled_blocks_per_sample(N, S, 4, uses_slab(B, N, 4));
+  const int napply = fine_blocks<float>(B);
   int nrz = vcycle<float, __nv_bfloat16>(B, rb[0], abf, sc, omega, st, nullptr, nullptr, z);
   scalar(B, sc, SM_RZ0, 0, 0, st, nrz);
   int rc = 0;
@@ -979,7 +994,7 @@ static cudaError_t pcg_inner_fused(SolverBufs& B, const float* a32, const __nv_b
     float* pnew;
     if (it == 0) {
       pnew = alias_first ? z : other(z, pold);
-      tiled_apply<float, float>(z, pold, alias_first ? nullptr : pnew, a32, q, B.partial, sc, N, bt, 1, st);
+      tiled_apply(z, pold, alias_first ? nullptr : pnew, a32, q, B.partial, sc, N, bt, 1, st);
     } else {
       pnew = other(z, pold);
       // the last pass needs only p.q (for alpha): with the slab passes q is not stored
@@ -1154,10 +1169,10 @@ cudaError_t ir_mixed(SolverBufs& B, const float* a32, const __nv_bfloat16* abf, 
       if (sres) {
         slab_res(d, p_last, last_inner <= 1, sci, step == 1 ? bdf : B.bdf, step == 1 ? bstride : nodes, B.bdf, xdf,
                  step == 1, a32, r32, B.partial, sco, N, B.batch(), st);
-        scalar(B, sco, SM_OUTER_CONV, tol2, cap, st, tiled_blocks_per_sample(N, S, 4, true));
+        scalar(B, sco, SM_OUTER_CONV, tol2, cap, st, tiled_blocks_per_sample(N, S, true));
       } else if (tiled) {
         tiled_res64(bdf, bstride, xdf, a32, r32, B.partial, sco, N, B.batch(), st);
-        scalar(B, sco, SM_OUTER_CONV, tol2, cap, st, tiled_blocks_per_sample(N, S, 8, false));
+        scalar(B, sco, SM_OUTER_CONV, tol2, cap, st, res64_blocks_per_sample(N, S));
       } else {
         launch("resid64", (double)(bstride ? B.n_act : 1) * nodes * 8 + nbytes<double, float>(N, B.n_act, 2, 1),
                k_residual64<float>, g(), kBlock, 0, st, b, bstride, (const double*)x_out, a32, r64, B.partial,

@@ -1,34 +1,13 @@
-// tiled.cu - z-marching shared-memory kernels for the fine-grid passes of the
-// solver (rows a4, a6) and for Phi / the adjoint right-hand side (row a5).
+// tiled.cu - z-marching shared-memory kernels for the refinement residual on grids without
+// a slab form and for Phi / the adjoint right-hand side (rows a4, a5), and the choice of
+// the FP32 passes' family.
 //
-// Layout: a block of 32 x 8 threads owns a 32 x 8 RY tile of interior nodes (RY
-// rows per thread: 4 for FP32 vectors, 2 for FP64; x0 = 1 + 32 bx, y0 = 1 + 8 RY by)
-// and marches along z over a chunk of interior planes.  Each node plane of an
-// input vector is staged once into shared memory with a one-node halo
-// (34 x (8 RY + 2)), each cell plane with a two-cell halo (36 x (8 RY + 3), from an
-// even x start), with cp.async into a five-plane ring that keeps two planes in
-// flight ahead of the stencil; the operand planes derived from them (three
-// planes) are kept in their own ring.  So every value is read from HBM about
-// once per pass (halos come from L2) and there is no integer division in the
-// index arithmetic.  Node (lx, ly) of the staged plane is the global node
-// (x0 - 1 + lx, y0 - 1 + ly); its eight surrounding cells are the staged cells
-// (lx + p, ly + q), p, q in {0, 1}, of two cell planes.
-//
-// Fused passes (FE operator A: see q1_row in internal.cuh; D = (h/3) sum_8 a, whose
-// inverse is precomputed per coefficient hierarchy and staged like a vector):
-//   APPLY : pn = z + beta p (pn = z on the first iteration); q = A pn;
-//           writes p = pn, q; partial p.q
-//   PRE   : x1 = omega D^{-1} r computed on the fly; t = r - A x1
-//   POST  : x2 = omega D^{-1} r + P e_c on the fly;
-//           z = x2 + omega D^{-1} (r - A x2); partial r.z
-//   (omega D^{-1} is precomputed per coefficient hierarchy and staged like a vector)
-//   RES64 : r = b - A x to FP64 accuracy in FP32 arithmetic: x and b are FP32 (hi, lo)
-//           pairs (staged as 8-byte words), a is FP32; writes r rounded to FP32 and the
-//           partial r.r
-// The fused passes write only interior nodes and zero-fill boundary nodes at staging
-// (like nodes outside the grid), so they never read a buffer's boundary values.
-#include <cstdio>
-#include <type_traits>
+// Layout: a block of 32 x 8 threads owns a tile of interior nodes (x0 = 1 + 32 bx, y0 = 1 +
+// (tile rows) by) and marches along z over a chunk of interior planes; each node plane is
+// staged once into shared memory with a one-node halo by cp.async, so every value is read
+// from HBM about once per pass (halos come from L2).  Node (lx, ly) of the staged plane is
+// the global node (x0 - 1 + lx, y0 - 1 + ly).  Boundary nodes are zero-filled at staging
+// (like nodes outside the grid) and not written.
 
 #include "internal.cuh"
 #include "kernels.h"
@@ -41,32 +20,6 @@ constexpr int TX = 32, TY = 8;
 constexpr int NPX = TX + 2;                     // staged node row: 34 nodes
 constexpr int NPY = TY + 2, NP = NPX * NPY;      // the Phi kernels' staged plane (one row per thread): 34 x 10
 constexpr int NT = TX * TY;
-
-enum TiledMode { TM_APPLY = 0, TM_PRE = 1, TM_POST = 2, TM_RES64 = 3, TM_PREU = 4, TM_APPLYX = 5 };
-
-struct TiledArgs {
-  const void* in0;   // APPLY: z   PRE/POST: r    RES64: x (FP64)
-  const void* in1;   // APPLY: p (old)                RES64: b (FP64)
-  const void* ec;    // POST: coarse correction (grid N/2)
-  const void* a;     // cell coefficient
-  const void* dinv;  // PRE/PREU/POST: omega D^{-1} per node (0 on the boundary)
-  void* out0;        // APPLY: q   PRE: t   POST: z   RES64: r
-  void* out1;        // APPLY: p (new)   PREU: r (new)
-  const void* q;     // PREU: A p of the current iteration
-  void* x;           // APPLYX: solution updated in place with alpha_prev * p_old
-  double* partial;   // [S][blocks per sample]
-  const SolveScalars* sc;
-  const int* act;    // launched samples (null: blockIdx.z / nzc itself)
-  long long bstride; // RES64: b stride per sample (0 = shared)
-  int N;
-  int nzc;           // z chunks per sample
-  int zc;            // planes per chunk (a multiple of kZSeg)
-  int nseg;          // partial-sum segments per sample column
-  int first;         // APPLY: first iteration (pn = z)
-  int xfirst;        // APPLYX: x not yet written (x = alpha_prev p_old)
-};
-
-__device__ __forceinline__ int ring3(int m) { return (m + 3) % 3; }
 
 // ---------------------------------------------------------------- async staging
 // cp.async (4- or 8-byte, zero-filled when the source is outside the grid)
@@ -88,381 +41,99 @@ __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_gr
 // batch size that chose the z chunking.
 constexpr int kZSeg = 8;
 
-constexpr int RING = 5;   // raw planes resident: k-1, k, k+1 + two in flight
+// The refinement residual on grids without a slab form: r = b - A x to FP64 accuracy with
+// x = hi + lo and b as FP32 pairs and FP32 cells, error-free products and compensated sums
+// (no FP64 instruction), rounded to FP32, and the partial r.r.  A tile of 32 x 16 nodes, two
+// rows per thread; the window is read from the staged planes themselves (five of them: three
+// in use, two in flight), so a plane takes one block barrier.  Bound by FP32 issue, some 400
+// operations per node.
+constexpr int kResRows = 2, kResTY = TY * kResRows, kResRing = 5;
+constexpr int kResNP = NPX * (kResTY + 2);                         // staged nodes: 34 x 18
+constexpr int kResCX = TX + 1, kResCP = kResCX * (kResTY + 1);     // staged cells: 33 x 17
+constexpr size_t kResSmem = kResRing * (sizeof(float2) * kResNP + sizeof(float) * kResCP);
 constexpr double kRes64OpsPerNode = 12 * 6 + 28 + 21 * 12 + 20;  // = 372 (see tiled_res64)
-constexpr int ERING = 4;  // coarse planes
-constexpr int CW = TX + 4;  // staged cell row: 36 cells from x0 - 3 (even start)
-constexpr int EWX = TX / 2 + 2;
 
-// Tile geometry for RY nodes per thread in y (block 32 x 8 threads, tile 32 x 8*RY nodes).
-template <int RY>
-struct Geo {
-  static constexpr int TYT = TY * RY;
-  static constexpr int NPYT = TYT + 2, NPL = NPX * NPYT;  // staged node plane (34 x (TYT+2))
-  static constexpr int CPYT = TYT + 3, CPL = CW * CPYT;   // staged cell plane (36 x (TYT+3))
-  static constexpr int EWYT = TYT / 2 + 2, EPL = EWX * EWYT;  // staged coarse plane
+struct ResArgs {
+  const float2 *x, *b;
+  const float* a;
+  float* r;
+  double* partial;
+  const SolveScalars* sc;
+  const int* act;
+  long long bstride;  // 0: one b for every sample
+  int N, nzc, zc, nseg;
 };
 
-template <typename T> struct RowsPerThread { static constexpr int value = 4; };
-template <> struct RowsPerThread<double> { static constexpr int value = 2; };
-
-template <typename T, typename TA, int MODE>
-struct TiledSmem {
-  static constexpr int RY = RowsPerThread<T>::value;
-  using G = Geo<RY>;
-  static constexpr bool kPre = (MODE == TM_PRE || MODE == TM_POST || MODE == TM_PREU);
-  static constexpr bool kApply = (MODE == TM_APPLY || MODE == TM_APPLYX);
-  static constexpr bool kRaw1 = kApply || MODE == TM_PREU;
-  static constexpr size_t raw0 = 0;
-  static constexpr size_t raw1 = raw0 + sizeof(T) * RING * G::NPL;
-  static constexpr size_t xs = raw1 + (kRaw1 ? sizeof(T) * RING * G::NPL : 0);
-  static constexpr size_t dv = xs + sizeof(T) * 3 * G::NPL;
-  static constexpr size_t ec = dv + (kPre ? sizeof(T) * RING * G::NPL : 0);
-  static constexpr size_t ep = ec + (MODE == TM_POST ? sizeof(T) * ERING * G::EPL : 0);
-  static constexpr size_t cells = ep + (MODE == TM_POST ? sizeof(T) * 2 * G::NPL : 0);
-  static constexpr size_t total = cells + sizeof(TA) * RING * G::CPL;
-};
-
-
-template <typename T, typename TA, int MODE>
-__global__ void __launch_bounds__(NT) k_tiled(TiledArgs A) {
+__global__ void __launch_bounds__(NT) k_res64(ResArgs A) {
   pdl_entry();
-  using L = TiledSmem<T, TA, MODE>;
-  constexpr int RY = L::RY;
-  using G = typename L::G;
-  constexpr int NPL = G::NPL, CPL = G::CPL, EPL = G::EPL;
-  constexpr bool kPre = L::kPre;
-  constexpr bool kPairs = sizeof(TA) == 2;                 // BF16 cells staged as 4-byte pairs
-  constexpr int NCE = kPairs ? CPL / 2 : CPL;              // cell staging entries per plane
-  constexpr int MN = (NPL + NT - 1) / NT, MC = (NCE + NT - 1) / NT, ME = (EPL + NT - 1) / NT;
-  // staging entries j < M - 1 always exist (only the last one per thread may not)
-  static_assert((MN - 1) * NT < NPL && (MC - 1) * NT < NCE && (ME - 1) * NT < EPL, "staging entries");
+  constexpr int RY = kResRows;
+  constexpr int MN = (kResNP + NT - 1) / NT, MC = (kResCP + NT - 1) / NT;
   extern __shared__ __align__(16) unsigned char smraw[];
-  T* raw0 = (T*)(smraw + L::raw0);
-  T* raw1 = (T*)(smraw + L::raw1);
-  T* xs = (T*)(smraw + L::xs);
-  T* dvs = (T*)(smraw + L::dv);
-  T* ecs = (T*)(smraw + L::ec);
-  T* eps = (T*)(smraw + L::ep);  // POST: two coarse planes interpolated in x and y to this tile's nodes
-  TA* cs = (TA*)(smraw + L::cells);
+  float2* xs = reinterpret_cast<float2*>(smraw);
+  float* cs = reinterpret_cast<float*>(smraw + kResRing * sizeof(float2) * kResNP);
   const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * TX + tx;
   const int N = A.N, n1 = N + 1;
   const int chunk = blockIdx.z % A.nzc;
   const int s = A.act != nullptr ? A.act[blockIdx.z / A.nzc] : (int)(blockIdx.z / A.nzc);
   if (A.sc != nullptr && !A.sc[s].active) return;
-  const int x0 = 1 + TX * blockIdx.x, y0 = 1 + G::TYT * blockIdx.y;
-  const long long nodes = (long long)n1 * n1 * n1, cells = (long long)N * N * N;
-  const int kbeg = 1 + chunk * A.zc;
-  const int kend = min(N - 1, kbeg + A.zc - 1);
-  const T scale = T(1.0 / (12.0 * N));
-  const T* in0 = (const T*)A.in0 + s * nodes;
-  constexpr bool kApply = L::kApply;
-  const T* in1 = kApply ? (const T*)A.in1 + s * nodes : (MODE == TM_PREU ? (const T*)A.q + s * nodes : in0);
-  const bool stage1 = (kApply && !A.first) || MODE == TM_PREU;  // raw1 holds p_old or q
-  const TA* a = (const TA*)A.a + s * cells;
-  const T* dvg = kPre ? (const T*)A.dinv + s * nodes : in0;
-  const int nc1 = N / 2 + 1;
-  const T* e0 = (MODE == TM_POST) ? (const T*)A.ec + s * (long long)nc1 * nc1 * nc1 : in0;
-  const int ex0 = (x0 - 1) / 2, ey0 = (y0 - 1) / 2;  // coarse tile origin
-  const long long pn = (long long)n1 * n1, pc = (long long)N * N, pe = (long long)nc1 * nc1;
-  T beta = T(0), alpha = T(0);
-  if (kApply && !A.first) beta = (T)A.sc[s].beta;
-  if (MODE == TM_APPLYX || MODE == TM_PREU) alpha = (T)A.sc[s].alpha;  // APPLYX: previous iteration's
-
-  // ---- per-thread staging entries, fixed for the whole march (only the plane offset moves)
-  int noff[MN], deb[MN];
-  unsigned char nflag[MN];  // bit0: entry exists, bit1: inside grid, bit2: interior (x,y), bit3/4: gi/gj odd
+  const int x0 = 1 + TX * blockIdx.x, y0 = 1 + kResTY * blockIdx.y;
+  const long long pn = (long long)n1 * n1, pc = (long long)N * N, nodes = pn * n1;
+  const int kbeg = 1 + chunk * A.zc, kend = min(N - 1, kbeg + A.zc - 1);
+  const float2* xg = A.x + s * nodes;
+  const float* ag = A.a + s * pc * N;
+  int noff[MN], coff[MC];  // offsets in a plane, -1: zero-filled
 #pragma unroll
   for (int j = 0; j < MN; ++j) {
-    const int e = tid + j * NT;
-    const int lx = e % NPX, ly = e / NPX;
-    const int gi = x0 - 1 + lx, gj = y0 - 1 + ly;
-    const bool has = e < NPL, in = has && gi <= N && gj <= N;
-    const bool inter = has && gi > 0 && gj > 0 && gi < N && gj < N;
-    nflag[j] = (has ? 1 : 0) | (in ? 2 : 0) | (inter ? 4 : 0) | ((gi & 1) ? 8 : 0) | ((gj & 1) ? 16 : 0);
-    noff[j] = in ? gi + n1 * gj : 0;
-    deb[j] = ((gi >> 1) - ex0) + EWX * ((gj >> 1) - ey0);
+    const int e = tid + j * NT, gi = x0 - 1 + e % NPX, gj = y0 - 1 + e / NPX;
+    noff[j] = (gi > 0 && gj > 0 && gi < N && gj < N) ? gi + n1 * gj : -1;
   }
-  int coff[MC], cdst[MC];
-  bool cok[MC], chas[MC];
 #pragma unroll
   for (int j = 0; j < MC; ++j) {
-    const int e = tid + j * NT;
-    const int cx = kPairs ? 2 * (e % (CW / 2)) : e % CW;
-    const int cy = kPairs ? e / (CW / 2) : e / CW;
-    const int gi = x0 - 3 + cx, gj = y0 - 2 + cy;
-    chas[j] = e < NCE;
-    cok[j] = chas[j] && gi >= 0 && gj >= 0 && gi + (kPairs ? 1 : 0) < N && gj < N;
-    coff[j] = cok[j] ? gi + N * gj : 0;
-    cdst[j] = cx + CW * cy;
+    const int e = tid + j * NT, gi = x0 - 1 + e % kResCX, gj = y0 - 1 + e / kResCX;
+    coff[j] = (gi < N && gj < N) ? gi + N * gj : -1;
   }
-  int eoff[ME];
-  bool eok[ME], ehas[ME];
-#pragma unroll
-  for (int j = 0; j < ME; ++j) {
-    const int e = tid + j * NT;
-    const int ci = ex0 + e % EWX, cj = ey0 + e / EWX;
-    ehas[j] = (MODE == TM_POST) && e < EPL;
-    eok[j] = ehas[j] && ci > 0 && cj > 0 && ci < nc1 - 1 && cj < nc1 - 1;  // coarse interior
-    eoff[j] = eok[j] ? ci + nc1 * cj : 0;
-  }
-  // POST: coarse plane c is staged once, by issue(2c - 2), and interpolated in x and y
-  // by derive(2c - 2), one fine plane before derive(2c - 1) first reads it (the
-  // barrier after each derive separates the two); the prologue stages and
-  // interpolates the planes of the first derived plane
-  auto stage_coarse = [&](int c) {
-    const bool cok2 = c > 0 && c < nc1 - 1;
-    const T* eb = e0 + (cok2 ? c * pe : 0);  // a plane inside the buffer; invalid entries are zero-filled
-#pragma unroll
-    for (int j = 0; j < ME; ++j) {
-      if (j == ME - 1 && !ehas[j]) continue;
-      cp_async<sizeof(T)>(ecs + (c & (ERING - 1)) * EPL + tid + j * NT, eb + eoff[j], cok2 && eok[j]);
-    }
-  };
-
-  auto issue = [&](int m, int slot) {
-    // every node vector here is zero on the Dirichlet boundary: boundary nodes are
-    // zero-filled like nodes outside the grid, so no buffer's boundary is ever read
-    const bool mok = m > 0 && m < N;
-    // plane bases inside the buffers (plane 0 when m is outside); every staged offset
-    // lies inside a plane, so each source address is valid and the flag alone decides
-    // between a copy and a zero fill
-    const long long mo = mok ? (long long)m * pn : 0;
-    const T* b0 = in0 + mo;
-    const T* b1 = in1 + mo;
-    const T* bd = dvg + mo;
+  auto issue = [&](int m, int slot) {  // node plane m, cell plane m
+    const bool mok = m > 0 && m < N, cok = m < N;
+    const float2* xb = xg + (mok ? m * pn : 0);
+    const float* ab = ag + (cok ? m * pc : 0);
 #pragma unroll
     for (int j = 0; j < MN; ++j) {
-      if (j == MN - 1 && !(nflag[j] & 1)) continue;
       const int e = tid + j * NT;
-      const bool ok = mok && (nflag[j] & 4);
-      cp_async<sizeof(T)>(raw0 + slot * NPL + e, b0 + noff[j], ok);
-      if (stage1) cp_async<sizeof(T)>(raw1 + slot * NPL + e, b1 + noff[j], ok);
-      if (kPre) cp_async<sizeof(T)>(dvs + slot * NPL + e, bd + noff[j], ok);
+      const bool ok = mok && noff[j] >= 0;
+      if (j < MN - 1 || e < kResNP) cp_async<8>(xs + slot * kResNP + e, xb + (ok ? noff[j] : 0), ok);
     }
-    const bool cmok = m >= 0 && m < N;
-    const TA* ab = a + (cmok ? (long long)m * pc : 0);
 #pragma unroll
     for (int j = 0; j < MC; ++j) {
-      if (j == MC - 1 && !chas[j]) continue;
-      cp_async<kPairs ? 4 : sizeof(TA)>(cs + slot * CPL + cdst[j], ab + coff[j], cmok && cok[j]);
+      const int e = tid + j * NT;
+      const bool ok = cok && coff[j] >= 0;
+      if (j < MC - 1 || e < kResCP) cp_async<4>(cs + slot * kResCP + e, ab + (ok ? coff[j] : 0), ok);
     }
-    if (MODE == TM_POST && !(m & 1)) stage_coarse((m >> 1) + 1);
     cp_async_commit();
   };
-
-  // POST: eps[c & 1] holds coarse plane c interpolated bilinearly in x and y at this
-  // tile's staged nodes; a fine plane m takes plane m/2 (m even) or the mean of planes
-  // (m-1)/2 and (m+1)/2 (m odd), so each coarse plane is interpolated once for two
-  // fine planes.  The tile origin is even (x0 - 1 = 32 bx, y0 - 1 = TYT by), so staged
-  // node (2a + p, 2b + q) lies in coarse cell (a, b) of the staged coarse tile: one
-  // work item per coarse cell writes its four nodes (odd index: halfway between two
-  // coarse nodes), every staged entry included.
-  auto interp_xy = [&](int c) {
-    const T* cp = ecs + (c & (ERING - 1)) * EPL;
-    T* ed = eps + (c & 1) * NPL;
-    constexpr int AX = EWX - 1, AY = G::EWYT - 1;  // 17 x (TYT/2 + 1) cells cover 34 x (TYT+2) nodes
-    // items NT.. go to the last threads (their warps stage one entry fewer in derive)
-    static_assert(AX * AY <= 2 * NT, "two rounds at most");
-#pragma unroll
-    for (int rd = 0; rd < 2; ++rd) {
-      const int wi = rd == 0 ? tid : 2 * NT - 1 - tid;
-      if (wi >= AX * AY || (rd == 1 && wi < NT)) continue;
-      const int ca = wi % AX, cb = wi / AX;
-      const T* q = cp + ca + EWX * cb;
-      const T e00 = q[0], e10 = q[1], e01 = q[EWX], e11 = q[EWX + 1];
-      const T r0 = (e00 + e10) * T(0.5), r1 = (e01 + e11) * T(0.5);
-      T* o = ed + 2 * ca + NPX * (2 * cb);
-      o[0] = e00;
-      o[1] = r0;
-      o[NPX] = (e00 + e01) * T(0.5);
-      o[NPX + 1] = (r0 + r1) * T(0.5);
-    }
-  };
-
-  // operand plane m from its staged raw plane (slot: its raw ring slot, r3: its xs slot)
-  auto derive = [&](int m, int slot, int r3) {
-    T* xp = xs + r3 * NPL;
-    const T* r0 = raw0 + slot * NPL;
-    if (kApply) {
-      const T* r1 = raw1 + slot * NPL;
-#pragma unroll
-      for (int j = 0; j < MN; ++j) {
-        if (j == MN - 1 && !(nflag[j] & 1)) continue;
-        const int e = tid + j * NT;
-        xp[e] = A.first ? r0[e] : r0[e] + beta * r1[e];
-      }
-    } else if (MODE == TM_RES64) {
-      // x is already an (hi, lo) pair: copy the 8-byte word
-#pragma unroll
-      for (int j = 0; j < MN; ++j)
-        if (j < MN - 1 || (nflag[j] & 1)) xp[tid + j * NT] = r0[tid + j * NT];
-    } else {
-      const T* dvp = dvs + slot * NPL;
-      const bool mint = m > 0 && m < N;
-      const int dk = m & 1, c0 = m >> 1;
-      // even m: coarse plane m/2 + 1 for the next (odd) plane, into the other eps slot
-      if (MODE == TM_POST && !dk) interp_xy(c0 + 1);
-      const T* e0p = eps + (c0 & 1) * NPL;
-      const T* e1p = eps + ((c0 + 1) & 1) * NPL;
-#pragma unroll
-      for (int j = 0; j < MN; ++j) {
-        if (j == MN - 1 && !(nflag[j] & 1)) continue;
-        const int e = tid + j * NT;
-        // branch-free: D^-1 is 0 on the boundary and zero-filled outside the grid (and
-        // so is r outside 0 < m < N), so only the coarse correction needs a mask
-        const T rn = (MODE == TM_PREU) ? r0[e] - alpha * raw1[slot * NPL + e] : r0[e];
-        T v = rn * dvp[e];
-        if (MODE == TM_POST) {
-          const T mk = (mint && (nflag[j] & 4)) ? T(1) : T(0);
-          v += mk * (dk ? (e0p[e] + e1p[e]) * T(0.5) : e0p[e]);
-        }
-        xp[e] = v;
-      }
-    }
-  };
-
-  // prologue: derive the planes before kbeg, keep two planes in flight
-  const int first_plane = kPre ? kbeg - 2 : kbeg - 1;
-  auto mod5 = [](int m) { return (m + 2 * RING) % RING; };
-  if (MODE == TM_POST) {  // committed with the first issue below
-    stage_coarse(first_plane >> 1);
-    if (first_plane & 1) stage_coarse((first_plane >> 1) + 1);
-  }
-  for (int m = first_plane; m <= kbeg + 2; ++m) issue(m, mod5(m));
-  cp_async_wait<2>();
-  __syncthreads();
-  if (MODE == TM_POST) {
-    interp_xy(first_plane >> 1);
-    if (first_plane & 1) interp_xy((first_plane >> 1) + 1);
-    __syncthreads();
-  }
-  for (int m = first_plane; m <= kbeg; ++m) {
-    derive(m, mod5(m), ring3(m));
-    __syncthreads();
-  }
-
-  // this thread's column: gi, rows gj = y0 + RY*ty + t (t < RY); staged node rows RY*ty + 1 + t
-  T red = T(0);
-  const int gi = x0 + tx;
-  const int gj0 = y0 + RY * ty;
+  for (int m = kbeg - 1; m <= kbeg + 2; ++m) issue(m, m % kResRing);  // planes past N are zero-filled
+  const int gi = x0 + tx, gj0 = y0 + RY * ty;
   const bool colok = gi < N;
-  const int xb = tx + NPX * (RY * ty);        // staged node (tx, RY*ty): top-left of the 3 x (RY+2) window
-  const int cbn = (tx + 2) + CW * (RY * ty + 1);  // staged cell (gi-1, gj0-1)
-  T* out0 = (T*)A.out0 + s * nodes + gi + (long long)n1 * gj0;
-  T* out1 = (kApply || MODE == TM_PREU) ? (T*)A.out1 + s * nodes + gi + (long long)n1 * gj0 : nullptr;
-  T* xio = (MODE == TM_APPLYX) ? (T*)A.x + s * nodes + gi + (long long)n1 * gj0 : nullptr;
-  const T* bptr = (MODE == TM_RES64) ? (const T*)A.in1 + s * A.bstride + gi + (long long)n1 * gj0 : nullptr;
-  float* r32o = (MODE == TM_RES64) ? (float*)A.out0 + s * nodes + gi + (long long)n1 * gj0 : nullptr;
-  float redf = 0.f;  // RES64: r.r of this thread in FP32
+  const int xb = tx + NPX * RY * ty, cbn = tx + kResCX * RY * ty;
+  const float2* bptr = A.b + s * A.bstride + gi + (long long)n1 * gj0;
+  float* r32o = A.r + s * nodes + gi + (long long)n1 * gj0;
+  float redf = 0.f;
   const double scd = 1.0 / (12.0 * N);
   const float sch = (float)scd, scl = (float)(scd - (double)sch);  // h/12 as an FP32 pair
-  // ring slots of plane k, maintained incrementally: s5 in the RING-plane raw/cell
-  // rings, r3 in the three-plane operand ring
-  int s5 = mod5(kbeg), r3 = ring3(kbeg);
+  int sl[3] = {(kbeg - 1) % kResRing, kbeg % kResRing, (kbeg + 1) % kResRing};  // slots of planes k - 1, k, k + 1
   for (int k = kbeg; k <= kend; ++k) {
-    const int s5p1 = s5 + 1 == RING ? 0 : s5 + 1;
-    const int s5p3 = s5 + 3 >= RING ? s5 + 3 - RING : s5 + 3;
-    const int s5m1 = s5 == 0 ? RING - 1 : s5 - 1;
-    const int r3p1 = r3 == 2 ? 0 : r3 + 1;
-    const int r3m1 = r3 == 0 ? 2 : r3 - 1;
-    const int r3s[3] = {r3m1, r3, r3p1};
-    const int c5s[2] = {s5m1, s5};
-    // APPLYX: fetch this plane's x early so the load overlaps the staging below
-    T xv[RY];
-    if (MODE == TM_APPLYX) {
+    float2 bv[RY];
 #pragma unroll
-      for (int t = 0; t < RY; ++t)
-        xv[t] = (colok && gj0 + t < N && !A.xfirst) ? xio[pn * k + n1 * t] : T(0);
-    }
-    issue(k + 3, s5p3);
-    cp_async_wait<2>();
-    __syncthreads();
-    derive(k + 1, s5p1, r3p1);
-    __syncthreads();
-    if constexpr (MODE == TM_RES64) {
-      if (colok) {
-        // b - A x with x = hi + lo (FP32 pairs) and FP32 cells, error-free products and
-        // compensated sums: exact pair sums of cells, exact products, one rounding of the
-        // unevaluated sum (S, comp) per term; the scale h/12 and the subtraction from b are
-        // done in the same pair arithmetic, so no FP64 instruction is executed.
-        float2 X[3][3][RY + 2];
-        float C[2][2][RY + 1];
-#pragma unroll
-        for (int pl = 0; pl < 3; ++pl) {
-          const float2* xp = reinterpret_cast<const float2*>(xs + r3s[pl] * NPL) + xb;
-#pragma unroll
-          for (int c = 0; c < 3; ++c)
-#pragma unroll
-            for (int rr = 0; rr < RY + 2; ++rr) X[pl][c][rr] = xp[c + NPX * rr];
-        }
-#pragma unroll
-        for (int r = 0; r < 2; ++r) {
-          const TA* cp = cs + c5s[r] * CPL + cbn;
-#pragma unroll
-          for (int p = 0; p < 2; ++p)
-#pragma unroll
-            for (int cr = 0; cr < RY + 1; ++cr) C[r][p][cr] = (float)cp[p + CW * cr];
-        }
-#pragma unroll
-        for (int t = 0; t < RY; ++t) {
-          if (gj0 + t >= N) break;
-          F2 pxy[2][2], pxz[2][2], pyz[2][2];
-#pragma unroll
-          for (int u = 0; u < 2; ++u)
-#pragma unroll
-            for (int v = 0; v < 2; ++v) {
-              pxy[v][u] = two_sum(C[0][u][t + v], C[1][u][t + v]);
-              pxz[v][u] = two_sum(C[v][u][t], C[v][u][t + 1]);
-              pyz[v][u] = two_sum(C[v][0][t + u], C[v][1][t + u]);
-            }
-          float S8 = 0.f, E8 = 0.f;
-#pragma unroll
-          for (int v = 0; v < 2; ++v)
-#pragma unroll
-            for (int u = 0; u < 2; ++u) {
-              const F2 q = two_sum(S8, pxy[v][u].h);
-              S8 = q.h;
-              E8 += q.l + pxy[v][u].l;
-            }
-          float S = 0.f, comp = 0.f;
-          df_term<false>(S, comp, F2{4.f * S8, 4.f * E8}, X[1][1][t + 1]);
-#pragma unroll
-          for (int v = 0; v < 2; ++v)
-#pragma unroll
-            for (int u = 0; u < 2; ++u) df_term<true>(S, comp, pxy[v][u], X[1][2 * u][t + 2 * v]);
-#pragma unroll
-          for (int r = 0; r < 2; ++r) {
-            const int pl = 2 * r;
-#pragma unroll
-            for (int u = 0; u < 2; ++u) {
-              df_term<true>(S, comp, pxz[r][u], X[pl][2 * u][t + 1]);
-              df_term<true>(S, comp, pyz[r][u], X[pl][1][t + 2 * u]);
-            }
-#pragma unroll
-            for (int q = 0; q < 2; ++q)
-#pragma unroll
-              for (int p = 0; p < 2; ++p) df_term<true>(S, comp, F2{C[r][p][t + q], 0.f}, X[pl][2 * p][t + 2 * q]);
-          }
-          // ax = (S + comp) (sch + scl), a pair (p, pe)
-          const F2 axs = two_sum(S, comp);
-          const float p = __fmul_rn(axs.h, sch);
-          const float pe = __fmaf_rn(axs.h, scl, __fmaf_rn(axs.l, sch, __fmaf_rn(axs.h, sch, -p)));
-          const long long o = pn * k + n1 * t;
-          const float2 bv = reinterpret_cast<const float2*>(bptr)[o];
-          const F2 d = two_sum(bv.x, -p);
-          const float rv = d.h + (d.l + (bv.y - pe));
-          r32o[o] = rv;  // the inner solve's FP32 residual
-          redf = __fmaf_rn(rv, rv, redf);
-        }
-      }
-    } else if (colok) {
-      // registers: operand window X[plane][col][row] (3 x 3 x (RY+2)), cells C[r][p][row] (2 x 2 x (RY+1))
-      T X[3][3][RY + 2];
-      T C[2][2][RY + 1];
+    for (int t = 0; t < RY; ++t)
+      bv[t] = (colok && gj0 + t < N) ? bptr[pn * k + n1 * t] : make_float2(0.f, 0.f);
+    cp_async_wait<1>();  // plane k + 1 has landed
+    __syncthreads();     // for every thread; plane k - 2 is no longer read
+    issue(k + 3, sl[2] + 2 >= kResRing ? sl[2] + 2 - kResRing : sl[2] + 2);
+    if (colok) {
+      float2 X[3][3][RY + 2];
+      float C[2][2][RY + 1];
 #pragma unroll
       for (int pl = 0; pl < 3; ++pl) {
-        const T* xp = xs + r3s[pl] * NPL + xb;
+        const float2* xp = xs + sl[pl] * kResNP + xb;
 #pragma unroll
         for (int c = 0; c < 3; ++c)
 #pragma unroll
@@ -470,87 +141,73 @@ __global__ void __launch_bounds__(NT) k_tiled(TiledArgs A) {
       }
 #pragma unroll
       for (int r = 0; r < 2; ++r) {
-        const TA* cp = cs + c5s[r] * CPL + cbn;
+        const float* cp = cs + sl[r] * kResCP + cbn;
 #pragma unroll
         for (int p = 0; p < 2; ++p)
 #pragma unroll
-          for (int cr = 0; cr < RY + 1; ++cr) C[r][p][cr] = smem_coef<T>(cp[p + CW * cr]);
+          for (int cr = 0; cr < RY + 1; ++cr) C[r][p][cr] = cp[p + kResCX * cr];
       }
-      const T* rk = raw0 + s5 * NPL + xb + 1 + NPX;
 #pragma unroll
       for (int t = 0; t < RY; ++t) {
         if (gj0 + t >= N) break;
-        // cells of node t: c[r][q][p] = C[r][p][t + q]; neighbour (du, dv) in plane pl: X[pl][1 + du][t + 1 + dv]
-        T pxy[2][2], pxz[2][2], pyz[2][2];
+        F2 pxy[2][2], pxz[2][2], pyz[2][2];
 #pragma unroll
         for (int u = 0; u < 2; ++u)
 #pragma unroll
           for (int v = 0; v < 2; ++v) {
-            pxy[v][u] = C[0][u][t + v] + C[1][u][t + v];   // cells (u, v, 0), (u, v, 1)
-            pxz[v][u] = C[v][u][t] + C[v][u][t + 1];       // cells (u, 0, v), (u, 1, v)
-            pyz[v][u] = C[v][0][t + u] + C[v][1][t + u];   // cells (0, u, v), (1, u, v)
+            pxy[v][u] = two_sum(C[0][u][t + v], C[1][u][t + v]);
+            pxz[v][u] = two_sum(C[v][u][t], C[v][u][t + 1]);
+            pyz[v][u] = two_sum(C[v][0][t + u], C[v][1][t + u]);
           }
-        const T sum8 = (pxy[0][0] + pxy[0][1]) + (pxy[1][0] + pxy[1][1]);
-        // three independent partial sums (centre plane, plane k-1, plane k+1): shorter
-        // dependency chains than one running accumulator
-        T accp[3];
-        accp[1] = T(4) * sum8 * X[1][1][t + 1];
+        float S8 = 0.f, E8 = 0.f;
 #pragma unroll
         for (int v = 0; v < 2; ++v)
 #pragma unroll
-          for (int u = 0; u < 2; ++u) accp[1] -= pxy[v][u] * X[1][2 * u][t + 2 * v];
+          for (int u = 0; u < 2; ++u) {
+            const F2 q = two_sum(S8, pxy[v][u].h);
+            S8 = q.h;
+            E8 += q.l + pxy[v][u].l;
+          }
+        float S = 0.f, comp = 0.f;
+        df_term<false>(S, comp, F2{4.f * S8, 4.f * E8}, X[1][1][t + 1]);
+#pragma unroll
+        for (int v = 0; v < 2; ++v)
+#pragma unroll
+          for (int u = 0; u < 2; ++u) df_term<true>(S, comp, pxy[v][u], X[1][2 * u][t + 2 * v]);
 #pragma unroll
         for (int r = 0; r < 2; ++r) {
-          const int pl = 2 * r;  // plane k-1 (r = 0) or k+1 (r = 1)
-          T a2 = T(0);
+          const int pl = 2 * r;
 #pragma unroll
           for (int u = 0; u < 2; ++u) {
-            a2 -= pxz[r][u] * X[pl][2 * u][t + 1];
-            a2 -= pyz[r][u] * X[pl][1][t + 2 * u];
+            df_term<true>(S, comp, pxz[r][u], X[pl][2 * u][t + 1]);
+            df_term<true>(S, comp, pyz[r][u], X[pl][1][t + 2 * u]);
           }
 #pragma unroll
           for (int q = 0; q < 2; ++q)
 #pragma unroll
-            for (int p = 0; p < 2; ++p) a2 -= C[r][p][t + q] * X[pl][2 * p][t + 2 * q];
-          accp[pl] = a2;
+            for (int p = 0; p < 2; ++p) df_term<true>(S, comp, F2{C[r][p][t + q], 0.f}, X[pl][2 * p][t + 2 * q]);
         }
-        const T ax = scale * (accp[1] + (accp[0] + accp[2]));
+        // ax = (S + comp) (sch + scl), a pair (p, pe)
+        const F2 axs = two_sum(S, comp);
+        const float p = __fmul_rn(axs.h, sch);
+        const float pe = __fmaf_rn(axs.h, scl, __fmaf_rn(axs.l, sch, __fmaf_rn(axs.h, sch, -p)));
         const long long o = pn * k + n1 * t;
-        if (kApply) {
-          const T pv = X[1][1][t + 1];
-          out0[o] = ax;
-          out1[o] = pv;
-          red += pv * ax;
-          if (MODE == TM_APPLYX) xio[o] = xv[t] + alpha * raw1[s5 * NPL + xb + 1 + NPX * (t + 1)];  // xv = 0 when A.xfirst
-        } else if (MODE == TM_PRE) {
-          out0[o] = rk[NPX * t] - ax;
-        } else if (MODE == TM_PREU) {
-          const T rn = rk[NPX * t] - alpha * raw1[s5 * NPL + xb + 1 + NPX * (t + 1)];
-          out0[o] = rn - ax;
-          out1[o] = rn;
-        } else if (MODE == TM_POST) {
-          const T rv = rk[NPX * t];
-          const T dk = dvs[s5 * NPL + xb + 1 + NPX * (t + 1)];
-          const T zv = X[1][1][t + 1] + (rv - ax) * dk;
-          out0[o] = zv;
-          red += rv * zv;
-        }
+        const F2 d = two_sum(bv[t].x, -p);
+        const float rv = d.h + (d.l + (bv[t].y - pe));
+        r32o[o] = rv;  // the inner solve's FP32 residual
+        redf = __fmaf_rn(rv, rv, redf);
       }
     }
-    if (MODE != TM_PRE && MODE != TM_PREU && (k == kend || (k - 1) % kZSeg == kZSeg - 1)) {
-      // end of a partial-sum segment (block-uniform condition)
-      const T b = block_sum(MODE == TM_RES64 ? (T)redf : red);
-      if (tid == 0) {
-        const int per = gridDim.x * gridDim.y * A.nseg;
-        const int bid = (((k - 1) / kZSeg) * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
-        A.partial[(long long)s * per + bid] = (double)b;
-      }
-      red = T(0);
+    if (k == kend || (k - 1) % kZSeg == kZSeg - 1) {  // end of a partial-sum segment (block-uniform)
+      const double b = block_sum((double)redf);
+      if (tid == 0)
+        A.partial[(long long)s * (gridDim.x * gridDim.y * A.nseg) +
+                  (((k - 1) / kZSeg) * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x] = b;
       redf = 0.f;
     }
-    __syncthreads();
-    s5 = s5p1;
-    r3 = r3p1;
+    sl[0] = sl[1];
+    sl[1] = sl[2];
+    sl[2] = sl[2] == kResRing - 1 ? 0 : sl[2] + 1;
   }
   cp_async_wait<0>();
 }
@@ -744,122 +401,65 @@ TiledShape tiled_shape(int N, int S, int ry, int zchunks) {
   return t;
 }
 
-// The tile shape follows the batch size bt.S (not the number of samples launched),
-// so a sample's partial sums, and with them its iterates, do not depend on how many
-// other samples are still active.
-template <typename T, typename TA, int MODE>
-static void run_tiled(const char* cls, double bytes, TiledArgs args, const Batch& bt, cudaStream_t st,
-                      double ops = 0.0) {
-  const TiledShape t = tiled_shape(args.N, bt.S, RowsPerThread<T>::value, bt.zchunks);
-  args.nzc = t.nzc;
-  args.zc = t.zc;
-  args.nseg = t.nseg;
-  args.act = bt.act;
-  const size_t smem = TiledSmem<T, TA, MODE>::total;  // up to ~91 KB (FP64): opt in above 48 KB
-  static bool smem_set = false;  // once per instantiation (capture-friendly)
-  if (smem > 48 * 1024 && !smem_set) {
-    cudaFuncSetAttribute(k_tiled<T, TA, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    smem_set = true;
-  }
-  launch_flops(cls, bytes, ops, k_tiled<T, TA, MODE>, dim3(t.bx, t.by, (unsigned)(bt.n * t.nzc)), dim3(TX, TY), smem,
-               st, args);
-}
-
-template <typename T, typename TA>
 static double vbytes(int N, int S, double vec, double coef) {
-  return (double)S * (vec * (double)nodes_of(N) * sizeof(T) + coef * (double)cells_of(N) * sizeof(TA));
-}
-
-template <typename T> const char* tag();
-template <> const char* tag<double>() { return "f64"; }
-template <> const char* tag<float>() { return "f32"; }
-static const char* name(const char* base, const char* t) {
-  static thread_local char buf[64];
-  snprintf(buf, sizeof(buf), "%s_%s", base, t);
-  return buf;
+  return (double)S * (vec * (double)nodes_of(N) * 4 + coef * (double)cells_of(N) * 4);
 }
 
 // p is double-buffered: neighbouring tiles read the old p in their halos while
 // this tile writes the new one.
 // FP32 vectors on 32^3 and 64^3 grids go to the whole-row slab passes (slab.cu)
-template <typename T, typename TA>
-void tiled_apply(const T* z, const T* pold, T* pnew, const TA* a, T* q, double* partial, const SolveScalars* sc, int N,
-                 const Batch& bt, int first, cudaStream_t st) {
-  if constexpr (std::is_same<T, float>::value && std::is_same<TA, float>::value) {
-    if (bt.stencil == 0 && slab_supported(N)) {
-      slab_apply(z, pold, pnew, a, q, nullptr, partial, sc, N, bt, first != 0, false, false, st);
-    } else {
-      tile32_apply(z, pold, pnew, a, q, nullptr, partial, sc, N, bt, first != 0, false, st);
-    }
-    return;
-  } else {
-  TiledArgs A{};
-  A.in0 = z; A.in1 = pold; A.a = a; A.out0 = q; A.out1 = pnew; A.partial = partial; A.sc = sc; A.N = N;
-  A.first = first;
-  run_tiled<T, TA, TM_APPLY>("apply_f64", vbytes<T, TA>(N, bt.n, first ? 3 : 4, 1), A, bt, st);
-  }
+static bool slab_pass(int N, const Batch& bt) { return bt.stencil == 0 && slab_supported(N); }
+void tiled_apply(const float* z, const float* pold, float* pnew, const float* a, float* q, double* partial,
+                 const SolveScalars* sc, int N, const Batch& bt, int first, cudaStream_t st) {
+  if (slab_pass(N, bt)) slab_apply(z, pold, pnew, a, q, nullptr, partial, sc, N, bt, first != 0, false, false, st);
+  else tile32_apply(z, pold, pnew, a, q, nullptr, partial, sc, N, bt, first != 0, false, st);
 }
-// fused variants of the mixed inner solve (see TM_PREU / TM_APPLYX)
+// fused variants of the mixed inner solve: x += alpha_prev p_old, and PREU
 void tiled_apply_x(const float* z, const float* pold, float* pnew, const float* a, float* q, float* x, double* partial,
                    const SolveScalars* sc, int N, const Batch& bt, cudaStream_t st, bool x_first) {
-  if (bt.stencil == 0 && slab_supported(N)) {
-    slab_apply(z, pold, pnew, a, q, x, partial, sc, N, bt, false, true, x_first, st);
-    return;
-  }
-  tile32_apply(z, pold, pnew, a, q, x, partial, sc, N, bt, false, x_first, st);
+  if (slab_pass(N, bt)) slab_apply(z, pold, pnew, a, q, x, partial, sc, N, bt, false, true, x_first, st);
+  else tile32_apply(z, pold, pnew, a, q, x, partial, sc, N, bt, false, x_first, st);
 }
 bool tiled_pre_update(const float* r, const float* q, const __nv_bfloat16* a, const float* dinv, float* t,
                       float* rnew, float* rc, const SolveScalars* sc, int N, const Batch& bt, cudaStream_t st) {
-  if (bt.stencil == 0 && slab_supported(N)) {
+  if (slab_pass(N, bt)) {
     slab_pre<__nv_bfloat16>(r, q, a, dinv, rnew, rc, sc, N, bt, st);
     return true;
   }
   tile32_pre<__nv_bfloat16>(r, q, a, dinv, t, rnew, sc, N, bt, st);
   return false;
 }
-
-template <typename T, typename TA>
-bool tiled_pre(const T* r, const TA* a, const T* dinv, T* t, T* rc, const SolveScalars* sc, int N, const Batch& bt,
-               cudaStream_t st) {
-  if constexpr (std::is_same<T, float>::value) {
-    if (bt.stencil == 0 && slab_supported(N)) {
-      slab_pre<TA>(r, nullptr, a, dinv, nullptr, rc, sc, N, bt, st);
-      return true;
-    }
-    tile32_pre<TA>(r, nullptr, a, dinv, t, nullptr, sc, N, bt, st);
-  } else {
-  TiledArgs A{};
-  A.in0 = r; A.a = a; A.dinv = dinv; A.out0 = t; A.sc = sc; A.N = N;
-  run_tiled<T, TA, TM_PRE>("pre_f64", vbytes<T, TA>(N, bt.n, 3, 1), A, bt, st);
+template <typename TA>
+bool tiled_pre(const float* r, const TA* a, const float* dinv, float* t, float* rc, const SolveScalars* sc, int N,
+               const Batch& bt, cudaStream_t st) {
+  if (slab_pass(N, bt)) {
+    slab_pre<TA>(r, nullptr, a, dinv, nullptr, rc, sc, N, bt, st);
+    return true;
   }
+  tile32_pre<TA>(r, nullptr, a, dinv, t, nullptr, sc, N, bt, st);
   return false;
 }
-template <typename T, typename TA>
-void tiled_post(const T* r, const TA* a, const T* dinv, const T* ec, T* z, double* partial, const SolveScalars* sc,
-                int N, const Batch& bt, cudaStream_t st) {
-  if constexpr (std::is_same<T, float>::value) {
-    if (bt.stencil == 0 && slab_supported(N)) {
-      slab_post<TA>(r, a, dinv, ec, z, partial, sc, N, bt, st);
-    } else {
-      tile32_post<TA>(r, a, dinv, ec, z, partial, sc, N, bt, st);
-    }
-  } else {
-  TiledArgs A{};
-  A.in0 = r; A.a = a; A.dinv = dinv; A.ec = ec; A.out0 = z; A.partial = partial; A.sc = sc; A.N = N;
-  run_tiled<T, TA, TM_POST>("post_f64", vbytes<T, TA>(N, bt.n, 3, 1) + vbytes<T, T>(N / 2, bt.n, 1, 0), A, bt, st);
-  }
+template <typename TA>
+void tiled_post(const float* r, const TA* a, const float* dinv, const float* ec, float* z, double* partial,
+                const SolveScalars* sc, int N, const Batch& bt, cudaStream_t st) {
+  if (slab_pass(N, bt)) slab_post<TA>(r, a, dinv, ec, z, partial, sc, N, bt, st);
+  else tile32_post<TA>(r, a, dinv, ec, z, partial, sc, N, bt, st);
 }
+
+// The tile shape follows the batch size bt.S (not the number of samples launched); the
+// partial sums do not depend on it.
 void tiled_res64(const float2* b, long long bstride, const float2* x, const float* a, float* r32, double* partial,
                  const SolveScalars* sc, int N, const Batch& bt, cudaStream_t st) {
-  TiledArgs A{};
-  A.in0 = x; A.in1 = b; A.bstride = bstride; A.a = a; A.out0 = r32; A.partial = partial; A.sc = sc; A.N = N;
+  const TiledShape t = tiled_shape(N, bt.S, kResRows, bt.zchunks);
+  const ResArgs A{x, b, a, r32, partial, sc, bt.act, bstride, N, t.nzc, t.zc, t.nseg};
   const double bb = (double)(bstride ? bt.n : 1) * nodes_of(N) * 8;
   // FP32 operations per interior node as written (no sharing between nodes): 12 exact
   // cell-pair sums (6 each), the 8-cell sum (28), 21 compensated product terms (12
   // each), the scaling, the subtraction from b and r.r (20)
   const double ops = (double)bt.n * (N - 1) * (N - 1) * (N - 1) * kRes64OpsPerNode;
-  run_tiled<double, float, TM_RES64>("resid64", bb + vbytes<double, float>(N, bt.n, 1, 1) + (double)bt.n * nodes_of(N) * 4,
-                                     A, bt, st, ops);
+  static_assert(kResSmem <= 48 * 1024, "no opt-in");
+  launch_flops("resid64", bb + vbytes(N, bt.n, 3, 1), ops, k_res64, dim3(t.bx, t.by, (unsigned)(bt.n * t.nzc)),
+               dim3(TX, TY), kResSmem, st, A);
 }
 
 int tiled_phi_df(const float2* y, int N, int S, const float2* gtab, const float2* mgtab, float2* badj,
@@ -883,28 +483,18 @@ int tiled_phi(const double* y, int N, int S, const double* gtab, const double* m
   return t.blocks_per_sample;
 }
 
-template void tiled_apply<float, float>(const float*, const float*, float*, const float*, float*, double*,
-                                        const SolveScalars*, int, const Batch&, int, cudaStream_t);
-template void tiled_apply<double, double>(const double*, const double*, double*, const double*, double*, double*,
-                                          const SolveScalars*, int, const Batch&, int, cudaStream_t);
-template bool tiled_pre<float, __nv_bfloat16>(const float*, const __nv_bfloat16*, const float*, float*, float*,
-                                              const SolveScalars*, int, const Batch&, cudaStream_t);
-template bool tiled_pre<float, float>(const float*, const float*, const float*, float*, float*, const SolveScalars*,
-                                      int, const Batch&, cudaStream_t);
-template void tiled_post<float, float>(const float*, const float*, const float*, const float*, float*, double*,
+template bool tiled_pre<__nv_bfloat16>(const float*, const __nv_bfloat16*, const float*, float*, float*,
                                        const SolveScalars*, int, const Batch&, cudaStream_t);
-template bool tiled_pre<double, double>(const double*, const double*, const double*, double*, double*,
+template bool tiled_pre<float>(const float*, const float*, const float*, float*, float*, const SolveScalars*, int,
+                               const Batch&, cudaStream_t);
+template void tiled_post<__nv_bfloat16>(const float*, const __nv_bfloat16*, const float*, const float*, float*, double*,
                                         const SolveScalars*, int, const Batch&, cudaStream_t);
-template void tiled_post<float, __nv_bfloat16>(const float*, const __nv_bfloat16*, const float*, const float*, float*,
-                                               double*, const SolveScalars*, int, const Batch&, cudaStream_t);
-template void tiled_post<double, double>(const double*, const double*, const double*, const double*, double*, double*,
-                                         const SolveScalars*, int, const Batch&, cudaStream_t);
+template void tiled_post<float>(const float*, const float*, const float*, const float*, float*, double*,
+                                const SolveScalars*, int, const Batch&, cudaStream_t);
 
-}  // namespace mlsgd
-
-namespace mlsgd {
-int tiled_blocks_per_sample(int N, int S, int elem, bool slab) {
-  if (elem == 4 && slab && slab_supported(N)) return slab_shape(N, S).blocks_per_sample;
-  return tiled_shape(N, S, elem == 8 ? RowsPerThread<double>::value : RowsPerThread<float>::value).blocks_per_sample;
+int tiled_blocks_per_sample(int N, int S, bool slab) {
+  return slab && slab_supported(N) ? slab_shape(N, S).blocks_per_sample : tiled_shape(N, S, 4).blocks_per_sample;
 }
+int res64_blocks_per_sample(int N, int S) { return tiled_shape(N, S, kResRows).blocks_per_sample; }
+
 }  // namespace mlsgd
