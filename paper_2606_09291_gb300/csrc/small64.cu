@@ -19,12 +19,17 @@
 //   x2 = w r + P e:            z = x2 + w (r - A x2) = (1 - omega) x2 + w (r + Off x2)
 //   q = D p - Off p
 // about 83 operations per node and iteration, of which the level-by-level kernels took
-// some 140.  The levels 4^3 and 2^3 are one warp's work in every block.
-// What is left is latency: barriers, dependent FMAs and the scalars' divisions.
+// some 140.  The levels 4^3 and 2^3 are one 27 x 27 matrix per sample, formed once.
+// What is left is latency: a warp alone issues one FP64 operation in 64 clocks, so every
+// step's length is the operations of its busiest warp, and three to four cluster barriers.
 // Measured: state and adjoint solves of 4 samples of 8^3 at rtol 1e-12 2.92 ms in passes,
-// 0.57 ms now; 16 samples of 16^3 with their 8^3 partners at 1e-10 10.1 -> 2.1 ms; with the
-// V-cycle below 32^3 9 samples of 64^3 and partners 36.2 -> 29.2 ms.
+// 0.54 ms with the coarse levels run step by step, two nodes per thread and clusters packed
+// onto SMs, 0.32 ms now; 64 samples 3.85, 0.68, 0.44; 16 samples of 16^3 with their 8^3
+// partners at 1e-10 10.1, 1.78, 1.45 ms.
 #include <cooperative_groups.h>
+
+#include <algorithm>
+#include <mutex>
 
 #include "internal.cuh"
 #include "kernels.h"
@@ -40,7 +45,8 @@ template <int N>
 struct Cfg {
   static constexpr int C = N / 2;               // blocks per sample (planes 2c + 1, 2c + 2)
   static constexpr int M = N - 1;               // interior nodes per side
-  static constexpr int NT = N == 16 ? 256 : 64;  // threads: M^2 columns
+  static constexpr int U = N == 16 ? 2 : 1;      // own nodes per thread: both planes of a column, or one
+  static constexpr int NT = N == 16 ? 256 : 128;  // threads: M^2 columns (8^3: for each of the two planes)
   static constexpr int n1 = N + 1, PL = n1 * n1, CP = N * N;
 };
 
@@ -50,7 +56,8 @@ struct Smem {
   using K = Cfg<N>;
   double r[4 * K::PL], op[4 * K::PL], wd[4 * K::PL];
   double c[3 * K::CP], fxy[2 * K::CP], fxz[3 * K::CP], fyz[3 * K::CP];  // scaled cells, face sums
-  double t8[729], x4[125], t4[125], z4[125], a4[64], wd4[125], a2[8];
+  double t8[729], z4[125], a4[64], wd4[125], a2[8];
+  double g4[27 * 27], inv4, part4[4 * 27];  // the V-cycle from 4^3 down as a matrix (coarse4_setup)
   double red[K::NT];
   double slot[3][K::C];  // partial sums of the blocks: r.r, r.z, p.q
   double bc;             // alpha or beta
@@ -65,8 +72,9 @@ template <int N, typename B>
 struct With8 : B {};
 template <typename B>
 struct With8<16, B> : B {  // the 8^3 level below a 16^3 one
-  double t[2 * 289];
-  double r8a[729], r8b[729], x8[729], wd8[729], a8[512];
+  double r8a[729], wd8[729], a8[512];
+  union { double r8b[729], x8[729]; };  // x8 once r8b has been added to r8a
+  double fxy8[3 * 64], fxz8[4 * 64], fyz8[4 * 64];  // face sums of the cell layers rank - 1 .. rank + 2
 };
 
 // Off x at an interior node: xq = &x[node], cq = &cells[lowest cell]; F: face sums
@@ -153,49 +161,97 @@ __device__ __forceinline__ double restrict27(const double* f) {
   return fma(0.5, a[0] + a[2], a[1]);
 }
 
-// levels 4^3 and 2^3 by warp 0 of every block: restricts M.t8, leaves the correction in M.z4
+// The V(1,1)-cycle from 4^3 down is a fixed linear map of the restricted residual r: with
+// w = omega/D, p the interpolation of the 2^3 node to 4^3 (and its transpose the
+// restriction), d the 2^3 diagonal and u = (1 - omega) p + w Off p,
+//   z4 = w ((2 - omega) r + Off (w r)) + u (u . r) / d = G r,
+// so the 27 x 27 matrix G is formed once and every cycle is one product with it: run step
+// by step the level took a third of an 8^3 iteration (11070 of 33800 clocks: 170
+// operations in a row in one warp, which alone issues one FP64 operation in 64 clocks).
+// a4 holds h/12 a of the 4^3 cells, wd4 omega/D, a2 the 2^3 cells; z4 is 0 on entry.
 template <typename SM>
-__device__ __forceinline__ void coarse4(SM& M, double omega) {
-  const int lane = threadIdx.x;
-  const int I = 1 + lane % 3, J = 1 + (lane / 3) % 3, K = 1 + lane / 9;
-  const int n = I + 5 * (J + 5 * K), c = (I - 1) + 4 * ((J - 1) + 4 * (K - 1));
-  const bool own = lane < 27;
-  double r = 0.0, w = 0.0, x = 0.0;
-  if (own) {
-    r = restrict27<9, 81>(M.t8 + 2 * I + 18 * J + 162 * K);
-    w = M.wd4[n];
-    x = w * r;
-    M.x4[n] = x;
-  }
-  __syncwarp();
-  if (own) M.t4[n] = off_cells<4>((1.0 - omega) * r, M.x4 + n, M.a4 + c);
-  __syncwarp();
-  const double r2 = restrict27<5, 25>(M.t4 + 62);
-  double s8 = 0.0;
+__device__ void coarse4_setup(SM& M, double omega, int nt) {
+  const int tid = threadIdx.x;
+  const int I = 1 + tid % 3, J = 1 + (tid / 3) % 3, K = 1 + tid / 9, n = I + 5 * (J + 5 * K);
+  const double p = ((I & 1) ? 0.5 : 1.0) * ((J & 1) ? 0.5 : 1.0) * ((K & 1) ? 0.5 : 1.0);
+  if (tid < 27) M.z4[n] = p;
+  if (tid == 32) {
+    double s8 = 0.0;
 #pragma unroll
-  for (int e = 0; e < 8; ++e) s8 += M.a2[e];
-  const double e2 = r2 / ((1.0 / 6.0) * s8);
-  if (own) {
-    x = fma(((I & 1) ? 0.5 : 1.0) * ((J & 1) ? 0.5 : 1.0) * ((K & 1) ? 0.5 : 1.0), e2, x);
-    M.x4[n] = x;
+    for (int e = 0; e < 8; ++e) s8 += M.a2[e];
+    M.inv4 = 6.0 / s8;
   }
-  __syncwarp();
-  if (own) M.z4[n] = fma(w, off_cells<4>(r, M.x4 + n, M.a4 + c), (1.0 - omega) * x);
+  __syncthreads();
+  if (tid < 27)
+    M.part4[tid] = fma(M.wd4[n], off_cells<4>(0.0, M.z4 + n, M.a4 + (I - 1) + 4 * ((J - 1) + 4 * (K - 1))), (1.0 - omega) * p);
+  __syncthreads();
+  for (int e = tid; e < 27 * 27; e += nt) {  // G[j][i]: a lane takes a row i
+    const int i = e % 27, j = e / 27;
+    const int xi = 1 + i % 3, yi = 1 + (i / 3) % 3, zi = 1 + i / 9;
+    const int du = 1 + j % 3 - xi, dv = 1 + (j / 3) % 3 - yi, dw = 1 + j / 9 - zi;
+    const double wi = M.wd4[xi + 5 * (yi + 5 * zi)], wj = M.wd4[(xi + du) + 5 * ((yi + dv) + 5 * (zi + dw))];
+    double g = M.part4[i] * (M.part4[j] * M.inv4);
+    if (i == j) g = fma(wi, 2.0 - omega, g);
+    const int zeros = (du == 0) + (dv == 0) + (dw == 0);
+    if (zeros <= 1 && abs(du) <= 1 && abs(dv) <= 1 && abs(dw) <= 1) {  // neighbours across a face or body diagonal
+      const int c0 = (du > 0 ? xi : xi - 1) + 4 * ((dv > 0 ? yi : yi - 1) + 4 * (dw > 0 ? zi : zi - 1));
+      double a = M.a4[c0];
+      if (zeros) a += M.a4[c0 + (du == 0 ? 1 : dv == 0 ? 4 : 16)];
+      g = fma(wi * a, wj, g);
+    }
+    M.g4[e] = g;
+  }
+}
+// restricts M.t8, leaves the correction in M.z4 (complete after the next block barrier);
+// called by every thread.  Four warps (one per quarter of the SM) share the sums.
+template <typename SM>
+__device__ __forceinline__ void coarse4(SM& M) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int I = 1 + lane % 3, J = 1 + (lane / 3) % 3, K = 1 + lane / 9;
+  const bool own = lane < 27;
+  if (own && w < 3) {  // the restriction's three planes
+    const double* f = M.t8 + 2 * I + 18 * J + 81 * (2 * K + w - 1);
+    double v = 0.0;
+#pragma unroll
+    for (int u = -1; u <= 1; ++u) {
+      const double* q = f + 9 * u;
+      v = fma(u == 0 ? 1.0 : 0.5, fma(0.5, q[-1] + q[1], q[0]), v);
+    }
+    M.part4[27 * w + lane] = v;
+  }
+  __syncthreads();
+  double z = 0.0;
+  if (w < 4) {  // columns 7 w .. 7 w + 6 of G
+    const double r = own ? fma(0.5, M.part4[lane] + M.part4[54 + lane], M.part4[27 + lane]) : 0.0;
+    const double* g = M.g4 + 7 * 27 * w + (own ? lane : 0);
+#pragma unroll
+    for (int jj = 0; jj < 7; ++jj) {
+      const double rj = __shfl_sync(0xffffffffu, r, (7 * w + jj) & 31);
+      if (7 * w + jj < 27) z = fma(g[27 * jj], rj, z);
+    }
+  }
+  __syncthreads();
+  if (own && w < 4) M.part4[27 * w + lane] = z;
+  __syncthreads();
+  if (own && w == 0)
+    M.z4[I + 5 * (J + 5 * K)] = (M.part4[lane] + M.part4[27 + lane]) + (M.part4[54 + lane] + M.part4[81 + lane]);
 }
 
-// One V(1,1)-cycle on M.r (own and halo planes): z of the own column's two nodes.
+// One V(1,1)-cycle on M.r (own and halo planes): z of the thread's own nodes, planes
+// 2 rank + 1 + u0 + (0 .. U - 1) of its column.
 // after_t runs between the barrier that publishes the restricted residual and the rest
 // (false: the cluster stops here).
 template <int N, typename SM, typename F>
 __device__ __forceinline__ bool vcycle(SM& M, cg::cluster_group& cl, int rank, bool col, int i, int j, double omega,
-                                       double z[2], F&& after_t) {
+                                       int u0, double (&z)[Cfg<N>::U], F&& after_t) {
   using K = Cfg<N>;
-  constexpr int S1 = K::n1, S2 = K::PL, C = K::C;
+  constexpr int S1 = K::n1, S2 = K::PL, C = K::C, U = K::U;
   const int tid = threadIdx.x, nb = i + S1 * j, cb = (i - 1) + N * (j - 1);
   const double om1 = 1.0 - omega;
+  const int l0 = 2 * u0;  // the thread's staged planes l0 .. l0 + 2 U - 1
   if (col) {
 #pragma unroll
-    for (int l = 0; l < 4; ++l) M.op[l * S2 + nb] = M.r[l * S2 + nb] * M.wd[l * S2 + nb];
+    for (int l = l0; l < l0 + 2 * U; ++l) M.op[l * S2 + nb] = M.r[l * S2 + nb] * M.wd[l * S2 + nb];
   }
   __syncthreads();
   auto off = [&](double acc, const double* v, int u) {  // node plane 2 rank + 1 + u
@@ -203,21 +259,22 @@ __device__ __forceinline__ bool vcycle(SM& M, cg::cluster_group& cl, int rank, b
                               M.fxz + u * K::CP + (i - 1) + N * j, M.fyz + u * K::CP + i + N * (j - 1));
   };
   const int nown = 2 * rank + 2 < N ? 2 : 1;  // the last block's second plane is the boundary
-  double t[2] = {0.0, 0.0};
+  double t[U] = {};
   if (col) {
 #pragma unroll
-    for (int u = 0; u < 2; ++u)
-      if (u < nown) t[u] = off(om1 * M.r[(u + 1) * S2 + nb], M.op, u);
+    for (int v = 0; v < U; ++v)
+      if (u0 + v < nown) t[v] = off(om1 * M.r[(u0 + v + 1) * S2 + nb], M.op, u0 + v);
   }
   if constexpr (N == 16) {
+    __syncthreads();  // op has been read: t takes its first two planes
     if (col) {
-      M.t[nb] = t[0];
-      M.t[S2 + nb] = t[1];
+      M.op[nb] = t[0];
+      M.op[S2 + nb] = t[U - 1];
     }
     __syncthreads();
     if (tid < 49) {  // coarse planes rank + 1 (planes 2 rank + 1, 2 rank + 2) and rank (half of plane 2 rank + 1)
       const int I = 1 + tid % 7, J = 1 + tid / 7;
-      const double* f = M.t + 2 * I + 17 * (2 * J);
+      const double* f = M.op + 2 * I + 17 * (2 * J);
       double a[3], b[3];
 #pragma unroll
       for (int u = -1; u <= 1; ++u) {
@@ -235,14 +292,20 @@ __device__ __forceinline__ bool vcycle(SM& M, cg::cluster_group& cl, int rank, b
       }
     }
   } else {
-    if (col) {
-      for (int q = 0; q < C; ++q) {
-        SM* R = cl.map_shared_rank(&M, q);
-        R->t8[nb + 81 * (2 * rank + 1)] = t[0];
-        if (nown == 2) R->t8[nb + 81 * (2 * rank + 2)] = t[1];
-      }
+    if (col && u0 < nown) {
+      for (int q = 0; q < C; ++q) cl.map_shared_rank(&M, q)->t8[nb + 81 * (2 * rank + 1 + u0)] = t[0];
     }
   }
+  // Off x8 at node (a, b, k) of the 8^3 level, k = rank .. rank + 2
+  auto off8 = [&](double acc, int a, int b, int k) {
+    if constexpr (N == 16) {
+      const int l = k - rank;
+      return off_row<9, 81, 8>(acc, M.x8 + a + 9 * b + 81 * k, M.a8 + (a - 1) + 8 * (b - 1) + 64 * (k - 1),
+                               M.fxy8 + 64 * l + (a - 1) + 8 * (b - 1), M.fxz8 + 64 * l + (a - 1) + 8 * b,
+                               M.fyz8 + 64 * l + a + 8 * (b - 1));
+    }
+    return acc;
+  };
   cl.sync();
   if (!after_t()) return false;
   if constexpr (N == 16) {
@@ -255,12 +318,12 @@ __device__ __forceinline__ bool vcycle(SM& M, cg::cluster_group& cl, int rank, b
     const int kt = rank + 1;  // the block's plane of the 8^3 residual
     if (kt < 8 && tid < 49) {
       const int a = 1 + tid % 7, b = 1 + tid / 7, n = a + 9 * b + 81 * kt;
-      const double v = off_cells<8>(om1 * M.r8a[n], M.x8 + n, M.a8 + (a - 1) + 8 * (b - 1) + 64 * (kt - 1));
+      const double v = off8(om1 * M.r8a[n], a, b, kt);
       for (int q = 0; q < C; ++q) cl.map_shared_rank(&M, q)->t8[n] = v;
     }
     cl.sync();
   }
-  if (tid < 32) coarse4(M, omega);
+  coarse4(M);
   __syncthreads();
   if constexpr (N == 16) {
     // corrected x8 on the planes the stencils of planes rank .. rank + 2 read, then z8 there
@@ -273,32 +336,45 @@ __device__ __forceinline__ bool vcycle(SM& M, cg::cluster_group& cl, int rank, b
     const int q0 = rank > 0 ? rank : 1, q1 = rank + 2 < 7 ? rank + 2 : 7;
     for (int e = tid; e < 49 * (q1 - q0 + 1); e += K::NT) {
       const int a = 1 + e % 7, b = 1 + (e / 7) % 7, k = q0 + e / 49, n = a + 9 * b + 81 * k;
-      const double s = off_cells<8>(M.r8a[n], M.x8 + n, M.a8 + (a - 1) + 8 * (b - 1) + 64 * (k - 1));
-      M.t8[n] = fma(M.wd8[n], s, om1 * M.x8[n]);
+      M.t8[n] = fma(M.wd8[n], off8(M.r8a[n], a, b, k), om1 * M.x8[n]);
     }
     __syncthreads();
   }
-  double x2[4];
+  double x2[2 * U];
   if (col) {
+    // staged plane l is node plane 2 rank + l: an even l takes coarse plane rank + l/2, an odd
+    // one the mean of it and the next; the sums over x and y are shared, weights come last
+    const double* e = N == 16 ? M.t8 : M.z4;
+    constexpr int E1 = N / 2 + 1, E2 = E1 * E1;
+    auto face = [&](int kc) {
+      if (kc > N / 2) return 0.0;
+      const double* q = e + (i >> 1) + E1 * (j >> 1) + E2 * kc;
+      double v = q[0];
+      if (i & 1) v += q[1];
+      if (j & 1) v += (i & 1) ? q[E1] + q[E1 + 1] : q[E1];
+      return v;
+    };
+    const double wf = ((i & 1) ? 0.5 : 1.0) * ((j & 1) ? 0.5 : 1.0);
+    double f = face(rank + u0);
 #pragma unroll
-    for (int l = 0; l < 4; ++l) {
-      const int k = 2 * rank + l;
-      double e = 0.0;
-      if (k > 0 && k < N) {
-        if constexpr (N == 16) e = interp<9, 81>(M.t8, i, j, k);
-        else e = interp<5, 25>(M.z4, i, j, k);
-      }
-      x2[l] = fma(M.wd[l * S2 + nb], M.r[l * S2 + nb], e);
-      M.op[l * S2 + nb] = x2[l];
+    for (int h = 0; h < U; ++h) {
+      const int l = l0 + 2 * h;
+      const double fn = face(rank + u0 + h + 1);
+      x2[2 * h] = fma(wf, f, M.wd[l * S2 + nb] * M.r[l * S2 + nb]);
+      x2[2 * h + 1] = fma(0.5 * wf, f + fn, M.wd[(l + 1) * S2 + nb] * M.r[(l + 1) * S2 + nb]);
+      if (2 * rank + l + 1 > N) x2[2 * h + 1] = 0.0;
+      M.op[l * S2 + nb] = x2[2 * h];
+      M.op[(l + 1) * S2 + nb] = x2[2 * h + 1];
+      f = fn;
     }
   }
   __syncthreads();
-  z[0] = z[1] = 0.0;
-  if (col) {
 #pragma unroll
-    for (int u = 0; u < 2; ++u)
-      if (u < nown)
-        z[u] = fma(M.wd[(u + 1) * S2 + nb], off(M.r[(u + 1) * S2 + nb], M.op, u), om1 * x2[u + 1]);
+  for (int v = 0; v < U; ++v) {
+    z[v] = 0.0;
+    const int l = u0 + v + 1;
+    if (col && u0 + v < nown)
+      z[v] = fma(M.wd[l * S2 + nb], off(M.r[l * S2 + nb], M.op, u0 + v), om1 * x2[l - l0]);
   }
   return true;
 }
@@ -319,6 +395,18 @@ __device__ void load_cells(SM& M, const double* a, int rank) {
     if (e < 2 * K::CP) M.fxy[e] = M.c[e] + M.c[e + K::CP];
     M.fxz[e] = j > 0 ? M.c[e - N] + M.c[e] : 0.0;
     M.fyz[e] = i > 0 ? M.c[e - 1] + M.c[e] : 0.0;
+  }
+}
+// face sums of the 8^3 level around planes rank .. rank + 2 from M.a8 (scaled)
+template <typename SM>
+__device__ void faces8(SM& M, int rank) {
+  for (int e = threadIdx.x; e < 4 * 64; e += 256) {
+    const int L = rank - 1 + e / 64, q = e & 63, i = q & 7, j = q >> 3;  // cell layer L at local layer e / 64
+    const bool in = L >= 0 && L < 8;
+    const double* c = M.a8 + 64 * (in ? L : 0) + q;
+    M.fxz8[e] = in && j > 0 ? c[-8] + c[0] : 0.0;
+    M.fyz8[e] = in && i > 0 ? c[-1] + c[0] : 0.0;
+    if (e < 3 * 64) M.fxy8[e] = in && L + 1 < 8 ? c[0] + c[64] : 0.0;
   }
 }
 // zero what the passes never write (boundary nodes)
@@ -364,11 +452,14 @@ __global__ void __launch_bounds__(256, 2) k_vcycle64(CoarseArgs64 A) {
   if (tid < 64) M.a4[tid] = (1.0 / 48.0) * A.a[2][(long long)s * 64 + tid];
   if (tid < 125) M.wd4[tid] = A.wd[2][(long long)s * 125 + tid];
   if (tid < 8) M.a2[tid] = A.a[3][(long long)s * 8 + tid];
+  __syncthreads();
+  faces8(M, rank);
+  coarse4_setup(M, A.omega, 256);
   cl.sync();  // every block's memory is ready for its neighbours' writes
   const int i = 1 + tid % 15, j = 1 + tid / 15;
   const bool col = tid < 225;
   double z[2];
-  vcycle<16>(M, cl, rank, col, i, j, A.omega, z, [] { return true; });
+  vcycle<16>(M, cl, rank, col, i, j, A.omega, 0, z, [] { return true; });
   double* zo = A.z + (long long)s * 4913 + (2 * rank + 1) * 289;
   if (col) {
     zo[i + 17 * j] = z[0];
@@ -409,11 +500,11 @@ __device__ __forceinline__ double omega_over_d(const double* c, int i, int j, in
 }
 
 template <int N>
-__global__ void __launch_bounds__(Cfg<N>::NT, N == 16 ? 2 : 8) k_small64(SolveArgs64 A) {
+__global__ void __launch_bounds__(Cfg<N>::NT, N == 16 ? 2 : 5) k_small64(SolveArgs64 A) {
   pdl_entry();
   using K = Cfg<N>;
   using SM = With8<N, SmemSolve<N>>;
-  constexpr int S1 = K::n1, S2 = K::PL, C = K::C, NT = K::NT;
+  constexpr int S1 = K::n1, S2 = K::PL, C = K::C, NT = K::NT, U = K::U;
   cg::cluster_group cl = cg::this_cluster();
   const int rank = (int)cl.block_rank(), s = blockIdx.x / C;
   extern __shared__ __align__(16) unsigned char smraw[];
@@ -454,23 +545,29 @@ __global__ void __launch_bounds__(Cfg<N>::NT, N == 16 ? 2 : 8) k_small64(SolveAr
       M.wd8[a + 9 * b + 81 * k] = omega_over_d<8>(M.a8, a, b, k, A.omega);
     }
   }
-  // this thread's column, its diagonal and right-hand side
-  const int i = 1 + tid % K::M, j = 1 + tid / K::M, nb = i + S1 * j, cb = (i - 1) + N * (j - 1);
-  const bool col = tid < K::M * K::M;
+  __syncthreads();
+  if constexpr (N == 16) faces8(M, rank);
+  coarse4_setup(M, A.omega, NT);
+  // this thread's column, its own planes u0 .. u0 + U - 1, their diagonal and right-hand side
+  const int u0 = U == 2 ? 0 : tid >> 6, tc = U == 2 ? tid : tid & 63;
+  const int i = 1 + tc % K::M, j = 1 + tc / K::M, nb = i + S1 * j, cb = (i - 1) + N * (j - 1);
+  const bool col = tc < K::M * K::M;
   const int nown = 2 * rank + 2 < N ? 2 : 1;
-  double D[2] = {0.0, 0.0}, x[2] = {0.0, 0.0};
+  double D[U] = {}, x[U] = {};
   double bb = 0.0;
   if (col) {
     auto sum4 = [&](const double* q) { return (q[0] + q[1]) + (q[N] + q[N + 1]); };
 #pragma unroll
-    for (int u = 0; u < 2; ++u)
+    for (int h = 0; h < U; ++h) {
+      const int u = u0 + h;
       if (u < nown) {
-        D[u] = 4.0 * sum4(M.fxy + u * K::CP + cb);
+        D[h] = 4.0 * sum4(M.fxy + u * K::CP + cb);
         const double v = bs[(2 * rank + 1 + u) * S2 + nb];
         M.r[(u + 1) * S2 + nb] = v;
         bb = fma(v, v, bb);
-        M.wd[(u + 1) * S2 + nb] = A.omega / D[u];
+        M.wd[(u + 1) * S2 + nb] = A.omega / D[h];
       }
+    }
     // halo planes: their diagonal from the cells in memory (one plane beyond the block's)
     const double h12 = 1.0 / (12.0 * N);
     auto halo = [&](int k, int l) {
@@ -479,8 +576,8 @@ __global__ void __launch_bounds__(Cfg<N>::NT, N == 16 ? 2 : 8) k_small64(SolveAr
       M.wd[l * S2 + nb] = A.omega / (4.0 * (h12 * (sum4(q) + sum4(q + K::CP))));
       M.r[l * S2 + nb] = bs[k * S2 + nb];
     };
-    halo(2 * rank, 0);
-    halo(2 * rank + 3, 3);
+    if (u0 == 0) halo(2 * rank, 0);
+    if (u0 == 2 - U) halo(2 * rank + 3, 3);
   }
   // block sum to every block's slot (complete after the next cluster barrier)
   auto push_sum = [&](double v, int which) {
@@ -519,8 +616,8 @@ __global__ void __launch_bounds__(Cfg<N>::NT, N == 16 ? 2 : 8) k_small64(SolveAr
   double rsum = 0.0;  // r.r of the own nodes
   for (int it = 0; go; ++it) {
     if (it > 0) push_sum(rsum, 0);
-    double z[2];
-    const bool on = vcycle<N>(M, cl, rank, col, i, j, A.omega, z, [&] {
+    double z[U];
+    const bool on = vcycle<N>(M, cl, rank, col, i, j, A.omega, u0, z, [&] {
       if (it == 0) return true;
       // stop test of the iterate before this V-cycle
       if (tid < 32) {
@@ -542,10 +639,11 @@ __global__ void __launch_bounds__(Cfg<N>::NT, N == 16 ? 2 : 8) k_small64(SolveAr
     // r.z, and z on the neighbours' halo planes
     double v = 0.0;
     if (col) {
-      v = M.r[S2 + nb] * z[0];
-      if (nown == 2) v = fma(M.r[2 * S2 + nb], z[1], v);
-      if (rank > 0) cl.map_shared_rank(&M, rank - 1)->zh[S2 + nb] = z[0];
-      if (rank + 1 < C) cl.map_shared_rank(&M, rank + 1)->zh[nb] = z[1];
+#pragma unroll
+      for (int h = 0; h < U; ++h)
+        if (u0 + h < nown) v = fma(M.r[(u0 + h + 1) * S2 + nb], z[h], v);
+      if (u0 == 0 && rank > 0) cl.map_shared_rank(&M, rank - 1)->zh[S2 + nb] = z[0];
+      if (u0 == 2 - U && rank + 1 < C) cl.map_shared_rank(&M, rank + 1)->zh[nb] = z[U - 1];
     }
     push_sum(v, 1);
     cl.sync();
@@ -559,26 +657,37 @@ __global__ void __launch_bounds__(Cfg<N>::NT, N == 16 ? 2 : 8) k_small64(SolveAr
     __syncthreads();
     const double beta = M.bc;
     if (col) {  // p = z + beta p on the own and the halo planes
-      const double zl[4] = {M.zh[nb], z[0], z[1], M.zh[S2 + nb]};
+      double zl[2 * U];  // the thread's staged planes 2 u0 .. 2 u0 + 2 U - 1
+      if constexpr (U == 2) {
+        zl[0] = M.zh[nb]; zl[1] = z[0]; zl[2] = z[1]; zl[3] = M.zh[S2 + nb];
+      } else {
+        zl[0] = u0 ? z[0] : M.zh[nb];
+        zl[1] = u0 ? M.zh[S2 + nb] : z[0];
+      }
 #pragma unroll
-      for (int l = 0; l < 4; ++l) M.p[l * S2 + nb] = it == 0 ? zl[l] : fma(beta, M.p[l * S2 + nb], zl[l]);
+      for (int h = 0; h < 2 * U; ++h) {
+        double* pl = M.p + (2 * u0 + h) * S2 + nb;
+        *pl = it == 0 ? zl[h] : fma(beta, *pl, zl[h]);
+      }
     }
     __syncthreads();
-    double q[2] = {0.0, 0.0};
+    double q[U] = {};
     v = 0.0;
     if (col) {
 #pragma unroll
-      for (int u = 0; u < 2; ++u)
+      for (int h = 0; h < U; ++h) {
+        const int u = u0 + h;
         if (u < nown) {
           const double pv = M.p[(u + 1) * S2 + nb];
           const double o = off_row<S1, S2, N>(0.0, M.p + (u + 1) * S2 + nb, M.c + u * K::CP + cb,
                                               M.fxy + u * K::CP + cb, M.fxz + u * K::CP + (i - 1) + N * j,
                                               M.fyz + u * K::CP + i + N * (j - 1));
-          q[u] = fma(D[u], pv, -o);
-          v = fma(pv, q[u], v);
+          q[h] = fma(D[h], pv, -o);
+          v = fma(pv, q[h], v);
         }
-      if (rank > 0) cl.map_shared_rank(&M, rank - 1)->qh[S2 + nb] = q[0];
-      if (rank + 1 < C) cl.map_shared_rank(&M, rank + 1)->qh[nb] = q[1];
+      }
+      if (u0 == 0 && rank > 0) cl.map_shared_rank(&M, rank - 1)->qh[S2 + nb] = q[0];
+      if (u0 == 2 - U && rank + 1 < C) cl.map_shared_rank(&M, rank + 1)->qh[nb] = q[U - 1];
     }
     push_sum(v, 2);
     cl.sync();
@@ -590,12 +699,22 @@ __global__ void __launch_bounds__(Cfg<N>::NT, N == 16 ? 2 : 8) k_small64(SolveAr
     const double alpha = M.bc;
     rsum = 0.0;
     if (col) {
-      const double ql[4] = {M.qh[nb], q[0], q[1], M.qh[S2 + nb]};
+      double ql[2 * U];
+      if constexpr (U == 2) {
+        ql[0] = M.qh[nb]; ql[1] = q[0]; ql[2] = q[1]; ql[3] = M.qh[S2 + nb];
+      } else {
+        ql[0] = u0 ? q[0] : M.qh[nb];
+        ql[1] = u0 ? M.qh[S2 + nb] : q[0];
+      }
 #pragma unroll
-      for (int l = 0; l < 4; ++l) M.r[l * S2 + nb] = fma(-alpha, ql[l], M.r[l * S2 + nb]);
+      for (int h = 0; h < 2 * U; ++h) {
+        double* rl = M.r + (2 * u0 + h) * S2 + nb;
+        *rl = fma(-alpha, ql[h], *rl);
+      }
 #pragma unroll
-      for (int u = 0; u < 2; ++u) {
-        x[u] = fma(alpha, M.p[(u + 1) * S2 + nb], x[u]);
+      for (int h = 0; h < U; ++h) {
+        const int u = u0 + h;
+        x[h] = fma(alpha, M.p[(u + 1) * S2 + nb], x[h]);
         const double rv = M.r[(u + 1) * S2 + nb];
         if (u < nown) rsum = fma(rv, rv, rsum);
       }
@@ -610,8 +729,9 @@ __global__ void __launch_bounds__(Cfg<N>::NT, N == 16 ? 2 : 8) k_small64(SolveAr
     if (rank == 0 && e < S2) xo[e] = 0.0;
   }
   if (col) {
-    xo[(long long)(2 * rank + 1) * S2 + nb] = x[0];
-    if (nown == 2) xo[(long long)(2 * rank + 2) * S2 + nb] = x[1];
+#pragma unroll
+    for (int h = 0; h < U; ++h)
+      if (u0 + h < nown) xo[(long long)(2 * rank + 1 + u0 + h) * S2 + nb] = x[h];
   }
   if (rank == 0 && tid == 0) {
     SolveScalars c;
@@ -624,21 +744,61 @@ __global__ void __launch_bounds__(Cfg<N>::NT, N == 16 ? 2 : 8) k_small64(SolveAr
 
 static_assert(sizeof(SmemV) <= 113 * 1024 && sizeof(With8<16, SmemSolve<16>>) <= 113 * 1024, "two blocks per SM");
 
-template <typename Kern>
-cudaError_t allow_smem(Kern* k, size_t bytes, bool& done) {
-  if (done) return cudaSuccess;
-  const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-  done = e == cudaSuccess;
-  return e;
+// Launches one cluster per sample, spread over as many SMs as one wave allows: blocks that
+// share an SM share its FP64 pipe, and the hardware fills an SM before it takes the next
+// (16 clusters of eight blocks went to 64 SMs).  The shared memory that is asked for sets
+// how many blocks an SM takes: the fewest with which every sample's cluster is resident.
+struct Spread {
+  std::once_flag once;
+  cudaError_t err = cudaSuccess;
+  int n = 0;
+  size_t smem[8];
+  int clusters[8];  // resident with at most i + 1 blocks per SM
+};
+template <typename Args>
+cudaError_t launch_spread(Spread& sp, const char* cls, double bytes, void (*k)(Args), int threads, int cluster,
+                          size_t smem, int most, int samples, cudaStream_t st, const Args& A) {
+  std::call_once(sp.once, [&] {
+    constexpr size_t kSm = 228 * 1024, kBlock = 1024;  // of an SM; reserved per block
+    sp.err = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)std::max(smem, kSm / 2 - kBlock + 16));
+    for (int occ = 1; occ <= most && sp.err == cudaSuccess; ++occ) {
+      const size_t want = std::max(smem, kSm / (occ + 1) - kBlock + 16);  // occ + 1 blocks don't fit
+      cudaLaunchAttribute at[1];
+      at[0].id = cudaLaunchAttributeClusterDimension;
+      at[0].val.clusterDim.x = (unsigned)cluster;
+      at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+      cudaLaunchConfig_t cfg{};
+      cfg.gridDim = dim3((unsigned)cluster);
+      cfg.blockDim = dim3((unsigned)threads);
+      cfg.dynamicSmemBytes = want;
+      cfg.attrs = at;
+      cfg.numAttrs = 1;
+      int c = 0;
+      if (cudaOccupancyMaxActiveClusters(&c, k, &cfg) != cudaSuccess) {
+        (void)cudaGetLastError();
+        c = 0;
+      }
+      sp.smem[sp.n] = want;
+      sp.clusters[sp.n++] = c;
+    }
+  });
+  if (sp.err != cudaSuccess) return sp.err;
+  size_t use = smem;
+  for (int i = 0; i < sp.n; ++i)
+    if (sp.clusters[i] >= samples) {
+      use = sp.smem[i];
+      break;
+    }
+  return launch_cluster(cls, bytes, k, dim3((unsigned)(samples * cluster)), dim3((unsigned)threads), (unsigned)cluster,
+                        use, st, A);
 }
 
 }  // namespace
 
 cudaError_t coarse_vcycle64(const double* r16, const double* const a[4], const double* const wd[3], double* z16,
                             const SolveScalars* sc, const Batch& bt, double omega, cudaStream_t st) {
-  static bool smem_set = false;  // once (capture-friendly)
-  const cudaError_t e = allow_smem(k_vcycle64, sizeof(SmemV), smem_set);
-  if (e != cudaSuccess) return e;
+  static Spread sp;
   CoarseArgs64 A{};
   A.r = r16;
   for (int l = 0; l < 4; ++l) A.a[l] = a[l];
@@ -646,7 +806,7 @@ cudaError_t coarse_vcycle64(const double* r16, const double* const a[4], const d
   A.z = z16; A.sc = sc; A.act = bt.act; A.omega = omega;
   // per sample: r, z and omega D^-1 of 16^3, the coefficient levels, omega D^-1 of 8^3 and 4^3
   const double bytes = (double)bt.n * 8 * (3.0 * 4913 + 4096 + 512 + 64 + 8 + 729 + 125);
-  return launch_cluster("coarse_f64", bytes, k_vcycle64, dim3((unsigned)bt.n * 8), dim3(256), 8, sizeof(SmemV), st, A);
+  return launch_spread(sp, "coarse_f64", bytes, k_vcycle64, 256, 8, sizeof(SmemV), 2, bt.n, st, A);
 }
 
 cudaError_t small_fp64(SolverBufs& B, const double* a64, const double* b, long long bstride, double* x_out,
@@ -654,18 +814,10 @@ cudaError_t small_fp64(SolverBufs& B, const double* a64, const double* b, long l
   const int N = B.N, S = B.S;
   SolveArgs64 A{a64, b, bstride, x_out, B.sc, prm.rtol * prm.rtol, prm.omega, prm.max_iter};
   const double bytes = (bstride ? S : 1) * (double)nodes_of(N) * 8 + (double)S * 8 * (nodes_of(N) + cells_of(N));
-  if (N == 16) {
-    using SM = With8<16, SmemSolve<16>>;
-    static bool smem_set = false;
-    const cudaError_t e = allow_smem(k_small64<16>, sizeof(SM), smem_set);
-    if (e != cudaSuccess) return e;
-    return launch_cluster("small_f64", bytes, k_small64<16>, dim3((unsigned)S * 8), dim3(256), 8, sizeof(SM), st, A);
-  }
-  using SM = With8<8, SmemSolve<8>>;
-  static bool smem_set8 = false;
-  const cudaError_t e = allow_smem(k_small64<8>, sizeof(SM), smem_set8);
-  if (e != cudaSuccess) return e;
-  return launch_cluster("small_f64", bytes, k_small64<8>, dim3((unsigned)S * 4), dim3(64), 4, sizeof(SM), st, A);
+  static Spread sp8, sp16;
+  if (N == 16)
+    return launch_spread(sp16, "small_f64", bytes, k_small64<16>, 256, 8, sizeof(With8<16, SmemSolve<16>>), 2, S, st, A);
+  return launch_spread(sp8, "small_f64", bytes, k_small64<8>, 128, 4, sizeof(With8<8, SmemSolve<8>>), 5, S, st, A);
 }
 
 }  // namespace mlsgd

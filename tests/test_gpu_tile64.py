@@ -62,3 +62,13 @@ def test_chunks_and_batches_leave_the_bits(lib, grid):
     for other in [_solve(lib, grid, 2, z, z_chunks=c) for c in (1, 3, 64)] + [_solve(lib, grid, 40, z)]:
         for a, b in zip(ref[1:], other[1:]):
             assert np.array_equal(a, b[:2])
+
+
+@pytest.mark.parametrize("grid", [0, 1])  # 8^3, 16^3
+def test_cluster_solves_do_not_depend_on_the_wave(lib, grid):
+    """The blocks per SM follow the sample count (one block on an SM, several, more than a wave): the same bits."""
+    z = inputs.z_test(32) + inputs.z_random(32, 3)
+    ref = _solve(lib, grid, 1, z)
+    for S in (15, 20, 40, 150, 250):
+        for a, b in zip(ref[1:], _solve(lib, grid, S, z)[1:]):
+            assert np.array_equal(a, b[:1])
