@@ -9,16 +9,17 @@
 // levels, operand and residuals on the SM and runs the refinement loop to the end:
 // coarse coefficients, FP32 inner PCG with its V(1,1)-cycle, FP64-accurate residual,
 // stop test.  What bounds it is the latency between block barriers (about 14 per inner
-// iteration) and, on 16^3, the shared-memory loads of three 21-point stencils.
+// iteration) and, on 16^3, the shared-memory loads of three 21-point stencils; FP64 in one
+// warp (64 clocks an operation) is kept out of the inner iterations.
 // Measured (three refinement steps of six iterations, state or adjoint): 1024 samples of
-// 8^3 400 us a solve against 2.2 ms in passes, 256 of 16^3 320 us against 3.1 ms, 64 of
+// 8^3 310 us a solve against 2.2 ms in passes, 256 of 16^3 320 us against 3.1 ms, 64 of
 // 16^3 200 us against 1.6 ms.
 //
-// Arithmetic: that of the pass-by-pass solver on the same grid, operation by operation
-// and sum by sum (solver.cu for 8^3: FP64 refinement residual and solution, partial sums
-// per 256 consecutive nodes; tiled.cu for 16^3: solution and b as FP32 pairs, partial
-// sums per thread over 8 planes and the rows of a thread), so a sample's iterates, its
-// iteration count and its result are the ones those passes give.
+// Arithmetic: that of the pass-by-pass solver on the same grid (solver.cu for 8^3: FP64
+// refinement residual and solution, partial sums per 256 consecutive nodes; tiled.cu for
+// 16^3: solution and b as FP32 pairs, partial sums per thread over 8 planes and the rows of
+// a thread), except that the 4^3 and 2^3 levels are one matrix (coarse4_build) and alpha and
+// beta are quotients of pairs.
 #include "internal.cuh"
 #include "kernels.h"
 #include "launch.h"
@@ -75,15 +76,28 @@ __device__ __forceinline__ double sum_groups(T v) {  // lane l holds warp l's su
   return (p0 + p2) + p1;
 }
 
+// floats of the levels from 8^3 down: x8, t8, t4, the 4^3 matrix and its vectors, a4, a2;
+// on 16^3 also r8 and a8
+constexpr int kLv8 = 2 * 729 + 125 + 27 * 27 + 54 + 64 + 8, kLv16 = kLv8 + 729 + 512;
+
+// a / b of two pairs (about 46 bits) rounded to FP32; 0 unless ok
+__device__ __forceinline__ float df_quotient(DF a, DF b, bool ok) {
+  if (!ok) return 0.f;
+  const float q = __fdiv_rn(a.h, b.h);
+  const float p = __fmul_rn(q, b.h), e = __fmaf_rn(q, b.h, -p);
+  const float rem = __fsub_rn(__fsub_rn(__fsub_rn(a.h, p), e), __fmaf_rn(q, b.l, -a.l));
+  const float c = __fdiv_rn(rem, b.h);
+  return fabsf(c) < INFINITY ? __fadd_rn(q, c) : q;
+}
+
 struct Smem8 {
   double xd[729];       // solution for the refinement residual
   double redd[24];
   float a32[512], abf[512];
   float op[729];        // operand of A p
   float r8[729];        // residual of the V-cycle
-  float lv[kCoarse8Own];
+  float lv[kLv8];
   float redf[2][24];
-  float bc;             // alpha or beta
   int go;
 };
 
@@ -97,23 +111,25 @@ __global__ void __launch_bounds__(kT8, 2) k_small8(SmallArgs A) {
     M.abf[c] = __bfloat162float(A.abf[(long long)s * 512 + c]);
   }
   if (n < 729) M.op[n] = M.r8[n] = 0.f;
-  for (int e = n; e < kCoarse8Own; e += kT8) M.lv[e] = 0.f;
+  for (int e = n; e < kLv8; e += kT8) M.lv[e] = 0.f;
   CoarseLevels L;
   L.r8 = M.r8; L.a8 = M.abf;
   L.x8 = M.lv; L.t8 = L.x8 + 729;
-  L.x4 = L.t8 + 729; L.t4 = L.x4 + 125;
-  float* a4 = L.t4 + 125;
+  L.t4 = L.t8 + 729; L.g4 = L.t4 + 125; L.s4 = L.g4 + 729;
+  float* a4 = L.s4 + 54;
   float* a2 = a4 + 64;
-  L.a4 = a4; L.a2 = a2;
+  L.x4 = nullptr; L.a4 = a4; L.a2 = a2;
   int i = 0, j = 0, k = 0;
   if (n < 729) node_ijk(n, 9, i, j, k);
   const bool in = n < 729 && interior(i, j, k, 8);
   const double bv = n < 729 ? A.b[s * A.bstride + n] : 0.0;
   __syncthreads();
   if (n < 64) a4[n] = coarsen_cell(M.abf, n, 4);
-  const float D = in ? diag_of<8>(M.abf, i, j, k) : 1.f;
+  const float w8 = in ? omega / diag_of<8>(M.abf, i, j, k) : 0.f;
   __syncthreads();
   if (n < 8) a2[n] = coarsen_cell(a4, n, 2);
+  __syncthreads();
+  coarse4_build<kT8>(L, omega);
   Outer o{0.0, 0.0, 0.0, 0, 0, 0};
   // block sum of a double, result in warp 0
   auto sum64 = [&](double v) {
@@ -122,15 +138,22 @@ __global__ void __launch_bounds__(kT8, 2) k_small8(SmallArgs A) {
     __syncthreads();
     return warp == 0 ? sum_groups<double>(lane < 24 ? M.redd[lane] : 0.0) : 0.0;
   };
+  // block sum of a float as a pair, in every thread: the three group sums are added exactly
+  // (FP64 additions and a division in one warp were a quarter of an iteration)
   int par = 0;
   auto sum32 = [&](float v) {
     v = warp_sum(v);
     if (lane == 0) M.redf[par][warp] = v;
     __syncthreads();
-    const double d = warp == 0 ? sum_groups<float>(lane < 24 ? M.redf[par][lane] : 0.f) : 0.0;
+    float g = lane < 24 ? M.redf[par][lane] : 0.f;
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) g += __shfl_xor_sync(0xffffffffu, g, o);
+    const float p0 = __shfl_sync(0xffffffffu, g, 0), p1 = __shfl_sync(0xffffffffu, g, 8),
+                p2 = __shfl_sync(0xffffffffu, g, 16);
     par ^= 1;
-    return d;
+    return df_add(df_add(DF{p0, 0.f}, DF{p2, 0.f}), DF{p1, 0.f});
   };
+  DF rz{0.f, 0.f};  // r . z
   {
     const double v = sum64(bv * bv);
     if (n == 0) {
@@ -176,20 +199,10 @@ __global__ void __launch_bounds__(kT8, 2) k_small8(SmallArgs A) {
     for (int it = 0;; ++it) {
       if (n < 729) M.r8[n] = r;
       __syncthreads();
-      const float z = vcycle8<kT8>(L, n, i, j, k, in, D, omega);
-      {
-        const double v = sum32(r * z);
-        if (n == 0) {
-          if (it == 0) o.rz = v;
-          else M.bc = pcg_beta(o, v);
-        }
-      }
-      if (it > 0) {
-        __syncthreads();
-        p = z + M.bc * p;
-      } else {
-        p = z;
-      }
+      const float z = vcycle8<kT8, true>(L, n, i, j, k, in, w8, omega);
+      const DF rzn = sum32(r * z);
+      p = it > 0 ? z + df_quotient(rzn, rz, rz.h != 0.f) * p : z;
+      rz = rzn;
       if (n < 729) M.op[n] = p;
       __syncthreads();
       float q = 0.f;
@@ -198,10 +211,8 @@ __global__ void __launch_bounds__(kT8, 2) k_small8(SmallArgs A) {
         cells8(C, M.a32, i, j, k, 8);
         q = float(1.0 / (12.0 * 8)) * q1_row(C, (const float*)M.op, i, j, k, 9);
       }
-      const double v = sum32(p * q);
-      if (n == 0) M.bc = pcg_alpha(o, v);
-      __syncthreads();
-      const float al = M.bc;
+      const DF pq = sum32(p * q);
+      const float al = df_quotient(rz, pq, pq.h > 0.f && rz.h != 0.f);
       d += al * p;
       if (it == inner - 1) break;
       r = r - al * q;
@@ -209,6 +220,7 @@ __global__ void __launch_bounds__(kT8, 2) k_small8(SmallArgs A) {
     x += (double)d;
     if (n == 0) { o.iters += 1; o.pad += inner; }
   }
+  o.rz = df_to_double(rz);
   if (n < 729) A.x64[(long long)s * 729 + n] = x;
   if (n == 0) store_scalars(A.sc + s, o);
 }
@@ -227,10 +239,9 @@ struct Smem16 {
   float b1[kN16];  // t, then r (dot)
   float b2[kN16];  // z, q or the refinement residual (dot)
   float a32[4096], abf[4096];
-  float lv[kCoarse8Floats];
+  float lv[kLv16];
   double redd[24];
   float redf[8];
-  float bc;
   int go;
 };
 static_assert(sizeof(Smem16) <= 227 * 1024, "shared memory");
@@ -296,14 +307,14 @@ __global__ void __launch_bounds__(kT16, 1) k_small16(SmallArgs A) {
     M.abf[c] = __bfloat162float(A.abf[(long long)s * 4096 + c]);
   }
   for (int e = tid; e < kN16; e += kT16) M.b0[e] = M.b1[e] = 0.f;
-  for (int e = tid; e < kCoarse8Floats; e += kT16) M.lv[e] = 0.f;
+  for (int e = tid; e < kLv16; e += kT16) M.lv[e] = 0.f;
   CoarseLevels L;
   L.r8 = M.lv; L.x8 = L.r8 + 729; L.t8 = L.x8 + 729;
   float* a8 = L.t8 + 729;
-  L.x4 = a8 + 512; L.t4 = L.x4 + 125;
-  float* a4 = L.t4 + 125;
+  L.t4 = a8 + 512; L.g4 = L.t4 + 125; L.s4 = L.g4 + 729;
+  float* a4 = L.s4 + 54;
   float* a2 = a4 + 64;
-  L.a8 = a8; L.a4 = a4; L.a2 = a2;
+  L.x4 = nullptr; L.a8 = a8; L.a4 = a4; L.a2 = a2;
   // the right-hand side's pair at node n of this sample
   auto b_pair = [&](int n) {
     return A.bp ? A.bp[s * A.bstride + n] : df_split(A.b[s * A.bstride + n]);
@@ -339,9 +350,11 @@ __global__ void __launch_bounds__(kT16, 1) k_small16(SmallArgs A) {
   int i8 = 0, j8 = 0, k8 = 0;
   if (tid < 729) node_ijk(tid, 9, i8, j8, k8);
   const bool in8 = tid < 729 && interior(i8, j8, k8, 8);
-  const float D8 = in8 ? diag_of<8>(a8, i8, j8, k8) : 1.f;
+  const float w8 = in8 ? omega / diag_of<8>(L.a8, i8, j8, k8) : 0.f;
   __syncthreads();
   if (tid < 8) a2[tid] = coarsen_cell(a4, tid, 2);
+  __syncthreads();
+  coarse4_build<kT16>(L, omega);
   Outer o{0.0, 0.0, 0.0, 0, 0, 0};
   // ||b||^2 as the solver's init pass sums it: three blocks of 256 threads, eight nodes a
   // thread at stride 256 (FP32 over the pair heads; FP64 for an FP64 right-hand side of its own)
@@ -384,7 +397,7 @@ __global__ void __launch_bounds__(kT16, 1) k_small16(SmallArgs A) {
   __syncthreads();
   // dot product of two shared vectors in the order of the tile passes: thread (tx, ty) of
   // segment sg sums rows 4 ty + 1 .. 4 ty + 4 over the segment's eight planes, then the
-  // block sum of the segment, then the two segments (result in warp 0)
+  // block sum of the segment, then the two segments (a pair, in every thread)
   auto dot = [&](const float* u, const float* v) {
     if (warp < 8) {
       const int sg = warp >> 2, ty = warp & 3;
@@ -404,13 +417,13 @@ __global__ void __launch_bounds__(kT16, 1) k_small16(SmallArgs A) {
       if (lane == 0) M.redf[warp] = red;
     }
     __syncthreads();
-    if (warp != 0) return 0.0;
     float w = lane < 8 ? M.redf[lane] : 0.f;
     w += __shfl_xor_sync(0xffffffffu, w, 2);
     w += __shfl_xor_sync(0xffffffffu, w, 1);
-    const double p0 = (double)__shfl_sync(0xffffffffu, w, 0), p1 = (double)__shfl_sync(0xffffffffu, w, 4);
-    return p0 + p1;
+    const float p0 = __shfl_sync(0xffffffffu, w, 0), p1 = __shfl_sync(0xffffffffu, w, 4);
+    return df_add(DF{p0, 0.f}, DF{p1, 0.f});
   };
+  DF rz{0.f, 0.f};  // r . z
   bool go = M.go != 0;
   const float2 zero2 = make_float2(0.f, 0.f);
   if (!go) {  // no step is taken: x = 0
@@ -493,7 +506,7 @@ __global__ void __launch_bounds__(kT16, 1) k_small16(SmallArgs A) {
         L.r8[tid] = v;
       }
       __syncthreads();
-      (void)vcycle8<kT16>(L, tid, i8, j8, k8, in8, D8, omega);
+      (void)vcycle8<kT16, true>(L, tid, i8, j8, k8, in8, w8, omega);
       __syncthreads();
       const int px = (xq + 1) & 1, py = (yq + 1) & 1;
       const float* e8 = L.t8 + ((xq + 1) >> 1) + 9 * ((yq + 1) >> 1);
@@ -524,20 +537,10 @@ __global__ void __launch_bounds__(kT16, 1) k_small16(SmallArgs A) {
           M.b2[n0 + 289 * u] = z[u];
         }
       __syncthreads();
-      {
-        const double v = dot(M.b1, M.b2);
-        if (tid == 0) {
-          if (it == 0) {
-            o.rz = v;
-            M.bc = 0.f;
-          } else {
-            M.bc = pcg_beta(o, v);
-          }
-        }
-      }
-      __syncthreads();
+      const DF rzn = dot(M.b1, M.b2);
       // p = z + beta p, q = A p
-      const float be = M.bc;
+      const float be = it == 0 ? 0.f : df_quotient(rzn, rz, rz.h != 0.f);
+      rz = rzn;
 #pragma unroll
       for (int u = 0; u < 4; ++u)
         if (u < nu) {
@@ -552,12 +555,8 @@ __global__ void __launch_bounds__(kT16, 1) k_small16(SmallArgs A) {
           M.b2[n0 + 289 * u] = q[u];
         }
       __syncthreads();
-      {
-        const double v = dot(M.b0, M.b2);
-        if (tid == 0) M.bc = pcg_alpha(o, v);
-      }
-      __syncthreads();
-      al = M.bc;
+      const DF pq = dot(M.b0, M.b2);
+      al = df_quotient(rz, pq, pq.h > 0.f && rz.h != 0.f);
       if (it == inner - 1) break;
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
@@ -584,6 +583,7 @@ __global__ void __launch_bounds__(kT16, 1) k_small16(SmallArgs A) {
         A.x64[e] = (double)v.x + (double)v.y;
       }
   }
+  o.rz = df_to_double(rz);
   if (tid == 0) store_scalars(A.sc + s, o);
 }
 
