@@ -883,57 +883,64 @@ __global__ void __launch_bounds__(kBlock) k_lvl_s2(const double* __restrict__ x,
   if (threadIdx.x == 0) partial[bid] = hf3 * bs;
 }
 // per control cell: batch mean = interpolated nodal mean; Chan merge with the old
-// field; block partials of h_c^3 delta^2 n_old S / n.  A block takes kLvlRows rows
-// (cy, cz) of control cells, 256 cells of a row per block in x; per row the
-// level-node columns are first interpolated in (y, z) into shared memory with their
-// differences, then each cell interpolates linearly in x between the two columns of its
-// level cell.  An empty record (n_old = 0) is not read.
+// field; block partials of h_c^3 delta^2 n_old S / n.  A block takes kLvlRows rows cy of a
+// plane cz of control cells, 256 cells of a row per block in x.  The node lines under it are
+// interpolated in z once, into shared memory; a thread interpolates a line in x at its cx
+// when it is reached, and a cell is then one FMA in y between the lines on either side
+// (1 + 3/r + 4 (Nf/256)(1/r + 1/16) FP64 operations a cell, the bound next to the store; one
+// interpolation in (y, z) per row, by one warp between three barriers, took 190 us on a
+// 256^3 control, about 75 us now).  An empty record (n_old = 0) is not read.
 constexpr int kLvlRows = 16;
 __global__ void __launch_bounds__(kBlock) k_lvl_field(const double* __restrict__ xm, int Nf, int Nc, int S,
                                                       const double* __restrict__ work, double* __restrict__ field,
                                                       double* __restrict__ partial) {
   pdl_entry();
-  extern __shared__ double col[];  // [2][Nf + 1]: the mean interpolated in (y, z), and its x differences
+  extern __shared__ double line[];  // [lines][Nf + 1]: the mean interpolated in z
   const int n1 = Nf + 1, r = Nc / Nf;
   const long long sz = (long long)n1 * n1;
   const float inv_r = 1.0f / (float)r;  // r a power of two: the weights are exact in FP32
   const double n_old = work[2], scale = work[1], a = work[3];
-  const int cx = blockIdx.x * blockDim.x + threadIdx.x;
-  const int ex = cx / r;
-  const double tx = f2d(((float)(cx - ex * r) + 0.5f) * inv_r);
-  const long long rows = (long long)Nc * Nc;
+  const int cx = blockIdx.x * blockDim.x + threadIdx.x, cz = blockIdx.z;
+  const int cy0 = blockIdx.y * kLvlRows, cy1 = min(Nc, cy0 + kLvlRows);
+  const int ey0 = cy0 / r, nl = (cy1 - 1) / r - ey0 + 2;
+  {
+    const int ez = cz / r;
+    const float tz = ((float)(cz - ez * r) + 0.5f) * inv_r;
+    const double w0 = f2d(1.f - tz), w1 = f2d(tz);
+    const double* b = xm + (long long)n1 * ey0 + sz * ez;
+    for (int c = threadIdx.x; c < nl * n1; c += blockDim.x) line[c] = fma(w1, b[sz + c], w0 * b[c]);
+  }
+  __syncthreads();
   double contrib = 0.0;
-  for (long long row = (long long)blockIdx.y * kLvlRows; row < rows && row < (long long)(blockIdx.y + 1) * kLvlRows;
-       ++row) {
-    const int cz = (int)((unsigned)row / (unsigned)Nc), cy = (int)row - cz * Nc;
-    const int ey = cy / r, ez = cz / r;
-    const float ty = ((float)(cy - ey * r) + 0.5f) * inv_r, tz = ((float)(cz - ez * r) + 0.5f) * inv_r;
-    const double w00 = f2d((1.f - ty) * (1.f - tz)), w10 = f2d(ty * (1.f - tz)), w01 = f2d((1.f - ty) * tz),
-                 w11 = f2d(ty * tz);
-    __syncthreads();  // the previous row's columns are no longer read
-    for (int c = threadIdx.x; c < n1; c += blockDim.x) {
-      const double* b = xm + c + (long long)n1 * ey + sz * ez;
-      col[c] = fma(w11, b[sz + n1], fma(w01, b[sz], fma(w10, b[n1], w00 * b[0])));
-    }
-    __syncthreads();
-    for (int c = threadIdx.x; c < Nf; c += blockDim.x) col[n1 + c] = col[c + 1] - col[c];
-    __syncthreads();
-    if (cx < Nc) {
-      const double mean = fma(tx, col[n1 + ex], col[ex]);
-      const long long c = cx + row * Nc;
+  if (cx < Nc) {
+    const int ex = cx / r;
+    const double tx = f2d(((float)(cx - ex * r) + 0.5f) * inv_r);
+    const double* l = line + ex;
+    auto at_x = [&](const double* q) { return fma(tx, q[1] - q[0], q[0]); };
+    double lo = 0.0, up = at_x(l), dy = 0.0;
+    double* f = field + cx + (long long)Nc * (cy0 + (long long)Nc * cz);
+    for (int cy = cy0; cy < cy1; ++cy, f += Nc) {
+      const int my = cy & (r - 1);
+      if (my == 0 || cy == cy0) {  // the next node line
+        lo = up;
+        l += n1;
+        up = at_x(l);
+        dy = up - lo;
+      }
+      const double mean = fma(f2d(((float)my + 0.5f) * inv_r), dy, lo);
       if (n_old > 0.0) {
-        const double delta = fma(field[c], scale, -mean);
-        field[c] = fma(a, delta, mean);
+        const double delta = fma(*f, scale, -mean);
+        *f = fma(a, delta, mean);
         contrib = fma(delta, delta, contrib);
       } else {
-        field[c] = mean;
+        *f = mean;
       }
     }
   }
   const double hc = 1.0 / Nc;
   contrib *= hc * hc * hc * a * S;
   const double bs = block_sum(contrib);
-  if (threadIdx.x == 0) partial[blockIdx.x + (long long)gridDim.x * blockIdx.y] = bs;
+  if (threadIdx.x == 0) partial[blockIdx.x + (long long)gridDim.x * (blockIdx.y + (long long)gridDim.y * blockIdx.z)] = bs;
 }
 
 // returns the number of block partials written (at most level_partial_cap(Nc, Nf))
@@ -958,10 +965,10 @@ static int launch_lvl(const void* qf, int Nf, const void* qc, int S, int Nc, con
   launch("level_nodes", (double)S * nodes * 8 + (double)nodes * 8, k_lvl_mean, dim3((unsigned)((nodes + 31) / 32)), kBlock,
          0, st, x, (int)nodes, S, 1.0 / S, mean);
   const unsigned fx = (unsigned)((Nc + kBlock - 1) / kBlock);
-  const unsigned fy = (unsigned)(((long long)Nc * Nc + kLvlRows - 1) / kLvlRows);
-  const long long nf = (long long)fx * fy;
-  launch("level_field", (double)nodes * 8 + (double)ncell * 16, k_lvl_field, dim3(fx, fy), kBlock,
-         (size_t)2 * (Nf + 1) * sizeof(double), st, (const double*)mean, Nf, Nc, S, work, field, partial);
+  const unsigned fy = (unsigned)((Nc + kLvlRows - 1) / kLvlRows);
+  const long long nf = (long long)fx * fy * Nc;
+  launch("level_field", (double)nodes * 8 + (double)ncell * 16, k_lvl_field, dim3(fx, fy, (unsigned)Nc),
+         kBlock, (size_t)((kLvlRows - 1) / r + 2 + (r < kLvlRows ? 1 : 0)) * (Nf + 1) * sizeof(double), st, (const double*)mean, Nf, Nc, S, work, field, partial);
   // samples spread over blocks within the partial buffer
   const long long room = level_partial_cap(Nc, Nf) - nf;
   const double sb = (double)S * nodes * 8 + (double)nodes * 8;
