@@ -62,8 +62,8 @@ inline long long level_partial_cap(int Nc, int Nf) {
   return (cells_of(Nc) + 255) / 256 + (cells_of(Nf) + 255) / 256 + 64;
 }
 
-// The samples one launch processes: a batch of S samples (the tile shapes and the
-// per-sample partial-sum layout follow S), of which n are launched, sample act[t] for
+// The samples one launch processes: a batch of S samples, of which n are launched (the z
+// chunks follow n; the per-sample partial-sum layout depends on neither), sample act[t] for
 // t < n (act null: samples 0..n-1, n == S).  The solver's host-checked modes compact
 // the still-active samples into act, so retired samples start no blocks.
 struct Batch {
@@ -72,7 +72,7 @@ struct Batch {
   const int* act;
   int* err;      // device flag a kernel sets when one of its bounded waits runs out
   int stencil;   // 0: slab passes where supported, 1: z-marching tiles only
-  int zchunks;   // z chunks per sample (0: chosen from S)
+  int zchunks;   // z chunks per sample (0: chosen from n)
 };
 
 // Buffers of one batched solve on a grid with N cells per side.  Vectors are

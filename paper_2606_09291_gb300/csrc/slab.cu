@@ -956,7 +956,10 @@ TiledShape slab_shape(int N, int S, int zchunks) {
 template <int N, typename TA, int MODE>
 static void run_slab(const char* cls, double bytes, SlabArgs args, const Batch& bt, cudaStream_t st,
                      double ops = 0.0) {
-  const TiledShape t = slab_shape(N, bt.S, bt.zchunks);
+  // the chunks follow the samples launched: a batch's few stragglers (one of 512 samples in a
+  // third refinement step) march 63 planes in four blocks otherwise, 56 us a pass instead of
+  // 10.  The partial sums do not depend on the chunking.
+  const TiledShape t = slab_shape(N, bt.n, bt.zchunks);
   args.nzc = t.nzc;
   args.zc = t.zc;
   args.nseg = t.nseg;

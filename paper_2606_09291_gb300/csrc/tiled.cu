@@ -446,11 +446,10 @@ void tiled_post(const float* r, const TA* a, const float* dinv, const float* ec,
   else tile32_post<TA>(r, a, dinv, ec, z, partial, sc, N, bt, st);
 }
 
-// The tile shape follows the batch size bt.S (not the number of samples launched); the
-// partial sums do not depend on it.
+// The z chunks follow the number of samples launched; the partial sums do not depend on them.
 void tiled_res64(const float2* b, long long bstride, const float2* x, const float* a, float* r32, double* partial,
                  const SolveScalars* sc, int N, const Batch& bt, cudaStream_t st) {
-  const TiledShape t = tiled_shape(N, bt.S, kResRows, bt.zchunks);
+  const TiledShape t = tiled_shape(N, bt.n, kResRows, bt.zchunks);
   const ResArgs A{x, b, a, r32, partial, sc, bt.act, bstride, N, t.nzc, t.zc, t.nseg};
   const double bb = (double)(bstride ? bt.n : 1) * nodes_of(N) * 8;
   // FP32 operations per interior node as written (no sharing between nodes): 12 exact
