@@ -71,22 +71,34 @@ __global__ void k_dot(const T* __restrict__ u, const T* __restrict__ v, double* 
   if (threadIdx.x == 0) partial[(long long)s * gridDim.x + blockIdx.x] = (double)b;
 }
 
-// x += alpha p; r -= alpha q; partial = r.r
+// x += alpha p; r -= alpha q; partial = r.r.  A thread takes kUpdNodes nodes: with one, the
+// five shuffled FP64 additions of the block sum were more than the update (9 samples of
+// 64^3: 45 us).
+constexpr int kUpdNodes = 8;
+static int update_blocks(int N) { return (int)((nodes_of(N) + kUpdNodes * kBlock - 1) / (kUpdNodes * kBlock)); }
 template <typename T, bool REDUCE>
-__global__ void k_update_xr(T* __restrict__ x, T* __restrict__ r, const T* __restrict__ p, const T* __restrict__ q,
-                            double* __restrict__ partial, const SolveScalars* __restrict__ sc, long long nodes,
-                            const int* __restrict__ act) {
+__global__ void __launch_bounds__(kBlock) k_update_xr(T* __restrict__ x, T* __restrict__ r, const T* __restrict__ p,
+                                                      const T* __restrict__ q, double* __restrict__ partial,
+                                                      const SolveScalars* __restrict__ sc, long long nodes,
+                                                      const int* __restrict__ act) {
   pdl_entry();
   SAMPLE_GUARD(sc);
-  const int n = blockIdx.x * blockDim.x + threadIdx.x;
   const T al = (T)sc[s].alpha;
+  const int n0 = blockIdx.x * (kUpdNodes * kBlock) + threadIdx.x;
+  x += s * nodes;
+  r += s * nodes;
+  p += s * nodes;
+  q += s * nodes;
   T contrib = T(0);
-  if (n < nodes) {
-    const long long o = s * nodes + n;
-    x[o] += al * p[o];
-    const T rn = r[o] - al * q[o];
-    r[o] = rn;
-    contrib = rn * rn;
+#pragma unroll 4
+  for (int t = 0; t < kUpdNodes; ++t) {
+    const int n = n0 + t * kBlock;
+    if (n < nodes) {
+      x[n] += al * p[n];
+      const T rn = r[n] - al * q[n];
+      r[n] = rn;
+      contrib += rn * rn;
+    }
   }
   if (REDUCE) {
     const T b = block_sum(contrib);
@@ -124,18 +136,21 @@ __global__ void k_init(const double* __restrict__ b, long long bstride, T* __res
   if (threadIdx.x == 0) partial[(long long)s * gridDim.x + blockIdx.x] = bs;
 }
 
-// one warp per launched sample: sum the block partials in a fixed order, then the
-// scalar update
-__global__ void k_scalar(const double* __restrict__ partial, int nblk, SolveScalars* __restrict__ sc, int n,
+// W warps per launched sample: sum the block partials in a fixed order, then the scalar
+// update.  Eight warps from kWideScalar partials on: one warp adds 2048 (256^3) in a chain of
+// 64, 6.3 us against 2.5 for a few.
+constexpr int kWideScalar = 256;
+template <int W>
+__global__ void __launch_bounds__(256) k_scalar(const double* __restrict__ partial, int nblk, SolveScalars* __restrict__ sc, int n,
                          const int* __restrict__ act, int mode, double tol2, int max_iter, int inner_iters,
                          const SolveScalars* __restrict__ outer) {
   pdl_entry();
-  const int t = blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5);
-  const int lane = threadIdx.x & 31;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int t = W == 1 ? blockIdx.x * 8 + warp : blockIdx.x;
   if (t >= n) return;
   const int s = act != nullptr ? act[t] : t;
   SolveScalars& c = sc[s];
-  if (mode == SM_INNER_BEGIN) {
+  if (mode == SM_INNER_BEGIN) {  // (no sums: one warp per sample)
     if (lane == 0) c.active = outer[s].active;
     return;
   }
@@ -145,8 +160,17 @@ __global__ void k_scalar(const double* __restrict__ partial, int nblk, SolveScal
   }
   if (mode != SM_INIT && !c.active) return;
   double v = 0.0;
-  for (int t = lane; t < nblk; t += 32) v += partial[(long long)s * nblk + t];
+  for (int t = W == 1 ? lane : (int)threadIdx.x; t < nblk; t += 32 * W) v += partial[(long long)s * nblk + t];
   v = warp_sum(v);
+  if constexpr (W > 1) {
+    __shared__ double sums[W];
+    if (lane == 0) sums[warp] = v;
+    __syncthreads();
+    if (warp != 0) return;
+    v = lane < W ? sums[lane] : 0.0;
+#pragma unroll
+    for (int o = W / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  }
   if (lane != 0) return;
   switch (mode) {
     case SM_INIT:
@@ -272,13 +296,19 @@ __global__ void k_restrict(const T* __restrict__ tf, T* __restrict__ rc, const S
 }
 
 // The same restriction marching in z: one thread per coarse node column (I, J) and
-// chunk of kRestrictPlanes coarse planes (blockIdx.z); the xy-weighted sum of fine
+// chunk of `planes` coarse planes (blockIdx.z); the xy-weighted sum of fine
 // plane 2K+1 serves coarse planes K and K+1, so a coarse node reads 18 fine values
-// instead of 27.  rc holds 0 on the coarse boundary.
-constexpr int kRestrictPlanes = 8;
+// instead of 27.  rc holds 0 on the coarse boundary.  Eight planes a chunk, fewer when
+// that gives less than about four blocks per SM (one 256^3 sample, 128^3 to 64^3: 153
+// blocks of eight planes are a chain of 17 loads, 8 us).
+static int restrict_planes(unsigned cols, int n, int Nc) {
+  int planes = 8;
+  while (planes > 2 && (long long)cols * n * ((Nc + planes) / planes) < 4 * 152) planes /= 2;
+  return planes;
+}
 template <typename T, int NCC>
 __global__ void k_restrict_zm(const T* __restrict__ tf, T* __restrict__ rc, const SolveScalars* __restrict__ sc,
-                              const int* __restrict__ act) {
+                              const int* __restrict__ act, int planes) {
   pdl_entry();
   SAMPLE_GUARD(sc);
   constexpr int Nc = NCC, n1c = Nc + 1, n1f = 2 * Nc + 1;
@@ -286,7 +316,7 @@ __global__ void k_restrict_zm(const T* __restrict__ tf, T* __restrict__ rc, cons
   const int col = blockIdx.x * blockDim.x + threadIdx.x;
   if (col >= n1c * n1c) return;
   const int I = col % n1c, J = col / n1c;
-  const int K0 = kRestrictPlanes * (int)blockIdx.z, K1 = min(Nc, K0 + kRestrictPlanes - 1);
+  const int K0 = planes * (int)blockIdx.z, K1 = min(Nc, K0 + planes - 1);
   T* out = rc + s * nc + col;
   if (I == 0 || J == 0 || I == Nc || J == Nc) {
     for (int K = K0; K <= K1; ++K) out[K * (n1c * n1c)] = T(0);
@@ -794,10 +824,11 @@ static int vcycle(SolverBufs& B, const T* r0, const TA0* a0, const SolveScalars*
       const double rb = nbytes<T, T>(Nj, n, 1, 0) + nbytes<T, T>(Nj / 2, n, 1, 0);
       if constexpr (NCC >= 32) {  // on smaller grids the per-node kernel has more threads in flight
         const int n1c = Nj / 2 + 1;
-        const dim3 gr((unsigned)((n1c * n1c + kBlock - 1) / kBlock), (unsigned)n,
-                      (unsigned)((Nj / 2 + kRestrictPlanes) / kRestrictPlanes));
+        const unsigned cols = (unsigned)((n1c * n1c + kBlock - 1) / kBlock);
+        const int planes = restrict_planes(cols, n, Nj / 2);
+        const dim3 gr(cols, (unsigned)n, (unsigned)((Nj / 2 + planes) / planes));
         launch(cls<T>("restrict", fine), rb, k_restrict_zm<T, NCC>, gr, kBlock, 0, st, (const T*)B.vt[j],
-               (T*)B.vr[j + 1], sc, act);
+               (T*)B.vr[j + 1], sc, act, planes);
       } else {
         launch(cls<T>("restrict", fine), rb, k_restrict<T, NCC>, grid_nodes(Nj / 2, n), kBlock, 0, st,
                (const T*)B.vt[j], (T*)B.vr[j + 1], sc, Nj / 2, act);
@@ -854,9 +885,9 @@ static int vcycle(SolverBufs& B, const T* r0, const TA0* a0, const SolveScalars*
 
 static void scalar(SolverBufs& B, SolveScalars* sc, int mode, double tol2, int max_iter, cudaStream_t st, int nblk,
                    int inner_iters = 0, const SolveScalars* outer = nullptr) {
-  const int warps = 8;
-  launch("scalar", 0.0, k_scalar, dim3((B.n_act + warps - 1) / warps), 32 * warps, 0, st, (const double*)B.partial,
-         nblk, sc, B.n_act, B.actp, mode, tol2, max_iter, inner_iters, outer);
+  const bool wide = nblk >= kWideScalar && mode != SM_INNER_BEGIN && mode != SM_OUTER_STEP;
+  launch("scalar", 0.0, wide ? k_scalar<8> : k_scalar<1>, dim3(wide ? B.n_act : (B.n_act + 7) / 8), 256, 0, st,
+         (const double*)B.partial, nblk, sc, B.n_act, B.actp, mode, tol2, max_iter, inner_iters, outer);
 }
 
 // All samples launched again (the start of a solve).
@@ -900,6 +931,7 @@ static cudaError_t pcg_loop(SolverBufs& B, const TAop* aop, const TA0* a0, T* x,
   T* q = (T*)B.q;
   const T* z = (const T*)B.vt[0];
   auto g = [&]() { return grid_nodes(N, B.n_act); };
+  auto gu = [&]() { return dim3((unsigned)update_blocks(N), (unsigned)B.n_act); };
   auto precondition = [&](int mode) {
     const int nrz = vcycle<T, TA0>(B, r, a0, sc, omega, st);
     if (nrz == 0) {
@@ -933,13 +965,13 @@ static cudaError_t pcg_loop(SolverBufs& B, const TAop* aop, const TA0* a0, T* x,
     }
     scalar(B, sc, SM_ALPHA, 0, 0, st, napply);
     if (fixed_iters > 0) {
-      launch(cls<T>("update", true), nbytes<T, T>(N, B.n_act, 6, 0), k_update_xr<T, false>, g(), kBlock, 0, st, x, r,
+      launch(cls<T>("update", true), nbytes<T, T>(N, B.n_act, 6, 0), k_update_xr<T, false>, gu(), kBlock, 0, st, x, r,
              (const T*)p, (const T*)q, B.partial, (const SolveScalars*)sc, nodes, B.actp);
       if (it == nit - 1) break;
     } else {
-      launch(cls<T>("update", true), nbytes<T, T>(N, B.n_act, 6, 0), k_update_xr<T, true>, g(), kBlock, 0, st, x, r,
+      launch(cls<T>("update", true), nbytes<T, T>(N, B.n_act, 6, 0), k_update_xr<T, true>, gu(), kBlock, 0, st, x, r,
              (const T*)p, (const T*)q, B.partial, (const SolveScalars*)sc, nodes, B.actp);
-      scalar(B, sc, SM_CONV, tol2, prm.max_iter, st, nb);
+      scalar(B, sc, SM_CONV, tol2, prm.max_iter, st, update_blocks(N));
       if ((it + 1) % prm.check_every == 0 || it + 1 == nit) {
         int n = 0;
         cudaError_t e = compact_active(B, sc, st, n);
