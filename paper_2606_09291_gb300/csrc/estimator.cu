@@ -650,16 +650,15 @@ __global__ void __launch_bounds__(kBlock) k_level_field(const void* __restrict__
   if (threadIdx.x == 0) partial[blockIdx.x] = hc * hc * hc * bs;
 }
 
-// k_level_field for pairs on both grids, the fine one RF (1 or 2) times coarser than the
-// control grid: the bulk of a difference level's statistics.  The FP32 pair arithmetic and
+// k_level_field for pairs on both grids, the fine one the control grid: the bulk of the
+// finest difference level's statistics.  The FP32 pair arithmetic and
 // the FP64 sums (four operations per cell and sample) take about the same time, and the
 // 16 scattered loads need threads in flight: 64 registers, four blocks per SM.  G = 4
 // splits the samples of a cell over four threads (their sums joined in a fixed order), for
 // batches on control grids too small to fill the SMs with one thread per cell: 512 samples
-// of 64^3 on a 64^3 control: 1.6 ms; 4
-// samples of 128^3 on 256^3: 2.8 ms with the divisions and a block sum per 256 cells, 0.94 ms now.
+// of 64^3 on a 64^3 control: 1.6 ms.
 constexpr int kPairBlocks = 4 * 152;
-template <int RF, int G>
+template <int G>
 __global__ void __launch_bounds__(kBlock, 4) k_level_pairs(const float2* __restrict__ qf, int Nf,
                                                            const float2* __restrict__ qc, int S, int Nc, double inv_s,
                                                            const double* __restrict__ work, double* __restrict__ field,
@@ -678,8 +677,8 @@ __global__ void __launch_bounds__(kBlock, 4) k_level_pairs(const float2* __restr
     const unsigned c = c0 + tc < ncell ? c0 + tc : ncell - 1;
     const unsigned row = c / (unsigned)Nc;
     const int cx = (int)(c - row * Nc), cz = (int)(row / (unsigned)Nc), cy = (int)(row - (unsigned)cz * Nc);
-    PairInterp<RF> Pf;
-    PairInterp<2 * RF> Pc;
+    PairInterp<1> Pf;
+    PairInterp<2> Pc;
     Pf.setup(Nf, cx, cy, cz);
     Pc.setup(Ncs, cx, cy, cz);
     auto value = [&](int s, const float2* f, const float2* k) {
@@ -754,7 +753,7 @@ __global__ void __launch_bounds__(kBlock) k_lvl_x(QF* __restrict__ qf, int Nf, c
                                                   const double* __restrict__ work) {
   pdl_entry();
   const int s = blockIdx.y;
-  const int n1 = Nf + 1, nodes = n1 * n1 * n1;  // at most 257^3 (the control grid is 4x finer)
+  const int n1 = Nf + 1, nodes = n1 * n1 * n1;  // at most 513^3 (the control grid is finer)
   const int n = blockIdx.x * blockDim.x + threadIdx.x;
   if (n >= nodes) return;
   int i, j, k;
@@ -1012,10 +1011,11 @@ void launch_level_stats(const double* qf, const double* phif, int Nf, const doub
   if (S == 0) return;
   launch("level_scalars", 0.0, k_level_scalars, dim3(1), kBlock, 0, st, phif, phic, S, theta, scalars, work, iters,
          status);
-  // levels at least 4x coarser than the control grid (per axis): statistics on the level
-  // grid (cost ~ level nodes and cells per sample instead of control cells per sample;
-  // at 2x the control-cell path in pair arithmetic is cheaper).  q_f is overwritten.
-  if (nodebuf && 4 * Nf <= Nc) {
+  // levels coarser than the control grid: statistics on the level grid (cost ~ level nodes
+  // per sample instead of control cells per sample; at 2x the whole FP64 level 3 of a run
+  // 18.87 -> 18.52 ms, 4 samples of 128^3 in pairs on a 256^3 control 11.63 -> 11.47, 300 of
+  // 32^3 on 64^3 7.83 -> 7.64).  q_f is overwritten.
+  if (nodebuf && 2 * Nf <= Nc) {
     const int nb = (qf_pairs && qc_pairs) ? launch_lvl<float2, float2>(qf, Nf, qc, S, Nc, work, field, partial, nodebuf, st)
                    : qf_pairs             ? launch_lvl<float2, double>(qf, Nf, qc, S, Nc, work, field, partial, nodebuf, st)
                                           : launch_lvl<double, double>(qf, Nf, qc, S, Nc, work, field, partial, nodebuf, st);
@@ -1026,13 +1026,12 @@ void launch_level_stats(const double* qf, const double* phif, int Nf, const doub
   const long long ncell = (long long)Nc * Nc * Nc;
   const int nblk = cell_blocks(ncell);
   const double qbytes = (double)S * 8 * (nodes_of(Nf) + (qc ? nodes_of(Ncoarse) : 0));
-  // both grids in pairs, the fine one the control grid or one level below it
-  if (qf_pairs && qc_pairs && (Nf == Nc || 2 * Nf == Nc)) {
+  // both grids in pairs, the fine one the control grid
+  if (qf_pairs && qc_pairs && Nf == Nc) {
     const bool split = S >= 16 && ncell < (long long)kPairBlocks * kBlock * 4;
     const int cb = split ? kBlock / 4 : kBlock;
     const int nb = (int)std::min<long long>((ncell + cb - 1) / cb, split ? kPairBlocks : cell_blocks(ncell));
-    auto kp = Nf == Nc ? (split ? k_level_pairs<1, 4> : k_level_pairs<1, 1>)
-                       : (split ? k_level_pairs<2, 4> : k_level_pairs<2, 1>);
+    auto kp = split ? k_level_pairs<4> : k_level_pairs<1>;
     launch_flops("level_field", qbytes + (double)ncell * 16, (double)S * ncell * 4.0, kp, dim3(nb), kBlock, 0, st,
                  (const float2*)qf, Nf, (const float2*)qc, S, Nc, 1.0 / S, (const double*)work, field, partial);
     launch("level_finish", 0.0, k_level_finish, dim3(1), kBlock, 0, st, (const double*)partial, nb, (const double*)work,
