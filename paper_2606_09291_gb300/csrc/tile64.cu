@@ -71,8 +71,10 @@ struct Args {
   int N, nzc, zc, nseg, first;
 };
 
-template <int MODE>
-__global__ void __launch_bounds__(kT, 2) k_tile64(Args A) {
+// OCC: blocks per SM the registers allow.  Three (80 registers, a few spilled) where the
+// launch has more than two blocks per SM, else two without spills.
+template <int MODE, int OCC>
+__global__ void __launch_bounds__(kT, OCC) k_tile64(Args A) {
   // launched after the kernel before has ended and without letting the next one's blocks in:
   // placed early, blocks share SMs unevenly (FP64 level 3 of a run: 22.7 ms, 20.7 without)
   extern __shared__ __align__(16) unsigned char smraw[];
@@ -328,6 +330,17 @@ int tiles_x(int N) { return (N - 1 + kW - 1) / kW; }
 int tiles_y(int N) { return (N - 1 + kH - 1) / kH; }
 int segments(int N) { return (N - 1 + kSeg - 1) / kSeg; }
 
+template <int MODE, int OCC>
+void run_occ(const char* cls, double bytes, const Args& A, dim3 grid, cudaStream_t st) {
+  constexpr size_t smem = sizeof(Smem<MODE>);
+  static_assert(smem + 1024 <= 228 * 1024 / 3, "three blocks per SM");
+  static bool smem_set = false;  // once per instantiation (capture-friendly)
+  if (!smem_set) {
+    cudaFuncSetAttribute(k_tile64<MODE, OCC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    smem_set = true;
+  }
+  launch_after(cls, bytes, k_tile64<MODE, OCC>, grid, dim3(kT), smem, st, A);
+}
 template <int MODE>
 void run(const char* cls, double bytes, Args A, const Batch& bt, cudaStream_t st) {
   const int bx = tiles_x(A.N), by = tiles_y(A.N), nseg = segments(A.N);
@@ -335,11 +348,11 @@ void run(const char* cls, double bytes, Args A, const Batch& bt, cudaStream_t st
   // fullest SM; a chunk costs about 0.6 planes more than it has (the cell layer and the
   // operand planes before its first), and one block alone leaves the pipe idle a quarter of
   // the time (9 samples of 64^3: 20.6 ms a solve pair with one block per SM, 17.7 with two).
+  auto per_sm = [&](int q) { return ((long long)bx * by * bt.n * ((nseg + q - 1) / q) + 151) / 152; };
   int spc = nseg;
   double best = 1e300;
   for (int q = 1; q <= nseg; ++q) {
-    const long long blocks = (long long)bx * by * bt.n * ((nseg + q - 1) / q);
-    const double cost = (blocks <= 152 ? 1.35 : (double)((blocks + 151) / 152)) * (kSeg * q + 0.6);
+    const double cost = (per_sm(q) == 1 ? 1.35 : (double)per_sm(q)) * (kSeg * q + 0.6);
     if (cost < best) { best = cost; spc = q; }
   }
   if (bt.zchunks > 0) spc = (nseg + bt.zchunks - 1) / bt.zchunks;
@@ -347,14 +360,12 @@ void run(const char* cls, double bytes, Args A, const Batch& bt, cudaStream_t st
   A.nzc = (nseg + spc - 1) / spc;
   A.zc = spc * kSeg;
   A.act = bt.act;
-  constexpr size_t smem = sizeof(Smem<MODE>);
-  static_assert(smem + 1024 <= 228 * 1024 / 3, "three blocks per SM");
-  static bool smem_set = false;  // once per instantiation (capture-friendly)
-  if (!smem_set) {
-    cudaFuncSetAttribute(k_tile64<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    smem_set = true;
-  }
-  launch_after(cls, bytes, k_tile64<MODE>, dim3(bx, by, (unsigned)(bt.n * A.nzc)), dim3(kT), smem, st, A);
+  const dim3 grid(bx, by, (unsigned)(bt.n * A.nzc));
+  // three blocks per SM against two, a solve pair: 3 samples of 64^3 7.1 against 8.5 ms, 16 25.9
+  // against 26.7, one of 128^3 15.2 against 16.0; with at most two there the spills cost:
+  // 9 of 64^3 14.5 against 14.3, 9 of 32^3 3.60 against 3.52
+  if (per_sm(spc) > 2) run_occ<MODE, 3>(cls, bytes, A, grid, st);
+  else run_occ<MODE, 2>(cls, bytes, A, grid, st);
 }
 
 double vbytes(int N, int n, double vec, double coef) {
