@@ -150,17 +150,18 @@ __global__ void __launch_bounds__(256) k_scalar(const double* __restrict__ parti
   if (t >= n) return;
   const int s = act != nullptr ? act[t] : t;
   SolveScalars& c = sc[s];
+  const SolveScalars o = c;  // read with the partial sums, not after them
   if (mode == SM_INNER_BEGIN) {  // (no sums: one warp per sample)
     if (lane == 0) c.active = outer[s].active;
     return;
   }
   if (mode == SM_OUTER_STEP) {
-    if (lane == 0 && c.active) { c.iters += 1; c.pad += inner_iters; }
+    if (lane == 0 && o.active) { c.iters = o.iters + 1; c.pad = o.pad + inner_iters; }
     return;
   }
-  if (mode != SM_INIT && !c.active) return;
   double v = 0.0;
   for (int t = W == 1 ? lane : (int)threadIdx.x; t < nblk; t += 32 * W) v += partial[(long long)s * nblk + t];
+  if (mode != SM_INIT && !o.active) return;
   v = warp_sum(v);
   if constexpr (W > 1) {
     __shared__ double sums[W];
@@ -179,20 +180,18 @@ __global__ void __launch_bounds__(256) k_scalar(const double* __restrict__ parti
       if (!(v < INFINITY)) { c.active = 0; c.status = 2; }
       break;
     case SM_RZ0: c.rz = v; break;
-    case SM_ALPHA: c.alpha = (v > 0.0 && c.rz != 0.0) ? c.rz / v : 0.0; break;
+    case SM_ALPHA: c.alpha = (v > 0.0 && o.rz != 0.0) ? o.rz / v : 0.0; break;
+    case SM_BETA: c.beta = (o.rz != 0.0) ? v / o.rz : 0.0; c.rz = v; break;
     case SM_CONV:
-      c.rr = v; c.iters += 1;
-      if (v <= tol2 * c.bb) c.active = 0;
-      else if (!(v < INFINITY)) { c.active = 0; c.status = 2; }
-      else if (c.iters >= max_iter) { c.active = 0; c.status = 1; }
-      break;
-    case SM_BETA: c.beta = (c.rz != 0.0) ? v / c.rz : 0.0; c.rz = v; break;
-    case SM_OUTER_CONV:
+    case SM_OUTER_CONV: {
+      const int iters = o.iters + (mode == SM_CONV ? 1 : 0);
       c.rr = v;
-      if (v <= tol2 * c.bb) c.active = 0;
+      c.iters = iters;
+      if (v <= tol2 * o.bb) c.active = 0;
       else if (!(v < INFINITY)) { c.active = 0; c.status = 2; }
-      else if (c.iters >= max_iter) { c.active = 0; c.status = 1; }
+      else if (iters >= max_iter) { c.active = 0; c.status = 1; }
       break;
+    }
   }
 }
 
