@@ -12,13 +12,13 @@
 // iteration) and, on 16^3, the shared-memory loads of three 21-point stencils; FP64 in one
 // warp (64 clocks an operation) is kept out of the inner iterations.
 // Measured (three refinement steps of six iterations, state or adjoint): 1024 samples of
-// 8^3 310 us a solve against 2.2 ms in passes, 256 of 16^3 320 us against 3.1 ms, 64 of
+// 8^3 180 us a solve (310 with a thread per node instead of per interior node) against 2.2 ms
+// in passes, 256 of 16^3 320 us against 3.1 ms, 64 of
 // 16^3 200 us against 1.6 ms.
 //
 // Arithmetic: that of the pass-by-pass solver on the same grid (solver.cu for 8^3: FP64
-// refinement residual and solution, partial sums per 256 consecutive nodes; tiled.cu for
-// 16^3: solution and b as FP32 pairs, partial sums per thread over 8 planes and the rows of
-// a thread), except that the 4^3 and 2^3 levels are one matrix (coarse4_build) and alpha and
+// refinement residual and solution; tiled.cu for 16^3: solution and b as FP32 pairs, partial
+// sums per thread over 8 planes and the rows of a thread), except that the 4^3 and 2^3 levels are one matrix (coarse4_build) and alpha and
 // beta are quotients of pairs.
 #include "internal.cuh"
 #include "kernels.h"
@@ -62,17 +62,15 @@ __device__ __forceinline__ float coarsen_cell(const float* af, int c, int Nc) {
 }
 
 // ---------------------------------------------------------------- 8^3
-// thread n < 729 owns node n; partial sums per 256 consecutive nodes (warps 0-7, 8-15,
-// 16-23), then over the three of them, as block_sum and k_scalar form them
-constexpr int kT8 = 768;
+// a thread per interior node (343): 11 warps and four blocks per SM, where one per node (729)
+// left half the lanes of every step idle in 24 warps and two blocks
+constexpr int kT8 = 352, kW8 = kT8 / 32;
 
-template <typename T>
-__device__ __forceinline__ double sum_groups(T v) {  // lane l holds warp l's sum (l < 24, else 0)
+__device__ __forceinline__ double sum_groups(double v) {  // lane l holds warp l's sum (l < 24, else 0)
 #pragma unroll
   for (int o = 4; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  double p = (double)v;  // lanes 8g: the block sum of group g
-  const double p0 = __shfl_sync(0xffffffffu, p, 0), p1 = __shfl_sync(0xffffffffu, p, 8),
-               p2 = __shfl_sync(0xffffffffu, p, 16);
+  const double p0 = __shfl_sync(0xffffffffu, v, 0), p1 = __shfl_sync(0xffffffffu, v, 8),
+               p2 = __shfl_sync(0xffffffffu, v, 16);  // lanes 8g: the block sum of group g
   return (p0 + p2) + p1;
 }
 
@@ -92,26 +90,32 @@ __device__ __forceinline__ float df_quotient(DF a, DF b, bool ok) {
 
 struct Smem8 {
   double xd[729];       // solution for the refinement residual
-  double redd[24];
+  double redd[kW8];
   float a32[512], abf[512];
   float op[729];        // operand of A p
   float r8[729];        // residual of the V-cycle
   float lv[kLv8];
-  float redf[2][24];
+  float redf[2][kW8];
   int go;
 };
 
-__global__ void __launch_bounds__(kT8, 2) k_small8(SmallArgs A) {
+__global__ void __launch_bounds__(kT8, 4) k_small8(SmallArgs A) {
   pdl_entry();
   __shared__ Smem8 M;
-  const int s = blockIdx.x, n = threadIdx.x, lane = n & 31, warp = n >> 5;
+  const int s = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const float omega = A.omega;
-  for (int c = n; c < 512; c += kT8) {
+  for (int c = tid; c < 512; c += kT8) {
     M.a32[c] = A.a32[(long long)s * 512 + c];
     M.abf[c] = __bfloat162float(A.abf[(long long)s * 512 + c]);
   }
-  if (n < 729) M.op[n] = M.r8[n] = 0.f;
-  for (int e = n; e < kLv8; e += kT8) M.lv[e] = 0.f;
+  const bool in = tid < 343;  // the thread's interior node
+  const int i = 1 + tid % 7, j = 1 + (tid / 7) % 7, k = 1 + tid / 49, n = in ? i + 9 * (j + 9 * k) : 0;
+  const double bv = in ? A.b[s * A.bstride + n] : 0.0;  // b is 0 on the boundary
+  for (int e = tid; e < 729; e += kT8) {
+    M.op[e] = M.r8[e] = 0.f;
+    M.xd[e] = 0.0;
+  }
+  for (int e = tid; e < kLv8; e += kT8) M.lv[e] = 0.f;
   CoarseLevels L;
   L.r8 = M.r8; L.a8 = M.abf;
   L.x8 = M.lv; L.t8 = L.x8 + 729;
@@ -119,15 +123,11 @@ __global__ void __launch_bounds__(kT8, 2) k_small8(SmallArgs A) {
   float* a4 = L.s4 + 54;
   float* a2 = a4 + 64;
   L.x4 = nullptr; L.a4 = a4; L.a2 = a2;
-  int i = 0, j = 0, k = 0;
-  if (n < 729) node_ijk(n, 9, i, j, k);
-  const bool in = n < 729 && interior(i, j, k, 8);
-  const double bv = n < 729 ? A.b[s * A.bstride + n] : 0.0;
   __syncthreads();
-  if (n < 64) a4[n] = coarsen_cell(M.abf, n, 4);
+  if (tid < 64) a4[tid] = coarsen_cell(M.abf, tid, 4);
   const float w8 = in ? omega / diag_of<8>(M.abf, i, j, k) : 0.f;
   __syncthreads();
-  if (n < 8) a2[n] = coarsen_cell(a4, n, 2);
+  if (tid < 8) a2[tid] = coarsen_cell(a4, tid, 2);
   __syncthreads();
   coarse4_build<kT8>(L, omega);
   Outer o{0.0, 0.0, 0.0, 0, 0, 0};
@@ -136,27 +136,32 @@ __global__ void __launch_bounds__(kT8, 2) k_small8(SmallArgs A) {
     v = warp_sum(v);
     if (lane == 0) M.redd[warp] = v;
     __syncthreads();
-    return warp == 0 ? sum_groups<double>(lane < 24 ? M.redd[lane] : 0.0) : 0.0;
+    double g = 0.0;
+    if (warp == 0) {
+      g = lane < kW8 ? M.redd[lane] : 0.0;
+#pragma unroll
+      for (int o = 8; o > 0; o >>= 1) g += __shfl_xor_sync(0xffffffffu, g, o);
+    }
+    return g;
   };
-  // block sum of a float as a pair, in every thread: the three group sums are added exactly
-  // (FP64 additions and a division in one warp were a quarter of an iteration)
+  // block sum of a float as a pair, in every thread (FP64 additions and a division in one
+  // warp were a quarter of an iteration)
   int par = 0;
   auto sum32 = [&](float v) {
     v = warp_sum(v);
     if (lane == 0) M.redf[par][warp] = v;
     __syncthreads();
-    float g = lane < 24 ? M.redf[par][lane] : 0.f;
+    DF g{lane < kW8 ? M.redf[par][lane] : 0.f, 0.f};
 #pragma unroll
-    for (int o = 4; o > 0; o >>= 1) g += __shfl_xor_sync(0xffffffffu, g, o);
-    const float p0 = __shfl_sync(0xffffffffu, g, 0), p1 = __shfl_sync(0xffffffffu, g, 8),
-                p2 = __shfl_sync(0xffffffffu, g, 16);
+    for (int o = 8; o > 0; o >>= 1)
+      g = df_add(g, DF{__shfl_xor_sync(0xffffffffu, g.h, o), __shfl_xor_sync(0xffffffffu, g.l, o)});
     par ^= 1;
-    return df_add(df_add(DF{p0, 0.f}, DF{p2, 0.f}), DF{p1, 0.f});
+    return DF{__shfl_sync(0xffffffffu, g.h, 0), __shfl_sync(0xffffffffu, g.l, 0)};
   };
   DF rz{0.f, 0.f};  // r . z
   {
     const double v = sum64(bv * bv);
-    if (n == 0) {
+    if (tid == 0) {
       o.bb = o.rr = v;
       bool go = v > 0.0;
       if (!(v < INFINITY)) { go = false; o.status = 2; }
@@ -169,7 +174,7 @@ __global__ void __launch_bounds__(kT8, 2) k_small8(SmallArgs A) {
   for (int step = 0; go; ++step) {
     double r64 = bv;
     if (step > 0) {  // r = b - A x in FP64
-      if (n < 729) M.xd[n] = x;
+      if (in) M.xd[n] = x;
       __syncthreads();
       r64 = 0.0;
       if (in) {
@@ -188,7 +193,7 @@ __global__ void __launch_bounds__(kT8, 2) k_small8(SmallArgs A) {
         r64 = bv - (1.0 / (12.0 * 8)) * q1_row(C, (const double*)M.xd, i, j, k, 9);
       }
       const double v = sum64(r64 * r64);
-      if (n == 0) M.go = outer_go(o, v, A.tol2, A.cap);
+      if (tid == 0) M.go = outer_go(o, v, A.tol2, A.cap);
       __syncthreads();
       go = M.go != 0;
       if (!go) break;
@@ -197,13 +202,13 @@ __global__ void __launch_bounds__(kT8, 2) k_small8(SmallArgs A) {
     const int inner = step == 0 ? A.inner : A.inner_next;
     float r = (float)r64, d = 0.f, p = 0.f;
     for (int it = 0;; ++it) {
-      if (n < 729) M.r8[n] = r;
+      if (in) M.r8[n] = r;
       __syncthreads();
       const float z = vcycle8<kT8, true>(L, n, i, j, k, in, w8, omega);
       const DF rzn = sum32(r * z);
       p = it > 0 ? z + df_quotient(rzn, rz, rz.h != 0.f) * p : z;
       rz = rzn;
-      if (n < 729) M.op[n] = p;
+      if (in) M.op[n] = p;
       __syncthreads();
       float q = 0.f;
       if (in) {
@@ -218,11 +223,14 @@ __global__ void __launch_bounds__(kT8, 2) k_small8(SmallArgs A) {
       r = r - al * q;
     }
     x += (double)d;
-    if (n == 0) { o.iters += 1; o.pad += inner; }
+    if (tid == 0) { o.iters += 1; o.pad += inner; }
   }
   o.rz = df_to_double(rz);
-  if (n < 729) A.x64[(long long)s * 729 + n] = x;
-  if (n == 0) store_scalars(A.sc + s, o);
+  __syncthreads();
+  if (in) M.xd[n] = x;  // the boundary is 0
+  __syncthreads();
+  for (int e = tid; e < 729; e += kT8) A.x64[(long long)s * 729 + e] = M.xd[e];
+  if (tid == 0) store_scalars(A.sc + s, o);
 }
 
 // ---------------------------------------------------------------- 16^3
@@ -385,7 +393,7 @@ __global__ void __launch_bounds__(kT16, 1) k_small16(SmallArgs A) {
     }
     __syncthreads();
     if (warp == 0) {
-      v = sum_groups<double>(lane < 24 ? M.redd[lane] : 0.0);
+      v = sum_groups(lane < 24 ? M.redd[lane] : 0.0);
       if (lane == 0) {
         o.bb = o.rr = v;
         bool go = v > 0.0;
