@@ -112,7 +112,7 @@ size_t level_bytes(const mlsgd_ctx* ctx, int level, int S) {
   b += al(kl_gemm_a_bytes(S, ctx->cfg.n_modes));
   b += solve_scratch_bytes(ctx, N, S);
   b += al((4 + 4 * (size_t)S) * 8) + al((size_t)level_partial_cap(ctx->Nc(), N) * 8);
-  b += al(2 * (size_t)nodes_of(N) * 8);
+  b += al((size_t)nodes_of(N) * 8);
   return b;
 }
 
@@ -665,7 +665,7 @@ mlsgd_status mlsgd_level_gradient(mlsgd_ctx* ctx, int iter, int level, int64_t f
     __nv_bfloat16* gemm_a = bp.take<__nv_bfloat16>((size_t)S * K);
     double* work = bp.take<double>(4 + 4 * (size_t)S);
     double* spartial = bp.take<double>((size_t)level_partial_cap(ctx->Nc(), N));
-    double* lvl_nodes = bp.take<double>(2 * (size_t)nodes_of(N));
+    double* lvl_nodes = bp.take<double>((size_t)nodes_of(N));
     char* scratch = bp.p;
     launch_draw_xi(ctx->cfg.seed, iter, level, first_sample + done, S, K, xi, st, ctx->xi_half_width());
     s = make_field(ctx, xi, level, S, ff, nullptr, st, gemm_a);

@@ -657,7 +657,6 @@ __global__ void __launch_bounds__(kBlock) k_level_field(const void* __restrict__
 // splits the samples of a cell over four threads (their sums joined in a fixed order), for
 // batches on control grids too small to fill the SMs with one thread per cell: 512 samples
 // of 64^3 on a 64^3 control: 1.6 ms.
-constexpr int kPairBlocks = 4 * 152;
 template <int G>
 __global__ void __launch_bounds__(kBlock, 4) k_level_pairs(const float2* __restrict__ qf, int Nf,
                                                            const float2* __restrict__ qc, int S, int Nc, double inv_s,
@@ -1030,7 +1029,8 @@ void launch_level_stats(const double* qf, const double* phif, int Nf, const doub
   if (qf_pairs && qc_pairs && Nf == Nc) {
     const bool split = S >= 16 && ncell < (long long)kPairBlocks * kBlock * 4;
     const int cb = split ? kBlock / 4 : kBlock;
-    const int nb = (int)std::min<long long>((ncell + cb - 1) / cb, split ? kPairBlocks : cell_blocks(ncell));
+    const int nb = (int)std::min<long long>({(ncell + cb - 1) / cb, split ? kPairBlocks : cell_blocks(ncell),
+                                             level_partial_cap(Nc, Nf)});
     auto kp = split ? k_level_pairs<4> : k_level_pairs<1>;
     launch_flops("level_field", qbytes + (double)ncell * 16, (double)S * ncell * 4.0, kp, dim3(nb), kBlock, 0, st,
                  (const float2*)qf, Nf, (const float2*)qc, S, Nc, 1.0 / S, (const double*)work, field, partial);

@@ -56,10 +56,13 @@ struct SolveScalars {
 __host__ __device__ inline long long nodes_of(int N) { return (long long)(N + 1) * (N + 1) * (N + 1); }
 __host__ __device__ inline long long cells_of(int N) { return (long long)N * N * N; }
 inline int node_blocks(int N) { return (int)((nodes_of(N) + 255) / 256); }
+constexpr int kPairBlocks = 4 * 152;  // at most, of the statistics that split a cell's samples over threads
 // block partials one level's statistics may write (control-cell blocks + level-cell
-// blocks + slack); the buffer is sized with this and the kernels stay within it
+// blocks + slack, or the split form's blocks, which are more on a 32^3 control grid: 512
+// against 320); the buffer is sized with this and every launch stays within it
 inline long long level_partial_cap(int Nc, int Nf) {
-  return (cells_of(Nc) + 255) / 256 + (cells_of(Nf) + 255) / 256 + 64;
+  const long long n = (cells_of(Nc) + 255) / 256 + (cells_of(Nf) + 255) / 256 + 64;
+  return Nf == Nc && Nc >= 32 && n < kPairBlocks ? kPairBlocks : n;
 }
 
 // The samples one launch processes: a batch of S samples, of which n are launched (the z
