@@ -18,8 +18,11 @@
 //
 // Arithmetic: that of the pass-by-pass solver on the same grid (solver.cu for 8^3: FP64
 // refinement residual and solution; tiled.cu for 16^3: solution and b as FP32 pairs, partial
-// sums per thread over 8 planes and the rows of a thread), except that the 4^3 and 2^3 levels are one matrix (coarse4_build) and alpha and
-// beta are quotients of pairs.
+// sums per thread over 8 planes and the rows of a thread), except that the 4^3 and 2^3 levels
+// are one matrix (coarse4_build) and that the sums of the FP32 partial sums of r.z and p.q, and
+// their quotients alpha and beta, are formed in FP32 pairs (46 bits) while those hold them, in
+// FP64 beyond (alpha64); alpha and beta are FP32 numbers either way.  30 drawn calls on 8^3 and
+// 16^3 against 64 bits: 1.001 times the pass-by-pass solver's error, by rtol in both.
 #include "internal.cuh"
 #include "kernels.h"
 #include "launch.h"
@@ -88,15 +91,46 @@ __device__ __forceinline__ float df_quotient(DF a, DF b, bool ok) {
   return fabsf(c) < INFINITY ? __fadd_rn(q, c) : q;
 }
 
+// alpha = rz / pq and beta = rz / rz_old from pairs; NaN where a sum is beyond FP32 (its pair is NaN)
+__device__ __forceinline__ float pair_alpha(DF rz, DF pq) {
+  return df_quotient(rz, pq, !(pq.h <= 0.f) && rz.h != 0.f);
+}
+__device__ __forceinline__ float pair_beta(DF rz, DF old) { return df_quotient(rz, old, old.h != 0.f); }
+// Then they are formed again from the partial sums, M.redf[0] of r.z and M.redf[1] of p.q, by
+// FP64 sums and quotients, those of the pass-by-pass solver (SM_ALPHA, SM_BETA in solver.cu):
+// a right-hand side whose products leave the FP32 range ends as it does there.  Small sums
+// need no such care: from 2^-100 down the pairs' error tends to 2^-149, still under the
+// rounding of the FP32 partial sums themselves.  Out of line and with no state but M.rz (the
+// last FP64 r.z), since the inner iterations have no register to spare: a level gradient of 1024
+// samples of 8^3 took 729 us without this and 735 with it, 64 samples of 16^3 the same (FP64
+// forms of the inner or the whole solve beside the pairs': 0.7 to 3% more on 8^3, 6% on 16^3).
+// Every thread calls them with the same values.
+template <typename SM>
+__device__ __noinline__ float alpha64(SM& M) {
+  const double rz = M.sum64(0), pq = M.sum64(1);
+  M.rz = rz;
+  return (float)((pq > 0.0 && rz != 0.0) ? rz / pq : 0.0);
+}
+template <typename SM>
+__device__ __noinline__ float beta64(SM& M, DF old) {
+  const double o = isnan(old.h) ? M.rz : df_to_double(old);
+  return (float)(o != 0.0 ? M.sum64(0) / o : 0.0);
+}
+
 struct Smem8 {
   double xd[729];       // solution for the refinement residual
-  double redd[kW8];
+  double redd[kW8], rz;
   float a32[512], abf[512];
   float op[729];        // operand of A p
   float r8[729];        // residual of the V-cycle
   float lv[kLv8];
   float redf[2][kW8];
   int go;
+  __device__ double sum64(int which) const {
+    double v = 0.0;
+    for (int w = 0; w < kW8; ++w) v += (double)redf[which][w];
+    return v;
+  }
 };
 
 __global__ void __launch_bounds__(kT8, 4) k_small8(SmallArgs A) {
@@ -146,16 +180,14 @@ __global__ void __launch_bounds__(kT8, 4) k_small8(SmallArgs A) {
   };
   // block sum of a float as a pair, in every thread (FP64 additions and a division in one
   // warp were a quarter of an iteration)
-  int par = 0;
-  auto sum32 = [&](float v) {
+  auto sum32 = [&](float v, int which) {  // 0: r.z, 1: p.q
     v = warp_sum(v);
-    if (lane == 0) M.redf[par][warp] = v;
+    if (lane == 0) M.redf[which][warp] = v;
     __syncthreads();
-    DF g{lane < kW8 ? M.redf[par][lane] : 0.f, 0.f};
+    DF g{lane < kW8 ? M.redf[which][lane] : 0.f, 0.f};
 #pragma unroll
     for (int o = 8; o > 0; o >>= 1)
       g = df_add(g, DF{__shfl_xor_sync(0xffffffffu, g.h, o), __shfl_xor_sync(0xffffffffu, g.l, o)});
-    par ^= 1;
     return DF{__shfl_sync(0xffffffffu, g.h, 0), __shfl_sync(0xffffffffu, g.l, 0)};
   };
   DF rz{0.f, 0.f};  // r . z
@@ -205,8 +237,10 @@ __global__ void __launch_bounds__(kT8, 4) k_small8(SmallArgs A) {
       if (in) M.r8[n] = r;
       __syncthreads();
       const float z = vcycle8<kT8, true>(L, n, i, j, k, in, w8, omega);
-      const DF rzn = sum32(r * z);
-      p = it > 0 ? z + df_quotient(rzn, rz, rz.h != 0.f) * p : z;
+      const DF rzn = sum32(r * z, 0);
+      float be = it > 0 ? pair_beta(rzn, rz) : 0.f;
+      if (isnan(be)) be = beta64(M, rz);
+      p = it > 0 ? z + be * p : z;
       rz = rzn;
       if (in) M.op[n] = p;
       __syncthreads();
@@ -216,8 +250,9 @@ __global__ void __launch_bounds__(kT8, 4) k_small8(SmallArgs A) {
         cells8(C, M.a32, i, j, k, 8);
         q = float(1.0 / (12.0 * 8)) * q1_row(C, (const float*)M.op, i, j, k, 9);
       }
-      const DF pq = sum32(p * q);
-      const float al = df_quotient(rz, pq, pq.h > 0.f && rz.h != 0.f);
+      const DF pq = sum32(p * q, 1);
+      float al = pair_alpha(rz, pq);
+      if (isnan(al)) al = alpha64(M);
       d += al * p;
       if (it == inner - 1) break;
       r = r - al * q;
@@ -248,9 +283,13 @@ struct Smem16 {
   float b2[kN16];  // z, q or the refinement residual (dot)
   float a32[4096], abf[4096];
   float lv[kLv16];
-  double redd[24];
-  float redf[8];
+  double redd[24], rz;
+  float redf[2][8];
   int go;
+  __device__ double sum64(int which) const {  // the block sums of the two segments, as `dot` forms them
+    const float* w = redf[which];
+    return (double)((w[0] + w[2]) + (w[1] + w[3])) + (double)((w[4] + w[6]) + (w[5] + w[7]));
+  }
 };
 static_assert(sizeof(Smem16) <= 227 * 1024, "shared memory");
 
@@ -406,7 +445,7 @@ __global__ void __launch_bounds__(kT16, 1) k_small16(SmallArgs A) {
   // dot product of two shared vectors in the order of the tile passes: thread (tx, ty) of
   // segment sg sums rows 4 ty + 1 .. 4 ty + 4 over the segment's eight planes, then the
   // block sum of the segment, then the two segments (a pair, in every thread)
-  auto dot = [&](const float* u, const float* v) {
+  auto dot = [&](const float* u, const float* v, int which) {  // 0: r.z, 1: p.q
     if (warp < 8) {
       const int sg = warp >> 2, ty = warp & 3;
       float red = 0.f;
@@ -422,10 +461,10 @@ __global__ void __launch_bounds__(kT16, 1) k_small16(SmallArgs A) {
             }
       }
       red = warp_sum(red);
-      if (lane == 0) M.redf[warp] = red;
+      if (lane == 0) M.redf[which][warp] = red;
     }
     __syncthreads();
-    float w = lane < 8 ? M.redf[lane] : 0.f;
+    float w = lane < 8 ? M.redf[which][lane] : 0.f;
     w += __shfl_xor_sync(0xffffffffu, w, 2);
     w += __shfl_xor_sync(0xffffffffu, w, 1);
     const float p0 = __shfl_sync(0xffffffffu, w, 0), p1 = __shfl_sync(0xffffffffu, w, 4);
@@ -545,9 +584,10 @@ __global__ void __launch_bounds__(kT16, 1) k_small16(SmallArgs A) {
           M.b2[n0 + 289 * u] = z[u];
         }
       __syncthreads();
-      const DF rzn = dot(M.b1, M.b2);
+      const DF rzn = dot(M.b1, M.b2, 0);
       // p = z + beta p, q = A p
-      const float be = it == 0 ? 0.f : df_quotient(rzn, rz, rz.h != 0.f);
+      float be = it == 0 ? 0.f : pair_beta(rzn, rz);
+      if (isnan(be)) be = beta64(M, rz);
       rz = rzn;
 #pragma unroll
       for (int u = 0; u < 4; ++u)
@@ -563,8 +603,9 @@ __global__ void __launch_bounds__(kT16, 1) k_small16(SmallArgs A) {
           M.b2[n0 + 289 * u] = q[u];
         }
       __syncthreads();
-      const DF pq = dot(M.b0, M.b2);
-      al = df_quotient(rz, pq, pq.h > 0.f && rz.h != 0.f);
+      const DF pq = dot(M.b0, M.b2, 1);
+      al = pair_alpha(rz, pq);
+      if (isnan(al)) al = alpha64(M);
       if (it == inner - 1) break;
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
