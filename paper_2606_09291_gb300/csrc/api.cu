@@ -116,7 +116,8 @@ size_t level_bytes(const mlsgd_ctx* ctx, int level, int S) {
   return b;
 }
 
-mlsgd_status ensure_ws(mlsgd_ctx* ctx, size_t bytes, cudaStream_t st) {
+// room: bytes to take beside them if the workspace has to grow anyway and the device has them
+mlsgd_status ensure_ws(mlsgd_ctx* ctx, size_t bytes, cudaStream_t st, size_t room = 0) {
   if (bytes <= ctx->ws_size) return MLSGD_OK;
   if (ctx->ws_external)
     return fail(ctx, MLSGD_ENOMEM, "the caller's workspace holds " + std::to_string(ctx->ws_size) + " bytes, " +
@@ -125,6 +126,13 @@ mlsgd_status ensure_ws(mlsgd_ctx* ctx, size_t bytes, cudaStream_t st) {
   if (ctx->ws) CK(cudaFree(ctx->ws));
   ctx->ws = nullptr;
   ctx->ws_size = 0;
+  if (room > 0) {
+    if (cudaMalloc(&ctx->ws, bytes + room) == cudaSuccess) {
+      ctx->ws_size = bytes + room;
+      return MLSGD_OK;
+    }
+    cudaGetLastError();
+  }
   if (cudaMalloc(&ctx->ws, bytes) != cudaSuccess) {
     cudaGetLastError();
     ctx->ws = nullptr;
@@ -132,6 +140,12 @@ mlsgd_status ensure_ws(mlsgd_ctx* ctx, size_t bytes, cudaStream_t st) {
   }
   ctx->ws_size = bytes;
   return MLSGD_OK;
+}
+// room in which B z on grid N is formed in one slab of control planes, where the solver's
+// vectors of S samples are less (at most 64 MB: slabs of that size cost nothing)
+size_t rhs_room(const mlsgd_ctx* ctx, int N, int S) {
+  const size_t b = rhs_slab_bytes(ctx->Nc(), N);
+  return b <= ((size_t)64 << 20) && b > solver_bytes(N, S, ctx->mixed() ? 4 : 8) ? b : 0;
 }
 
 struct GridFields {
@@ -185,12 +199,13 @@ mlsgd_status solve_verdict(mlsgd_ctx* ctx, int flags, const char* who) {
   return MLSGD_OK;
 }
 
-// state + Phi + adjoint for S samples on grid N; scratch carved from bp (not kept).
+// state + Phi + adjoint for S samples on grid N; scratch carved from `scratch` (not kept), of
+// which ws_end is the end.
 // want_pairs (internal callers): on tiled grids of the mixed path, y stays and q is
 // returned as FP32 (hi, lo) pairs in the FP64 buffers' storage (*pairs_out = true),
 // and Phi / the adjoint right-hand side are formed in pair arithmetic.
 mlsgd_status solve_grid(mlsgd_ctx* ctx, int N, int S, const GridFields& f, const double* z, double* y, double* q,
-                        double* phi, int* iters, int* status, char* scratch, cudaStream_t st,
+                        double* phi, int* iters, int* status, char* scratch, char* ws_end, cudaStream_t st,
                         bool want_pairs = false, bool* pairs_out = nullptr) {
   const size_t nodes = (size_t)nodes_of(N);
   char* p = scratch;
@@ -208,8 +223,11 @@ mlsgd_status solve_grid(mlsgd_ctx* ctx, int N, int S, const GridFields& f, const
   PcgParams prm{ctx->cfg.rtol, ctx->cfg.max_iter, ctx->cfg.omega > 0 ? ctx->cfg.omega : 0.6, 4};
   const int inner = ctx->cfg.inner_iters > 0 ? ctx->cfg.inner_iters : 6;
   const int inner2 = ctx->cfg.inner_iters_next > 0 ? ctx->cfg.inner_iters_next : inner;
-  // B z first: the solver's vectors, not yet in use, are its scratch
-  launch_rhs_state(z, ctx->Nc(), N, b, scratch, (size_t)(p - scratch), st);
+  // B z first: its scratch are the solver's vectors, not yet in use, or what is left behind
+  // everything if that is more
+  const size_t behind = ws_end > bp.p ? (size_t)(ws_end - bp.p) : 0;
+  const bool back = behind > (size_t)(p - scratch);
+  launch_rhs_state(z, ctx->Nc(), N, b, back ? bp.p : scratch, back ? behind : (size_t)(p - scratch), st);
   const bool small = small_supported(N);  // 8^3, 16^3: a solve is one launch
   if (!small && ctx->mixed()) build_hierarchy_mixed(B, f.abf, prm.omega, st);
   if (!small && !ctx->mixed()) build_hierarchy_fp64(B, f.a64, prm.omega, st);
@@ -517,13 +535,13 @@ mlsgd_status mlsgd_solve_state_adjoint(mlsgd_ctx* ctx, int grid, int n_samples, 
   const int N = ctx->N(grid);
   const int S = n_samples;
   const size_t need = field_bytes(ctx, N, S) + solve_scratch_bytes(ctx, N, S);
-  mlsgd_status s = ensure_ws(ctx, need, st);
+  mlsgd_status s = ensure_ws(ctx, need, st, rhs_room(ctx, N, S));
   if (s != MLSGD_OK) return s;
   Bump bp{ctx->ws};
   GridFields f = carve_fields(ctx, N, S, bp);
   FieldOut o{nullptr, f.a64, f.a32, f.abf};
   launch_exp_field(log_a_dev, o, (long long)S * cells_of(N), st);
-  s = solve_grid(ctx, N, S, f, z_dev, y_dev, q_dev, phi_dev, iters_dev, status_dev, bp.p, st);
+  s = solve_grid(ctx, N, S, f, z_dev, y_dev, q_dev, phi_dev, iters_dev, status_dev, bp.p, ctx->ws + ctx->ws_size, st);
   if (s != MLSGD_OK) return s;
   // report non-convergence / non-finite solves (synchronous check of the status flags)
   std::vector<int> h(S);
@@ -600,7 +618,8 @@ mlsgd_status mlsgd_solve_state_adjoint_noalloc(mlsgd_ctx* ctx, int grid, int n_s
   GridFields f = carve_fields(ctx, N, S, bp);
   FieldOut o{nullptr, f.a64, f.a32, f.abf};
   launch_exp_field(log_a_dev, o, (long long)S * cells_of(N), st);
-  s = solve_grid(ctx, N, S, f, z_dev, y_dev, q_dev, phi_dev, iters_dev, status_dev, bp.p, st);
+  s = solve_grid(ctx, N, S, f, z_dev, y_dev, q_dev, phi_dev, iters_dev, status_dev, bp.p,
+                 scratch + MLSGD_NOALLOC_SCRATCH_BYTES, st);
   if (s != MLSGD_OK) return s;
   // the OR of the per-sample flags is formed on the device and one int read back
   // through the context's pinned word (no allocation, any batch size)
@@ -643,9 +662,11 @@ mlsgd_status mlsgd_level_gradient(mlsgd_ctx* ctx, int iter, int level, int64_t f
     return fail(ctx, MLSGD_EINVAL, "mlsgd_level_gradient: bad arguments");
   if (n_samples == 0) return MLSGD_OK;
   const int chunk = std::min(n_samples, ctx->cfg.max_batch);
-  mlsgd_status s = ensure_ws(ctx, level_bytes(ctx, level, chunk), st);
-  if (s != MLSGD_OK) return s;
   const int N = ctx->N(level), K = ctx->cfg.n_modes;
+  const size_t room = std::max(rhs_room(ctx, N, chunk), level > 0 ? rhs_room(ctx, N / 2, chunk) : 0);
+  mlsgd_status s = ensure_ws(ctx, level_bytes(ctx, level, chunk), st, room);
+  if (s != MLSGD_OK) return s;
+  char* ws_end = ctx->ws + ctx->ws_size;
   for (int64_t done = 0; done < n_samples; done += chunk) {
     const int S = (int)std::min<int64_t>(chunk, n_samples - done);
     Bump bp{ctx->ws};
@@ -671,12 +692,12 @@ mlsgd_status mlsgd_level_gradient(mlsgd_ctx* ctx, int iter, int level, int64_t f
     s = make_field(ctx, xi, level, S, ff, nullptr, st, gemm_a);
     if (s != MLSGD_OK) return s;
     bool pf = false, pc = false;
-    s = solve_grid(ctx, N, S, ff, z_dev, nullptr, qf, phif, iters, status, scratch, st, true, &pf);
+    s = solve_grid(ctx, N, S, ff, z_dev, nullptr, qf, phif, iters, status, scratch, ws_end, st, true, &pf);
     if (s != MLSGD_OK) return s;
     if (level > 0) {
       s = make_field(ctx, xi, level - 1, S, fc, nullptr, st, gemm_a);
       if (s != MLSGD_OK) return s;
-      s = solve_grid(ctx, N / 2, S, fc, z_dev, nullptr, qc, phic, iters + S, status + S, scratch, st, true, &pc);
+      s = solve_grid(ctx, N / 2, S, fc, z_dev, nullptr, qc, phic, iters + S, status + S, scratch, ws_end, st, true, &pc);
       if (s != MLSGD_OK) return s;
     }
     launch_level_stats(qf, phif, N, qc, phic, N / 2, S, ctx->Nc(), ctx->cfg.theta, stats->field_dev,

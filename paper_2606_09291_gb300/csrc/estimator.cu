@@ -56,10 +56,12 @@ __global__ void k_rhs_state(const double* __restrict__ z, int Nc, int N, double*
 // Bound: FP64 issue, then one read of z.  Contracted axis by axis every control cell
 // costs two FMAs (to the two nodes of its level cell along y), where contracting the
 // (2r)^2 rows of each node row's support costs 4 (and reads z four times).
-// k_rhs_xy: one block per (level cell row ey, control plane cz) contracts y, then x, into
-// u[cz][ey][side][i]; k_rhs_z contracts z.  A 256^3 control onto 8^3: 615 us by node
-// rows, 116 us now.
-__global__ void __launch_bounds__(kBlock) k_rhs_xy(const double* __restrict__ z, int Nc, int N,
+// k_rhs_xy: one block per (level cell row ey, control plane z0 + cz) contracts y, then x,
+// into u[cz][ey][side][i]; k_rhs_z contracts z, slab after slab of the control planes that u
+// has room for (the order of the sums does not depend on the slabs).  A 256^3 control onto
+// 8^3: 615 us by node rows, 116 us by axis; a whole FP64 state and adjoint solve of one 8^3
+// sample under it 862 and 358 us.
+__global__ void __launch_bounds__(kBlock) k_rhs_xy(const double* __restrict__ z, int Nc, int N, int z0,
                                                    double* __restrict__ u) {
   pdl_entry();
   extern __shared__ double sm[];  // t[r], left and right sums [2][Nc]
@@ -70,7 +72,7 @@ __global__ void __launch_bounds__(kBlock) k_rhs_xy(const double* __restrict__ z,
   const double inv_r = 1.0 / r;
   for (int m = threadIdx.x; m < r; m += blockDim.x) t[m] = (m + 0.5) * inv_r;
   __syncthreads();
-  const double* zp = z + (long long)Nc * ((long long)r * ey + (long long)Nc * cz);
+  const double* zp = z + (long long)Nc * ((long long)r * ey + (long long)Nc * (z0 + cz));
   for (int cx = threadIdx.x; cx < Nc; cx += blockDim.x) {
     double all = 0.0, right = 0.0;
 #pragma unroll 4
@@ -94,8 +96,10 @@ __global__ void __launch_bounds__(kBlock) k_rhs_xy(const double* __restrict__ z,
     ub[e] = v;
   }
 }
-// node (i, j, k): the right side of cell row j - 1 and the left side of row j, over 2r planes
-__global__ void __launch_bounds__(kBlock) k_rhs_z(const double* __restrict__ u, int Nc, int N,
+// node (i, j, k): the right side of cell row j - 1 and the left side of row j, over those of
+// its 2r control planes that are among z0 .. z0 + planes - 1; b holds the sum so far between
+// two slabs
+__global__ void __launch_bounds__(kBlock) k_rhs_z(const double* __restrict__ u, int Nc, int N, int z0, int planes,
                                                   double* __restrict__ b) {
   pdl_entry();
   const int n1 = N + 1, r = Nc / N;
@@ -103,18 +107,23 @@ __global__ void __launch_bounds__(kBlock) k_rhs_z(const double* __restrict__ u, 
   if (n >= n1 * n1 * n1) return;
   int i, j, k;
   node_ijk(n, n1, i, j, k);
-  double v = 0.0;
-  if (interior(i, j, k, N)) {
-    const long long plane = (long long)N * 2 * n1;
-    const double* up = u + (long long)r * (k - 1) * plane + (long long)(2 * (j - 1) + 1) * n1 + i;
-    const double inv_r = 1.0 / r;
-    for (int m = 0; m < 2 * r; ++m, up += plane) {
-      const double w = m < r ? (m + 0.5) * inv_r : 2.0 - (m + 0.5) * inv_r;
-      v = fma(w, up[0] + up[n1], v);
-    }
-    const double hc = 1.0 / Nc;
-    v *= hc * hc * hc;
+  if (!interior(i, j, k, N)) {
+    if (z0 == 0) b[n] = 0.0;
+    return;
   }
+  const int first = r * (k - 1), m0 = max(0, z0 - first), m1 = min(2 * r, z0 + planes - first);
+  if (m0 >= m1) return;
+  const long long plane = (long long)N * 2 * n1;
+  const double* up = u + (long long)(first + m0 - z0) * plane + (long long)(2 * (j - 1) + 1) * n1 + i;
+  const double inv_r = 1.0 / r;
+  double v = m0 > 0 ? b[n] : 0.0;
+#pragma unroll 8
+  for (int m = m0; m < m1; ++m, up += plane) {
+    const double w = m < r ? (m + 0.5) * inv_r : 2.0 - (m + 0.5) * inv_r;
+    v = fma(w, up[0] + up[n1], v);
+  }
+  const double hc = 1.0 / Nc;
+  if (m1 == 2 * r) v *= hc * hc * hc;
   b[n] = v;
 }
 // Control and level grid equal: (B z)_n = h^3 / 8 sum of the eight cells, summed along y,
@@ -152,15 +161,13 @@ __global__ void __launch_bounds__(kBlock) k_rhs_equal(const double* __restrict__
   }
 }
 
-// The by-axis form from r = Nc / N = 4 on.  At r = 2 it takes about as many operations as
-// the node rows (145 against 156 us of FP64 issue for a 256^3 control on 128^3), which
-// need no scratch.
-constexpr int kRhsAxisR = 4;
-size_t rhs_scratch_bytes(int Nc, int N) {  // u of k_rhs_xy
-  return Nc >= kRhsAxisR * N ? (size_t)Nc * N * 2 * (N + 1) * sizeof(double) : 0;
-}
+// The by-axis form from r = Nc / N = 8 on.  Below, the node rows, which need no scratch, are as
+// fast or faster: at r = 2 145 against 156 us of FP64 issue for a 256^3 control on 128^3, at
+// r = 4 a state and adjoint solve of one 64^3 sample under a 256^3 control 1912 against 1934 us
+// (mixed), 3919 against 3947 (FP64), of 8^3 to 32^3 the same within 0.5%.
+constexpr int kRhsAxisR = 8;
 
-// The form of r = 2, and without scratch of any r: one block per node row (j, k); threads along cx contract the
+// The form of r = 2 and 4: one block per node row (j, k); threads along cx contract the
 // (2r)^2 control rows (cy, cz) of the row's support with w(y) w(z) into a column sum per
 // cx, then each node i of the row contracts its 2r columns with w(x).
 __global__ void __launch_bounds__(kBlock) k_rhs_rows(const double* __restrict__ z, int Nc, int N,
@@ -204,7 +211,11 @@ __global__ void __launch_bounds__(kBlock) k_rhs_rows(const double* __restrict__ 
   }
 }
 
-// scratch: memory the launch may overwrite (the by-axis form needs rhs_scratch_bytes)
+size_t rhs_slab_bytes(int Nc, int N) {  // u of all control planes
+  return Nc >= kRhsAxisR * N ? (size_t)Nc * N * 2 * (N + 1) * sizeof(double) : 0;
+}
+
+// scratch: memory the launch may overwrite, at least 16 N (N + 1) bytes (a control plane of u)
 void launch_rhs_state(const double* z, int Nc, int N, double* b, void* scratch, size_t scratch_bytes,
                       cudaStream_t st) {
   const double bytes = (double)cells_of(Nc) * 8 + (double)nodes_of(N) * 8;
@@ -214,13 +225,20 @@ void launch_rhs_state(const double* z, int Nc, int N, double* b, void* scratch, 
     launch("rhs", bytes, k_rhs_equal,
            dim3((unsigned)(((N + 1) * (N + 1) + kBlock - 1) / kBlock), (unsigned)((N + kRhsPlanes) / kRhsPlanes)), kBlock,
            0, st, z, N, b);
-  } else if (Nc >= kRhsAxisR * N && rhs_scratch_bytes(Nc, N) <= scratch_bytes) {
+  } else if (Nc >= kRhsAxisR * N) {
+    // slabs of control planes, as many and as equal as the scratch asks for
+    const size_t plane = (size_t)N * 2 * (N + 1) * sizeof(double);
+    const int fit = (int)std::min<size_t>(Nc, std::max<size_t>(1, scratch_bytes / plane));
+    const int slabs = (Nc + fit - 1) / fit, planes = (Nc + slabs - 1) / slabs;
     double* u = (double*)scratch;
-    const double ub = (double)rhs_scratch_bytes(Nc, N);
-    launch("rhs", (double)cells_of(Nc) * 8 + ub, k_rhs_xy, dim3((unsigned)N, (unsigned)Nc), kBlock,
-           (size_t)(Nc / N + 2 * Nc) * sizeof(double), st, z, Nc, N, u);
-    launch("rhs", ub + (double)nodes_of(N) * 8, k_rhs_z, dim3(node_blocks(N)), kBlock, 0, st, (const double*)u, Nc, N,
-           b);
+    for (int z0 = 0; z0 < Nc; z0 += planes) {
+      const int n = std::min(planes, Nc - z0);
+      const double ub = (double)n * plane;
+      launch("rhs", (double)n * Nc * Nc * 8 + ub, k_rhs_xy, dim3((unsigned)N, (unsigned)n), kBlock,
+             (size_t)(Nc / N + 2 * Nc) * sizeof(double), st, z, Nc, N, z0, u);
+      launch("rhs", ub + (double)nodes_of(N) * 8, k_rhs_z, dim3(node_blocks(N)), kBlock, 0, st, (const double*)u, Nc, N,
+             z0, n, b);
+    }
   } else {
     const size_t smem = (size_t)(2 * (Nc / N) + Nc) * sizeof(double);
     launch("rhs", bytes, k_rhs_rows, dim3((unsigned)(N + 1), (unsigned)(N + 1)), kBlock, smem, st, z, Nc, N, b);

@@ -251,9 +251,9 @@ cudaError_t kl_gemm(const double* xi, const double* scale, int S, int K, const _
                     __nv_bfloat16* A_scratch, __nv_bfloat16* abf, float* loga, int* err, cudaStream_t st);
 
 // ---------------------------------------------------------------- estimator
-// scratch: scratch_bytes of device memory the launch may overwrite (rhs_scratch_bytes for
-// the by-axis form of a finer control grid; less falls back to a slower form)
-size_t rhs_scratch_bytes(int Nc, int N);
+// scratch: scratch_bytes of device memory the launch may overwrite, at least 16 N (N + 1)
+// (more mean fewer launches, up to rhs_slab_bytes; b's bits do not depend on it)
+size_t rhs_slab_bytes(int Nc, int N);
 void launch_rhs_state(const double* z, int Nc, int N, double* b, void* scratch, size_t scratch_bytes, cudaStream_t st);
 // Phi = 1/2 e^T M e, badj = M e (interior rows), e = y - g_h
 void launch_phi_adjrhs(const double* y, int N, int S, double* badj, double* phi, double* partial,
