@@ -55,6 +55,7 @@ struct Cand { double key; int i, j, k; };
 KLTable build_kl_table(double corr_len, int K) {
   KLTable T;
   int n1d = 4;
+  while (n1d * n1d * n1d < K) ++n1d;  // at least K candidates
   for (;;) {
     kl_modes_1d(corr_len, n1d, T.omega, T.lam1, T.norm);
     std::vector<Cand> cand;
