@@ -86,6 +86,7 @@ struct SolverBufs {
   const int* actp = nullptr; // their indices (null: all S)
   int* act = nullptr;        // [S] device list the compaction writes
   int* err = nullptr;        // device error flag (bounded waits that ran out)
+  cudaError_t failed = cudaSuccess;  // of a V-cycle step that could not be launched: the solve returns it
   int stencil = 0;           // see Batch
   int zchunks = 0;
   Batch batch() const { return Batch{S, n_act, actp, err, stencil, zchunks}; }

@@ -749,41 +749,45 @@ static_assert(sizeof(SmemV) <= 113 * 1024 && sizeof(With8<16, SmemSolve<16>>) <=
 // (16 clusters of eight blocks went to 64 SMs).  The shared memory that is asked for sets
 // how many blocks an SM takes: the fewest with which every sample's cluster is resident.
 struct Spread {
-  std::once_flag once;
-  cudaError_t err = cudaSuccess;
-  int n = 0;
+  std::mutex m;
+  int n = 0;  // 0: not set up (again after a failure)
   size_t smem[8];
   int clusters[8];  // resident with at most i + 1 blocks per SM
 };
 template <typename Args>
 cudaError_t launch_spread(Spread& sp, const char* cls, double bytes, void (*k)(Args), int threads, int cluster,
                           size_t smem, int most, int samples, cudaStream_t st, const Args& A) {
-  std::call_once(sp.once, [&] {
-    constexpr size_t kSm = 228 * 1024, kBlock = 1024;  // of an SM; reserved per block
-    sp.err = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)std::max(smem, kSm / 2 - kBlock + 16));
-    for (int occ = 1; occ <= most && sp.err == cudaSuccess; ++occ) {
-      const size_t want = std::max(smem, kSm / (occ + 1) - kBlock + 16);  // occ + 1 blocks don't fit
-      cudaLaunchAttribute at[1];
-      at[0].id = cudaLaunchAttributeClusterDimension;
-      at[0].val.clusterDim.x = (unsigned)cluster;
-      at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-      cudaLaunchConfig_t cfg{};
-      cfg.gridDim = dim3((unsigned)cluster);
-      cfg.blockDim = dim3((unsigned)threads);
-      cfg.dynamicSmemBytes = want;
-      cfg.attrs = at;
-      cfg.numAttrs = 1;
-      int c = 0;
-      if (cudaOccupancyMaxActiveClusters(&c, k, &cfg) != cudaSuccess) {
-        (void)cudaGetLastError();
-        c = 0;
+  {
+    std::lock_guard<std::mutex> lock(sp.m);
+    if (sp.n == 0) {
+      constexpr size_t kSm = 228 * 1024, kBlock = 1024;  // of an SM; reserved per block
+      const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                 (int)std::max(smem, kSm / 2 - kBlock + 16));
+      if (e != cudaSuccess) return e;
+      for (int occ = 1; occ <= most; ++occ) {
+        const size_t want = std::max(smem, kSm / (occ + 1) - kBlock + 16);  // occ + 1 blocks don't fit
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = (unsigned)cluster;
+        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = dim3((unsigned)cluster);
+        cfg.blockDim = dim3((unsigned)threads);
+        cfg.dynamicSmemBytes = want;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        int c = 0;  // without an answer the least shared memory is taken
+        const bool clean = cudaPeekAtLastError() == cudaSuccess;
+        if (cudaOccupancyMaxActiveClusters(&c, k, &cfg) != cudaSuccess) {
+          if (clean) (void)cudaGetLastError();  // an earlier call's error stays
+          c = 0;
+        }
+        sp.smem[occ - 1] = want;
+        sp.clusters[occ - 1] = c;
       }
-      sp.smem[sp.n] = want;
-      sp.clusters[sp.n++] = c;
+      sp.n = most;
     }
-  });
-  if (sp.err != cudaSuccess) return sp.err;
+  }
   size_t use = smem;
   for (int i = 0; i < sp.n; ++i)
     if (sp.clusters[i] >= samples) {

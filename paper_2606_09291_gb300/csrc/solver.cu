@@ -760,6 +760,10 @@ void build_hierarchy_mixed(SolverBufs& B, const __nv_bfloat16* abf, double omega
 // passes; the V-cycle from 32^3 down 18 us against 38 us in three passes, 38 us at 38.
 constexpr int kCluster32Max = 32;
 
+static void note(SolverBufs& B, cudaError_t e) {
+  if (B.failed == cudaSuccess) B.failed = e;
+}
+
 // One V(1,1)-cycle on r0 (level-0 coefficient a0); the result is left in vt[0].
 // Grids with N >= kTiledMinN run the fine level with the tiled passes (PRE
 // fuses the pre-smoothing into the residual, POST fuses prolongation,
@@ -841,9 +845,9 @@ static int vcycle(SolverBufs& B, const T* r0, const TA0* a0, const SolveScalars*
     if constexpr (std::is_same<T, double>::value) {
       (void)below;
       const double* const wd[3] = {(const double*)B.dinv[jc], (const double*)B.vx[jc + 1], (const double*)B.vx[jc + 2]};
-      (void)coarse_vcycle64(rin(jc), al, wd, (double*)B.vt[jc], sc, bt, (double)omega, st);  // checked by the caller
+      note(B, coarse_vcycle64(rin(jc), al, wd, (double*)B.vt[jc], sc, bt, (double)omega, st));
     } else if (from32) {
-      (void)vcycle32(rin(jc), al[0], (const float*)B.dinv[jc], below, (float*)B.vt[jc], sc, bt, (double)omega, st);
+      note(B, vcycle32(rin(jc), al[0], (const float*)B.dinv[jc], below, (float*)B.vt[jc], sc, bt, (double)omega, st));
     } else {
       coarse_vcycle(rin(jc), al, (T*)B.vt[jc], sc, bt, (double)omega, st);
     }
@@ -982,8 +986,9 @@ static cudaError_t pcg_loop(SolverBufs& B, const TAop* aop, const TA0* a0, T* x,
     if (!tiled)
       launch(cls<T>("pupdate", true), nbytes<T, T>(N, B.n_act, 3, 0), k_p_update<T>, g(), kBlock, 0, st, pbuf[0], z,
              (const SolveScalars*)sc, nodes, 0, B.actp);
+    if (B.failed != cudaSuccess) break;
   }
-  return cudaGetLastError();
+  return B.failed != cudaSuccess ? B.failed : cudaGetLastError();
 }
 
 // Mixed inner solve on a tiled grid, `iters` PCG iterations with the vector
@@ -1053,7 +1058,7 @@ static cudaError_t pcg_inner_fused(SolverBufs& B, const float* a32, const __nv_b
     rc ^= 1;
     scalar(B, sc, SM_BETA, 0, 0, st, nrz);
   }
-  return cudaGetLastError();
+  return B.failed != cudaSuccess ? B.failed : cudaGetLastError();
 }
 
 // Buffers the tiled passes write only on interior nodes must hold zero

@@ -65,6 +65,7 @@ class Host:
     def reset(self):
         self.L.fake_reset()
         self.L.fake_refuse_opt_in(b"")
+        self.L.fake_refuse_occupancy(0)
         self.L.cudaGetLastError()
 
     def close(self):

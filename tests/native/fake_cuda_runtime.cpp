@@ -25,6 +25,7 @@ struct State {
   std::map<std::pair<const void*, int>, int> smem;  // opt-in per kernel and device
   std::vector<Launch> launches;
   std::string fail;     // kernels whose opt-in is refused
+  bool no_occupancy = false;
   int device = 0;
   cudaError_t last = cudaSuccess;
 };
@@ -58,6 +59,7 @@ const char* fake_launch(int i, unsigned v[8]) {
 }
 void fake_reset() { S().launches.clear(); }
 void fake_refuse_opt_in(const char* kernel) { S().fail = kernel; }
+void fake_refuse_occupancy(int on) { S().no_occupancy = on != 0; }
 void fake_set_last_error(int e) { S().last = (cudaError_t)e; }
 long long fake_level_partial_cap(int Nc, int Nf) { return mlsgd::level_partial_cap(Nc, Nf); }
 
@@ -80,7 +82,11 @@ cudaError_t cudaFuncSetAttribute(const void* f, cudaFuncAttribute a, int v) {
   if (a == cudaFuncAttributeMaxDynamicSharedMemorySize) S().smem[{f, S().device}] = v;
   return cudaSuccess;
 }
-cudaError_t cudaOccupancyMaxActiveClusters(int* n, const void*, const cudaLaunchConfig_t*) { *n = 16; return cudaSuccess; }
+cudaError_t cudaOccupancyMaxActiveClusters(int* n, const void*, const cudaLaunchConfig_t*) {
+  if (S().no_occupancy) return set(cudaErrorUnknown);
+  *n = 16;
+  return cudaSuccess;
+}
 cudaError_t cudaMalloc(void** p, size_t n) { *p = calloc(1, n); return *p ? cudaSuccess : set(cudaErrorMemoryAllocation); }
 cudaError_t cudaFree(void* p) { free(p); return cudaSuccess; }
 cudaError_t cudaHostAlloc(void** p, size_t n, unsigned) { return cudaMalloc(p, n); }
