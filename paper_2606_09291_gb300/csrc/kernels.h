@@ -80,6 +80,7 @@ struct Batch {
 
 // Buffers of one batched solve on a grid with N cells per side.  Vectors are
 // [S][nodes] (stride nodes_of(N)), coefficients [S][cells].
+constexpr int kMaxMg = 10;   // MG levels of a 1024^3 grid
 struct SolverBufs {
   int N, S, J;               // MG levels j = 0..J, N_j = N >> j, N_J = 2
   int n_act = 0;             // samples launched by the masked kernels (host-known)
@@ -91,11 +92,11 @@ struct SolverBufs {
   int zchunks = 0;
   Batch batch() const { return Batch{S, n_act, actp, err, stencil, zchunks}; }
   // MG hierarchy (j >= 1 coarse; j = 0 uses the caller's operator coefficient)
-  void* acoef[8];            // coefficient per MG level (j = 0: the V-cycle's own copy, may alias)
-  void* vx[8];               // V-cycle iterate per level
-  void* vt[8];               // V-cycle temporary / output per level
-  void* vr[8];               // restricted residual (j >= 1)
-  void* dinv[8];             // D^{-1} of levels run with the tiled passes (0 at boundary nodes), else null
+  void* acoef[kMaxMg];            // coefficient per MG level (j = 0: the V-cycle's own copy, may alias)
+  void* vx[kMaxMg];               // V-cycle iterate per level
+  void* vt[kMaxMg];               // V-cycle temporary / output per level
+  void* vr[kMaxMg];               // restricted residual (j >= 1)
+  void* dinv[kMaxMg];             // D^{-1} of levels run with the tiled passes (0 at boundary nodes), else null
   float2* bdf;               // mixed tiled solves: b as FP32 (hi, lo) pairs [S][nodes]; with the slab
                              // refinement step, the residual pairs of the step
   float2* bsh;               // the same for a b shared by every sample: [nodes]

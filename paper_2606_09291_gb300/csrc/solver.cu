@@ -634,7 +634,7 @@ void carve_solver(SolverBufs& B, int N, int S, int elem, char*& ptr) {
     B.vx[j] = take(vj); B.vt[j] = take(vj); B.vr[j] = take(vj);
     B.acoef[j] = take((size_t)S * cells_of(Nj) * elem);
   }
-  for (int j = 0; j < 8; ++j) B.dinv[j] = nullptr;
+  for (int j = 0; j < kMaxMg; ++j) B.dinv[j] = nullptr;
   for (int j = 0; j <= B.J; ++j)
     if (tiled_level(N, j)) B.dinv[j] = take((size_t)S * nodes_of(N >> j) * elem + kVecSlack);
   B.bdf = (elem == 4 && tiled_level(N, 0)) ? (float2*)take((size_t)S * nodes_of(N) * sizeof(float2)) : nullptr;

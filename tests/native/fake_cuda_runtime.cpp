@@ -4,6 +4,7 @@
 // made to fail.  Linked with the library's object files in place of libcudart.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstdlib>
 #include <cstring>
 #include <map>
@@ -61,6 +62,29 @@ void fake_reset() { S().launches.clear(); }
 void fake_refuse_opt_in(const char* kernel) { S().fail = kernel; }
 void fake_refuse_occupancy(int on) { S().no_occupancy = on != 0; }
 void fake_set_last_error(int e) { S().last = (cudaError_t)e; }
+// 0 when the vectors of a solve on an N^3 grid lie side by side within solver_bytes
+int fake_check_carve(int N, int S, int elem) {
+  mlsgd::SolverBufs B;
+  char* const base = (char*)4096;
+  char* p = base;
+  mlsgd::carve_solver(B, N, S, elem, p);
+  if (p < base || (size_t)(p - base) > mlsgd::solver_bytes(N, S, elem)) return 1;
+  std::vector<std::pair<char*, size_t>> v;
+  const auto add = [&](void* q, long long n) { if (q) v.push_back({(char*)q, (size_t)n}); };
+  const size_t e = (size_t)elem * S;
+  for (void* q : {B.x, B.r, B.r2, B.p, B.q}) add(q, e * mlsgd::nodes_of(N));
+  for (int j = 0; j <= B.J; ++j) {
+    const int M = N >> j;
+    for (void* q : {B.vx[j], B.vt[j], B.vr[j], B.dinv[j]}) add(q, e * mlsgd::nodes_of(M));
+    add(B.acoef[j], e * mlsgd::cells_of(M));
+  }
+  std::sort(v.begin(), v.end());
+  for (size_t i = 0; i < v.size(); ++i) {
+    char* const end = i + 1 < v.size() ? v[i + 1].first : (char*)B.partial;
+    if (v[i].first < base || v[i].first + v[i].second > end) return 2;
+  }
+  return 0;
+}
 long long fake_level_partial_cap(int Nc, int Nf) { return mlsgd::level_partial_cap(Nc, Nf); }
 
 // ---- the runtime
