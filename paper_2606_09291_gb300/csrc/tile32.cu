@@ -503,7 +503,8 @@ int chunk_segments(long long tiles, int nseg) {
 template <typename TA, int MODE>
 void run(const char* cls, double bytes, Args args, const Batch& bt, cudaStream_t st) {
   const TiledShape t = tiled_shape(args.N, bt.S, 4);
-  const int spc = bt.zchunks > 0 ? (t.nseg + bt.zchunks - 1) / bt.zchunks : chunk_segments((long long)t.bx * t.by * bt.n, t.nseg);
+  int spc = chunk_segments((long long)t.bx * t.by * bt.n, t.nseg);
+  if (bt.zchunks > 0) spc = bt.zchunks < t.nseg ? (t.nseg + bt.zchunks - 1) / bt.zchunks : 1;
   args.nzc = (t.nseg + spc - 1) / spc;
   args.zc = spc * kSegPlanes;
   args.nseg = t.nseg;

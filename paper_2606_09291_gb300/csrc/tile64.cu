@@ -355,7 +355,7 @@ void run(const char* cls, double bytes, Args A, const Batch& bt, cudaStream_t st
     const double cost = (per_sm(q) == 1 ? 1.35 : (double)per_sm(q)) * (kSeg * q + 0.6);
     if (cost < best) { best = cost; spc = q; }
   }
-  if (bt.zchunks > 0) spc = (nseg + bt.zchunks - 1) / bt.zchunks;
+  if (bt.zchunks > 0) spc = bt.zchunks < nseg ? (nseg + bt.zchunks - 1) / bt.zchunks : 1;
   A.nseg = nseg;
   A.nzc = (nseg + spc - 1) / spc;
   A.zc = spc * kSeg;
