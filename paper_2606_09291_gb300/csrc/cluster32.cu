@@ -718,20 +718,12 @@ __global__ void __launch_bounds__(kNT, 1) k_solve32(SArgs A) {
   cl.sync();  // no block leaves while others may still write to it
 }
 
-template <typename Kern>
-cudaError_t allow_smem(Kern* k, size_t bytes, bool& done) {
-  if (done) return cudaSuccess;
-  const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-  done = e == cudaSuccess;
-  return e;
-}
-
 }  // namespace
 
 cudaError_t vcycle32(const float* r, const float* a, const float* dinv, const float* const below[4], float* z,
                      const SolveScalars* sc, const Batch& bt, double omega, cudaStream_t st) {
-  static bool smem_set = false;  // once (capture-friendly)
-  const cudaError_t e = allow_smem(k_vcycle32, sizeof(SmemV<float>), smem_set);
+  static SmemOptIn opt_in;
+  const cudaError_t e = opt_in(k_vcycle32, sizeof(SmemV<float>));
   if (e != cudaSuccess) return e;
   VArgs A{r, a, dinv, below[0], below[1], below[2], below[3], z, sc, bt.act, (float)omega};
   const double bytes = (double)bt.n * 4 * (3.0 * kNodes + 32768 + 4096 + 512 + 64 + 8);
@@ -741,8 +733,8 @@ cudaError_t vcycle32(const float* r, const float* a, const float* dinv, const fl
 
 cudaError_t solve32(SolverBufs& B, const float* a32, const __nv_bfloat16* abf, const float2* rr_in, long long rr_stride,
                     float2* x, const PcgParams& prm, int inner, int inner_next, int fixed_steps, cudaStream_t st) {
-  static bool smem_set = false;
-  const cudaError_t e = allow_smem(k_solve32, sizeof(SmemS), smem_set);
+  static SmemOptIn opt_in;
+  const cudaError_t e = opt_in(k_solve32, sizeof(SmemS));
   if (e != cudaSuccess) return e;
   SArgs A{};
   A.a32 = a32; A.abf = abf; A.dinv = (const float*)B.dinv[0];

@@ -136,11 +136,8 @@ bool coarse_vcycle_applies(int N, int j) { return j >= 1 && (N >> j) == 16; }
 void coarse_vcycle(const float* r16, const float* const a[4], float* z16, const SolveScalars* sc, const Batch& bt,
                    double omega, cudaStream_t st) {
   using M = CoarseSmem<float>;
-  static bool smem_set = false;  // once (capture-friendly)
-  if (!smem_set) {
-    cudaFuncSetAttribute(k_coarse_vcycle<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)M::bytes);
-    smem_set = true;
-  }
+  static SmemOptIn opt_in;
+  (void)opt_in(k_coarse_vcycle<float>, M::bytes);  // a launch without it is refused
   CoarseArgs A{};
   A.r = r16;
   for (int l = 0; l < 4; ++l) A.a[l] = a[l];

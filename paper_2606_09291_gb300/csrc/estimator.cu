@@ -991,11 +991,8 @@ static int launch_lvl(const void* qf, int Nf, const void* qc, int S, int Nc, con
   if (Nf <= 16) {
     const int g = (int)std::min<long long>(S, room);
     const size_t smem = 3 * (size_t)nodes * sizeof(double);
-    static bool smem_set = false;  // once (capture-friendly)
-    if (smem > 48 * 1024 && !smem_set) {
-      cudaFuncSetAttribute(k_lvl_s2_small, cudaFuncAttributeMaxDynamicSharedMemorySize, 3 * 17 * 17 * 17 * 8);
-      smem_set = true;
-    }
+    static SmemOptIn opt_in;
+    if (smem > 48 * 1024) (void)opt_in(k_lvl_s2_small, smem);  // a launch without it is refused
     launch("level_cells", sb, k_lvl_s2_small, dim3((unsigned)g), kBlock, smem, st, x, Nf, S, (const double*)mean, 2.0 * A, B,
            hf3, partial + nf);
     return (int)(nf + g);

@@ -240,11 +240,10 @@ cudaError_t launch_field(const double* xi, int K, const ModeTable& mt, const dou
   if (!out.log_a && !out.a64 && (out.a32 || out.abf) && N % 4 == 0) {
     const size_t smem = 2 * sizeof(float2) * (size_t)((K + 1) & ~1) +
                         sizeof(float) * (2 * (size_t)mt.n1x * N + 2 * (size_t)mt.n1d * N);
-    static size_t smem_df = 48 * 1024;
-    if (smem > smem_df) {
-      cudaError_t e = cudaFuncSetAttribute(k_field_df, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    static SmemOptIn opt_in;
+    if (smem > 48 * 1024) {
+      const cudaError_t e = opt_in(k_field_df, smem);
       if (e != cudaSuccess) return e;
-      smem_df = smem;
     }
     const double cells = (double)S * N * N * N;
     int planes = kFieldPlanes;
@@ -258,12 +257,11 @@ cudaError_t launch_field(const double* xi, int K, const ModeTable& mt, const dou
   // pairs of planes while two blocks fit an SM and the pairs fill the SMs
   const bool two = field_smem_bytes(mt, K, N, 2) <= 110 * 1024 && (long long)S * (N / 2) >= 2 * 152;
   const size_t smem = field_smem_bytes(mt, K, N, two ? 2 : 1);
-  static size_t smem_set[2] = {48 * 1024, 48 * 1024};  // raised once per size (not on every enqueue: capture-friendly)
+  static SmemOptIn opt_in[2];
   auto kern = two ? k_field<2> : k_field<1>;
-  if (smem > smem_set[two]) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (smem > 48 * 1024) {
+    const cudaError_t e = opt_in[two](kern, smem);
     if (e != cudaSuccess) return e;
-    smem_set[two] = smem;
   }
   const double cells = (double)S * N * N * N;
   const double outb = cells * ((out.log_a ? 8 : 0) + (out.a64 ? 8 : 0) + (out.a32 ? 4 : 0) + (out.abf ? 2 : 0));

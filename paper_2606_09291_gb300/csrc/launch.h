@@ -5,12 +5,38 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include <atomic>
+#include <mutex>
 #include <utility>
 
 namespace mlsgd {
 
 void prof_begin(const char* cls, cudaStream_t st);
 void prof_end(const char* cls, cudaStream_t st, double bytes, double flops);
+
+// A kernel's opt-in to more dynamic shared memory than the default: once per device (and
+// again when a call needs more, never to less), from any thread; no call on every enqueue.
+// A refusal is returned and tried again by the next call.
+struct SmemOptIn {
+  static constexpr int kDevices = 64;
+  std::atomic<int> bytes[kDevices];  // static storage: 0
+  std::mutex m;
+  template <typename... KArgs>
+  cudaError_t operator()(void (*kern)(KArgs...), size_t need, bool carveout = false) {
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev < 0 || dev >= kDevices) return cudaErrorInvalidDevice;
+    if (bytes[dev].load(std::memory_order_acquire) >= (int)need) return cudaSuccess;
+    std::lock_guard<std::mutex> lock(m);
+    if (bytes[dev].load(std::memory_order_relaxed) >= (int)need) return cudaSuccess;
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)need);
+    if (e == cudaSuccess && carveout)
+      e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+    if (e == cudaSuccess) bytes[dev].store((int)need, std::memory_order_release);
+    return e;
+  }
+};
 
 // Launches `kern` in clusters of `cluster` consecutive blocks (0: none), as a
 // programmatic dependent of the work before it in the stream: its blocks may start while

@@ -966,13 +966,8 @@ static void run_slab(const char* cls, double bytes, SlabArgs args, const Batch& 
   args.act = bt.act;
   args.scale = (float)(1.0 / (12.0 * N));
   const size_t smem = SlabSmem<N, TA, MODE>::total;
-  static bool smem_set = false;  // once per instantiation (capture-friendly)
-  if (!smem_set) {
-    cudaFuncSetAttribute(k_slab<N, TA, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    cudaFuncSetAttribute(k_slab<N, TA, MODE>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                         cudaSharedmemCarveoutMaxShared);
-    smem_set = true;
-  }
+  static SmemOptIn opt_in;
+  (void)opt_in(k_slab<N, TA, MODE>, smem, true);  // a launch without it is refused
   launch_flops(cls, bytes, ops, k_slab<N, TA, MODE>, dim3(1, t.by, (unsigned)(bt.n * t.nzc)), dim3(256), smem, st,
                args);
 }

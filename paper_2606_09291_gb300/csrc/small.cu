@@ -661,13 +661,9 @@ cudaError_t small_mixed(SolverBufs& B, const float* a32, const __nv_bfloat16* ab
   if (N == 8) {
     launch("small_f32", bytes, k_small8, dim3((unsigned)S), dim3(kT8), 0, st, A);
   } else {
-    static bool smem_set = false;  // once (capture-friendly)
-    if (!smem_set) {
-      const cudaError_t e =
-          cudaFuncSetAttribute(k_small16, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Smem16));
-      if (e != cudaSuccess) return e;
-      smem_set = true;
-    }
+    static SmemOptIn opt_in;
+    const cudaError_t e = opt_in(k_small16, sizeof(Smem16));
+    if (e != cudaSuccess) return e;
     launch("small_f32", bytes, k_small16, dim3((unsigned)S), dim3(kT16), sizeof(Smem16), st, A);
   }
   return cudaGetLastError();

@@ -748,15 +748,20 @@ static_assert(sizeof(SmemV) <= 113 * 1024 && sizeof(With8<16, SmemSolve<16>>) <=
 // share an SM share its FP64 pipe, and the hardware fills an SM before it takes the next
 // (16 clusters of eight blocks went to 64 SMs).  The shared memory that is asked for sets
 // how many blocks an SM takes: the fewest with which every sample's cluster is resident.
-struct Spread {
+struct Spread {  // of one device
   std::mutex m;
   int n = 0;  // 0: not set up (again after a failure)
   size_t smem[8];
   int clusters[8];  // resident with at most i + 1 blocks per SM
 };
 template <typename Args>
-cudaError_t launch_spread(Spread& sp, const char* cls, double bytes, void (*k)(Args), int threads, int cluster,
+cudaError_t launch_spread(Spread (&spreads)[SmemOptIn::kDevices], const char* cls, double bytes, void (*k)(Args), int threads, int cluster,
                           size_t smem, int most, int samples, cudaStream_t st, const Args& A) {
+  int dev = 0;
+  const cudaError_t ed = cudaGetDevice(&dev);
+  if (ed != cudaSuccess) return ed;
+  if (dev < 0 || dev >= SmemOptIn::kDevices) return cudaErrorInvalidDevice;
+  Spread& sp = spreads[dev];
   {
     std::lock_guard<std::mutex> lock(sp.m);
     if (sp.n == 0) {
@@ -802,7 +807,7 @@ cudaError_t launch_spread(Spread& sp, const char* cls, double bytes, void (*k)(A
 
 cudaError_t coarse_vcycle64(const double* r16, const double* const a[4], const double* const wd[3], double* z16,
                             const SolveScalars* sc, const Batch& bt, double omega, cudaStream_t st) {
-  static Spread sp;
+  static Spread sp[SmemOptIn::kDevices];
   CoarseArgs64 A{};
   A.r = r16;
   for (int l = 0; l < 4; ++l) A.a[l] = a[l];
@@ -818,7 +823,7 @@ cudaError_t small_fp64(SolverBufs& B, const double* a64, const double* b, long l
   const int N = B.N, S = B.S;
   SolveArgs64 A{a64, b, bstride, x_out, B.sc, prm.rtol * prm.rtol, prm.omega, prm.max_iter};
   const double bytes = (bstride ? S : 1) * (double)nodes_of(N) * 8 + (double)S * 8 * (nodes_of(N) + cells_of(N));
-  static Spread sp8, sp16;
+  static Spread sp8[SmemOptIn::kDevices], sp16[SmemOptIn::kDevices];
   if (N == 16)
     return launch_spread(sp16, "small_f64", bytes, k_small64<16>, 256, 8, sizeof(With8<16, SmemSolve<16>>), 2, S, st, A);
   return launch_spread(sp8, "small_f64", bytes, k_small64<8>, 128, 4, sizeof(With8<8, SmemSolve<8>>), 5, S, st, A);

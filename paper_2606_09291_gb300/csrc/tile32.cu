@@ -512,12 +512,8 @@ void run(const char* cls, double bytes, Args args, const Batch& bt, cudaStream_t
   args.err = bt.err;
   constexpr size_t smem = sizeof(Smem<TA, MODE>);
   static_assert((sizeof(TA) == 4 && MODE == T_POST) || smem + 1024 <= 228 * 1024 / 3, "three blocks per SM");
-  static bool smem_set = false;  // once per instantiation (capture-friendly)
-  if (!smem_set) {
-    cudaFuncSetAttribute(k_tile32<TA, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    cudaFuncSetAttribute(k_tile32<TA, MODE>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
-    smem_set = true;
-  }
+  static SmemOptIn opt_in;
+  (void)opt_in(k_tile32<TA, MODE>, smem, true);  // a launch without it is refused
   launch(cls, bytes, k_tile32<TA, MODE>, dim3(t.bx, t.by, (unsigned)(bt.n * args.nzc)), dim3(256), smem, st, args);
 }
 

@@ -334,11 +334,8 @@ template <int MODE, int OCC>
 void run_occ(const char* cls, double bytes, const Args& A, dim3 grid, cudaStream_t st) {
   constexpr size_t smem = sizeof(Smem<MODE>);
   static_assert(smem + 1024 <= 228 * 1024 / 3, "three blocks per SM");
-  static bool smem_set = false;  // once per instantiation (capture-friendly)
-  if (!smem_set) {
-    cudaFuncSetAttribute(k_tile64<MODE, OCC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    smem_set = true;
-  }
+  static SmemOptIn opt_in;
+  (void)opt_in(k_tile64<MODE, OCC>, smem);  // a launch without it is refused
   launch_after(cls, bytes, k_tile64<MODE, OCC>, grid, dim3(kT), smem, st, A);
 }
 template <int MODE>

@@ -464,11 +464,8 @@ void tiled_res64(const float2* b, long long bstride, const float2* x, const floa
 int tiled_phi_df(const float2* y, int N, int S, const float2* gtab, const float2* mgtab, float2* badj,
                  double* partial, cudaStream_t st) {
   const TiledShape t = tiled_shape(N, S, kPhiRows);
-  static bool smem_set = false;  // once (capture-friendly)
-  if (!smem_set) {
-    cudaFuncSetAttribute(k_phi_tiled_df, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPhiSmem);
-    smem_set = true;
-  }
+  static SmemOptIn opt_in;
+  (void)opt_in(k_phi_tiled_df, kPhiSmem);  // a launch without it is refused
   launch("phi_adjrhs", (double)S * nodes_of(N) * 16, k_phi_tiled_df, dim3(t.bx, t.by, (unsigned)(S * t.nzc)),
          dim3(TX, TY), kPhiSmem, st, y, N, gtab, mgtab, badj, partial, t.nzc, t.zc, t.nseg);
   return t.blocks_per_sample;
