@@ -35,9 +35,11 @@ template <typename T> __device__ __forceinline__ T smem_coef(__nv_bfloat16 v) { 
 // First statement of every kernel: waits until the kernels before it in the stream have
 // completed and their writes are visible (nothing is read or written before), then lets
 // the next kernel's blocks be launched as soon as all of this kernel's have started, so
-// that their launch latency is hidden (launch.h sets the attribute).
+// that their launch latency is hidden (launch.h sets the attribute).  A kernel that does
+// not let the next one in early begins with the wait alone.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
 __device__ __forceinline__ void pdl_entry() {
-  asm volatile("griddepcontrol.wait;\n" ::: "memory");
+  pdl_wait();
   asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
 }
 

@@ -40,7 +40,7 @@ struct SmemOptIn {
 
 // Launches `kern` in clusters of `cluster` consecutive blocks (0: none), as a
 // programmatic dependent of the work before it in the stream: its blocks may start while
-// the kernel before drains (every kernel begins with pdl_entry, which waits for it).
+// the kernel before drains (every kernel begins with pdl_entry or pdl_wait, which wait for it).
 // !early: not before that kernel has ended (a kernel whose time is that of the fullest SM
 // wants its blocks spread over idle SMs, not placed where the kernel before leaves room).
 template <typename... KArgs, typename... Args>

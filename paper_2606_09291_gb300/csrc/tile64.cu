@@ -76,7 +76,9 @@ struct Args {
 template <int MODE, int OCC>
 __global__ void __launch_bounds__(kT, OCC) k_tile64(Args A) {
   // launched after the kernel before has ended and without letting the next one's blocks in:
-  // placed early, blocks share SMs unevenly (FP64 level 3 of a run: 22.7 ms, 20.7 without)
+  // placed early, blocks share SMs unevenly (FP64 level 3 of a run: 22.7 ms, 20.7 without); the
+  // wait holds whatever the launch
+  pdl_wait();
   extern __shared__ __align__(16) unsigned char smraw[];
   Smem<MODE>& M = *reinterpret_cast<Smem<MODE>*>(smraw);
   const int tid = threadIdx.x, tx = tid & 31, ty = tid >> 5;
