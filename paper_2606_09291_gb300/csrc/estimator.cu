@@ -759,9 +759,14 @@ __global__ void __launch_bounds__(kBlock, 4) k_level_pairs(const float2* __restr
 // axis) to the deviations from the mean, where the 8 x 8 matrix per level cell took 64 per
 // cell.  Values given as FP32 pairs enter FP64 by integer instructions (f2d) and one addition.
 __device__ __forceinline__ double ldq(const double* p, long long i) { return p[i]; }
+__device__ __forceinline__ double f2d_all(float f) {  // f2d, subnormals too: scaled into its range
+  const bool small = fabsf(f) < 0x1p-126f;
+  const double d = f2d(small ? f * 0x1p64f : f);
+  return small && f != 0.f ? __hiloint2double(__double2hiint(d) - (64 << 20), __double2loint(d)) : d;
+}
 __device__ __forceinline__ double ldq(const float2* p, long long i) {
   const float2 v = p[i];
-  return f2d(v.x) + f2d(v.y);
+  return f2d_all(v.x) + f2d_all(v.y);
 }
 // x_s at every node of the level grid, written over q_f (same 8-byte slots; q_f is
 // not needed after the statistics)
