@@ -59,8 +59,8 @@ __global__ void k_rhs_state(const double* __restrict__ z, int Nc, int N, double*
 // k_rhs_xy: one block per (level cell row ey, control plane z0 + cz) contracts y, then x,
 // into u[cz][ey][side][i]; k_rhs_z contracts z, slab after slab of the control planes that u
 // has room for (the order of the sums does not depend on the slabs).  A 256^3 control onto
-// 8^3: 615 us by node rows, 116 us by axis; a whole FP64 state and adjoint solve of one 8^3
-// sample under it 862 and 358 us.
+// 8^3: 615 us by node rows, about 105 us by axis; a whole FP64 state and adjoint solve of one
+// 8^3 sample under it 862 and 343 us.
 __global__ void __launch_bounds__(kBlock) k_rhs_xy(const double* __restrict__ z, int Nc, int N, int z0,
                                                    double* __restrict__ u) {
   pdl_entry();
@@ -98,8 +98,11 @@ __global__ void __launch_bounds__(kBlock) k_rhs_xy(const double* __restrict__ z,
 }
 // node (i, j, k): the right side of cell row j - 1 and the left side of row j, over those of
 // its 2r control planes that are among z0 .. z0 + planes - 1; b holds the sum so far between
-// two slabs
-__global__ void __launch_bounds__(kBlock) k_rhs_z(const double* __restrict__ u, int Nc, int N, int z0, int planes,
+// two slabs.  One warp per block: a warp alone issues an FP64 operation in 64 clocks and eight
+// of an SM share its pipe, so the few nodes of a coarse grid are spread over SMs (8^3 under
+// 256^3: 15 us less than with 256 threads a block).
+constexpr int kRhsZBlock = 32;
+__global__ void __launch_bounds__(kRhsZBlock) k_rhs_z(const double* __restrict__ u, int Nc, int N, int z0, int planes,
                                                   double* __restrict__ b) {
   pdl_entry();
   const int n1 = N + 1, r = Nc / N;
@@ -236,8 +239,8 @@ void launch_rhs_state(const double* z, int Nc, int N, double* b, void* scratch, 
       const double ub = (double)n * plane;
       launch("rhs", (double)n * Nc * Nc * 8 + ub, k_rhs_xy, dim3((unsigned)N, (unsigned)n), kBlock,
              (size_t)(Nc / N + 2 * Nc) * sizeof(double), st, z, Nc, N, z0, u);
-      launch("rhs", ub + (double)nodes_of(N) * 8, k_rhs_z, dim3(node_blocks(N)), kBlock, 0, st, (const double*)u, Nc, N,
-             z0, n, b);
+      launch("rhs", ub + (double)nodes_of(N) * 8, k_rhs_z, dim3((unsigned)((nodes_of(N) + kRhsZBlock - 1) / kRhsZBlock)),
+             kRhsZBlock, 0, st, (const double*)u, Nc, N, z0, n, b);
     }
   } else {
     const size_t smem = (size_t)(2 * (Nc / N) + Nc) * sizeof(double);
