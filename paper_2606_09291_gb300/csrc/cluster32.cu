@@ -14,7 +14,7 @@
 // memory (L2); their halo planes are updated along with the own ones.
 //
 // What bounds it: the latency of barriers and shared memory; a block of 1024 threads has
-// one SM to itself.  It wins while the clusters make few waves (see cluster32_applies).
+// one SM to itself.  It wins while the clusters make few waves (kCluster32Max in solver.cu).
 //
 // Arithmetic: that of the slab passes (slab.cu), the fused coarse V-cycle (coarse.cu) and
 // the refinement step on the same level, operation by operation, with the order of their

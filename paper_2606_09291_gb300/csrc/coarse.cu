@@ -18,9 +18,6 @@
 // divides by D as the level-by-level kernels do, and pre- and post-smoothing take
 // the same D, so the preconditioner stays symmetric.  Boundary nodes hold 0 in every
 // array.  The operator rows are those of the assembled Q1 stiffness (q1_row).
-#include <cstdio>
-#include <type_traits>
-
 #include "internal.cuh"
 #include "kernels.h"
 #include "launch.h"
@@ -32,8 +29,7 @@ namespace {
 
 constexpr int kCT = 768;  // threads per block (24 warps: two blocks per SM hide the shared-memory latency)
 
-// shared-memory layout (elements of T)
-template <typename T>
+// shared-memory layout (floats)
 struct CoarseSmem {
   using L16 = Lv<16>;
   using L8 = Lv<8>;
@@ -45,88 +41,86 @@ struct CoarseSmem {
   static constexpr int r4 = a8 + L8::cells, x4 = r4 + L4::nodes, t4 = x4 + L4::nodes, a4 = t4 + L4::nodes;
   static constexpr int r2 = a4 + L4::cells, x2 = r2 + L2::nodes, a2 = x2 + L2::nodes;
   static constexpr int total = a2 + L2::cells;
-  static constexpr size_t bytes = sizeof(T) * (size_t)total;
+  static constexpr size_t bytes = sizeof(float) * (size_t)total;
 };
 
-// asynchronous element copy into shared memory (4 or 8 bytes; the thread waits for its
-// own copies, a block barrier then publishes them)
-template <typename T>
-__device__ __forceinline__ void cp_async_elem(T* dst, const T* src) {
+// asynchronous element copy into shared memory (the thread waits for its own copies, a block
+// barrier then publishes them)
+__device__ __forceinline__ void cp_async_elem(float* dst, const float* src) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], %2;\n" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src),
-               "n"(sizeof(T))
+               "n"(sizeof(float))
                : "memory");
 }
 
 struct CoarseArgs {
-  const void* r;      // restricted residual on the 16^3 level, [S][17^3]
-  const void* a[4];   // cell coefficient of the levels 16^3, 8^3, 4^3, 2^3, [S][cells]
-  void* z;            // the V-cycle's correction on the 16^3 level, [S][17^3]
+  const float* r;     // restricted residual on the 16^3 level, [S][17^3]
+  const float* a[4];  // cell coefficient of the levels 16^3, 8^3, 4^3, 2^3, [S][cells]
+  float* z;           // the V-cycle's correction on the 16^3 level, [S][17^3]
   const SolveScalars* sc;
   const int* act;
-  double omega;
+  float omega;
 };
 
-template <typename T>
 __global__ void __launch_bounds__(kCT, 2) k_coarse_vcycle(CoarseArgs A) {
   pdl_entry();
-  using M = CoarseSmem<T>;
+  using M = CoarseSmem;
   const int s = A.act != nullptr ? A.act[blockIdx.x] : (int)blockIdx.x;
   if (A.sc != nullptr && !A.sc[s].active) return;
   extern __shared__ __align__(16) unsigned char smraw[];
-  T* sm = (T*)smraw;
-  const T omega = (T)A.omega;
+  float* sm = reinterpret_cast<float*>(smraw);
+  const float omega = A.omega;
   // r and the four coefficient levels, all copies in flight at once
-  const T* rg = (const T*)A.r + (long long)s * Lv<16>::nodes;
+  const float* rg = A.r + (long long)s * Lv<16>::nodes;
   for (int n = threadIdx.x; n < Lv<16>::nodes; n += kCT) cp_async_elem(sm + M::r16 + n, rg + n);
   const int aoff[4] = {M::a16, M::a8, M::a4, M::a2};
   const int acnt[4] = {Lv<16>::cells, Lv<8>::cells, Lv<4>::cells, Lv<2>::cells};
 #pragma unroll
   for (int l = 0; l < 4; ++l) {
-    const T* ag = (const T*)A.a[l] + (long long)s * acnt[l];
+    const float* ag = A.a[l] + (long long)s * acnt[l];
     for (int n = threadIdx.x; n < acnt[l]; n += kCT) cp_async_elem(sm + aoff[l] + n, ag + n);
   }
   asm volatile("cp.async.commit_group;\n" ::: "memory");
   asm volatile("cp.async.wait_all;\n" ::: "memory");
   __syncthreads();
-  dinv_level<kCT, T>(sm + M::a16, sm + M::d16);
+  dinv_level<kCT, float>(sm + M::a16, sm + M::d16);
   __syncthreads();
   // down: 16^3, 8^3, 4^3
-  pre_level<kCT, 16, true, T>(sm + M::r16, sm + M::a16, sm + M::d16, sm + M::x16, sm + M::t16, omega);
+  pre_level<kCT, 16, true, float>(sm + M::r16, sm + M::a16, sm + M::d16, sm + M::x16, sm + M::t16, omega);
   __syncthreads();
-  restrict_level<kCT, 8, T>(sm + M::t16, sm + M::r8);
+  restrict_level<kCT, 8, float>(sm + M::t16, sm + M::r8);
   __syncthreads();
-  pre_level<kCT, 8, false, T>(sm + M::r8, sm + M::a8, nullptr, sm + M::x8, sm + M::t8, omega);
+  pre_level<kCT, 8, false, float>(sm + M::r8, sm + M::a8, nullptr, sm + M::x8, sm + M::t8, omega);
   __syncthreads();
-  restrict_level<kCT, 4, T>(sm + M::t8, sm + M::r4);
+  restrict_level<kCT, 4, float>(sm + M::t8, sm + M::r4);
   __syncthreads();
-  pre_level<kCT, 4, false, T>(sm + M::r4, sm + M::a4, nullptr, sm + M::x4, sm + M::t4, omega);
+  pre_level<kCT, 4, false, float>(sm + M::r4, sm + M::a4, nullptr, sm + M::x4, sm + M::t4, omega);
   __syncthreads();
-  restrict_level<kCT, 2, T>(sm + M::t4, sm + M::r2);
+  restrict_level<kCT, 2, float>(sm + M::t4, sm + M::r2);
   __syncthreads();
   // 2^3: the single interior unknown (node 13), x = r / D
   for (int n = threadIdx.x; n < Lv<2>::nodes; n += kCT) {
-    T v = T(0);
+    float v = 0.f;
     if (n == 13) {
-      Cells8<T, T> C;
+      Cells8<float, float> C;
       cells8(C, sm + M::a2, 1, 1, 1, 2);
-      v = sm[M::r2 + 13] / (T(1.0 / 6.0) * C.sum);
+      v = sm[M::r2 + 13] / (float(1.0 / 6.0) * C.sum);
     }
     sm[M::x2 + n] = v;
   }
   __syncthreads();
   // up: 4^3, 8^3 (the smoothed corrections overwrite the dead residuals t), then 16^3
-  prolong_level<kCT, 4, T>(sm + M::x4, sm + M::x2);
+  prolong_level<kCT, 4, float>(sm + M::x4, sm + M::x2);
   __syncthreads();
-  post_level<kCT, 4, false, T>(sm + M::r4, sm + M::a4, nullptr, sm + M::x4, sm + M::t4, omega);
+  post_level<kCT, 4, false, float>(sm + M::r4, sm + M::a4, nullptr, sm + M::x4, sm + M::t4, omega);
   __syncthreads();
-  prolong_level<kCT, 8, T>(sm + M::x8, sm + M::t4);
+  prolong_level<kCT, 8, float>(sm + M::x8, sm + M::t4);
   __syncthreads();
-  post_level<kCT, 8, false, T>(sm + M::r8, sm + M::a8, nullptr, sm + M::x8, sm + M::t8, omega);
+  post_level<kCT, 8, false, float>(sm + M::r8, sm + M::a8, nullptr, sm + M::x8, sm + M::t8, omega);
   __syncthreads();
-  prolong_level<kCT, 16, T>(sm + M::x16, sm + M::t8);
+  prolong_level<kCT, 16, float>(sm + M::x16, sm + M::t8);
   __syncthreads();
-  post_level<kCT, 16, true, T>(sm + M::r16, sm + M::a16, sm + M::d16, sm + M::x16,
-                          (T*)A.z + (long long)s * Lv<16>::nodes, omega);
+  post_level<kCT, 16, true, float>(sm + M::r16, sm + M::a16, sm + M::d16, sm + M::x16,
+                          A.z + (long long)s * Lv<16>::nodes, omega);
 }
 
 }  // namespace
@@ -135,20 +129,20 @@ bool coarse_vcycle_applies(int N, int j) { return j >= 1 && (N >> j) == 16; }
 
 void coarse_vcycle(const float* r16, const float* const a[4], float* z16, const SolveScalars* sc, const Batch& bt,
                    double omega, cudaStream_t st) {
-  using M = CoarseSmem<float>;
+  using M = CoarseSmem;
   static SmemOptIn opt_in;
-  (void)opt_in(k_coarse_vcycle<float>, M::bytes);  // a launch without it is refused
+  (void)opt_in(k_coarse_vcycle, M::bytes);  // a launch without it is refused
   CoarseArgs A{};
   A.r = r16;
   for (int l = 0; l < 4; ++l) A.a[l] = a[l];
   A.z = z16;
   A.sc = sc;
   A.act = bt.act;
-  A.omega = omega;
+  A.omega = (float)omega;
   // per sample: r and z on 17^3 nodes, the four coefficient levels
   const double bytes = (double)bt.n * sizeof(float) *
                        (2.0 * Lv<16>::nodes + Lv<16>::cells + Lv<8>::cells + Lv<4>::cells + Lv<2>::cells);
-  launch("coarse_f32", bytes, k_coarse_vcycle<float>, dim3((unsigned)bt.n), dim3(kCT), M::bytes, st, A);
+  launch("coarse_f32", bytes, k_coarse_vcycle, dim3((unsigned)bt.n), dim3(kCT), M::bytes, st, A);
 }
 
 }  // namespace mlsgd

@@ -29,7 +29,6 @@ __device__ __forceinline__ void cells8(Cells8<T, T>& C, const T* a, int i, int j
       }
 }
 
-__device__ __forceinline__ double rcp(double x) { return 1.0 / x; }
 __device__ __forceinline__ float rcp(float x) { return __fdividef(1.0f, x); }
 
 // D^-1 of the 16^3 level at every node (0 on the boundary)

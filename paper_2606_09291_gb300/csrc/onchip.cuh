@@ -24,7 +24,6 @@ struct CoarseLevels {
   float *g4, *s4;                   // with MATRIX: the matrix [27 x 27], u and omega/D [2 x 27]
 };
 constexpr int kCoarse8Floats = 3 * 729 + 512 + 2 * 125 + 64 + 8;
-constexpr int kCoarse8Own = 2 * 729 + 2 * 125 + 64 + 8;  // without r8 and a8
 
 template <int N>
 __device__ __forceinline__ float diag_of(const float* a, int i, int j, int k) {  // D = (h/3) sum_8 a

@@ -12,9 +12,9 @@
 // iteration) and, on 16^3, the shared-memory loads of three 21-point stencils; FP64 in one
 // warp (64 clocks an operation) is kept out of the inner iterations.
 // Measured (three refinement steps of six iterations, state or adjoint): 1024 samples of
-// 8^3 180 us a solve (310 with a thread per node instead of per interior node) against 2.2 ms
-// in passes, 256 of 16^3 320 us against 3.1 ms, 64 of
-// 16^3 200 us against 1.6 ms.
+// 8^3 180 us a solve (310 with a thread per node instead of per interior node; at about 300
+// samples, where both are one wave, 117 against 115) against 2.2 ms in passes, 256 of 16^3
+// 320 us against 3.1 ms, 64 of 16^3 200 us against 1.6 ms.
 //
 // Arithmetic: that of the pass-by-pass solver on the same grid (solver.cu for 8^3: FP64
 // refinement residual and solution; tiled.cu for 16^3: solution and b as FP32 pairs, partial

@@ -565,11 +565,11 @@ __global__ void k_accumulate(double* __restrict__ x, const float* __restrict__ d
 static inline dim3 grid_nodes(int N, int S) { return dim3((unsigned)node_blocks(N), (unsigned)S); }
 
 // f(std::integral_constant<int, N>) for the grids of the hierarchies (N a power of two,
-// 16 .. 256), f(std::integral_constant<int, 0>) (N at run time) otherwise
-template <typename F>
+// LEAST .. 256), f(std::integral_constant<int, 0>) (N at run time) otherwise
+template <int LEAST, typename F>
 static void with_grid(int N, F&& f) {
   switch (N) {
-    case 16: f(std::integral_constant<int, 16>()); break;
+    case 16: f(std::integral_constant<int, LEAST <= 16 ? 16 : 0>()); break;
     case 32: f(std::integral_constant<int, 32>()); break;
     case 64: f(std::integral_constant<int, 64>()); break;
     case 128: f(std::integral_constant<int, 128>()); break;
@@ -822,7 +822,7 @@ static int vcycle(SolverBufs& B, const T* r0, const TA0* a0, const SolveScalars*
              st, rin(j), (const T*)B.vx[j], aj, (T*)B.vt[j], sc, Nj, omega, act);
     }
     if (restricted) continue;
-    with_grid(Nj / 2, [&](auto c) {
+    with_grid<16>(Nj / 2, [&](auto c) {
       constexpr int NCC = decltype(c)::value;
       const double rb = nbytes<T, T>(Nj, n, 1, 0) + nbytes<T, T>(Nj / 2, n, 1, 0);
       if constexpr (NCC >= 32) {  // on smaller grids the per-node kernel has more threads in flight
@@ -1046,7 +1046,7 @@ static cudaError_t pcg_inner_fused(SolverBufs& B, const float* a32, const __nv_b
         *p_last = pnew;
         break;
       }
-      with_grid(N, [&](auto c) {
+      with_grid<32>(N, [&](auto c) {
         launch("finish_step", (double)n * nodes * ((iters > 1 ? 4 : 0) + 4 + (assign_out ? 8 : 16)),
                k_finish_step<decltype(c)::value>, grid_nodes(N, n), kBlock, 0, st, x_out, (const float*)x,
                (const float*)pnew, (const SolveScalars*)sc, sco, nodes, N, assign_out ? 1 : 0, iters > 1 ? 0 : 1,
@@ -1167,7 +1167,7 @@ cudaError_t ir_mixed(SolverBufs& B, const float* a32, const __nv_bfloat16* abf, 
   int last_inner = inner_iters;  // inner iterations of the step the next refinement pass completes
   if (tiled) {
     const dim3 gi((unsigned)init_blocks(N), (unsigned)S);
-    with_grid(N, [&](auto c) {
+    with_grid<32>(N, [&](auto c) {
       constexpr int NN = decltype(c)::value;
       if (b_pair) {
         launch("init_f32", bb + nbytes<float, float>(N, S, 1, 0), k_init32<true, NN>, gi, kBlock, 0, st, b, b_pair,

@@ -31,8 +31,8 @@
 // Partial sums are formed per (tile, segment of kSeg planes) whatever the chunk, so the
 // iterates do not depend on the batch or the chunking.
 // Measured: FP64 level 3 of an optimisation run (9 samples of 64^3 with 32^3 partners, 24
-// iterations) 28.6 ms with the node-by-node passes, 20.2 ms now; state and adjoint of one
-// 128^3 sample at rtol 1e-10 17.3 ms.
+// iterations) 28.6 ms with the node-by-node passes, 20.2 ms when they were replaced (18.6 with
+// what followed elsewhere); state and adjoint of one 128^3 sample at rtol 1e-10 15.2 ms.
 #include "internal.cuh"
 #include "kernels.h"
 #include "launch.h"
