@@ -13,8 +13,9 @@
 // vectors a thread reads only at its own nodes (r, p, the correction) stay in global
 // memory (L2); their halo planes are updated along with the own ones.
 //
-// What bounds it: the latency of barriers and shared memory; a block of 1024 threads has
-// one SM to itself.  It wins while the clusters make few waves (kCluster32Max in solver.cu).
+// What bounds it (ncu, 16 samples): the latency of barriers and of the vectors in L2 (6.4 and
+// 5.6 of 24 cycles per instruction of a warp); a block of 1024 threads has one SM to
+// itself and issues in 33% of its cycles.  It wins while the clusters make few waves (kCluster32Max in solver.cu).
 //
 // Arithmetic: that of the slab passes (slab.cu), the fused coarse V-cycle (coarse.cu) and
 // the refinement step on the same level, operation by operation, with the order of their

@@ -8,9 +8,11 @@
 // block (8^3: 27 KB; 16^3: 108 KB), so here a block keeps its sample's coefficient
 // levels, operand and residuals on the SM and runs the refinement loop to the end:
 // coarse coefficients, FP32 inner PCG with its V(1,1)-cycle, FP64-accurate residual,
-// stop test.  What bounds it is the latency between block barriers (about 14 per inner
-// iteration) and, on 16^3, the shared-memory loads of three 21-point stencils; FP64 in one
-// warp (64 clocks an operation) is kept out of the inner iterations.
+// stop test.  What bounds it (ncu, 1024 samples of 8^3 and 64 of 16^3): latency, of shared
+// memory and of about 14 block barriers per inner iteration (8 and 5 of 21 cycles per
+// instruction of a warp on 8^3, 3 and 4 of 15 on 16^3); issue is 45 and 53% busy.  FP64 in one
+// warp (64 clocks an operation) is kept out of the inner iterations; the FP64 refinement
+// residuals of 8^3 take 45% of that pipe.
 // Measured (three refinement steps of six iterations, state or adjoint): 1024 samples of
 // 8^3 180 us a solve (310 with a thread per node instead of per interior node; at about 300
 // samples, where both are one wave, 117 against 115) against 2.2 ms in passes, 256 of 16^3
